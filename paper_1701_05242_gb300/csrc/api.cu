@@ -262,14 +262,16 @@ extern "C" int dcm_grid_dims(const dcm_params* p, int64_t* cells3, int64_t* boxe
 
 struct ScratchPlan {
   int64_t n_max, ncell, nbox, scan_cap, red_cap, rsize, flags, nblk;
+  int64_t tile_cap;  // pair tiles (0: not served)
+  int64_t red_slots() const { return red_cap > tile_cap ? red_cap : tile_cap; }
   double skin;
   int32_t min_component, segmentation, ms_outer;
   int64_t total() const {
     return 4 * 4 + 16 + 3 * 4 * n_max + 4 * (ncell + 1) + 4 * ncell + 8 * (scan_cap + 1) + 3 * 4 * nbox + 2 * nbox +
-           2 * rsize * nbox + 4 * flags + 4 * (int64_t)kHistCap + 4 * 8 + 8 * 3 * red_cap + 8 * 8 + 8 * 8 * 256 +
+           2 * rsize * nbox + 4 * flags + 4 * (int64_t)kHistCap + 4 * 8 + 8 * 3 * red_slots() + 8 * 8 + 8 * 8 * 256 +
            8 * 32 * red_cap + 8 * 48 + (skin > 0 ? 8 * n_max + 8 * (n_max / 32 + 16) + 4 * rsize * n_max + 32 : 0) +
            (min_component > 0 ? 9 * nbox + 4 * 80 : 0) + 13 * nbox + 4 * (flags + 2) + 4 * nblk +
-           4 * tile_scratch_ints(n_max) +
+           4 * tile_scratch_ints(n_max) + (tile_cap > 0 ? 4 * tile_ints(tile_cap) : 0) +
            (segmentation ? 6 * rsize * nbox + 32 * ms_outer + 16 + 4 * (ms_outer + 2) : 0);
   }
 };
@@ -293,6 +295,8 @@ static ScratchPlan plan_of(const dcm_params* p) {
   s.min_component = p->min_component;
   s.segmentation = p->segmentation;
   s.ms_outer = p->ms_outer;
+  const TilePlan tp = tile_plan(*p, nc, s.n_max);
+  s.tile_cap = tp.usable ? tp.slots : 0;
   s.nblk = adjoint_blocks(p, 0) * adjoint_blocks(p, 1) * adjoint_blocks(p, 2);
   return s;
 }
@@ -317,7 +321,7 @@ extern "C" void dcm_destroy(dcm_ctx* ctx) {
                  ctx->D[1], ctx->flags, ctx->hist, ctx->thr, ctx->red, ctx->totals, ctx->D[0], ctx->red_tmp, ctx->adj_part, ctx->adj_pairs,
                  ctx->nnb, ctx->nimg, ctx->capw, ctx->offw, ctx->list, ctx->xbuild, ctx->dmax, ctx->lflag,
                  ctx->cc_lab, ctx->cc_cnt, ctx->cc_flags, ctx->cc_s0, ctx->dq[0], ctx->dq[1], ctx->dqlen,
-                 ctx->dstamp, ctx->dfixed, ctx->blk_max, ctx->tile_scratch, ctx->ms_u, ctx->ms_ub, ctx->ms_p, ctx->ms_w,
+                 ctx->dstamp, ctx->dfixed, ctx->blk_max, ctx->tile_scratch, ctx->tiles, ctx->ms_u, ctx->ms_ub, ctx->ms_p, ctx->ms_w,
                  ctx->ms_sums, ctx->ms_c, ctx->ms_flags};
   for (void* q : dev)
     if (q) cudaFree(q);
@@ -376,7 +380,7 @@ extern "C" int dcm_create(const dcm_params* p, dcm_ctx** out) {
   alloc((void**)&ctx->flags, 4 * s.flags);
   alloc((void**)&ctx->hist, 4 * (int64_t)kHistCap);
   alloc((void**)&ctx->thr, 4 * 8);
-  alloc((void**)&ctx->red, 8 * 3 * s.red_cap);
+  alloc((void**)&ctx->red, 8 * 3 * s.red_slots());
   alloc((void**)&ctx->totals, 8 * 8);
   alloc((void**)&ctx->red_tmp, 8 * 8 * 256);
   alloc((void**)&ctx->adj_part, 8 * 32 * s.red_cap);
@@ -414,6 +418,10 @@ extern "C" int dcm_create(const dcm_params* p, dcm_ctx** out) {
   ctx->nblk = s.nblk;
   alloc((void**)&ctx->blk_max, 4 * s.nblk);
   alloc((void**)&ctx->tile_scratch, 4 * tile_scratch_ints(s.n_max));
+  if (s.tile_cap > 0) {
+    alloc((void**)&ctx->tiles, 4 * tile_ints(s.tile_cap));
+    ctx->tile_cap = s.tile_cap;
+  }
   if (ok && cudaMallocHost((void**)&ctx->host_status, 16) != cudaSuccess) ok = false;
   if (!ok) {
     cudaGetLastError();

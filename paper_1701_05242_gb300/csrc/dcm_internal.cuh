@@ -117,6 +117,8 @@ struct dcm_ctx {
   int64_t red_cap;          // number of partial slots in red (per quantity)
   int32_t* blk_max;         // nblk: largest cutoff (float bits) per adjoint block
   int32_t* tile_scratch;    // tile_scratch_ints(n_max): launch order of the force and adjoint tiles
+  int32_t* tiles;           // tile_ints(tile_cap): counters, slots in use, slots left to the row walk, particles of the slots
+  int64_t tile_cap;         // pair tile slots (0: tiles not served)
   int nblk3[3];             // adjoint blocks per dimension (edge >= 1.001 rc_max)
   int64_t nblk;
   int64_t scan_cap;
@@ -244,6 +246,31 @@ template <typename R>
 int lj_forces(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, const R* rc,
               const int32_t* cell_start, typename RT<R>::R4* force, double* totals, cudaStream_t st,
               bool energies = true);
+
+// forces_tiles.cu
+// Geometry of the pair tiles (pair_tiles.cuh), fixed per context.
+struct TileCfg {
+  int ry, rz;      // cell rows of a bundle along y and z
+  int nby, nbz;    // bundles along y and z
+  int cap;         // longest tile, in cells along x
+  int cmax;        // spare tile slots per bundle (tiles that are not full)
+  float scale;     // power of two that takes rc_max into [4, 8)
+};
+struct TilePlan {
+  TileCfg cfg;
+  int64_t slots;   // tile slots, and partial sums per quantity, for n particles
+  bool usable;
+};
+TilePlan tile_plan(const dcm_params& p, const int64_t* nc, int64_t n);
+constexpr int64_t tile_ints(int64_t slots) { return 4 + 34 * slots; }
+bool tiles_serve(const dcm_ctx* ctx, int64_t n);  // whether lj_forces runs over tiles
+template <typename R>
+struct ForceArgs;
+// Forces (and with part, 3 quantities of tile_plan(...).slots partials) over tiles.
+template <typename R>
+int tile_forces(dcm_ctx* ctx, bool typed, bool ew, int64_t n, const typename RT<R>::R4* pos, const R* rc,
+                const int32_t* cell_start, const ForceArgs<R>& a, typename RT<R>::R4* force, double* part,
+                cudaStream_t st);
 
 // adjoint.cu
 template <typename R>

@@ -189,6 +189,18 @@ int lj_forces(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, const R* r
   a.rc_max = (R)ctx->p.rc_max;
   const bool typed = lj_general(t);
   const int kind = resolve_force_kernel(ctx);
+  // AUTO runs over tiles where they serve: the default accumulation (the
+  // packed pair loop, its sums carried by the same Kahan compensation), or FP64
+  if (ctx->p.force_kernel == DCM_FORCE_AUTO && tiles_serve(ctx, n) &&
+      (sizeof(R) == 8 || (kind == DCM_FORCE_PACKED && resolve_accumulation(ctx) == DCM_ACC_PLANE_KAHAN))) {
+    double* part = totals ? ctx->red : nullptr;
+    stage_begin(ctx, DCM_STAGE_FORCES, st);
+    int r = tile_forces<R>(ctx, typed, energies || totals, n, pos, rc, cell_start, a, force, part, st);
+    stage_end(ctx, DCM_STAGE_FORCES, st);
+    if (r) return r;
+    if (totals) return reduce_partials(ctx, part, tile_plan(ctx->p, ctx->nc, n).slots, 3, totals, false, st);
+    return DCM_OK;
+  }
   const int block = kind == DCM_FORCE_PACKED ? kX2Block : kForceBlock;
   const int64_t nwarp = (n + block - 1) / block * (block / 32);
   if (totals && nwarp > ctx->red_cap)

@@ -88,6 +88,41 @@ struct Acc {
   int np = 0;
 };
 
+// One pair of the scalar loop: r_ij = (dx, dy, dz), pjw the partner's type.
+template <typename R, bool TYPED>
+__device__ __forceinline__ void pair_one(R dx, R dy, R dz, R pjw, R rc2, int ti, const ForceArgs<R>& a,
+                                         const R* ushift, Acc<R>& c) {
+  R r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+  bool acc = r2 < rc2;
+  R inv = recip(r2);
+  inv = acc ? inv : (R)0;
+  if (TYPED) {
+    int tj = type_of(pjw, a.ntypes);
+    int tp = ti * a.ntypes + tj;
+    R s2 = a.sig2[tp] * inv;
+    R s6 = s2 * s2 * s2;
+    R pv = a.eps24[tp] * s6 * fma((R)2, s6, (R)-1);  // r . F_ij
+    R fs = pv * inv;
+    c.fx = fma(fs, dx, c.fx);
+    c.fy = fma(fs, dy, c.fy);
+    c.fz = fma(fs, dz, c.fz);
+    R us = tj == 0 ? ushift[0] : (tj == 1 ? ushift[1] : (tj == 2 ? ushift[2] : ushift[3]));
+    R u = a.eps4[tp] * s6 * (s6 - (R)1);
+    c.en += acc ? u - us : (R)0;
+    c.vir += pv;
+  } else {
+    R s6 = inv * inv * inv;
+    R pv = s6 * fma((R)2, s6, (R)-1);  // r . F_ij / 24
+    R q = pv * inv;                    // |F_ij| / (24 r)
+    c.fx = fma(q, dx, c.fx);
+    c.fy = fma(q, dy, c.fy);
+    c.fz = fma(q, dz, c.fz);
+    c.en += fma(s6, s6, -s6);          // U / 4
+    c.vir += pv;
+  }
+  c.np += acc ? 1 : 0;
+}
+
 // Pairs of particle i (coordinates xi, yi, zi in the image frame of the
 // segment) with sorted particles [lo, hi).  SJ: the segment's j coordinates
 // need the exact -L image shift (sh); otherwise they are used as loaded.
@@ -108,35 +143,7 @@ __device__ __forceinline__ void pair_range(const typename RT<R>::R4* __restrict_
       dy = yi - pj.y;
       dz = zi - pj.z;
     }
-    R r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-    bool acc = r2 < rc2;
-    R inv = recip(r2);
-    inv = acc ? inv : (R)0;
-    if (TYPED) {
-      int tj = type_of(pj.w, a.ntypes);
-      int tp = ti * a.ntypes + tj;
-      R s2 = a.sig2[tp] * inv;
-      R s6 = s2 * s2 * s2;
-      R pv = a.eps24[tp] * s6 * fma((R)2, s6, (R)-1);  // r . F_ij
-      R fs = pv * inv;
-      c.fx = fma(fs, dx, c.fx);
-      c.fy = fma(fs, dy, c.fy);
-      c.fz = fma(fs, dz, c.fz);
-      R us = tj == 0 ? ushift[0] : (tj == 1 ? ushift[1] : (tj == 2 ? ushift[2] : ushift[3]));
-      R u = a.eps4[tp] * s6 * (s6 - (R)1);
-      c.en += acc ? u - us : (R)0;
-      c.vir += pv;
-    } else {
-      R s6 = inv * inv * inv;
-      R pv = s6 * fma((R)2, s6, (R)-1);  // r . F_ij / 24
-      R q = pv * inv;                    // |F_ij| / (24 r)
-      c.fx = fma(q, dx, c.fx);
-      c.fy = fma(q, dy, c.fy);
-      c.fz = fma(q, dz, c.fz);
-      c.en += fma(s6, s6, -s6);          // U / 4
-      c.vir += pv;
-    }
-    c.np += acc ? 1 : 0;
+    pair_one<R, TYPED>(dx, dy, dz, pj.w, rc2, ti, a, ushift, c);
   }
 }
 
@@ -553,29 +560,13 @@ __device__ __forceinline__ R clamp_cutoff(R rc_in, R rc_max) {
   return rci;
 }
 
-// Forces, energy and virial of particle `self` (position pi, cutoff rc_in)
-// over the cell grid g whose cell starts are start[0 .. ncell] (positions
-// pos, sorted by cell), with the per-particle sums of accumulation form M.
-// Returns the force and writes e_i, w_i (in FP64: the totals are reduced
-// from them in FP64) and the accepted-pair count.
-// Without EW (the packed loop only) the energy, the virial and the pair
-// count are not summed: e_out, w_out, np_out and the force's w are zero.
-template <typename R, bool TYPED, bool X2 = false, Accum M = Accum::kPlain, bool NC = true, bool EW = true>
-__device__ __forceinline__ typename RT<R>::R4 force_one(const typename RT<R>::R4* __restrict__ pos,
-                                                        const int32_t* __restrict__ start, const Grid<R>& g,
-                                                        const ForceArgs<R>& a, int self,
-                                                        const typename RT<R>::R4& pi, R rc_in, double& e_out,
-                                                        double& w_out, int& np_out) {
-  static_assert(!X2 || sizeof(R) == 4, "the packed loop serves FP32 only (with types: at most two)");
-  static_assert(M == Accum::kPlain || sizeof(R) == 4, "accumulation forms apply to FP32 pair math only");
-  static_assert(X2 || plain_loop(M), "the pair forms run on the packed loop");
-  Acc<R> c;
-  Acc2 c2;
-  Sums<M> S;
-  const R rci = clamp_cutoff<R>(rc_in, a.rc_max);
-  const R rc2 = rci * rci;
-  const int ti = TYPED ? type_of(pi.w, a.ntypes) : 0;
-  R ushift[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+// Constants of particle i's pair loop in k8: the energy shifts per partner
+// type in k8[0 .. 3], or for the packed typed loop (one or two types) the row
+// k8[t], k8[2 + t], k8[4 + t], k8[6 + t] of pair_range_x2t.
+template <typename R, bool TYPED, bool X2>
+__device__ __forceinline__ void row_constants(const ForceArgs<R>& a, int ti, R rc2, R (&ushift)[8]) {
+#pragma unroll
+  for (int t = 0; t < 8; ++t) ushift[t] = (R)0;
   if (a.shift && rc2 > (R)0) {  // no pairs at rc = 0: no shift either
     for (int t = 0; t < (TYPED ? a.ntypes : 1); ++t) {
       int tp = ti * a.ntypes + t;
@@ -594,10 +585,15 @@ __device__ __forceinline__ typename RT<R>::R4 force_one(const typename RT<R>::R4
       ushift[6 + t] = a.eps4[tp];
     }
   }
-  static_assert(EW || X2, "the scalar loop always sums energy and virial");
-  walk_rows<R, TYPED, X2, M, NC, Walk::kAll, EW>(pos, start, g, a, self, pi, rci, ti, ushift, c, c2, S);
-  // The five sums (fx, fy, fz, en, vir) of the form, in FP64 where the form
-  // keeps them so; the packed loop sums the sign-flipped differences r_j - r_i.
+}
+
+// Force, energy and virial from a particle's sums.  The five sums (fx, fy,
+// fz, en, vir) of the form, in FP64 where the form keeps them so; the packed
+// loop sums the sign-flipped differences r_j - r_i.
+template <typename R, bool TYPED, bool X2, Accum M, bool EW>
+__device__ __forceinline__ typename RT<R>::R4 finish_sums(const Acc<R>& c, const Acc2& c2, const Sums<M>& S,
+                                                          const R* ushift, double& e_out, double& w_out,
+                                                          int& np_out) {
   using V = std::conditional_t<f64_form(M), double, R>;
   V v[5];
   const int np = X2 ? c2.np : c.np;
@@ -648,6 +644,35 @@ __device__ __forceinline__ typename RT<R>::R4 force_one(const typename RT<R>::R4
   out.w = (R)e_out;
   np_out = np;
   return out;
+}
+
+// Forces, energy and virial of particle `self` (position pi, cutoff rc_in)
+// over the cell grid g whose cell starts are start[0 .. ncell] (positions
+// pos, sorted by cell), with the per-particle sums of accumulation form M.
+// Returns the force and writes e_i, w_i (in FP64: the totals are reduced
+// from them in FP64) and the accepted-pair count.
+// Without EW (the packed loop only) the energy, the virial and the pair
+// count are not summed: e_out, w_out, np_out and the force's w are zero.
+template <typename R, bool TYPED, bool X2 = false, Accum M = Accum::kPlain, bool NC = true, bool EW = true>
+__device__ __forceinline__ typename RT<R>::R4 force_one(const typename RT<R>::R4* __restrict__ pos,
+                                                        const int32_t* __restrict__ start, const Grid<R>& g,
+                                                        const ForceArgs<R>& a, int self,
+                                                        const typename RT<R>::R4& pi, R rc_in, double& e_out,
+                                                        double& w_out, int& np_out) {
+  static_assert(!X2 || sizeof(R) == 4, "the packed loop serves FP32 only (with types: at most two)");
+  static_assert(M == Accum::kPlain || sizeof(R) == 4, "accumulation forms apply to FP32 pair math only");
+  static_assert(X2 || plain_loop(M), "the pair forms run on the packed loop");
+  Acc<R> c;
+  Acc2 c2;
+  Sums<M> S;
+  const R rci = clamp_cutoff<R>(rc_in, a.rc_max);
+  const R rc2 = rci * rci;
+  const int ti = TYPED ? type_of(pi.w, a.ntypes) : 0;
+  R ushift[8];
+  row_constants<R, TYPED, X2>(a, ti, rc2, ushift);
+  static_assert(EW || X2, "the scalar loop always sums energy and virial");
+  walk_rows<R, TYPED, X2, M, NC, Walk::kAll, EW>(pos, start, g, a, self, pi, rci, ti, ushift, c, c2, S);
+  return finish_sums<R, TYPED, X2, M, EW>(c, c2, S, ushift, e_out, w_out, np_out);
 }
 
 }  // namespace dcm
