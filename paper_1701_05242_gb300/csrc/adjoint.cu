@@ -380,15 +380,69 @@ struct AdjRow {
   float sg[2], e24[2], cu[2], cd[2];
 };
 
+// One packed step on the differences d = r_j - r_k of two candidates (v0, v1:
+// whether each slot holds a real one) with cutoffs rc0, rc1, types w0, w1 and
+// upstream gradients a0, a1.
+__device__ __forceinline__ void adj_pair_x2(float2 dx, float2 dy, float2 dz, bool v0, bool v1, float rc0, float rc1,
+                                            float w0, float w1, const float4& a0, const float4& a1, float rck2,
+                                            const float4& ak, float half_dlde, const AdjRow& k, AdjAcc2& c) {
+  const float2 two = make_float2(2.f, 2.f), one = make_float2(1.f, 1.f);
+  const float2 akx = make_float2(ak.x, ak.x), aky = make_float2(ak.y, ak.y), akz = make_float2(ak.z, ak.z);
+  const float hd2 = 4.f * half_dlde;
+  const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+  const bool f0 = v0 && r2.x < rck2, f1 = v1 && r2.y < rck2;
+  const bool b0 = v0 && r2.x < rc0 * rc0, b1 = v1 && r2.y < rc1 * rc1;
+  float y0, y1;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(r2.x));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y1) : "f"(r2.y));
+  float2 y = make_float2(y0, y1);
+  const float2 e = __ffma2_rn(make_float2(-r2.x, -r2.y), y, one);
+  y = __ffma2_rn(y, e, y);
+  y = make_float2(f0 || b0 ? y.x : 0.f, f1 || b1 ? y.y : 0.f);
+  const bool t0 = w0 >= 1.f, t1 = w1 >= 1.f;
+  const float2 sg = make_float2(t0 ? k.sg[1] : k.sg[0], t1 ? k.sg[1] : k.sg[0]);
+  const float2 e24 = make_float2(t0 ? k.e24[1] : k.e24[0], t1 ? k.e24[1] : k.e24[0]);
+  const float2 s2 = __fmul2_rn(sg, y);
+  const float2 s6 = __fmul2_rn(__fmul2_rn(s2, s2), s2), s12 = __fmul2_rn(s6, s6);
+  const float2 ey = __fmul2_rn(e24, y);
+  const float2 g = __fmul2_rn(ey, __ffma2_rn(two, s12, make_float2(-s6.x, -s6.y)));        // 24 eps (2 s12 - s6) / r^2
+  const float2 gp = __fmul2_rn(__fmul2_rn(ey, y),
+                               __ffma2_rn(make_float2(-28.f, -28.f), s12, __fmul2_rn(make_float2(8.f, 8.f), s6)));
+  const float2 fw = make_float2(f0 ? 1.f : 0.f, f1 ? 1.f : 0.f), rv = make_float2(b0 ? 1.f : 0.f, b1 ? 1.f : 0.f);
+  const float2 dak = __ffma2_rn(dx, akx, __ffma2_rn(dy, aky, __fmul2_rn(dz, akz)));
+  const float2 ajx = make_float2(a0.x, a1.x), ajy = make_float2(a0.y, a1.y), ajz = make_float2(a0.z, a1.z);
+  const float2 daj = __ffma2_rn(dx, ajx, __ffma2_rn(dy, ajy, __fmul2_rn(dz, ajz)));
+  const float2 gf = __fmul2_rn(g, fw), gr = __fmul2_rn(g, rv);
+  // coefficient of d: g'/r (fwd d.A_k - rev d.A_j) + (fwd + rev) dLdE/2 g
+  const float2 cd = __ffma2_rn(gp, __ffma2_rn(fw, dak, __fmul2_rn(make_float2(-rv.x, -rv.y), daj)),
+                               __fmul2_rn(__fadd2_rn(fw, rv), __fmul2_rn(make_float2(half_dlde, half_dlde), g)));
+  c.gx = __fadd2_rn(c.gx, __ffma2_rn(cd, dx, __ffma2_rn(gf, akx, __fmul2_rn(make_float2(-gr.x, -gr.y), ajx))));
+  c.gy = __fadd2_rn(c.gy, __ffma2_rn(cd, dy, __ffma2_rn(gf, aky, __fmul2_rn(make_float2(-gr.x, -gr.y), ajy))));
+  c.gz = __fadd2_rn(c.gz, __ffma2_rn(cd, dz, __ffma2_rn(gf, akz, __fmul2_rn(make_float2(-gr.x, -gr.y), ajz))));
+  // parameter sums of the forward pairs, by partner type
+  const float2 rfa = __fmul2_rn(__fmul2_rn(y, make_float2(-dak.x, -dak.y)), make_float2(24.f, 24.f));  // 24 y (r.A_k)
+  const float2 ue = __fadd2_rn(s12, make_float2(-s6.x, -s6.y));                                      // s12 - s6
+  const float2 us = __ffma2_rn(make_float2(12.f, 12.f), s12, __fmul2_rn(make_float2(-6.f, -6.f), s6));
+  const float2 cu = make_float2(t0 ? k.cu[1] : k.cu[0], t1 ? k.cu[1] : k.cu[0]);
+  const float2 cdd = make_float2(t0 ? k.cd[1] : k.cd[0], t1 ? k.cd[1] : k.cd[0]);
+  const float2 hd = make_float2(hd2, hd2);
+  const float2 te = __fmul2_rn(fw, __ffma2_rn(rfa, __ffma2_rn(two, s12, make_float2(-s6.x, -s6.y)),
+                                              __fmul2_rn(hd, __fadd2_rn(ue, make_float2(-cu.x, -cu.y)))));
+  const float2 u24 = __ffma2_rn(make_float2(24.f, 24.f), s12, __fmul2_rn(make_float2(-6.f, -6.f), s6));
+  const float2 ts = __fmul2_rn(fw, __ffma2_rn(rfa, u24, __fmul2_rn(hd, __fadd2_rn(us, make_float2(-cdd.x, -cdd.y)))));
+  // slot a of the packed pair belongs to partner type t_a
+  c.de[0] = __fadd2_rn(c.de[0], make_float2(t0 ? 0.f : te.x, t1 ? 0.f : te.y));
+  c.de[1] = __fadd2_rn(c.de[1], make_float2(t0 ? te.x : 0.f, t1 ? te.y : 0.f));
+  c.ds[0] = __fadd2_rn(c.ds[0], make_float2(t0 ? 0.f : ts.x, t1 ? 0.f : ts.y));
+  c.ds[1] = __fadd2_rn(c.ds[1], make_float2(t0 ? ts.x : 0.f, t1 ? ts.y : 0.f));
+}
+
 template <bool SJ>
 __device__ __forceinline__ void adj_range_x2(const float4* __restrict__ pos, const float* __restrict__ rc,
                                              const float4* __restrict__ A, int lo, int hi, int self, float xi,
                                              float yi, float zi, float shx, float shy, float shz, float rck2,
                                              float rc_max, const float4& ak, float half_dlde, const AdjRow& k,
                                              AdjAcc2& c) {
-  const float2 two = make_float2(2.f, 2.f), m1 = make_float2(-1.f, -1.f), one = make_float2(1.f, 1.f);
-  const float2 akx = make_float2(ak.x, ak.x), aky = make_float2(ak.y, ak.y), akz = make_float2(ak.z, ak.z);
-  const float hd2 = 4.f * half_dlde;
   for (int j = lo; j < hi; j += 2) {
     const bool has1 = j + 1 < hi;
     const int j1 = has1 ? j + 1 : j;
@@ -405,53 +459,7 @@ __device__ __forceinline__ void adj_range_x2(const float4* __restrict__ pos, con
       dy = make_float2(p0.y - yi, p1.y - yi);
       dz = make_float2(p0.z - zi, p1.z - zi);
     }
-    const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
-    const bool v0 = j != self, v1 = has1 && j1 != self;
-    const bool f0 = v0 && r2.x < rck2, f1 = v1 && r2.y < rck2;
-    const bool b0 = v0 && r2.x < rc0 * rc0, b1 = v1 && r2.y < rc1 * rc1;
-    float y0, y1;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(r2.x));
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y1) : "f"(r2.y));
-    float2 y = make_float2(y0, y1);
-    const float2 e = __ffma2_rn(make_float2(-r2.x, -r2.y), y, one);
-    y = __ffma2_rn(y, e, y);
-    y = make_float2(f0 || b0 ? y.x : 0.f, f1 || b1 ? y.y : 0.f);
-    const bool t0 = p0.w >= 1.f, t1 = p1.w >= 1.f;
-    const float2 sg = make_float2(t0 ? k.sg[1] : k.sg[0], t1 ? k.sg[1] : k.sg[0]);
-    const float2 e24 = make_float2(t0 ? k.e24[1] : k.e24[0], t1 ? k.e24[1] : k.e24[0]);
-    const float2 s2 = __fmul2_rn(sg, y);
-    const float2 s6 = __fmul2_rn(__fmul2_rn(s2, s2), s2), s12 = __fmul2_rn(s6, s6);
-    const float2 ey = __fmul2_rn(e24, y);
-    const float2 g = __fmul2_rn(ey, __ffma2_rn(two, s12, make_float2(-s6.x, -s6.y)));        // 24 eps (2 s12 - s6) / r^2
-    const float2 gp = __fmul2_rn(__fmul2_rn(ey, y),
-                                 __ffma2_rn(make_float2(-28.f, -28.f), s12, __fmul2_rn(make_float2(8.f, 8.f), s6)));
-    const float2 fw = make_float2(f0 ? 1.f : 0.f, f1 ? 1.f : 0.f), rv = make_float2(b0 ? 1.f : 0.f, b1 ? 1.f : 0.f);
-    const float2 dak = __ffma2_rn(dx, akx, __ffma2_rn(dy, aky, __fmul2_rn(dz, akz)));
-    const float2 ajx = make_float2(a0.x, a1.x), ajy = make_float2(a0.y, a1.y), ajz = make_float2(a0.z, a1.z);
-    const float2 daj = __ffma2_rn(dx, ajx, __ffma2_rn(dy, ajy, __fmul2_rn(dz, ajz)));
-    const float2 gf = __fmul2_rn(g, fw), gr = __fmul2_rn(g, rv);
-    // coefficient of d: g'/r (fwd d.A_k - rev d.A_j) + (fwd + rev) dLdE/2 g
-    const float2 cd = __ffma2_rn(gp, __ffma2_rn(fw, dak, __fmul2_rn(make_float2(-rv.x, -rv.y), daj)),
-                                 __fmul2_rn(__fadd2_rn(fw, rv), __fmul2_rn(make_float2(half_dlde, half_dlde), g)));
-    c.gx = __fadd2_rn(c.gx, __ffma2_rn(cd, dx, __ffma2_rn(gf, akx, __fmul2_rn(make_float2(-gr.x, -gr.y), ajx))));
-    c.gy = __fadd2_rn(c.gy, __ffma2_rn(cd, dy, __ffma2_rn(gf, aky, __fmul2_rn(make_float2(-gr.x, -gr.y), ajy))));
-    c.gz = __fadd2_rn(c.gz, __ffma2_rn(cd, dz, __ffma2_rn(gf, akz, __fmul2_rn(make_float2(-gr.x, -gr.y), ajz))));
-    // parameter sums of the forward pairs, by partner type
-    const float2 rfa = __fmul2_rn(__fmul2_rn(y, make_float2(-dak.x, -dak.y)), make_float2(24.f, 24.f));  // 24 y (r.A_k)
-    const float2 ue = __fadd2_rn(s12, make_float2(-s6.x, -s6.y));                                      // s12 - s6
-    const float2 us = __ffma2_rn(make_float2(12.f, 12.f), s12, __fmul2_rn(make_float2(-6.f, -6.f), s6));
-    const float2 cu = make_float2(t0 ? k.cu[1] : k.cu[0], t1 ? k.cu[1] : k.cu[0]);
-    const float2 cdd = make_float2(t0 ? k.cd[1] : k.cd[0], t1 ? k.cd[1] : k.cd[0]);
-    const float2 hd = make_float2(hd2, hd2);
-    const float2 te = __fmul2_rn(fw, __ffma2_rn(rfa, __ffma2_rn(two, s12, make_float2(-s6.x, -s6.y)),
-                                                __fmul2_rn(hd, __fadd2_rn(ue, make_float2(-cu.x, -cu.y)))));
-    const float2 u24 = __ffma2_rn(make_float2(24.f, 24.f), s12, __fmul2_rn(make_float2(-6.f, -6.f), s6));
-    const float2 ts = __fmul2_rn(fw, __ffma2_rn(rfa, u24, __fmul2_rn(hd, __fadd2_rn(us, make_float2(-cdd.x, -cdd.y)))));
-    // slot a of the packed pair belongs to partner type t_a
-    c.de[0] = __fadd2_rn(c.de[0], make_float2(t0 ? 0.f : te.x, t1 ? 0.f : te.y));
-    c.de[1] = __fadd2_rn(c.de[1], make_float2(t0 ? te.x : 0.f, t1 ? te.y : 0.f));
-    c.ds[0] = __fadd2_rn(c.ds[0], make_float2(t0 ? 0.f : ts.x, t1 ? 0.f : ts.y));
-    c.ds[1] = __fadd2_rn(c.ds[1], make_float2(t0 ? ts.x : 0.f, t1 ? ts.y : 0.f));
+    adj_pair_x2(dx, dy, dz, j != self, has1 && j1 != self, rc0, rc1, p0.w, p1.w, a0, a1, rck2, ak, half_dlde, k, c);
   }
 }
 
@@ -564,6 +572,161 @@ __global__ void __launch_bounds__(kAdjX2Block) k_adjoint_x2(int64_t n, const flo
   }
 }
 
+// The packed adjoint of a small system, one warp per particle: the lanes
+// take the rows of the walk (radius `reach`), write their candidates into a
+// list in shared memory and then share the list, two candidates per lane and
+// step.  A launch of 2,000 particles lasts as long as one particle's walk: 435 us
+// with one thread per particle.  The sums of the lanes are added in a fixed tree.
+constexpr int kAdjWarps = 4, kAdjList = 1024;  // particles per block; candidates listed at a time
+
+__global__ void __launch_bounds__(32 * kAdjWarps) k_adjoint_warp(
+    int64_t n, const float4* __restrict__ pos, const float* __restrict__ rc, const int32_t* __restrict__ start,
+    ForceArgs<float> a, const float4* __restrict__ A, float half_dlde, float4* __restrict__ G,
+    double* __restrict__ part, int64_t nslot, BlockGrid bg, const int32_t* __restrict__ bmax) {
+  __shared__ uint32_t list_sh[kAdjWarps][kAdjList];  // particle, and its image along x, y, z (adjoint code) per entry
+  __shared__ uint8_t code_sh[kAdjWarps][kAdjList];
+  __shared__ double sum_sh[kAdjWarps][8];
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  uint32_t* list = list_sh[wid];
+  uint8_t* codes = code_sh[wid];
+  const int64_t i = (int64_t)blockIdx.x * kAdjWarps + wid;
+  const int nt = a.ntypes;
+  const Grid<float>& g = a.g;
+  AdjAcc2 c;
+  int tk = 0;
+  if (i < n) {
+    const float4 pi = __ldg(pos + i), ak = __ldg(A + i);
+    const float rck = clamp_cutoff<float>(__ldg(rc + i), a.rc_max), rck2 = rck * rck;
+    // the largest cutoff of the 27 blocks around (reverse_reach), one block per lane
+    float m = 0.f;
+    if (lane < 27) {
+      const int b0 = block_coord(pi.x, bg.inv_be[0], bg.nb[0]) + lane % 3 - 1,
+                b1 = block_coord(pi.y, bg.inv_be[1], bg.nb[1]) + lane / 3 % 3 - 1,
+                b2 = block_coord(pi.z, bg.inv_be[2], bg.nb[2]) + lane / 9 - 1;
+      const int xx = (b0 + bg.nb[0]) % bg.nb[0], yy = (b1 + bg.nb[1]) % bg.nb[1], zz = (b2 + bg.nb[2]) % bg.nb[2];
+      m = __int_as_float(__ldg(bmax + xx + bg.nb[0] * (yy + bg.nb[1] * zz)));
+    }
+    m = __int_as_float(__reduce_max_sync(full, __float_as_int(m)));  // cutoffs are not negative
+    const float reach = fmaxf(fminf(m, a.rc_max), rck);
+    const float reach2s = reach * reach * 1.000004f;
+    tk = type_of(pi.w, nt);
+    AdjRow k;
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      const int tc = t < nt ? t : nt - 1, p = tk * nt + tc;
+      k.sg[t] = a.sig2[p];
+      k.e24[t] = a.eps24[p];
+      k.cu[t] = k.cd[t] = 0.f;
+      if (a.shift && rck2 > 0.f) {
+        const float c2 = a.sig2[p] / rck2, c6 = c2 * c2 * c2, c12 = c6 * c6;
+        k.cu[t] = c12 - c6;
+        k.cd[t] = 12.f * c12 - 6.f * c6;
+      }
+    }
+    const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
+    const float l = g.edge, il = g.inv_edge, ilx = g.inv_edge_x;
+    const int cx = cell_coord<float>(pi.x, g.edge_x, ilx, nx), cy = cell_coord<float>(pi.y, l, il, ny),
+              cz = cell_coord<float>(pi.z, l, il, nz);
+    const int H = (int)ceilf(reach * il), Hx = (int)ceilf(reach * ilx), side = 2 * H + 1;
+    int listed = 0;
+    auto visit = [&]() {
+      __syncwarp();
+      for (int q = 2 * lane; q < listed; q += 64) {
+        const bool has1 = q + 1 < listed;
+        const int q1 = has1 ? q + 1 : q;
+        const int j0 = (int)list[q], j1 = (int)list[q1];
+        const uint32_t e0 = codes[q], e1 = codes[q1];
+        const float4 p0 = __ldg(pos + j0), p1 = __ldg(pos + j1), a0 = __ldg(A + j0), a1 = __ldg(A + j1);
+        const float rc0 = clamp_cutoff<float>(__ldg(rc + j0), a.rc_max), rc1 = clamp_cutoff<float>(__ldg(rc + j1), a.rc_max);
+        // an image at -L shifts j, one at +L shifts the particle itself
+        auto diff = [&](float pj, float pk, float L, uint32_t e) {
+          return (e & 1u ? pj - L : pj) - (e & 2u ? pk - L : pk);
+        };
+        const float2 dx = make_float2(diff(p0.x, pi.x, g.L[0], e0), diff(p1.x, pi.x, g.L[0], e1)),
+                     dy = make_float2(diff(p0.y, pi.y, g.L[1], e0 >> 2), diff(p1.y, pi.y, g.L[1], e1 >> 2)),
+                     dz = make_float2(diff(p0.z, pi.z, g.L[2], e0 >> 4), diff(p1.z, pi.z, g.L[2], e1 >> 4));
+        adj_pair_x2(dx, dy, dz, !(j0 == i && e0 == 0), has1 && !(j1 == i && e1 == 0), rc0, rc1, p0.w, p1.w, a0, a1,
+                    rck2, ak, half_dlde, k, c);
+      }
+      __syncwarp();
+      listed = 0;
+    };
+    // the rows, each in up to three pieces along x (image at -L, the box, image at +L)
+    const int nitem = 3 * side * side;
+    for (int it0 = 0; it0 < nitem; it0 += 32) {
+      const int it = it0 + lane;
+      int j0 = 0, cnt = 0;
+      uint32_t code = 0;
+      if (it < nitem) {
+        const int piece = it % 3, row = it / 3, uy = cy - H + row % side, uz = cz - H + row / side;
+        const float gz = uz > cz ? (float)uz * l - pi.z : (uz < cz ? pi.z - (float)(uz + 1) * l : 0.f);
+        const float gy = uy > cy ? (float)uy * l - pi.y : (uy < cy ? pi.y - (float)(uy + 1) * l : 0.f);
+        const float g2 = gz * gz + gy * gy;
+        if (g2 < reach2s) {
+          const float wx = sqrtf(reach2s - g2);
+          const int ulo = max(ufloor<float>((pi.x - wx) * ilx - 5e-4f), cx - Hx);
+          const int uhi = min(ufloor<float>((pi.x + wx) * ilx + 5e-4f), cx + Hx);
+          // a coordinate outside [0, L): no window
+          const int lo = piece == 0 ? ulo : (piece == 1 ? max(ulo, 0) : max(ulo, nx));
+          const int hi = piece == 0 ? min(uhi, -1) : (piece == 1 ? min(uhi, nx - 1) : uhi);
+          if (lo <= hi) {
+            const int wy = uy < 0 ? uy + ny : (uy >= ny ? uy - ny : uy), wz = uz < 0 ? uz + nz : (uz >= nz ? uz - nz : uz);
+            const int base = nx * (wy + ny * wz) + (piece == 0 ? nx : (piece == 2 ? -nx : 0));
+            j0 = __ldg(start + base + lo);
+            cnt = max(__ldg(start + base + hi + 1) - j0, 0);
+            code = (piece == 0 ? 1u : (piece == 2 ? 2u : 0u)) | (uy < 0 ? 4u : (uy >= ny ? 8u : 0u)) |
+                   (uz < 0 ? 16u : (uz >= nz ? 32u : 0u));
+          }
+        }
+      }
+      int incl = cnt;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(full, incl, o);
+        if (lane >= o) incl += u;
+      }
+      const int off = incl - cnt, total = __shfl_sync(full, incl, 31);
+      for (int done = 0; done < total;) {
+        const int take = min(total - done, kAdjList - listed);
+        for (int q = max(done - off, 0); q < min(done + take - off, cnt); ++q) {
+          list[listed + off + q - done] = (uint32_t)(j0 + q);
+          codes[listed + off + q - done] = (uint8_t)code;
+        }
+        listed += take;
+        done += take;
+        if (listed == kAdjList) visit();
+      }
+    }
+    visit();
+  }
+  float v[7] = {c.gx.x + c.gx.y, c.gy.x + c.gy.y, c.gz.x + c.gz.y, c.de[0].x + c.de[0].y, c.de[1].x + c.de[1].y,
+                c.ds[0].x + c.ds[0].y, c.ds[1].x + c.ds[1].y};
+#pragma unroll
+  for (int q = 0; q < 7; ++q)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(full, v[q], o);
+  if (i < n && lane == 0) G[i] = make_float4(v[0], v[1], v[2], 0.f);
+  if (part) {  // per block, in FP64, in the order of the particles
+    if (lane < 8) {
+      const int p = lane & 3, q = lane >> 2;  // type pair, eps or sigma
+      double t = 0.0;
+      if (p < nt * nt && i < n && tk == p / nt) {
+        const bool t1 = p % nt == 1;
+        t = q ? (double)(t1 ? v[6] : v[5]) * 0.25 * (double)a.eps4[p] / sqrt((double)a.sig2[p])  // eps_p / sigma_p
+              : (double)(t1 ? v[4] : v[3]);
+      }
+      sum_sh[wid][lane] = t;
+    }
+    __syncthreads();
+    if (threadIdx.x < 8 && (threadIdx.x & 3) < nt * nt) {
+      double t = 0.0;
+      for (int w = 0; w < kAdjWarps; ++w) t += sum_sh[w][threadIdx.x];
+      part[(int64_t)(16 * (threadIdx.x >> 2) + (threadIdx.x & 3)) * nslot + blockIdx.x] = t;
+    }
+  }
+}
+
 // Cost key of the adjoint's tiles (tile_order.cuh): the largest reverse reach
 // among a tile's particles, the radius of its widest walk.
 template <typename R>
@@ -619,9 +782,12 @@ int lj_adjoint(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, const R* 
   a.shift = ctx->p.shift_energy;
   a.rc_max = (R)ctx->p.rc_max;
   constexpr int kBlock = adj_block<R>();
-  int64_t nblk = (n + kBlock - 1) / kBlock, nwarp = nblk * (kBlock / 32);
+  // the packed loop (FP32, one or two types), else the scalar loop; small
+  // systems of the packed loop take a warp per particle
+  const bool x2 = sizeof(R) == 4 && nt <= 2, small = x2 && n <= kAdjWarpMaxN;
+  const int64_t nblk = (n + kBlock - 1) / kBlock, nwarp = small ? adj_warp_slots(n) : nblk * (kBlock / 32);
   bool want = dparams != nullptr;
-  if (want && nwarp > ctx->red_cap)
+  if (want && nwarp > ctx->adj_cap)
     return set_error(ctx, DCM_ERR_CAPACITY, "adjoint reduction needs %lld partials", (long long)nwarp);
   double* part = want ? ctx->adj_part : nullptr;  // [32][nwarp]: de pairs 0..15, ds pairs 16..31
   BlockGrid bg;
@@ -631,16 +797,15 @@ int lj_adjoint(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, const R* 
   }
   DCM_CUDA_TRY(ctx, cudaMemsetAsync(ctx->blk_max, 0, sizeof(int32_t) * ctx->nblk, st));
   DCM_LAUNCH(ctx, k_block_max<R>, (unsigned)((n + 255) / 256), 256, 0, st, n, pos, rc, a.rc_max, bg, ctx->blk_max);
-  // the packed loop (FP32, one or two types), else the scalar loop
-  const bool x2 = sizeof(R) == 4 && nt <= 2;
   const int tb = x2 ? kAdjX2Block : kBlock;
   const void* kern = x2 ? (const void*)k_adjoint_x2
                         : (lj_general(t) ? (const void*)k_adjoint<R, true> : (const void*)k_adjoint<R, false>);
+  static_assert(kAdjWarps == 4, "adj_warp_slots");
   static_assert(kAdjX2Block == adj_block<float>(), "the partials layout assumes equal blocks");
   // launch order of the tiles, the widest walks first, where that pays
   const TileOrder to = tile_order_layout(ctx->tile_scratch, (n + tb - 1) / tb);
   const int32_t* order = nullptr;
-  if (tile_order_pays(kern, tb, to.ntile)) {
+  if (!small && tile_order_pays(kern, tb, to.ntile)) {
     int r0 = tile_order_begin(ctx, to, st);
     if (r0) return r0;
     DCM_LAUNCH(ctx, k_adj_tile_key<R>, (unsigned)to.ntile, tb, 0, st, n, pos, rc, a.rc_max, bg,
@@ -649,7 +814,10 @@ int lj_adjoint(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, const R* 
     order = to.order;
   }
   if constexpr (sizeof(R) == 4) {
-    if (x2)
+    if (small)
+      DCM_LAUNCH(ctx, k_adjoint_warp, (unsigned)adj_warp_slots(n), 32 * kAdjWarps, 0, st, n, pos, rc, cell_start, a, A,
+                 (float)(0.5 * dlde), G, part, nwarp, bg, (const int32_t*)ctx->blk_max);
+    else if (x2)
       DCM_LAUNCH(ctx, k_adjoint_x2, (unsigned)to.ntile, kAdjX2Block, 0, st, n, pos, rc, cell_start, a, A,
                  (float)(0.5 * dlde), G, part, nwarp, bg, (const int32_t*)ctx->blk_max, order);
   }

@@ -263,13 +263,20 @@ extern "C" int dcm_grid_dims(const dcm_params* p, int64_t* cells3, int64_t* boxe
 struct ScratchPlan {
   int64_t n_max, ncell, nbox, scan_cap, red_cap, rsize, flags, nblk;
   int64_t tile_cap;  // pair tiles (0: not served)
-  int64_t red_slots() const { return red_cap > tile_cap ? red_cap : tile_cap; }
+  int64_t red_slots() const {
+    const int64_t a = red_cap > tile_cap ? red_cap : tile_cap, b = plane_slots(n_max < kPlanesMaxN ? n_max : kPlanesMaxN);
+    return a > b ? a : b;
+  }
+  int64_t adj_slots() const {
+    const int64_t b = adj_warp_slots(n_max < kAdjWarpMaxN ? n_max : kAdjWarpMaxN);
+    return red_cap > b ? red_cap : b;
+  }
   double skin;
   int32_t min_component, segmentation, ms_outer;
   int64_t total() const {
     return 4 * 4 + 16 + 3 * 4 * n_max + 4 * (ncell + 1) + 4 * ncell + 8 * (scan_cap + 1) + 3 * 4 * nbox + 2 * nbox +
            2 * rsize * nbox + 4 * flags + 4 * (int64_t)kHistCap + 4 * 8 + 8 * 3 * red_slots() + 8 * 8 + 8 * 8 * 256 +
-           8 * 32 * red_cap + 8 * 48 + (skin > 0 ? 8 * n_max + 8 * (n_max / 32 + 16) + 4 * rsize * n_max + 32 : 0) +
+           8 * 32 * adj_slots() + 8 * 48 + (skin > 0 ? 8 * n_max + 8 * (n_max / 32 + 16) + 4 * rsize * n_max + 32 : 0) +
            (min_component > 0 ? 9 * nbox + 4 * 80 : 0) + 13 * nbox + 4 * (flags + 2) + 4 * nblk +
            4 * tile_scratch_ints(n_max) + (tile_cap > 0 ? 4 * tile_ints(tile_cap) : 0) +
            (segmentation ? 6 * rsize * nbox + 32 * ms_outer + 16 + 4 * (ms_outer + 2) : 0);
@@ -383,7 +390,8 @@ extern "C" int dcm_create(const dcm_params* p, dcm_ctx** out) {
   alloc((void**)&ctx->red, 8 * 3 * s.red_slots());
   alloc((void**)&ctx->totals, 8 * 8);
   alloc((void**)&ctx->red_tmp, 8 * 8 * 256);
-  alloc((void**)&ctx->adj_part, 8 * 32 * s.red_cap);
+  alloc((void**)&ctx->adj_part, 8 * 32 * s.adj_slots());
+  ctx->adj_cap = s.adj_slots();
   if (p->skin > 0.0) {
     alloc((void**)&ctx->nnb, 4 * nm);
     alloc((void**)&ctx->nimg, 4 * nm);

@@ -110,7 +110,8 @@ struct dcm_ctx {
   int32_t* thr;             // [8]: gmin, gmax, T, sweeps, ...
   double* red;              // reduction partials
   double* red_tmp;          // [8 * 256] first-level chunk sums
-  double* adj_part;         // [32][red_cap] adjoint parameter-gradient partials
+  double* adj_part;         // [32][adj_cap] adjoint parameter-gradient partials
+  int64_t adj_cap;
   double* adj_pairs;        // [48]: per-pair eps sums, per-pair sigma sums, eps values
   double* totals;           // [4]
   int32_t* host_status;     // pinned host mirror
@@ -247,6 +248,17 @@ int lj_forces(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, const R* r
               const int32_t* cell_start, typename RT<R>::R4* force, double* totals, cudaStream_t st,
               bool energies = true);
 
+// Systems of at most kPlanesMaxN particles (mixed form, default accumulation)
+// take 16 lanes per particle in the forces (k_forces_planes), whose blocks of 8
+// particles each leave one partial sum.
+constexpr int64_t kPlanesMaxN = 32768;
+constexpr int kPlaneLanes = 16, kPlaneBlock = 128;  // lanes per particle, threads per block
+constexpr int64_t plane_slots(int64_t n) { return (n + 7) / 8; }
+// Systems of at most kAdjWarpMaxN particles take a warp per particle in the
+// packed adjoint (k_adjoint_warp, blocks of 4 particles).
+constexpr int64_t kAdjWarpMaxN = 49152;
+constexpr int64_t adj_warp_slots(int64_t n) { return (n + 3) / 4; }
+
 // forces_tiles.cu
 // Geometry of the pair tiles (pair_tiles.cuh), fixed per context.
 struct TileCfg {
@@ -262,7 +274,7 @@ struct TilePlan {
   bool usable;
 };
 TilePlan tile_plan(const dcm_params& p, const int64_t* nc, int64_t n);
-constexpr int64_t tile_ints(int64_t slots) { return 4 + 34 * slots; }
+constexpr int64_t tile_ints(int64_t slots) { return 8 + 34 * slots; }
 bool tiles_serve(const dcm_ctx* ctx, int64_t n);  // whether lj_forces runs over tiles
 template <typename R>
 struct ForceArgs;

@@ -475,6 +475,92 @@ __device__ __forceinline__ void segment(const typename RT<R>::R4* __restrict__ p
 // of a window beyond either x end).
 enum class Walk { kAll, kImagesOnly };
 
+// What the row walk of one particle works with (cell (cx, cy, cz), stencil half
+// widths H and Hx in cells, squared cutoff with and without the culling slack).
+template <typename R>
+struct Walker {
+  int cx, cy, cz, H, Hx;
+  R rc2, rc2s;
+  __device__ __forceinline__ Walker(const Grid<R>& g, const typename RT<R>::R4& pi, R rci) {
+    rc2 = rci * rci;
+    rc2s = rc2 * (R)1.000004;  // culling slack; the pair test is exact
+    cx = cell_coord<R>(pi.x, g.edge_x, g.inv_edge_x, g.n[0]);
+    cy = cell_coord<R>(pi.y, g.edge, g.inv_edge, g.n[1]);
+    cz = cell_coord<R>(pi.z, g.edge, g.inv_edge, g.n[2]);
+    H = (int)ceil(rci * g.inv_edge);
+    Hx = (int)ceil(rci * g.inv_edge_x);
+  }
+};
+
+// The rows of the z-plane uz of particle `self`'s walk (walk_rows); false if
+// the plane is out of reach.
+template <typename R, bool TYPED, bool X2, Accum M, bool NC = true, Walk MODE = Walk::kAll, bool EW = true>
+__device__ __forceinline__ bool walk_plane(const typename RT<R>::R4* __restrict__ pos,
+                                           const int32_t* __restrict__ start, const Grid<R>& g,
+                                           const ForceArgs<R>& a, int self, const typename RT<R>::R4& pi,
+                                           const Walker<R>& wk, int uz, int ti, const R* ushift, Acc<R>& c, Acc2& c2,
+                                           Sums<M>& S) {
+  constexpr bool kImg = MODE == Walk::kImagesOnly;
+  const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
+  const R l = g.edge, il = g.inv_edge, ilx = g.inv_edge_x;
+  const int cx = wk.cx, cy = wk.cy, cz = wk.cz, H = wk.H, Hx = wk.Hx;
+  const R rc2 = wk.rc2, rc2s = wk.rc2s;
+  R gz = uz > cz ? (R)uz * l - pi.z : (uz < cz ? pi.z - (R)(uz + 1) * l : (R)0);
+  R gz2 = gz * gz;
+  if (gz2 >= rc2s) return false;
+  int wz = uz < 0 ? uz + nz : (uz >= nz ? uz - nz : uz);
+  R zi = uz >= nz ? pi.z - g.L[2] : pi.z;  // image +L: shift i
+  R zsh = uz < 0 ? -g.L[2] : (R)0;          // image -L: shift j
+  for (int uy = cy - H; uy <= cy + H; ++uy) {
+    R gy = uy > cy ? (R)uy * l - pi.y : (uy < cy ? pi.y - (R)(uy + 1) * l : (R)0);
+    R gyz2 = gz2 + gy * gy;
+    if (gyz2 >= rc2s) continue;
+    int wy = uy < 0 ? uy + ny : (uy >= ny ? uy - ny : uy);
+    R yi = uy >= ny ? pi.y - g.L[1] : pi.y;
+    R ysh = uy < 0 ? -g.L[1] : (R)0;
+    R wx = window_half_width(rc2s - gyz2);
+    int ulo = ufloor<R>((pi.x - wx) * ilx - (R)5e-4);
+    int uhi = ufloor<R>((pi.x + wx) * ilx + (R)5e-4);
+    // both ends clamped into [cx - Hx - 1, cx + Hx + 1]: for a coordinate
+    // outside [0, L) (its cell clamped into the grid, its window not) the
+    // segments come out empty and every index stays in range
+    ulo = min(max(ulo, cx - Hx), cx + Hx + 1);
+    uhi = max(min(uhi, cx + Hx), cx - Hx - 1);
+    // 32-bit: parameter validation keeps the cell count below 2^31 - 1
+    const int row = nx * (wy + ny * wz);
+    // segment u < 0: image -L (shift j)
+    if (ulo < 0) {
+      int a1 = min(uhi, -1);
+      int j0 = ld_start<NC>(start + row + ulo + nx), j1 = ld_start<NC>(start + row + a1 + nx + 1);
+      segment<R, true, TYPED, X2, M, NC, EW>(pos, j0, j1, pi.x, yi, zi, -g.L[0], ysh, zsh, rc2, ti, a, ushift, c, c2, S);
+    }
+    // segment 0 <= u < nx: no x shift; the particle itself is skipped
+    const bool img_row = uy < 0 || uy >= ny || uz < 0 || uz >= nz;
+    if (!kImg || img_row) {
+      int a0 = max(ulo, 0), a1 = min(uhi, nx - 1);
+      if (a0 <= a1) {
+        int j0 = ld_start<NC>(start + row + a0), j1 = ld_start<NC>(start + row + a1 + 1);
+        if (!kImg && uy == cy && uz == cz) {  // the particle's own row: cut it out
+          segment<R, false, TYPED, X2, M, NC, EW>(pos, j0, min(j1, self), pi.x, yi, zi, 0, 0, 0, rc2, ti, a, ushift, c, c2, S);
+          segment<R, false, TYPED, X2, M, NC, EW>(pos, max(j0, self + 1), j1, pi.x, yi, zi, 0, 0, 0, rc2, ti, a, ushift, c,
+                                       c2, S);
+        } else if (ysh == (R)0 && zsh == (R)0) {
+          segment<R, false, TYPED, X2, M, NC, EW>(pos, j0, j1, pi.x, yi, zi, 0, 0, 0, rc2, ti, a, ushift, c, c2, S);
+        } else {
+          segment<R, true, TYPED, X2, M, NC, EW>(pos, j0, j1, pi.x, yi, zi, (R)0, ysh, zsh, rc2, ti, a, ushift, c, c2, S);
+        }
+      }
+    }
+    // segment u >= nx: image +L (shift i)
+    if (uhi >= nx) {
+      int a0 = max(ulo, nx);
+      int j0 = ld_start<NC>(start + row + a0 - nx), j1 = ld_start<NC>(start + row + uhi - nx + 1);
+      segment<R, true, TYPED, X2, M, NC, EW>(pos, j0, j1, pi.x - g.L[0], yi, zi, (R)0, ysh, zsh, rc2, ti, a, ushift, c, c2, S);
+    }
+  }
+  return true;
+}
+
 // The culled cell-row walk of particle `self` (position pi, clamped cutoff
 // rci) over the cell grid g whose cell starts are start[0 .. ncell] (positions
 // pos sorted by cell), accumulating into c (scalar loop) or c2 (packed).
@@ -483,69 +569,9 @@ __device__ __forceinline__ void walk_rows(const typename RT<R>::R4* __restrict__
                                           const int32_t* __restrict__ start, const Grid<R>& g,
                                           const ForceArgs<R>& a, int self, const typename RT<R>::R4& pi, R rci,
                                           int ti, const R* ushift, Acc<R>& c, Acc2& c2, Sums<M>& S) {
-  constexpr bool kImg = MODE == Walk::kImagesOnly;
-  const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
-  const R l = g.edge, il = g.inv_edge, ilx = g.inv_edge_x;
-  const R rc2 = rci * rci;
-  const R rc2s = rc2 * (R)1.000004;  // culling slack; the pair test is exact
-  const int cx = cell_coord<R>(pi.x, g.edge_x, ilx, nx);
-  const int cy = cell_coord<R>(pi.y, l, il, ny);
-  const int cz = cell_coord<R>(pi.z, l, il, nz);
-  const int H = (int)ceil(rci * il), Hx = (int)ceil(rci * ilx);
-  for (int uz = cz - H; uz <= cz + H; ++uz) {
-    R gz = uz > cz ? (R)uz * l - pi.z : (uz < cz ? pi.z - (R)(uz + 1) * l : (R)0);
-    R gz2 = gz * gz;
-    if (gz2 >= rc2s) continue;
-    int wz = uz < 0 ? uz + nz : (uz >= nz ? uz - nz : uz);
-    R zi = uz >= nz ? pi.z - g.L[2] : pi.z;  // image +L: shift i
-    R zsh = uz < 0 ? -g.L[2] : (R)0;          // image -L: shift j
-    for (int uy = cy - H; uy <= cy + H; ++uy) {
-      R gy = uy > cy ? (R)uy * l - pi.y : (uy < cy ? pi.y - (R)(uy + 1) * l : (R)0);
-      R gyz2 = gz2 + gy * gy;
-      if (gyz2 >= rc2s) continue;
-      int wy = uy < 0 ? uy + ny : (uy >= ny ? uy - ny : uy);
-      R yi = uy >= ny ? pi.y - g.L[1] : pi.y;
-      R ysh = uy < 0 ? -g.L[1] : (R)0;
-      R wx = window_half_width(rc2s - gyz2);
-      int ulo = ufloor<R>((pi.x - wx) * ilx - (R)5e-4);
-      int uhi = ufloor<R>((pi.x + wx) * ilx + (R)5e-4);
-      // both ends clamped into [cx - Hx - 1, cx + Hx + 1]: for a coordinate
-      // outside [0, L) (its cell clamped into the grid, its window not) the
-      // segments come out empty and every index stays in range
-      ulo = min(max(ulo, cx - Hx), cx + Hx + 1);
-      uhi = max(min(uhi, cx + Hx), cx - Hx - 1);
-      // 32-bit: parameter validation keeps the cell count below 2^31 - 1
-      const int row = nx * (wy + ny * wz);
-      // segment u < 0: image -L (shift j)
-      if (ulo < 0) {
-        int a1 = min(uhi, -1);
-        int j0 = ld_start<NC>(start + row + ulo + nx), j1 = ld_start<NC>(start + row + a1 + nx + 1);
-        segment<R, true, TYPED, X2, M, NC, EW>(pos, j0, j1, pi.x, yi, zi, -g.L[0], ysh, zsh, rc2, ti, a, ushift, c, c2, S);
-      }
-      // segment 0 <= u < nx: no x shift; the particle itself is skipped
-      const bool img_row = uy < 0 || uy >= ny || uz < 0 || uz >= nz;
-      if (!kImg || img_row) {
-        int a0 = max(ulo, 0), a1 = min(uhi, nx - 1);
-        if (a0 <= a1) {
-          int j0 = ld_start<NC>(start + row + a0), j1 = ld_start<NC>(start + row + a1 + 1);
-          if (!kImg && uy == cy && uz == cz) {  // the particle's own row: cut it out
-            segment<R, false, TYPED, X2, M, NC, EW>(pos, j0, min(j1, self), pi.x, yi, zi, 0, 0, 0, rc2, ti, a, ushift, c, c2, S);
-            segment<R, false, TYPED, X2, M, NC, EW>(pos, max(j0, self + 1), j1, pi.x, yi, zi, 0, 0, 0, rc2, ti, a, ushift, c,
-                                         c2, S);
-          } else if (ysh == (R)0 && zsh == (R)0) {
-            segment<R, false, TYPED, X2, M, NC, EW>(pos, j0, j1, pi.x, yi, zi, 0, 0, 0, rc2, ti, a, ushift, c, c2, S);
-          } else {
-            segment<R, true, TYPED, X2, M, NC, EW>(pos, j0, j1, pi.x, yi, zi, (R)0, ysh, zsh, rc2, ti, a, ushift, c, c2, S);
-          }
-        }
-      }
-      // segment u >= nx: image +L (shift i)
-      if (uhi >= nx) {
-        int a0 = max(ulo, nx);
-        int j0 = ld_start<NC>(start + row + a0 - nx), j1 = ld_start<NC>(start + row + uhi - nx + 1);
-        segment<R, true, TYPED, X2, M, NC, EW>(pos, j0, j1, pi.x - g.L[0], yi, zi, (R)0, ysh, zsh, rc2, ti, a, ushift, c, c2, S);
-      }
-    }
+  const Walker<R> wk(g, pi, rci);
+  for (int uz = wk.cz - wk.H; uz <= wk.cz + wk.H; ++uz) {
+    if (!walk_plane<R, TYPED, X2, M, NC, MODE, EW>(pos, start, g, a, self, pi, wk, uz, ti, ushift, c, c2, S)) continue;
     if constexpr (plane_form(M)) flush_partials<M, R, X2, EW>(c, c2, S);
   }
 }

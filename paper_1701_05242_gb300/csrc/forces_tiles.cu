@@ -19,7 +19,7 @@ namespace dcm {
 // ---------------------------------------------------------------------------
 
 // Counters of a launch.
-enum { kTileFirst = 0, kTileLater = 1, kTileQueue = 2, kTileRest = 3, kTileCounters = 4 };
+enum { kTileFirst = 0, kTileLater = 1, kTileQueue = 2, kTileRest = 3, kTileOutside = 4, kTileCounters = 8 };
 
 // One warp per bundle: deals the bundle's particles, in the order of their
 // cell step along x, into tiles of 32 (a tile ends early only where it would
@@ -27,17 +27,21 @@ enum { kTileFirst = 0, kTileLater = 1, kTileQueue = 2, kTileRest = 3, kTileCount
 // tile in slot s are idx[32 s .. 32 s + 31] (-1: none).  Slots follow the
 // particles (those before the bundle / 32, plus cmax per bundle, which covers the
 // tiles that are not full), so sums kept per slot do not depend on timing; the
-// list of the slots in use does (bundles append to it as they finish).  Tiles
-// whose first or 16th particle has a cutoff above `wide` are listed from the
-// front, the others from the back: the costly ones start first, so that a launch of
-// few tiles per warp does not end on them (260K particles, mixed: see the
-// kernel below).  NR: cell rows of a bundle, at most; the starts of the next 32
+// list of the slots in use does (bundles append to it as they finish).  Full
+// tiles whose first or 16th particle has a cutoff above `wide` are listed from
+// the front, the others from the back: the costly ones start first, so that a
+// launch of few tiles per warp does not end on them (a tile of the vapor, cut
+// off at its longest, has a wide cutoff but few candidates).  Coordinates
+// outside the box are looked for in the boundary cells, the only ones that may
+// hold them.  NR: cell rows of a bundle, at most; the starts of the next 32
 // steps are loaded while these are dealt.
 template <typename R, int NR>
-__global__ void __launch_bounds__(128) k_tile_cut(const int32_t* __restrict__ start, const R* __restrict__ rc, R wide,
-                                                  int nx, int ny, int nz, TileCfg cfg, int32_t* __restrict__ idx,
-                                                  int32_t* __restrict__ list, int32_t* __restrict__ counters,
-                                                  int64_t nslot) {
+__global__ void __launch_bounds__(128) k_tile_cut(const int32_t* __restrict__ start,
+                                                  const typename RT<R>::R4* __restrict__ pos,
+                                                  const R* __restrict__ rc, R wide, Grid<R> g, TileCfg cfg,
+                                                  int32_t* __restrict__ idx, int32_t* __restrict__ list,
+                                                  int32_t* __restrict__ counters, int64_t nslot) {
+  const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const int b = blockIdx.x * 4 + (threadIdx.x >> 5);
@@ -53,8 +57,14 @@ __global__ void __launch_bounds__(128) k_tile_cut(const int32_t* __restrict__ st
   }
   const int plane = __ldg(start + nx * ny * z0);
   int row[NR];
+  unsigned outer = 0;  // rows of boundary cells
 #pragma unroll
-  for (int r = 0; r < NR; ++r) row[r] = nx * (y0 + r % nr_y + ny * (z0 + r / nr_y));
+  for (int r = 0; r < NR; ++r) {
+    const int y = y0 + r % nr_y, z = z0 + r / nr_y;
+    row[r] = nx * (y + ny * z);
+    if (y == 0 || y == ny - 1 || z == 0 || z == nz - 1) outer |= 1u << r;
+  }
+  bool outside = false;
   int from[NR], to[NR];  // the particles of the lane's cells
   auto load = [&](int x) {
 #pragma unroll
@@ -102,9 +112,16 @@ __global__ void __launch_bounds__(128) k_tile_cut(const int32_t* __restrict__ st
     S += __shfl_sync(full, s, 31);
 #pragma unroll
     for (int r = 0; r < NR; ++r)
-      for (int k = k0[r]; k < k1[r]; ++k, ++place)
+      for (int k = k0[r]; k < k1[r]; ++k, ++place) {
         if (place < lim) idx[place] = k;
+        if ((outer >> r & 1u) || x == 0 || x == nx - 1) {
+          const auto q = ldg4(pos + k);
+          outside = outside || !(q.x >= (R)0 && q.x < g.L[0] && q.y >= (R)0 && q.y < g.L[1] && q.z >= (R)0 &&
+                                 q.z < g.L[2]);
+        }
+      }
   }
+  if (outside) counters[kTileOutside] = 1;
   if (S + lane < B && S + lane < lim) idx[S + lane] = -1;
   __syncwarp();
   const int nt = min(B, lim) >> 5;
@@ -114,7 +131,7 @@ __global__ void __launch_bounds__(128) k_tile_cut(const int32_t* __restrict__ st
     if (t < nt) {
       const volatile int32_t* m = idx + 32 * t;  // written by other lanes of this warp
       const int i0 = m[0], i1 = m[15];
-      is_wide = rc[max(i0, 0)] > wide || rc[max(i1, 0)] > wide;
+      is_wide = m[31] >= 0 && (rc[i0] > wide || rc[i1] > wide);
     }
     const unsigned w = __ballot_sync(full, t < nt && is_wide), v = __ballot_sync(full, t < nt && !is_wide);
     int at = 0;
@@ -241,7 +258,7 @@ __device__ __forceinline__ void tile_partials(double e, double w, int np, double
 template <typename R>
 constexpr int tile_warps() {
   constexpr int fit = 227 * 1024 / (int)sizeof(TileSmem<R>);
-  constexpr int most = sizeof(R) == 4 ? 20 : 8;
+  constexpr int most = sizeof(R) == 4 ? 16 : 8;
   return fit < most ? fit : most;
 }
 
@@ -260,6 +277,7 @@ __global__ void __launch_bounds__(32 * tile_warps<R>(), 1) k_forces_tiles(
   const int lane = threadIdx.x & 31;
   const Grid<R>& g = a.g;
   const int nfirst = __ldg(counters + kTileFirst), ntile = nfirst + __ldg(counters + kTileLater);
+  if (__ldg(counters + kTileOutside)) return;  // all tiles go to the row walk
   auto take = [&]() {
     int t = 0;
     if (lane == 0) t = atomicAdd(counters + kTileQueue, 1);
@@ -329,19 +347,22 @@ __global__ void __launch_bounds__(32 * tile_warps<R>(), 1) k_forces_tiles(
   }
 }
 
-// The tiles that the filter does not serve, by the row walk.
+// The tiles that the filter does not serve, by the row walk: those left over,
+// or all of them if a coordinate lies outside the box.
 template <typename R, bool TYPED, bool EW>
 __global__ void __launch_bounds__(64) k_forces_rest(const typename RT<R>::R4* __restrict__ pos,
                                                     const R* __restrict__ rc, const int32_t* __restrict__ start,
                                                     ForceArgs<R> a, const int32_t* __restrict__ idx,
-                                                    const int32_t* __restrict__ rest,
+                                                    const int32_t* __restrict__ list, const int32_t* __restrict__ rest,
                                                     const int32_t* __restrict__ counters,
                                                     typename RT<R>::R4* __restrict__ force, double* __restrict__ part,
                                                     int64_t nslot) {
   constexpr bool kX2 = sizeof(R) == 4;
-  const int n = __ldg(counters + kTileRest), lane = threadIdx.x & 31;
+  const bool all = __ldg(counters + kTileOutside) != 0;
+  const int nfirst = __ldg(counters + kTileFirst), lane = threadIdx.x & 31;
+  const int n = all ? nfirst + __ldg(counters + kTileLater) : __ldg(counters + kTileRest);
   for (int k = blockIdx.x * 2 + (threadIdx.x >> 5); k < n; k += gridDim.x * 2) {
-    const int slot = __ldg(rest + k), i = __ldg(idx + 32 * (int64_t)slot + lane);
+    const int slot = __ldg(!all ? rest + k : (k < nfirst ? list + k : list + (nslot - 1 - (k - nfirst)))), i = __ldg(idx + 32 * (int64_t)slot + lane);
     double e = 0, w = 0;
     int np = 0;
     if (i >= 0)
@@ -403,8 +424,8 @@ int tile_forces(dcm_ctx* ctx, bool typed, bool ew, int64_t n, const typename RT<
   DCM_CUDA_TRY(ctx, cudaMemsetAsync(counters, 0, kTileCounters * sizeof(int32_t), st));
   if (part) DCM_CUDA_TRY(ctx, cudaMemsetAsync(part, 0, 3 * sizeof(double) * (size_t)tp.slots, st));
   auto kc = tp.cfg.ry * tp.cfg.rz <= 4 ? k_tile_cut<R, 4> : k_tile_cut<R, 16>;
-  DCM_LAUNCH(ctx, kc, (unsigned)((nb + 3) / 4), 128, 0, st, cell_start, rc, (R)(1.2 * ctx->p.rc_min), (int)ctx->nc[0],
-             (int)ctx->nc[1], (int)ctx->nc[2], tp.cfg, idx, list, counters, tp.slots);
+  DCM_LAUNCH(ctx, kc, (unsigned)((nb + 3) / 4), 128, 0, st, cell_start, pos, rc, (R)(1.2 * ctx->p.rc_min), a.g, tp.cfg,
+             idx, list, counters, tp.slots);
   auto k = typed ? (ew ? k_forces_tiles<R, true, true> : k_forces_tiles<R, true, false>)
                  : (ew ? k_forces_tiles<R, false, true> : k_forces_tiles<R, false, false>);
   auto kr = typed ? (ew ? k_forces_rest<R, true, true> : k_forces_rest<R, true, false>)
@@ -417,7 +438,7 @@ int tile_forces(dcm_ctx* ctx, bool typed, bool ew, int64_t n, const typename RT<
   DCM_LAUNCH(ctx, k, grid, 32 * warps, smem, st, pos, rc, cell_start, a, tp.cfg, idx, list, rest, counters, force,
              part, tp.slots);
   DCM_LAUNCH(ctx, kr, (unsigned)std::min<int64_t>((tp.slots + 1) / 2, 8 * sms), 64, 0, st, pos, rc, cell_start, a, idx,
-             rest, counters, force, part, tp.slots);
+             list, rest, counters, force, part, tp.slots);
   return check_launch(ctx, "tile_forces");
 }
 

@@ -37,8 +37,10 @@
 // staged as x_j - L; a tile whose cells reach past +L moves its whole frame by
 // -L (x_i - L and, inside the box, x_j - L, both exact because the tile and
 // everything within its cutoffs lie in the upper half).  A tile that reaches
-// past both ends of an axis, or holds or meets coordinates outside the box
-// (or NaN), is left to the per-particle row walk.
+// past both ends of an axis is left to the per-particle row walk, and so is
+// every tile of a system in which a coordinate lies outside the box (or is
+// NaN): binning puts such particles into the boundary cells, where the kernel that
+// cuts the tiles looks for them.
 #pragma once
 
 #include <cuda_fp16.h>
@@ -247,16 +249,13 @@ __device__ __forceinline__ bool tile_candidates(TileSmem<R>& sm, const typename 
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const float Lf[3] = {(float)g.L[0], (float)g.L[1], (float)g.L[2]};
-  bool in_box = true;
   float lo[3], hi[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    in_box = in_box && xi[d] >= (R)0 && xi[d] < g.L[d];
     const float v = (float)xi[d];
     lo[d] = active ? v : Lf[d];
     hi[d] = active ? v : 0.f;
   }
-  if (!__all_sync(full, !active || in_box)) return false;
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     lo[d] = warp_min_nonneg(lo[d]);
@@ -269,7 +268,7 @@ __device__ __forceinline__ bool tile_candidates(TileSmem<R>& sm, const typename 
   const float ie[3] = {(float)g.inv_edge_x, (float)g.inv_edge, (float)g.inv_edge};
   const float rs = rmax * 1.000004f;
   int u0[3], u1[3];
-  bool upper[3], cross[3], ok = true, edge = false;  // edge: boundary cells, the only ones that may hold coordinates outside the box
+  bool upper[3], cross[3], ok = true;
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     const float eps = 5e-4f + 4e-7f * Lf[d] * ie[d];
@@ -277,7 +276,6 @@ __device__ __forceinline__ bool tile_candidates(TileSmem<R>& sm, const typename 
     u1[d] = (int)floorf((hi[d] + rs) * ie[d] + eps);
     upper[d] = u1[d] >= g.n[d];
     cross[d] = upper[d] || u0[d] < 0;
-    edge = edge || u0[d] <= 0 || u1[d] >= g.n[d] - 1;
     // one image per axis, and a frame moved by -L only where that is exact
     ok = ok && !(upper[d] && u0[d] < 0) && !(upper[d] && !(lo[d] - rs >= 0.5f * Lf[d])) && u0[d] >= -g.n[d] &&
          u1[d] < 2 * g.n[d];
@@ -300,6 +298,7 @@ __device__ __forceinline__ bool tile_candidates(TileSmem<R>& sm, const typename 
   // for the fullest list of each chunk).
   const int nyr = u1[1] - u0[1] + 1, nzr = u1[2] - u0[2] + 1, nseg = cross[0] ? 2 : 1;
   const int nyh = (nyr + 1) >> 1, nhalf = nyh * nzr * nseg;
+  const bool images = cross[0] || cross[1] || cross[2];
   // the lane's own row among the items, on the side inside the box
   int own = -1, own_half = 0;
   if (active && row_y >= u0[1] && row_y <= u1[1] && row_z >= u0[2] && row_z <= u1[2]) {
@@ -396,15 +395,9 @@ __device__ __forceinline__ bool tile_candidates(TileSmem<R>& sm, const typename 
         if (most > 24)
           for (int q = 24; q < most; q += 8) copy_if<sizeof(R4), 0>(dst + (uint32_t)(q * sizeof(R4)), p + q, nn - q);
       }
-      if (edge) {  // look for coordinates outside the box, then shift the image rows in place
+      if (images) {  // shift the image rows in place
         copy_async_wait();
         __syncwarp();
-        bool in = true;
-        for (int q = staged + lane; q < staged + take; q += 32) {
-          const R4 p = sm.pos[q];
-          in = in && p.x >= (R)0 && p.x < g.L[0] && p.y >= (R)0 && p.y < g.L[1] && p.z >= (R)0 && p.z < g.L[2];
-        }
-        if (!__all_sync(full, in)) return false;
         for (unsigned rows = __ballot_sync(full, im != 0 && len > 0); rows; rows &= rows - 1) {
           const int src = __ffs(rows) - 1;
           const int nn = __shfl_sync(full, len, src), tt = __shfl_sync(full, to, src);

@@ -1,8 +1,8 @@
 """The tiled force kernels (tensor-core pair filter) against the row walk.
 
 DCM_FORCE_AUTO runs over tiles of 32 particles where they serve (boxes of at
-least 4 rc_max, at least 4,000 particles); DCM_FORCE_PACKED and
-DCM_FORCE_THREAD run the row walk.  Both accept the same pairs and evaluate each
+least 4 rc_max, more than 32,768 particles in the mixed form); DCM_FORCE_PACKED
+and DCM_FORCE_THREAD run the row walk.  Both accept the same pairs and evaluate each
 with the same roundings, and differ in the order of the sums only.
 
 Tolerances, from the order of the sums: a particle's force is a sum of partial
@@ -71,12 +71,12 @@ def forces(D, box, pos, rc, types=None, prec="mixed", **kw):
 CASES = [
     # box, cell edges, cutoffs, two types, shift: bundles with a last single
     # row, rows of one cell step, several cells per rc, cells as wide as rc
-    ((36.0, 36.0, 36.0), dict(), "ramp", False, 0),
-    ((25.5, 31.5, 40.5), dict(lx=0.5), "ramp", False, 1),
-    ((24.0, 25.5, 61.5), dict(lx=0.75), "mixed", True, 1),
-    ((27.0, 24.0, 30.0), dict(l=0.75), "ramp", True, 0),
-    ((30.0, 30.0, 27.0), dict(l=3.0), "uniform", False, 1),
-    ((96.0, 24.0, 24.0), dict(lx=0.5), "mixed", False, 0),
+    ((48.0, 45.0, 51.0), dict(), "ramp", False, 0),
+    ((25.5, 64.5, 70.5), dict(lx=0.5), "ramp", False, 1),
+    ((24.0, 61.5, 75.0), dict(lx=0.75), "mixed", True, 1),
+    ((48.0, 46.5, 49.5), dict(l=0.75), "ramp", True, 0),
+    ((48.0, 51.0, 45.0), dict(l=3.0, h=1.5), "uniform", False, 1),
+    ((192.0, 24.0, 25.5), dict(lx=0.5), "mixed", False, 0),
 ]
 
 
@@ -86,7 +86,7 @@ def test_tiles_equal_the_row_walk(D, box, edges, kind, typed, shift, prec):
     pos = lattice(box, 3)
     rng = np.random.default_rng(4)
     rc = cutoffs(pos, box, kind, rng)
-    assert len(pos) >= 4000
+    assert len(pos) > 32768
     kw = dict(edges, shift_energy=shift)
     types = None
     if typed:
@@ -109,7 +109,7 @@ def test_tiles_crowded_cells_and_empty_regions(D):
     """One cell with hundreds of particles (several full tiles from one cell
     step), everything else a thin gas: tiles end at their longest, lists
     overflow their chunk many times."""
-    box = (60.0, 30.0, 24.0)
+    box = (96.0, 60.0, 60.0)
     rng = np.random.default_rng(8)
     g = np.stack(np.meshgrid(*[np.arange(9)] * 3, indexing="ij"), -1).reshape(-1, 3)
     clump = np.array([30.1, 15.1, 12.1]) + 0.15 * g + rng.uniform(-0.03, 0.03, (len(g), 3))
@@ -120,7 +120,7 @@ def test_tiles_crowded_cells_and_empty_regions(D):
     pos = np.concatenate([clump, gas, fill]).astype(np.float32)
     pos = pos[rng.permutation(len(pos))]
     rc = rng.choice([3.0, 6.0], len(pos))
-    assert len(pos) >= 4000
+    assert len(pos) > 32768
     F0, t0 = forces(D, box, pos, rc, force_kernel=D.DCM_FORCE_PACKED, lx=0.5)
     F1, t1 = forces(D, box, pos, rc, lx=0.5)
     assert t1[2] == t0[2]
@@ -128,11 +128,11 @@ def test_tiles_crowded_cells_and_empty_regions(D):
     assert np.abs(F1 - F0)[:, :3].max() <= 1e-6 * scale
 
 
-@pytest.mark.parametrize("bad", [np.nan, np.inf, -3.0, 41.0, 1e30])
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -3.0, 50.0, 1e30])
 def test_tiles_coordinates_outside_the_box(D, bad):
     """A coordinate that is not in the box sends its own tile and every tile
     that meets it to the row walk: same NaN set, same values elsewhere."""
-    box = (36.0, 30.0, 30.0)
+    box = (48.0, 45.0, 48.0)
     pos = lattice(box, 5)
     rng = np.random.default_rng(6)
     for k in rng.choice(len(pos), 7, replace=False):
