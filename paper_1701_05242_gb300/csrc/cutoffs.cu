@@ -11,7 +11,7 @@ namespace dcm {
 template <typename R>
 __device__ __forceinline__ void centre_coord(R x, R h, R inv_h, int& k, R& t) {
   R q = floor(x * inv_h - (R)0.5);
-  k = (int)q;
+  k = (int)fmin(fmax(q, (R)-1e9), (R)1e9);  // room for the steps below (NaN: -1e9)
   if (((R)k + (R)0.5) * h > x)
     --k;
   else if (((R)k + (R)1.5) * h <= x)
@@ -30,13 +30,20 @@ __global__ void k_cutoffs(int64_t n, const typename RT<R>::R4* __restrict__ pos,
   centre_coord<R>(p.x, h, inv_h, kx, tx);
   centre_coord<R>(p.y, h, inv_h, ky, ty);
   centre_coord<R>(p.z, h, inv_h, kz, tz);
-  // periodic wrap (a true modulo, so positions outside the box stay in range)
-  auto wrapk = [](int k, int n) { k %= n; return k < 0 ? k + n : k; };
+  // periodic wrap: k is -1 .. n - 1 inside the box; a true modulo elsewhere, so
+  // that positions outside the box stay in range
+  auto wrapk = [](int k, int n) {
+    if (k >= 0 && k < n) return k;
+    if (k == -1) return n - 1;
+    if (k == n) return 0;
+    k %= n;
+    return k < 0 ? k + n : k;
+  };
   int x0 = wrapk(kx, nx), x1 = wrapk(kx + 1, nx);
   int y0 = wrapk(ky, ny), y1 = wrapk(ky + 1, ny);
   int z0 = wrapk(kz, nz), z1 = wrapk(kz + 1, nz);
   auto at = [&](int x, int y, int z) {
-    R v = D[x + (int64_t)nx * (y + (int64_t)ny * z)];
+    R v = __ldg(D + (x + nx * (y + ny * z)));  // fewer than 2^31 boxes
     return v < r_grid ? v : r_grid;
   };
   // nested linear interpolation: a + t (b - a)
@@ -48,7 +55,9 @@ __global__ void k_cutoffs(int64_t n, const typename RT<R>::R4* __restrict__ pos,
   R c0 = lerp(c00, c10, ty), c1 = lerp(c01, c11, ty);
   R delta = lerp(c0, c1, tz);
   R r;
-  if (ramp > (R)0) {
+  if (ramp > (R)0 && delta >= (R)1.001 * ramp) {
+    r = rc_min;  // what the ramp gives there, without its division (the bulk of the liquid)
+  } else if (ramp > (R)0) {
     r = rc_max - (rc_max - rc_min) * delta / ramp;
     r = r < rc_min ? rc_min : (r > rc_max ? rc_max : r);
   } else {

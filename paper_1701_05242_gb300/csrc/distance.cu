@@ -12,30 +12,16 @@
 // whose update can differ from the previous sweep's, so the iterates are
 // those of full Jacobi sweeps while the work follows the moving front (the
 // paper's queue Q); the MPI_Allreduce of the paper's version becomes the
-// queue length in device memory.  dcm_distance launches one kernel per sweep
-// and checks convergence on the host every eight sweeps; the timestep runs
-// every sweep in one cooperative launch with a grid barrier between sweeps
-// (no host wait), until a sweep changes nothing or iter_max sweeps have run.
+// queue length in device memory.  The initial values and sweep 0 are one pass
+// over the grid, the later sweeps one cooperative launch with a grid barrier
+// between them, until a sweep changes nothing or iter_max sweeps have run;
+// dcm_distance then reads the outcome on the host, the timestep does not.
 #include <algorithm>
 
 #include "dcm_internal.cuh"
 #include "grid_sync.cuh"
 
 namespace dcm {
-
-template <typename R>
-__global__ void k_dist_init(const uint8_t* __restrict__ s, const uint8_t* __restrict__ iface, int64_t nbox,
-                            R* __restrict__ D0, R* __restrict__ D1, uint8_t* __restrict__ fixed0,
-                            int32_t* __restrict__ stamp) {
-  int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= nbox) return;
-  bool z = !s[b] || iface[b];
-  R v = z ? (R)0 : RT<R>::inf();
-  D0[b] = v;
-  D1[b] = v;
-  fixed0[b] = (uint8_t)z;
-  stamp[b] = -1;
-}
 
 // Godunov upwind update of |grad d| = 1 with spacing h from the three axis
 // minima a (any order).  Returns +inf if all are +inf.
@@ -61,22 +47,46 @@ __device__ __forceinline__ R godunov3(R a0, R a1, R a2, R h) {
 }
 
 // Queue the high-density boxes among b and its six neighbours for sweep it+1
-// (each box once: stamp holds the last sweep a box was queued for).
-__device__ __forceinline__ void dist_push(int64_t b, int x, int y, int z, int nx, int ny, int nz,
+// (each box once: stamp holds the last sweep a box was queued for).  Called by
+// every lane of a warp (push: whether this lane's box
+// changed): the lanes take their queue places together, one atomic per warp and
+// neighbour (the queue of a 51,200-box front takes about 200,000 entries per
+// sweep, each of which was an atomic on the queue's length).
+__device__ __forceinline__ void dist_push(bool push, int b, int x, int y, int z, int nx, int ny, int nz,
                                           const uint8_t* __restrict__ fixed0, int32_t* __restrict__ stamp,
                                           int32_t* __restrict__ qout, int32_t* __restrict__ qlen, int it) {
-  const int64_t nxy = (int64_t)nx * ny;
-  int64_t nb[7] = {b,
-                   x == 0 ? b + nx - 1 : b - 1,
-                   x == nx - 1 ? b - x : b + 1,
-                   y == 0 ? b + (int64_t)(ny - 1) * nx : b - nx,
-                   y == ny - 1 ? b - (int64_t)y * nx : b + nx,
-                   z == 0 ? b + (int64_t)(nz - 1) * nxy : b - nxy,
-                   z == nz - 1 ? b - (int64_t)z * nxy : b + nxy};
+  const unsigned warp = 0xffffffffu;
+  if (!__any_sync(warp, push)) return;
+  const int nxy = nx * ny;  // fewer than 2^31 boxes in all
+  const int nb[7] = {b,
+                     x == 0 ? b + nx - 1 : b - 1,
+                     x == nx - 1 ? b - x : b + 1,
+                     y == 0 ? b + (ny - 1) * nx : b - nx,
+                     y == ny - 1 ? b - y * nx : b + nx,
+                     z == 0 ? b + (nz - 1) * nxy : b - nxy,
+                     z == nz - 1 ? b - z * nxy : b + nxy};
+  bool take[7];
+#pragma unroll
+  for (int k = 0; k < 7; ++k) take[k] = push && !fixed0[nb[k]];
+#pragma unroll
+  for (int k = 0; k < 7; ++k)
+    if (take[k]) take[k] = atomicExch(stamp + nb[k], it + 1) != it + 1;
+  const int lane = threadIdx.x & 31;
+  unsigned m[7];
+  int total = 0;
+#pragma unroll
   for (int k = 0; k < 7; ++k) {
-    int64_t q = nb[k];
-    if (fixed0[q]) continue;
-    if (atomicExch(stamp + q, it + 1) != it + 1) qout[atomicAdd(qlen + it + 1, 1)] = (int32_t)q;
+    m[k] = __ballot_sync(warp, take[k]);
+    total += __popc(m[k]);
+  }
+  if (!total) return;
+  int at = 0;
+  if (lane == 0) at = atomicAdd(qlen + it + 1, total);
+  at = __shfl_sync(warp, at, 0);
+#pragma unroll
+  for (int k = 0; k < 7; ++k) {
+    if (take[k]) qout[at + __popc(m[k] & ((1u << lane) - 1u))] = nb[k];
+    at += __popc(m[k]);
   }
 }
 
@@ -107,55 +117,65 @@ __device__ __forceinline__ bool dist_update(const R* Din, R* Dout, int64_t b, in
   return ch;
 }
 
-// Sweep 0 over the whole grid.  Grid-stride over (row, chunk) work items.
+// Initial values and sweep 0 in one pass: before sweep 0 a box is 0 (low
+// density or interface) or +inf, so the sweep reads the bytes of s and iface
+// instead of the first iterate.  A thread marches along z.  HBM-bound: 33 MB read,
+// 211 MB written for 16.4M boxes (60 + 122 us as two passes).
 template <typename R>
-__global__ void k_dist_sweep0(const R* __restrict__ Din, R* __restrict__ Dout, int nx, int ny, int nz, R h, R r_grid,
-                              const uint8_t* __restrict__ fixed0, int32_t* __restrict__ stamp,
-                              int32_t* __restrict__ qout, int32_t* __restrict__ qlen, int32_t* __restrict__ flags) {
-  const int chunks = (nx + blockDim.x - 1) / blockDim.x;
-  const int64_t items = (int64_t)ny * nz * chunks;
-  bool changed = false;
-  for (int64_t w = blockIdx.x; w < items; w += gridDim.x) {
-    int yz = (int)(w / chunks);
-    int x = (int)(w - (int64_t)yz * chunks) * blockDim.x + threadIdx.x;
-    if (x >= nx) continue;
-    int y = yz % ny, z = yz / ny;
-    int64_t b = x + (int64_t)nx * yz;
-    if (fixed0[b]) continue;  // interface / low-density boxes are fixed at 0 in both buffers
-    if (dist_update<R>(Din, Dout, b, x, y, z, nx, ny, nz, h, r_grid)) {
-      changed = true;
-      dist_push(b, x, y, z, nx, ny, nz, fixed0, stamp, qout, qlen, 0);
+__global__ void __launch_bounds__(256) k_dist_first(const uint8_t* __restrict__ s, const uint8_t* __restrict__ iface,
+                                                    R* __restrict__ D0, R* __restrict__ D1, int nx, int ny, int nz,
+                                                    int zc, R h, R r_grid, uint8_t* __restrict__ fixed0) {
+  const int x = blockIdx.x * 32 + (threadIdx.x & 31), y = blockIdx.y * 8 + (threadIdx.x >> 5);
+  if (x >= nx || y >= ny) return;
+  const int z0 = blockIdx.z * zc, z1 = min(z0 + zc, nz);
+  const int nxy = nx * ny, col = x + nx * y;
+  auto zero = [&](int b) { return __ldg(s + b) == 0 || __ldg(iface + b) != 0; };
+  const int xm = x == 0 ? nx - 1 : -1, xp = x == nx - 1 ? 1 - nx : 1;
+  const int ym = y == 0 ? (ny - 1) * nx : -nx, yp = y == ny - 1 ? -(ny - 1) * nx : nx;
+  bool below = zero(col + nxy * (z0 == 0 ? nz - 1 : z0 - 1)), here = zero(col + nxy * z0);
+  for (int z = z0; z < z1; ++z) {
+    const int b = col + nxy * z;
+    const bool above = zero(col + nxy * (z == nz - 1 ? 0 : z + 1));
+    const R inf = RT<R>::inf(), cur = here ? (R)0 : inf;
+    R v = cur;
+    if (!here) {
+      const R a0 = zero(b + xm) || zero(b + xp) ? (R)0 : inf, a1 = zero(b + ym) || zero(b + yp) ? (R)0 : inf,
+              a2 = below || above ? (R)0 : inf;
+      const R d = godunov3<R>(a0, a1, a2, h);
+      v = d < cur && d <= r_grid ? d : cur;
     }
+    D0[b] = cur;
+    D1[b] = v;
+    fixed0[b] = (uint8_t)here;
+    below = here;
+    here = above;
   }
-  if (__any_sync(0xffffffffu, changed) && (threadIdx.x & 31) == 0) flags[0] = 1;
 }
 
-// Sweep it >= 1 over its queue (grid-stride; an empty queue means converged).
+// The queue of sweep 1: the boxes that sweep 0 changed and their neighbours.
+// Apart from the pass above, whose warps it would hold up at every front box.
 template <typename R>
-__global__ void k_dist_sweep_queue(const R* __restrict__ Din, R* __restrict__ Dout, int nx, int ny, int nz, R h,
-                                   R r_grid, const uint8_t* __restrict__ fixed0, int32_t* __restrict__ stamp,
-                                   const int32_t* __restrict__ qin, int32_t* __restrict__ qout,
-                                   int32_t* __restrict__ qlen, int32_t* __restrict__ flags, int it) {
-  const int32_t n = qlen[it];
-  bool changed = false;
-  const int64_t nxy = (int64_t)nx * ny;
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
-    int64_t b = qin[k];
-    int x = (int)(b % nx), y = (int)((b / nx) % ny), z = (int)(b / nxy);
-    if (dist_update<R>(Din, Dout, b, x, y, z, nx, ny, nz, h, r_grid)) {
-      changed = true;
-      dist_push(b, x, y, z, nx, ny, nz, fixed0, stamp, qout, qlen, it);
-    }
+__global__ void __launch_bounds__(256) k_dist_queue0(const R* __restrict__ D1, int64_t nbox, int nx, int ny, int nz,
+                                                     const uint8_t* __restrict__ fixed0, int32_t* __restrict__ stamp,
+                                                     int32_t* __restrict__ qout, int32_t* __restrict__ qlen,
+                                                     int32_t* __restrict__ flags) {
+  const int64_t gs = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t b0 = (int64_t)blockIdx.x * blockDim.x; b0 < nbox; b0 += gs) {
+    const int64_t b = b0 + threadIdx.x;
+    // changed from +inf: finite and not fixed at 0
+    const bool changed = b < nbox && D1[b] > (R)0 && D1[b] < RT<R>::inf();
+    if (!__any_sync(0xffffffffu, changed)) continue;
+    const int x = (int)(b % nx), y = (int)((b / nx) % ny), z = (int)(b / ((int64_t)nx * ny));
+    dist_push(changed, (int)b, x, y, z, nx, ny, nz, fixed0, stamp, qout, qlen, 0);
+    if ((threadIdx.x & 31) == 0) flags[0] = 1;
   }
-  if (__any_sync(0xffffffffu, changed) && (threadIdx.x & 31) == 0) flags[it] = 1;
 }
 
-// All sweeps in one cooperative launch (every block resident): sweep 0 over
-// the whole grid, then the queue sweeps, a bounded grid barrier after each,
-// until a sweep changes nothing or `budget` sweeps have run.  The same
-// iterates as one launch per sweep (bit for bit); the loop needs no host
-// check and launches nothing per sweep.  A barrier wait that runs past
-// budget_ns records DCM_ERR_TIMEOUT and ends the launch.
+// The sweeps after sweep 0 in one cooperative launch (every block resident):
+// each over its queue, a bounded grid barrier after it, until a sweep changes
+// nothing or `budget` sweeps have run.  The loop needs no host check and
+// launches nothing per sweep.  A barrier wait that runs past budget_ns records
+// DCM_ERR_TIMEOUT and ends the launch.
 template <typename R>
 __global__ void __launch_bounds__(256) k_dist_coop(R* D0, R* D1, int nx, int ny, int nz, R h, R r_grid,
                                                    const uint8_t* __restrict__ fixed0, int32_t* stamp, int32_t* q0,
@@ -163,26 +183,6 @@ __global__ void __launch_bounds__(256) k_dist_coop(R* D0, R* D1, int nx, int ny,
                                                    uint32_t* sync, int64_t budget_ns, int32_t* status) {
   const unsigned full = 0xffffffffu;
   const uint32_t expected = gridDim.x;
-  const int64_t nxy = (int64_t)nx * ny;
-  {
-    const int chunks = (nx + blockDim.x - 1) / blockDim.x;
-    const int64_t items = (int64_t)ny * nz * chunks;
-    bool changed = false;
-    for (int64_t w = blockIdx.x; w < items; w += gridDim.x) {
-      const int yz = (int)(w / chunks);
-      const int x = (int)(w - (int64_t)yz * chunks) * blockDim.x + threadIdx.x;
-      if (x >= nx) continue;
-      const int y = yz % ny, z = yz / ny;
-      const int64_t b = x + (int64_t)nx * yz;
-      if (fixed0[b]) continue;
-      if (dist_update<R, true>(D0, D1, b, x, y, z, nx, ny, nz, h, r_grid)) {
-        changed = true;
-        dist_push(b, x, y, z, nx, ny, nz, fixed0, stamp, q1, qlen, 0);
-      }
-    }
-    if (__any_sync(full, changed) && (threadIdx.x & 31) == 0) flags[0] = 1;
-  }
-  if (!grid_sync(sync, expected, budget_ns, status)) return;
   const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, gs = (int64_t)gridDim.x * blockDim.x;
   for (int it = 1; it < budget; ++it) {
     if (((volatile int32_t*)flags)[it - 1] == 0) break;  // the previous sweep changed nothing
@@ -191,31 +191,42 @@ __global__ void __launch_bounds__(256) k_dist_coop(R* D0, R* D1, int nx, int ny,
     const int32_t* qin = (it & 1) ? q1 : q0;
     int32_t* qout = (it & 1) ? q0 : q1;
     const int32_t n = ((volatile int32_t*)qlen)[it];
-    bool changed = false;
-    for (int64_t k = gt; k < n; k += gs) {
-      const int64_t b = __ldcg(qin + k);
-      const int x = (int)(b % nx), y = (int)((b / nx) % ny), z = (int)(b / nxy);
-      if (dist_update<R, true>(Din, Dout, b, x, y, z, nx, ny, nz, h, r_grid)) {
-        changed = true;
-        dist_push(b, x, y, z, nx, ny, nz, fixed0, stamp, qout, qlen, it);
+    bool any = false;
+    for (int64_t k = gt; k - (threadIdx.x & 31) < n; k += gs) {  // whole warps
+      bool changed = false;
+      int b = 0, x = 0, y = 0, z = 0;
+      if (k < n) {
+        b = __ldcg(qin + k);
+        const int yz = b / nx;
+        x = b - yz * nx;
+        z = yz / ny;
+        y = yz - z * ny;
+        changed = dist_update<R, true>(Din, Dout, b, x, y, z, nx, ny, nz, h, r_grid);
       }
+      any |= changed;
+      dist_push(changed, b, x, y, z, nx, ny, nz, fixed0, stamp, qout, qlen, it);
     }
-    if (__any_sync(full, changed) && (threadIdx.x & 31) == 0) flags[it] = 1;
+    if (__any_sync(full, any) && (threadIdx.x & 31) == 0) flags[it] = 1;
     if (!grid_sync(sync, expected, budget_ns, status)) return;
   }
 }
 
 // iters = 1 + index of the first sweep that changed nothing (or -1), and a
-// device status if the budget ran out.
-__global__ void k_dist_finish(const int32_t* flags, int sweeps, int32_t* iters, int32_t* status) {
+// device status if the budget ran out.  One warp; result (device, nullable)
+// gets the same number as iters.
+__global__ void k_dist_finish(const int32_t* flags, int sweeps, int32_t* iters, int32_t* result, int32_t* status) {
+  const int lane = threadIdx.x;
   int first = -1;
-  for (int k = 0; k < sweeps; ++k)
-    if (flags[k] == 0) {
-      first = k;
-      break;
-    }
-  if (iters) *iters = first >= 0 ? first + 1 : -1;
-  if (first < 0) raise_status(status, DCM_ERR_NOT_CONVERGED);
+  for (int k0 = 0; k0 < sweeps && first < 0; k0 += 32) {
+    const unsigned m = __ballot_sync(0xffffffffu, k0 + lane < sweeps && flags[k0 + lane] == 0);
+    if (m) first = k0 + __ffs(m) - 1;
+  }
+  if (lane == 0) {
+    const int v = first >= 0 ? first + 1 : -1;
+    if (iters) *iters = v;
+    if (result) *result = v;
+    if (first < 0) raise_status(status, DCM_ERR_NOT_CONVERGED);
+  }
 }
 
 template <typename R>
@@ -226,71 +237,54 @@ int distance_sweeps(dcm_ctx* ctx, const uint8_t* s, const uint8_t* iface, R* D, 
   R h = (R)ctx->p.h, rg = (R)ctx->p.r_grid;
   R* buf[2] = {D, (R*)ctx->D[1]};
   int32_t* q[2] = {ctx->dq[0], ctx->dq[1]};
-  unsigned nb = (unsigned)((nbox + 255) / 256);
-  int64_t items = (int64_t)ny * nz * ((nx + 127) / 128);
-  unsigned sg = (unsigned)std::min<int64_t>(items, 152 * 16);
-  const unsigned qg = 152 * 8;  // queue sweeps: grid-stride over the queue length read on the device
-  int iter_max = ctx->p.iter_max;
+  const int iter_max = ctx->p.iter_max;
+  // without a host check the budget is rounded up to an even number of sweeps,
+  // so that the last iterate is in D wherever the sweeps end
+  const int budget = host_check ? iter_max : iter_max + (iter_max & 1);
   DCM_CUDA_TRY(ctx, cudaMemsetAsync(ctx->flags, 0, sizeof(int32_t) * (size_t)(iter_max + 2), st));
   DCM_CUDA_TRY(ctx, cudaMemsetAsync(ctx->dqlen, 0, sizeof(int32_t) * (size_t)(iter_max + 2), st));
-  DCM_LAUNCH(ctx, k_dist_init<R>, nb, 256, 0, st, s, iface, nbox, buf[0], buf[1], ctx->dfixed, ctx->dstamp);
-  auto sweep = [&](int it) -> int {
-    if (it == 0)
-      DCM_LAUNCH(ctx, k_dist_sweep0<R>, sg, 128, 0, st, buf[0], buf[1], nx, ny, nz, h, rg, ctx->dfixed, ctx->dstamp,
-                 q[1], ctx->dqlen, ctx->flags);
-    else
-      DCM_LAUNCH(ctx, k_dist_sweep_queue<R>, qg, 256, 0, st, buf[it & 1], buf[(it + 1) & 1], nx, ny, nz, h, rg,
-                 ctx->dfixed, ctx->dstamp, q[it & 1], q[(it + 1) & 1], ctx->dqlen, ctx->flags, it);
-    return DCM_OK;
-  };
-  int done = 0;
+  DCM_CUDA_TRY(ctx, cudaMemsetAsync(ctx->dstamp, 0xff, sizeof(int32_t) * (size_t)nbox, st));
+  const int64_t cols = (int64_t)((nx + 31) / 32) * ((ny + 7) / 8);
+  const int zc = (int)std::max<int64_t>(1, std::min<int64_t>(64, (int64_t)nz * cols / (152 * 8)));
+  if ((ny + 7) / 8 > 65535 || (nz + zc - 1) / zc > 65535)
+    return set_error(ctx, DCM_ERR_CAPACITY, "distance sweeps: density grid too long");
+  DCM_LAUNCH(ctx, k_dist_first<R>, dim3((nx + 31) / 32, (ny + 7) / 8, (nz + zc - 1) / zc), 256, 0, st, s, iface, buf[0],
+             buf[1], nx, ny, nz, zc, h, rg, ctx->dfixed);
+  DCM_LAUNCH(ctx, k_dist_queue0<R>, (unsigned)std::min<int64_t>((nbox + 255) / 256, 152 * 8), 256, 0, st, buf[1], nbox,
+             nx, ny, nz, ctx->dfixed, ctx->dstamp, q[1], ctx->dqlen, ctx->flags);
+  auto kern = k_dist_coop<R>;
+  int per_sm = 0, sms = 0, dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, 0) != cudaSuccess || per_sm < 1)
+    return set_error(ctx, DCM_ERR_CUDA, "distance sweeps: occupancy query failed");
+  cudaLaunchConfig_t cfg = {};
+  // no more blocks than boxes to sweep: the barrier costs by the block
+  cfg.gridDim = dim3((unsigned)std::min<int64_t>((nbox + 255) / 256, std::min(per_sm, 4) * sms));
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = 0;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  DCM_CUDA_TRY(ctx, cudaMemsetAsync(ctx->coop_sync, 0, 4 * sizeof(uint32_t), st));
+  ++ctx->launches;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, kern, buf[0], buf[1], nx, ny, nz, h, rg, (const uint8_t*)ctx->dfixed,
+                                     ctx->dstamp, q[0], q[1], ctx->dqlen, ctx->flags, budget, ctx->coop_sync,
+                                     (int64_t)2000000000, ctx->status);
+  if (e != cudaSuccess) return set_error(ctx, DCM_ERR_CUDA, "distance sweeps: %s", cudaGetErrorString(e));
+  DCM_LAUNCH(ctx, k_dist_finish, 1, 32, 0, st, ctx->flags, budget, iters, host_check ? ctx->thr + 3 : nullptr,
+             ctx->status);
   if (host_check) {
-    // chunks of 8 sweeps, then look at the last flag of the chunk on the host
-    const int chunk = 8;
-    bool converged = false;
-    while (done < iter_max && !converged) {
-      int m = std::min(chunk, iter_max - done);
-      for (int k = 0; k < m; ++k, ++done) sweep(done);
-      DCM_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->host_status, ctx->flags + done - 1, sizeof(int32_t),
-                                        cudaMemcpyDeviceToHost, st));
-      DCM_CUDA_TRY(ctx, cudaStreamSynchronize(st));
-      converged = ctx->host_status[0] == 0;
-    }
-    DCM_LAUNCH(ctx, k_dist_finish, 1, 1, 0, st, ctx->flags, done, iters, ctx->status);
-    if (!converged) {
-      if (done & 1) DCM_CUDA_TRY(ctx, cudaMemcpyAsync(D, buf[1], sizeof(R) * nbox, cudaMemcpyDeviceToDevice, st));
+    DCM_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->host_status, ctx->thr + 3, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+    DCM_CUDA_TRY(ctx, cudaStreamSynchronize(st));
+    if (ctx->host_status[0] < 0) {
+      if (iter_max & 1) DCM_CUDA_TRY(ctx, cudaMemcpyAsync(D, buf[1], sizeof(R) * nbox, cudaMemcpyDeviceToDevice, st));
       check_launch(ctx, "distance_sweeps");
       return set_error(ctx, DCM_ERR_NOT_CONVERGED, "fast sweeping did not converge in %d sweeps", iter_max);
     }
-  } else {
-    // every sweep in one cooperative launch, until one changes nothing or
-    // the even budget iter_max (rounded up) runs out (the last iterate then
-    // in buf[0] = D); no host check
-    const int budget = iter_max + (iter_max & 1);
-    auto kern = k_dist_coop<R>;
-    int per_sm = 0, sms = 0, dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, 0) != cudaSuccess || per_sm < 1)
-      return set_error(ctx, DCM_ERR_CUDA, "distance sweeps: occupancy query failed");
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(std::min(per_sm, 4) * sms));
-    cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    DCM_CUDA_TRY(ctx, cudaMemsetAsync(ctx->coop_sync, 0, 4 * sizeof(uint32_t), st));
-    ++ctx->launches;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, kern, buf[0], buf[1], nx, ny, nz, h, rg, (const uint8_t*)ctx->dfixed,
-                                       ctx->dstamp, q[0], q[1], ctx->dqlen, ctx->flags, budget, ctx->coop_sync,
-                                       (int64_t)2000000000, ctx->status);
-    if (e != cudaSuccess) return set_error(ctx, DCM_ERR_CUDA, "distance sweeps: %s", cudaGetErrorString(e));
-    done = budget;
-    DCM_LAUNCH(ctx, k_dist_finish, 1, 1, 0, st, ctx->flags, done, iters, ctx->status);
   }
   return check_launch(ctx, "distance_sweeps");
 }
