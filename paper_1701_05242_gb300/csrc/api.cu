@@ -279,7 +279,7 @@ struct ScratchPlan {
            8 * 32 * adj_slots() + 8 * 48 + (skin > 0 ? 8 * n_max + 8 * (n_max / 32 + 16) + 4 * rsize * n_max + 32 : 0) +
            (min_component > 0 ? 9 * nbox + 4 * 80 : 0) + 13 * nbox + 4 * (flags + 2) + 4 * nblk +
            4 * tile_scratch_ints(n_max) + (tile_cap > 0 ? 4 * tile_ints(tile_cap) : 0) +
-           (segmentation ? 6 * rsize * nbox + 32 * ms_outer + 16 + 4 * (ms_outer + 2) : 0);
+           (segmentation ? 10 * rsize * nbox + 32 * ms_outer + 16 + 4 * (ms_outer + 2) : 0);
   }
 };
 
@@ -414,8 +414,8 @@ extern "C" int dcm_create(const dcm_params* p, dcm_ctx** out) {
   }
   if (p->segmentation) {
     alloc(&ctx->ms_u, s.rsize * s.nbox);
-    alloc(&ctx->ms_ub, s.rsize * s.nbox);
-    alloc(&ctx->ms_p, 3 * s.rsize * s.nbox);
+    alloc(&ctx->ms_ub, 2 * s.rsize * s.nbox);
+    alloc(&ctx->ms_p, 6 * s.rsize * s.nbox);
     alloc(&ctx->ms_w, s.rsize * s.nbox);
     alloc((void**)&ctx->ms_sums, 32 * (int64_t)p->ms_outer);
     alloc((void**)&ctx->ms_c, 16);

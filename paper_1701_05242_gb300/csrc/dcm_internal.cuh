@@ -148,8 +148,8 @@ struct dcm_ctx {
   int list_valid;
   // regularised segmentation (params.segmentation = 1)
   void* ms_u;               // nbox reals: relaxed volume u
-  void* ms_ub;              // nbox reals: extrapolated u
-  void* ms_p;               // 3 nbox reals: dual value per face
+  void* ms_ub;              // 2 x nbox reals: extrapolated u, old and new
+  void* ms_p;               // 2 x 3 nbox reals: dual value per face (x, then y, then z), old and new
   void* ms_w;               // nbox reals: data weights
   unsigned long long* ms_sums;  // [ms_outer][4]: n0, S0, n1, S1
   double* ms_c;             // [2]: phase values of the last outer iteration
