@@ -17,27 +17,33 @@ class LJForces(torch.autograd.Function):
     @staticmethod
     def forward(fctx, pos4, eps, sigma, rc, cell_start, ctx):
         n = pos4.shape[0]
-        D.dcm_set_lj(ctx, eps.detach().cpu().tolist(), sigma.detach().cpu().tolist())
+        nt = eps.shape[0]
+        if eps.device == sigma.device and eps.dtype == sigma.dtype:  # one wait for the device, not two
+            lj = torch.cat([eps.detach(), sigma.detach()]).tolist()
+        else:
+            lj = eps.detach().tolist() + sigma.detach().tolist()
+        D.dcm_set_lj(ctx, lj[:nt], lj[nt:])
         force = torch.empty_like(pos4)
-        totals = torch.zeros(3, dtype=torch.float64, device=pos4.device)
+        totals = torch.empty(3, dtype=torch.float64, device=pos4.device)
         D.dcm_forces(ctx, n, pos4.detach().contiguous(), rc, cell_start, force, totals)
         fctx.save_for_backward(pos4, rc, cell_start)
         fctx.dcm = ctx
-        fctx.nt = eps.shape[0]
+        fctx.nt = nt
         return force[:, :3], totals[0].to(pos4.dtype)
 
     @staticmethod
     def backward(fctx, gF, gE):
         pos4, rc, cell_start = fctx.saved_tensors
         n = pos4.shape[0]
-        A = torch.zeros_like(pos4)
-        if gF is not None:
+        if gF is None:
+            A = torch.zeros_like(pos4)
+        else:
+            A = torch.empty_like(pos4)  # the fourth column is not read
             A[:, :3] = gF
         dE = 0.0 if gE is None else float(gE)
-        G = torch.empty_like(pos4)
-        dpar = torch.zeros(2 * fctx.nt, dtype=torch.float64, device=pos4.device)
+        G = torch.empty_like(pos4)  # the adjoint writes zero into its fourth column
+        dpar = torch.empty(2 * fctx.nt, dtype=torch.float64, device=pos4.device)
         D.dcm_forces_backward(fctx.dcm, n, pos4.detach().contiguous(), rc, cell_start, A, dE, G, dpar)
-        G[:, 3] = 0
         nt = fctx.nt
         return G, dpar[:nt].to(pos4.dtype), dpar[nt:].to(pos4.dtype), None, None, None
 

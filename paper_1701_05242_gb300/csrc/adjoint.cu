@@ -33,6 +33,7 @@
 #include <algorithm>
 
 #include "forces_core.cuh"
+#include "pair_tiles.cuh"
 #include "tile_order.cuh"
 
 namespace dcm {
@@ -352,7 +353,7 @@ __global__ void __launch_bounds__(adj_block<R>()) k_adjoint(int64_t n, const typ
         // eps_p / sigma_p, the factor taken out of the d/dsigma terms
         const double f = TYPED ? 0.25 * (double)a.eps4[p] / sqrt((double)a.sig2[p]) : 1.0;
         part[(int64_t)p * nwarp + w] = (double)de;
-        part[(int64_t)(16 + p) * nwarp + w] = (double)ds * f;
+        part[(int64_t)(np + p) * nwarp + w] = (double)ds * f;
       }
     }
   }
@@ -505,6 +506,69 @@ __device__ __forceinline__ void adj_shell(const float4* __restrict__ pos, const 
   }
 }
 
+// Particle i's constants for the packed loop.
+__device__ __forceinline__ AdjRow adj_row(const ForceArgs<float>& a, int tk, float rck2) {
+  AdjRow k;
+#pragma unroll
+  for (int t = 0; t < 2; ++t) {
+    const int tc = t < a.ntypes ? t : a.ntypes - 1, p = tk * a.ntypes + tc;
+    k.sg[t] = a.sig2[p];
+    k.e24[t] = a.eps24[p];
+    k.cu[t] = k.cd[t] = 0.f;
+    if (a.shift && rck2 > 0.f) {
+      const float c2 = a.sig2[p] / rck2, c6 = c2 * c2 * c2, c12 = c6 * c6;
+      k.cu[t] = c12 - c6;
+      k.cd[t] = 12.f * c12 - 6.f * c6;
+    }
+  }
+  return k;
+}
+
+// The packed row walk of particle i; returns its type.
+__device__ __forceinline__ int adj_one_x2(const float4* __restrict__ pos, const float* __restrict__ rc,
+                                          const int32_t* __restrict__ start, const ForceArgs<float>& a,
+                                          const float4* __restrict__ A, float half_dlde, const BlockGrid& bg,
+                                          const int32_t* __restrict__ bmax, int64_t i, AdjAcc2& c) {
+  const float4 pi = __ldg(pos + i), ak = __ldg(A + i);
+  const float rck = clamp_cutoff<float>(__ldg(rc + i), a.rc_max), rck2 = rck * rck;
+  const float reach = reverse_reach<float>(pi, rck, a.rc_max, bg, bmax);
+  const int tk = type_of(pi.w, a.ntypes);
+  const AdjRow k = adj_row(a, tk, rck2);
+  adj_walk2<float>(
+      start, a.g, pi, rck, reach, (int)i,
+      [&](int lo, int hi, int self, float xi, float yi, float zi, float shx, float shy, float shz) {
+        if (shx == 0.f && shy == 0.f && shz == 0.f)
+          adj_range_x2<false>(pos, rc, A, lo, hi, self, xi, yi, zi, shx, shy, shz, rck2, a.rc_max, ak, half_dlde, k, c);
+        else
+          adj_range_x2<true>(pos, rc, A, lo, hi, self, xi, yi, zi, shx, shy, shz, rck2, a.rc_max, ak, half_dlde, k, c);
+      },
+      [&](int lo, int hi, int self, float xi, float yi, float zi, float shx, float shy, float shz) {
+        adj_shell(pos, rc, A, lo, hi, self, xi, yi, zi, shx, shy, shz, rck2, a.rc_max, ak, half_dlde, k, c);
+      });
+  return tk;
+}
+
+// A warp's parameter sums per type pair p (eps, then sigma), in FP32 across the
+// warp, into slot w of the partials.  mine: the lane holds a particle of type tk.
+__device__ __forceinline__ void adj_warp_partials(const ForceArgs<float>& a, bool mine, int tk, const AdjAcc2& c,
+                                                  double* __restrict__ part, int64_t nslot, int64_t w) {
+  const int nt = a.ntypes, np = nt * nt;
+  for (int p = 0; p < np; ++p) {
+    const bool own = mine && tk == p / nt, t1 = p % nt == 1;
+    const float2 de2 = t1 ? c.de[1] : c.de[0], ds2 = t1 ? c.ds[1] : c.ds[0];
+    float de = own ? de2.x + de2.y : 0.f, ds = own ? ds2.x + ds2.y : 0.f;
+    for (int o = 16; o > 0; o >>= 1) {
+      de += __shfl_xor_sync(0xffffffffu, de, o);
+      ds += __shfl_xor_sync(0xffffffffu, ds, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+      const double f = 0.25 * (double)a.eps4[p] / sqrt((double)a.sig2[p]);  // eps_p / sigma_p
+      part[(int64_t)p * nslot + w] = (double)de;
+      part[(int64_t)(np + p) * nslot + w] = (double)ds * f;
+    }
+  }
+}
+
 constexpr int kAdjX2Block = 64;
 
 __global__ void __launch_bounds__(kAdjX2Block) k_adjoint_x2(int64_t n, const float4* __restrict__ pos,
@@ -516,59 +580,130 @@ __global__ void __launch_bounds__(kAdjX2Block) k_adjoint_x2(int64_t n, const flo
                                                             const int32_t* __restrict__ bmax,
                                                             const int32_t* __restrict__ order) {
   const int64_t i = (int64_t)(order ? __ldg(order + blockIdx.x) : (int32_t)blockIdx.x) * blockDim.x + threadIdx.x;
-  const int nt = a.ntypes;
   AdjAcc2 c;
   int tk = 0;
   if (i < n) {
-    const float4 pi = __ldg(pos + i);
-    const float4 ak = __ldg(A + i);
-    const float rck = clamp_cutoff<float>(__ldg(rc + i), a.rc_max), rck2 = rck * rck;
-    const float reach = reverse_reach<float>(pi, rck, a.rc_max, bg, bmax);
-    tk = type_of(pi.w, nt);
-    AdjRow k;
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-      const int tc = t < nt ? t : nt - 1, p = tk * nt + tc;
-      k.sg[t] = a.sig2[p];
-      k.e24[t] = a.eps24[p];
-      k.cu[t] = k.cd[t] = 0.f;
-      if (a.shift && rck2 > 0.f) {
-        const float c2 = a.sig2[p] / rck2, c6 = c2 * c2 * c2, c12 = c6 * c6;
-        k.cu[t] = c12 - c6;
-        k.cd[t] = 12.f * c12 - 6.f * c6;
-      }
-    }
-    adj_walk2<float>(
-        start, a.g, pi, rck, reach, (int)i,
-        [&](int lo, int hi, int self, float xi, float yi, float zi, float shx, float shy, float shz) {
-          if (shx == 0.f && shy == 0.f && shz == 0.f)
-            adj_range_x2<false>(pos, rc, A, lo, hi, self, xi, yi, zi, shx, shy, shz, rck2, a.rc_max, ak, half_dlde,
-                                k, c);
-          else
-            adj_range_x2<true>(pos, rc, A, lo, hi, self, xi, yi, zi, shx, shy, shz, rck2, a.rc_max, ak, half_dlde, k,
-                               c);
-        },
-        [&](int lo, int hi, int self, float xi, float yi, float zi, float shx, float shy, float shz) {
-          adj_shell(pos, rc, A, lo, hi, self, xi, yi, zi, shx, shy, shz, rck2, a.rc_max, ak, half_dlde, k, c);
-        });
+    tk = adj_one_x2(pos, rc, start, a, A, half_dlde, bg, bmax, i, c);
     G[i] = make_float4(c.gx.x + c.gx.y, c.gy.x + c.gy.y, c.gz.x + c.gz.y, 0.f);
   }
-  if (part) {
-    const int64_t w = i >> 5;
-    for (int p = 0; p < nt * nt; ++p) {
-      const bool mine = i < n && tk == p / nt, t1 = p % nt == 1;
-      const float2 de2 = t1 ? c.de[1] : c.de[0], ds2 = t1 ? c.ds[1] : c.ds[0];
-      float de = mine ? de2.x + de2.y : 0.f, ds = mine ? ds2.x + ds2.y : 0.f;
-      for (int o = 16; o > 0; o >>= 1) {
-        de += __shfl_xor_sync(0xffffffffu, de, o);
-        ds += __shfl_xor_sync(0xffffffffu, ds, o);
+  if (part) adj_warp_partials(a, i < n, tk, c, part, nwarp, i >> 5);
+}
+
+// ----------------------------------------------------------------------------
+// The packed adjoint over tiles (pair_tiles.cuh): the filter keeps, per
+// particle, the candidates within its reverse reach, and the packed step above
+// runs on those alone (the row walk evaluates every candidate of the inner
+// window, forward and reverse, 2.1 per accepted pair, with 51% of the lanes
+// active).  Staged per candidate: position and type, upstream gradient, cutoff.
+// ----------------------------------------------------------------------------
+struct __align__(32) AdjRec {
+  float x, y, z, w, ax, ay, az, rc;
+};
+
+__global__ void __launch_bounds__(256) k_adj_records(int64_t n, const float4* __restrict__ pos,
+                                                     const float* __restrict__ rc, const float4* __restrict__ A,
+                                                     float rc_max, AdjRec* __restrict__ rec) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const float4 p = __ldg(pos + i), v = __ldg(A + i);
+  float4* q = reinterpret_cast<float4*>(rec + i);
+  q[0] = p;
+  q[1] = make_float4(v.x, v.y, v.z, clamp_cutoff<float>(__ldg(rc + i), rc_max));
+}
+
+// Largest cutoff of the 27 blocks around each block.
+__global__ void k_block_reach(const int32_t* __restrict__ bmax, BlockGrid bg, int32_t* __restrict__ reach) {
+  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  const int nx = bg.nb[0], ny = bg.nb[1], nz = bg.nb[2];
+  if (b >= nx * ny * nz) return;
+  const int x = b % nx, y = b / nx % ny, z = b / (nx * ny);
+  int m = 0;  // the order of nonnegative floats is that of their bits
+  for (int k = 0; k < 27; ++k) {
+    const int xx = (x + k % 3 - 1 + nx) % nx, yy = (y + k / 3 % 3 - 1 + ny) % ny, zz = (z + k / 9 - 1 + nz) % nz;
+    m = max(m, bmax[xx + nx * (yy + ny * zz)]);
+  }
+  reach[b] = m;
+}
+
+constexpr int kAdjTileWarps = 12;  // three per scheduler: the pair step wants up to 168 registers
+
+__global__ void __launch_bounds__(32 * kAdjTileWarps, 1) k_adjoint_tiles(
+    const AdjRec* __restrict__ rec, const int32_t* __restrict__ start, const __grid_constant__ ForceArgs<float> a,
+    TileCfg cfg, TileTable t, float half_dlde, BlockGrid bg, const int32_t* __restrict__ block_reach,
+    float4* __restrict__ G, double* __restrict__ part, int64_t nslot) {
+  const unsigned full = 0xffffffffu;
+  extern __shared__ __align__(32) unsigned char smem_raw[];
+  TileSmem<AdjRec>& sm = reinterpret_cast<TileSmem<AdjRec>*>(smem_raw)[threadIdx.x >> 5];
+  const int lane = threadIdx.x & 31;
+  const int nfirst = __ldg(t.counters + kTileFirst), ntile = nfirst + __ldg(t.counters + kTileLater);
+  if (__ldg(t.counters + kTileOutside)) return;  // all tiles go to the row walk
+  auto take = [&]() {
+    int q = 0;
+    if (lane == 0) q = atomicAdd(t.counters + kTileQueue, 1);
+    return q;
+  };
+  auto slot_of = [&](int q0) {
+    const int q = __shfl_sync(full, q0, 0);
+    return q < ntile ? __ldg(q < nfirst ? t.list + q : t.list + (nslot - 1 - (q - nfirst))) : -1;
+  };
+  int slot = slot_of(take());
+  while (slot >= 0) {
+    const int t1 = take();  // the next tile, asked for early
+    const int i = __ldg(t.idx + 32 * (int64_t)slot + lane);
+    const bool active = i >= 0;
+    const float4* self = reinterpret_cast<const float4*>(rec + max(i, 0));
+    const float4 pi = __ldg(self), ak = __ldg(self + 1);  // ak.w: the cutoff
+    const float rck = ak.w, rck2 = rck * rck;
+    const int b0 = block_coord(pi.x, bg.inv_be[0], bg.nb[0]), b1 = block_coord(pi.y, bg.inv_be[1], bg.nb[1]),
+              b2 = block_coord(pi.z, bg.inv_be[2], bg.nb[2]);
+    const float reach =
+        fmaxf(fminf(__int_as_float(__ldg(block_reach + b0 + bg.nb[0] * (b1 + bg.nb[1] * b2))), a.rc_max), rck);
+    const int tk = type_of(pi.w, a.ntypes);
+    const AdjRow k = adj_row(a, tk, rck2);
+    AdjAcc2 c;
+    float xi[3] = {pi.x, pi.y, pi.z};
+    const bool done = tile_candidates<float, AdjRec>(sm, rec, start, a.g, cfg, active, i, xi, rck, reach,
+                                                          [](const AdjRec& q) { return q.rc; }, []() {}, [&](int last) {
+      ListWalk l;
+      l.begin(shared_addr(&sm.list[0][lane]), last);
+      while (l.more()) {
+        const uint32_t q0 = l.next(5), q1 = l.next(5);
+        const float4 p0 = lds4(q0), a0 = lds4(q0 + 16), p1 = lds4(q1), a1 = lds4(q1 + 16);
+        adj_pair_x2(make_float2(p0.x - xi[0], p1.x - xi[0]), make_float2(p0.y - xi[1], p1.y - xi[1]),
+                    make_float2(p0.z - xi[2], p1.z - xi[2]), true, true, a0.w, a1.w, p0.w, p1.w, a0, a1, rck2, ak,
+                    half_dlde, k, c);
       }
-      if ((threadIdx.x & 31) == 0) {
-        const double f = 0.25 * (double)a.eps4[p] / sqrt((double)a.sig2[p]);  // eps_p / sigma_p
-        part[(int64_t)p * nwarp + w] = (double)de;
-        part[(int64_t)(16 + p) * nwarp + w] = (double)ds * f;
-      }
+    });
+    if (done) {
+      if (active) G[i] = make_float4(c.gx.x + c.gx.y, c.gy.x + c.gy.y, c.gz.x + c.gz.y, 0.f);
+      if (part) adj_warp_partials(a, active, tk, c, part, nslot, slot);
+    } else if (lane == 0) {
+      t.rest[atomicAdd(t.counters + kTileRest, 1)] = slot;
     }
+    slot = slot_of(t1);
+  }
+}
+
+// The tiles that the filter does not serve, by the row walk.
+__global__ void __launch_bounds__(64) k_adjoint_rest(const float4* __restrict__ pos, const float* __restrict__ rc,
+                                                     const int32_t* __restrict__ start, ForceArgs<float> a, TileTable t,
+                                                     const float4* __restrict__ A, float half_dlde,
+                                                     float4* __restrict__ G, double* __restrict__ part, int64_t nslot,
+                                                     BlockGrid bg, const int32_t* __restrict__ bmax) {
+  const bool all = __ldg(t.counters + kTileOutside) != 0;
+  const int nfirst = __ldg(t.counters + kTileFirst), lane = threadIdx.x & 31;
+  const int n = all ? nfirst + __ldg(t.counters + kTileLater) : __ldg(t.counters + kTileRest);
+  for (int q = blockIdx.x * 2 + (threadIdx.x >> 5); q < n; q += gridDim.x * 2) {
+    const int slot = __ldg(!all ? t.rest + q : (q < nfirst ? t.list + q : t.list + (nslot - 1 - (q - nfirst))));
+    const int i = __ldg(t.idx + 32 * (int64_t)slot + lane);
+    AdjAcc2 c;
+    int tk = 0;
+    if (i >= 0) {
+      tk = adj_one_x2(pos, rc, start, a, A, half_dlde, bg, bmax, i, c);
+      G[i] = make_float4(c.gx.x + c.gx.y, c.gy.x + c.gy.y, c.gz.x + c.gz.y, 0.f);
+    }
+    __syncwarp();
+    if (part) adj_warp_partials(a, i >= 0, tk, c, part, nslot, slot);
   }
 }
 
@@ -611,19 +746,7 @@ __global__ void __launch_bounds__(32 * kAdjWarps) k_adjoint_warp(
     const float reach = fmaxf(fminf(m, a.rc_max), rck);
     const float reach2s = reach * reach * 1.000004f;
     tk = type_of(pi.w, nt);
-    AdjRow k;
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-      const int tc = t < nt ? t : nt - 1, p = tk * nt + tc;
-      k.sg[t] = a.sig2[p];
-      k.e24[t] = a.eps24[p];
-      k.cu[t] = k.cd[t] = 0.f;
-      if (a.shift && rck2 > 0.f) {
-        const float c2 = a.sig2[p] / rck2, c6 = c2 * c2 * c2, c12 = c6 * c6;
-        k.cu[t] = c12 - c6;
-        k.cd[t] = 12.f * c12 - 6.f * c6;
-      }
-    }
+    const AdjRow k = adj_row(a, tk, rck2);
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
     const float l = g.edge, il = g.inv_edge, ilx = g.inv_edge_x;
     const int cx = cell_coord<float>(pi.x, g.edge_x, ilx, nx), cy = cell_coord<float>(pi.y, l, il, ny),
@@ -722,7 +845,7 @@ __global__ void __launch_bounds__(32 * kAdjWarps) k_adjoint_warp(
     if (threadIdx.x < 8 && (threadIdx.x & 3) < nt * nt) {
       double t = 0.0;
       for (int w = 0; w < kAdjWarps; ++w) t += sum_sh[w][threadIdx.x];
-      part[(int64_t)(16 * (threadIdx.x >> 2) + (threadIdx.x & 3)) * nslot + blockIdx.x] = t;
+      part[(int64_t)(nt * nt * (threadIdx.x >> 2) + (threadIdx.x & 3)) * nslot + blockIdx.x] = t;
     }
   }
 }
@@ -742,24 +865,37 @@ __global__ void k_adj_tile_key(int64_t n, const typename RT<R>::R4* __restrict__
   tile_key_of_block(r, (float)rc_max, key, cnt, nchunk);
 }
 
+struct TypeEps {
+  double e[4];
+};
+
 // Per-type gradients from per-type-pair sums: eps_ab = sqrt(eps_a eps_b),
 // sigma_ab = (sigma_a + sigma_b) / 2.  pair_de/ds: [ntypes^2]; out: [2 ntypes].
-__global__ void k_mix_chain(const double* pair_de, const double* pair_ds, int nt, const double* eps, double* out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  for (int a = 0; a < 2 * nt; ++a) out[a] = 0.0;
+__global__ void k_mix_chain(const double* pair_de, const double* pair_ds, int nt, TypeEps eps, double* out) {
+  // one thread per output; each sums its pairs in the order of the pairs
+  const int q = threadIdx.x, t = q % nt;
+  if (q >= 2 * nt) return;
+  double v = 0.0;
   for (int a = 0; a < nt; ++a)
     for (int b = 0; b < nt; ++b) {
-      int p = a * nt + b;
-      if (a == b) {
-        out[a] += pair_de[p];
-        out[nt + a] += pair_ds[p];
+      const int p = a * nt + b;
+      if (q < nt) {
+        if (a == b) {
+          if (t == a) v += pair_de[p];
+        } else {
+          if (t == a) v += pair_de[p] * 0.5 * sqrt(eps.e[b] / eps.e[a]);
+          if (t == b) v += pair_de[p] * 0.5 * sqrt(eps.e[a] / eps.e[b]);
+        }
       } else {
-        out[a] += pair_de[p] * 0.5 * sqrt(eps[b] / eps[a]);
-        out[b] += pair_de[p] * 0.5 * sqrt(eps[a] / eps[b]);
-        out[nt + a] += 0.5 * pair_ds[p];
-        out[nt + b] += 0.5 * pair_ds[p];
+        if (a == b) {
+          if (t == a) v += pair_ds[p];
+        } else {
+          if (t == a) v += 0.5 * pair_ds[p];
+          if (t == b) v += 0.5 * pair_ds[p];
+        }
       }
     }
+  out[q] = v;
 }
 
 template <typename R>
@@ -785,11 +921,14 @@ int lj_adjoint(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, const R* 
   // the packed loop (FP32, one or two types), else the scalar loop; small
   // systems of the packed loop take a warp per particle
   const bool x2 = sizeof(R) == 4 && nt <= 2, small = x2 && n <= kAdjWarpMaxN;
-  const int64_t nblk = (n + kBlock - 1) / kBlock, nwarp = small ? adj_warp_slots(n) : nblk * (kBlock / 32);
+  const TilePlan tp = tile_plan(ctx->p, ctx->nc, n);
+  const bool tiled = x2 && !small && ctx->adj_rec && tp.usable;
+  const int64_t nblk = (n + kBlock - 1) / kBlock;
+  const int64_t nwarp = small ? adj_warp_slots(n) : (tiled ? tp.slots : nblk * (kBlock / 32));
   bool want = dparams != nullptr;
-  if (want && nwarp > ctx->adj_cap)
+  if (want && (tiled ? 8 * nwarp > ctx->adj_doubles : nwarp > ctx->adj_cap))
     return set_error(ctx, DCM_ERR_CAPACITY, "adjoint reduction needs %lld partials", (long long)nwarp);
-  double* part = want ? ctx->adj_part : nullptr;  // [32][nwarp]: de pairs 0..15, ds pairs 16..31
+  double* part = want ? ctx->adj_part : nullptr;  // [2 nt^2][nwarp]: eps sums per type pair, then sigma sums
   BlockGrid bg;
   for (int d = 0; d < 3; ++d) {
     bg.nb[d] = ctx->nblk3[d];
@@ -802,10 +941,31 @@ int lj_adjoint(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, const R* 
                         : (lj_general(t) ? (const void*)k_adjoint<R, true> : (const void*)k_adjoint<R, false>);
   static_assert(kAdjWarps == 4, "adj_warp_slots");
   static_assert(kAdjX2Block == adj_block<float>(), "the partials layout assumes equal blocks");
+  if constexpr (sizeof(R) == 4) {
+    if (tiled) {
+      AdjRec* rec = (AdjRec*)ctx->adj_rec;
+      TileTable tt;
+      int r0 = tile_cut<float>(ctx, tp, pos, rc, cell_start, a.g, tt, st);
+      if (r0) return r0;
+      if (part) DCM_CUDA_TRY(ctx, cudaMemsetAsync(part, 0, sizeof(double) * (size_t)(2 * nt * nt * nwarp), st));
+      DCM_LAUNCH(ctx, k_adj_records, (unsigned)((n + 255) / 256), 256, 0, st, n, pos, rc, A, a.rc_max, rec);
+      DCM_LAUNCH(ctx, k_block_reach, (unsigned)((ctx->nblk + 127) / 128), 128, 0, st, (const int32_t*)ctx->blk_max, bg,
+                 ctx->blk_max + ctx->nblk);
+      const int smem = kAdjTileWarps * (int)sizeof(TileSmem<AdjRec>);
+      DCM_CUDA_TRY(ctx, cudaFuncSetAttribute(k_adjoint_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+      int sms = 0;
+      DCM_CUDA_TRY(ctx, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
+      DCM_LAUNCH(ctx, k_adjoint_tiles, (unsigned)std::min<int64_t>((nwarp + kAdjTileWarps - 1) / kAdjTileWarps, sms),
+                 32 * kAdjTileWarps, smem, st, rec, cell_start, a, tp.cfg, tt, (float)(0.5 * dlde), bg,
+                 (const int32_t*)(ctx->blk_max + ctx->nblk), G, part, nwarp);
+      DCM_LAUNCH(ctx, k_adjoint_rest, 8 * sms, 64, 0, st, pos, rc, cell_start, a, tt, A, (float)(0.5 * dlde), G, part,
+                 nwarp, bg, (const int32_t*)ctx->blk_max);
+    }
+  }
   // launch order of the tiles, the widest walks first, where that pays
   const TileOrder to = tile_order_layout(ctx->tile_scratch, (n + tb - 1) / tb);
   const int32_t* order = nullptr;
-  if (!small && tile_order_pays(kern, tb, to.ntile)) {
+  if (!small && !tiled && tile_order_pays(kern, tb, to.ntile)) {
     int r0 = tile_order_begin(ctx, to, st);
     if (r0) return r0;
     DCM_LAUNCH(ctx, k_adj_tile_key<R>, (unsigned)to.ntile, tb, 0, st, n, pos, rc, a.rc_max, bg,
@@ -817,7 +977,7 @@ int lj_adjoint(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, const R* 
     if (small)
       DCM_LAUNCH(ctx, k_adjoint_warp, (unsigned)adj_warp_slots(n), 32 * kAdjWarps, 0, st, n, pos, rc, cell_start, a, A,
                  (float)(0.5 * dlde), G, part, nwarp, bg, (const int32_t*)ctx->blk_max);
-    else if (x2)
+    else if (x2 && !tiled)
       DCM_LAUNCH(ctx, k_adjoint_x2, (unsigned)to.ntile, kAdjX2Block, 0, st, n, pos, rc, cell_start, a, A,
                  (float)(0.5 * dlde), G, part, nwarp, bg, (const int32_t*)ctx->blk_max, order);
   }
@@ -828,15 +988,13 @@ int lj_adjoint(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, const R* 
   }
   int r = check_launch(ctx, "lj_adjoint");
   if (r || !want) return r;
-  int npair = nt * nt;
-  for (int p = 0; p < npair; p += 4) {
-    int q = std::min(4, npair - p);
-    if ((r = reduce_partials(ctx, part + (int64_t)p * nwarp, nwarp, q, ctx->adj_pairs + p, false, st))) return r;
-    if ((r = reduce_partials(ctx, part + (int64_t)(16 + p) * nwarp, nwarp, q, ctx->adj_pairs + 16 + p, false, st)))
+  const int rows = 2 * nt * nt;  // eps sums, then sigma sums
+  for (int p = 0; p < rows; p += 8)
+    if ((r = reduce_partials(ctx, part + (int64_t)p * nwarp, nwarp, std::min(8, rows - p), ctx->adj_pairs + p, false, st)))
       return r;
-  }
-  DCM_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->adj_pairs + 32, ctx->p.eps, sizeof(double) * nt, cudaMemcpyHostToDevice, st));
-  DCM_LAUNCH(ctx, k_mix_chain, 1, 1, 0, st, ctx->adj_pairs, ctx->adj_pairs + 16, nt, ctx->adj_pairs + 32, dparams);
+  TypeEps eps;
+  for (int k = 0; k < 4; ++k) eps.e[k] = ctx->p.eps[k];
+  DCM_LAUNCH(ctx, k_mix_chain, 1, 32, 0, st, ctx->adj_pairs, ctx->adj_pairs + nt * nt, nt, eps, dparams);
   return check_launch(ctx, "lj_adjoint mix");
 }
 

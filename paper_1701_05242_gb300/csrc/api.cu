@@ -271,13 +271,19 @@ struct ScratchPlan {
     const int64_t b = adj_warp_slots(n_max < kAdjWarpMaxN ? n_max : kAdjWarpMaxN);
     return red_cap > b ? red_cap : b;
   }
+  // the tiled adjoint: mixed form, systems that the warp-per-particle kernel is too slow for
+  bool adj_tiles() const { return rsize == 4 && tile_cap > 0 && n_max > kAdjWarpMaxN; }
+  int64_t adj_doubles() const {
+    const int64_t a = 32 * adj_slots(), b = adj_tiles() ? 8 * tile_cap : 0;
+    return a > b ? a : b;
+  }
   double skin;
   int32_t min_component, segmentation, ms_outer;
   int64_t total() const {
     return 4 * 4 + 16 + 3 * 4 * n_max + 4 * (ncell + 1) + 4 * ncell + 8 * (scan_cap + 1) + 3 * 4 * nbox + 2 * nbox +
            2 * rsize * nbox + 4 * flags + 4 * (int64_t)kHistCap + 4 * 8 + 8 * 3 * red_slots() + 8 * 8 + 8 * 8 * 256 +
-           8 * 32 * adj_slots() + 8 * 48 + (skin > 0 ? 8 * n_max + 8 * (n_max / 32 + 16) + 4 * rsize * n_max + 32 : 0) +
-           (min_component > 0 ? 9 * nbox + 4 * 80 : 0) + 13 * nbox + 4 * (flags + 2) + 4 * nblk +
+           8 * adj_doubles() + (adj_tiles() ? 32 * n_max : 0) + 8 * 48 + (skin > 0 ? 8 * n_max + 8 * (n_max / 32 + 16) + 4 * rsize * n_max + 32 : 0) +
+           (min_component > 0 ? 9 * nbox + 4 * 80 : 0) + 13 * nbox + 4 * (flags + 2) + 8 * nblk +
            4 * tile_scratch_ints(n_max) + (tile_cap > 0 ? 4 * tile_ints(tile_cap) : 0) +
            (segmentation ? 10 * rsize * nbox + 32 * ms_outer + 16 + 4 * (ms_outer + 2) : 0);
   }
@@ -328,7 +334,7 @@ extern "C" void dcm_destroy(dcm_ctx* ctx) {
                  ctx->D[1], ctx->flags, ctx->hist, ctx->thr, ctx->red, ctx->totals, ctx->D[0], ctx->red_tmp, ctx->adj_part, ctx->adj_pairs,
                  ctx->nnb, ctx->nimg, ctx->capw, ctx->offw, ctx->list, ctx->xbuild, ctx->dmax, ctx->lflag,
                  ctx->cc_lab, ctx->cc_cnt, ctx->cc_flags, ctx->cc_s0, ctx->dq[0], ctx->dq[1], ctx->dqlen,
-                 ctx->dstamp, ctx->dfixed, ctx->blk_max, ctx->tile_scratch, ctx->tiles, ctx->ms_u, ctx->ms_ub, ctx->ms_p, ctx->ms_w,
+                 ctx->dstamp, ctx->dfixed, ctx->blk_max, ctx->tile_scratch, ctx->tiles, ctx->adj_rec, ctx->ms_u, ctx->ms_ub, ctx->ms_p, ctx->ms_w,
                  ctx->ms_sums, ctx->ms_c, ctx->ms_flags};
   for (void* q : dev)
     if (q) cudaFree(q);
@@ -390,8 +396,10 @@ extern "C" int dcm_create(const dcm_params* p, dcm_ctx** out) {
   alloc((void**)&ctx->red, 8 * 3 * s.red_slots());
   alloc((void**)&ctx->totals, 8 * 8);
   alloc((void**)&ctx->red_tmp, 8 * 8 * 256);
-  alloc((void**)&ctx->adj_part, 8 * 32 * s.adj_slots());
+  alloc((void**)&ctx->adj_part, 8 * s.adj_doubles());
   ctx->adj_cap = s.adj_slots();
+  ctx->adj_doubles = s.adj_doubles();
+  if (s.adj_tiles()) alloc(&ctx->adj_rec, 32 * nm);
   if (p->skin > 0.0) {
     alloc((void**)&ctx->nnb, 4 * nm);
     alloc((void**)&ctx->nimg, 4 * nm);
@@ -424,7 +432,7 @@ extern "C" int dcm_create(const dcm_params* p, dcm_ctx** out) {
   alloc((void**)&ctx->adj_pairs, 8 * 48);
   for (int d = 0; d < 3; ++d) ctx->nblk3[d] = (int)adjoint_blocks(p, d);  // as counted in the plan
   ctx->nblk = s.nblk;
-  alloc((void**)&ctx->blk_max, 4 * s.nblk);
+  alloc((void**)&ctx->blk_max, 8 * s.nblk);
   alloc((void**)&ctx->tile_scratch, 4 * tile_scratch_ints(s.n_max));
   if (s.tile_cap > 0) {
     alloc((void**)&ctx->tiles, 4 * tile_ints(s.tile_cap));

@@ -111,12 +111,14 @@ struct dcm_ctx {
   double* red;              // reduction partials
   double* red_tmp;          // [8 * 256] first-level chunk sums
   double* adj_part;         // [32][adj_cap] adjoint parameter-gradient partials
-  int64_t adj_cap;
-  double* adj_pairs;        // [48]: per-pair eps sums, per-pair sigma sums, eps values
+  int64_t adj_cap;          // partial slots per quantity
+  int64_t adj_doubles;      // doubles in adj_part
+  void* adj_rec;            // n_max x 32 bytes: what the tiled adjoint stages per particle (or null: not served)
+  double* adj_pairs;        // [48]: per-pair eps sums, per-pair sigma sums
   double* totals;           // [4]
   int32_t* host_status;     // pinned host mirror
   int64_t red_cap;          // number of partial slots in red (per quantity)
-  int32_t* blk_max;         // nblk: largest cutoff (float bits) per adjoint block
+  int32_t* blk_max;         // 2 nblk: largest cutoff (float bits) per adjoint block, and of the 27 around it
   int32_t* tile_scratch;    // tile_scratch_ints(n_max): launch order of the force and adjoint tiles
   int32_t* tiles;           // tile_ints(tile_cap): counters, slots in use, slots left to the row walk, particles of the slots
   int64_t tile_cap;         // pair tile slots (0: tiles not served)

@@ -18,9 +18,6 @@ namespace dcm {
 // tiles
 // ---------------------------------------------------------------------------
 
-// Counters of a launch.
-enum { kTileFirst = 0, kTileLater = 1, kTileQueue = 2, kTileRest = 3, kTileOutside = 4, kTileCounters = 8 };
-
 // One warp per bundle: deals the bundle's particles, in the order of their
 // cell step along x, into tiles of 32 (a tile ends early only where it would
 // grow longer than cfg.cap cells, and at the bundle's end).  The particles of the
@@ -257,7 +254,7 @@ __device__ __forceinline__ void tile_partials(double e, double w, int np, double
 // memory holds, one block per SM.
 template <typename R>
 constexpr int tile_warps() {
-  constexpr int fit = 227 * 1024 / (int)sizeof(TileSmem<R>);
+  constexpr int fit = 227 * 1024 / (int)sizeof(TileSmem<typename RT<R>::R4>);
   constexpr int most = sizeof(R) == 4 ? 16 : 8;
   return fit < most ? fit : most;
 }
@@ -273,7 +270,7 @@ __global__ void __launch_bounds__(32 * tile_warps<R>(), 1) k_forces_tiles(
   constexpr Accum M = kX2 ? Accum::kPlaneKahan : Accum::kPlain;
   const unsigned full = 0xffffffffu;
   extern __shared__ __align__(32) unsigned char smem_raw[];
-  TileSmem<R>& sm = reinterpret_cast<TileSmem<R>*>(smem_raw)[threadIdx.x >> 5];
+  TileSmem<R4>& sm = reinterpret_cast<TileSmem<R4>*>(smem_raw)[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
   const Grid<R>& g = a.g;
   const int nfirst = __ldg(counters + kTileFirst), ntile = nfirst + __ldg(counters + kTileLater);
@@ -315,7 +312,7 @@ __global__ void __launch_bounds__(32 * tile_warps<R>(), 1) k_forces_tiles(
     R xi[3] = {pi.x, pi.y, pi.z};
     // the FP64 cutoff rounded up
     const float rf = sizeof(R) == 4 ? (float)rci : __double2float_ru((double)rci);
-    const bool done = tile_candidates<R>(sm, pos, start, g, cfg, active, i, xi, rf, ahead, [&](int last) {
+    const bool done = tile_candidates<R, R4>(sm, pos, start, g, cfg, active, i, xi, rf, rf, NoCutoff{}, ahead, [&](int last) {
       ListWalk l;
       l.begin(shared_addr(&sm.list[0][lane]), last);
       if constexpr (kX2)
@@ -415,30 +412,45 @@ bool tiles_serve(const dcm_ctx* ctx, int64_t n) {
 
 
 template <typename R>
+int tile_cut(dcm_ctx* ctx, const TilePlan& tp, const typename RT<R>::R4* pos, const R* rc, const int32_t* cell_start,
+             const Grid<R>& g, TileTable& t, cudaStream_t st) {
+  t.counters = ctx->tiles;
+  t.list = t.counters + kTileCounters;
+  t.rest = t.list + tp.slots;
+  t.idx = t.rest + tp.slots;
+  const int64_t nb = (int64_t)tp.cfg.nby * tp.cfg.nbz;
+  DCM_CUDA_TRY(ctx, cudaMemsetAsync(t.counters, 0, kTileCounters * sizeof(int32_t), st));
+  auto kc = tp.cfg.ry * tp.cfg.rz <= 4 ? k_tile_cut<R, 4> : k_tile_cut<R, 16>;
+  DCM_LAUNCH(ctx, kc, (unsigned)((nb + 3) / 4), 128, 0, st, cell_start, pos, rc, (R)(1.2 * ctx->p.rc_min), g, tp.cfg,
+             t.idx, t.list, t.counters, tp.slots);
+  return DCM_OK;
+}
+template int tile_cut<float>(dcm_ctx*, const TilePlan&, const float4*, const float*, const int32_t*,
+                             const Grid<float>&, TileTable&, cudaStream_t);
+
+template <typename R>
 int tile_forces(dcm_ctx* ctx, bool typed, bool ew, int64_t n, const typename RT<R>::R4* pos, const R* rc,
                 const int32_t* cell_start, const ForceArgs<R>& a, typename RT<R>::R4* force, double* part,
                 cudaStream_t st) {
   const TilePlan tp = tile_plan(ctx->p, ctx->nc, n);
-  int32_t *counters = ctx->tiles, *list = counters + kTileCounters, *rest = list + tp.slots, *idx = rest + tp.slots;
-  const int64_t nb = (int64_t)tp.cfg.nby * tp.cfg.nbz;
-  DCM_CUDA_TRY(ctx, cudaMemsetAsync(counters, 0, kTileCounters * sizeof(int32_t), st));
   if (part) DCM_CUDA_TRY(ctx, cudaMemsetAsync(part, 0, 3 * sizeof(double) * (size_t)tp.slots, st));
-  auto kc = tp.cfg.ry * tp.cfg.rz <= 4 ? k_tile_cut<R, 4> : k_tile_cut<R, 16>;
-  DCM_LAUNCH(ctx, kc, (unsigned)((nb + 3) / 4), 128, 0, st, cell_start, pos, rc, (R)(1.2 * ctx->p.rc_min), a.g, tp.cfg,
-             idx, list, counters, tp.slots);
+  TileTable t;
+  int r = tile_cut<R>(ctx, tp, pos, rc, cell_start, a.g, t, st);
+  if (r) return r;
   auto k = typed ? (ew ? k_forces_tiles<R, true, true> : k_forces_tiles<R, true, false>)
                  : (ew ? k_forces_tiles<R, false, true> : k_forces_tiles<R, false, false>);
   auto kr = typed ? (ew ? k_forces_rest<R, true, true> : k_forces_rest<R, true, false>)
                   : (ew ? k_forces_rest<R, false, true> : k_forces_rest<R, false, false>);
-  constexpr int warps = tile_warps<R>(), smem = warps * (int)sizeof(TileSmem<R>);
+  constexpr int warps = tile_warps<R>(), smem = warps * (int)sizeof(TileSmem<typename RT<R>::R4>);
   DCM_CUDA_TRY(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   int sms = 0;
   DCM_CUDA_TRY(ctx, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
   const unsigned grid = (unsigned)std::min<int64_t>((tp.slots + warps - 1) / warps, sms);
-  DCM_LAUNCH(ctx, k, grid, 32 * warps, smem, st, pos, rc, cell_start, a, tp.cfg, idx, list, rest, counters, force,
+  DCM_LAUNCH(ctx, k, grid, 32 * warps, smem, st, pos, rc, cell_start, a, tp.cfg, t.idx, t.list, t.rest,
+             t.counters, force,
              part, tp.slots);
-  DCM_LAUNCH(ctx, kr, (unsigned)std::min<int64_t>((tp.slots + 1) / 2, 8 * sms), 64, 0, st, pos, rc, cell_start, a, idx,
-             list, rest, counters, force, part, tp.slots);
+  DCM_LAUNCH(ctx, kr, (unsigned)std::min<int64_t>((tp.slots + 1) / 2, 8 * sms), 64, 0, st, pos, rc, cell_start, a,
+             t.idx, t.list, t.rest, t.counters, force, part, tp.slots);
   return check_launch(ctx, "tile_forces");
 }
 

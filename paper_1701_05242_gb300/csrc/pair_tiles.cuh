@@ -53,13 +53,28 @@ constexpr int kTileCand = 384;               // candidates staged at a time: hal
 constexpr int kTileGroups = kTileCand / 32;  // mask words per lane
 constexpr int kTileEnd = 4;                  // candidates a list may be read past its end
 
-// Shared memory of one warp.
-template <typename R>
+// Shared memory of one warp.  E: what is staged per candidate, a position
+// (x, y, z first) with whatever else the caller's pairs need.
+template <typename E>
 struct TileSmem {
-  typename RT<R>::R4 pos[kTileCand + kTileEnd];  // staged candidates; the last ones are far away and never accepted
+  E pos[kTileCand + kTileEnd];  // staged candidates; the last ones are far away and never accepted
   uint2 list[kTileGroups + 2][32];  // per lane: mask of a group, shared address of its first candidate
-  uint4 frag[32];                   // the filter's operand of the group at work
+  uint4 frag[32 * (sizeof(E) == sizeof(float4) ? 1 : 2)];  // the filter's operands of the group at work
 };
+
+// Counters of a launch.
+enum { kTileFirst = 0, kTileLater = 1, kTileQueue = 2, kTileRest = 3, kTileOutside = 4, kTileCounters = 8 };
+
+// The tiles of a launch (forces_tiles.cu): the slots in use are list[0 ..
+// counters[kTileFirst]) and list[nslot - counters[kTileLater] .. nslot) from its
+// end, slot s holds particles idx[32 s .. 32 s + 31], rest takes the slots that a
+// kernel leaves to the row walk.
+struct TileTable {
+  int32_t *counters, *list, *rest, *idx;
+};
+template <typename R>
+int tile_cut(dcm_ctx* ctx, const TilePlan& tp, const typename RT<R>::R4* pos, const R* rc, const int32_t* cell_start,
+             const Grid<R>& g, TileTable& t, cudaStream_t st);
 
 // First bit (from the most significant) of a nonzero word.
 __device__ __forceinline__ int first_bit(uint32_t w) {
@@ -108,6 +123,7 @@ struct TileFilter {
   float s, ox, oy, oz;  // x' = x s + o
   uint32_t a[4];        // rows g, g + 8, g + 16, g + 24: two of the eight k slots
   float c[4];           // |x_i'|^2 - rc_i'^2 - slack of those rows
+  float c2[4];          // |x_i'|^2 - slack, for candidates with a cutoff of their own (filter_group2)
   uint32_t wr, rd[4];   // shared addresses: where the lane stores its candidate's operand, and its fragments
 };
 
@@ -140,7 +156,10 @@ __device__ __forceinline__ void filter_begin(TileFilter& f, uint4* frag, float x
   const uint32_t xy = pack_half(fmaf(x, f.s, f.ox), fmaf(y, f.s, f.oy)), zz = pack_half(fmaf(z, f.s, f.oz), 0.f);
   const float2 hxy = unpack_half(xy), hz = unpack_half(zz);
   float ni = fmaf(hxy.x, hxy.x, fmaf(hxy.y, hxy.y, hz.x * hz.x)) - r * r - slack;
-  if (!(rc >= 0.f)) ni = kNever;
+  const float nn2 = fmaf(hxy.x, hxy.x, fmaf(hxy.y, hxy.y, hz.x * hz.x)) -
+                    (fmaf(2.f * rmax * scale, e, e * e) + qj * 0x1p-16f + 0x1p-10f);
+  const bool none = !(rc >= 0.f);
+  if (none) ni = kNever;
   const __half2 m2 = __floats2half2_rn(-2.f, -2.f);
   const __half2 axy = __hmul2(*reinterpret_cast<const __half2*>(&xy), m2);
   uint4 w;
@@ -157,6 +176,7 @@ __device__ __forceinline__ void filter_begin(TileFilter& f, uint4* frag, float x
     const int owner = (lane & ~3) + k;
     f.a[k] = t < 3 ? q[owner * 4 + t] : 0u;
     f.c[k] = __uint_as_float(q[owner * 4 + 3]);
+    f.c2[k] = __shfl_sync(0xffffffffu, none ? kNever : nn2, owner);
   }
   // candidate 8 t' + 2 k + e of a group is column 2 t' + e of product k, so that
   // the bits arrive in candidate order; the slot order keeps stores and loads
@@ -167,24 +187,17 @@ __device__ __forceinline__ void filter_begin(TileFilter& f, uint4* frag, float x
   for (int k = 0; k < 4; ++k) f.rd[k] = shared_addr(q + (8 * k + (g ^ (2 * k))) * 4 + t);
 }
 
-// One group of 32 candidates, candidate `lane` at (x, y, z): the mask of this
-// lane's particle, bit 31 - k for candidate k.
-__device__ __forceinline__ uint32_t filter_group(TileFilter& f, float x, float y, float z) {
+// The signs of one product of the group's operand (at byte `at` behind the
+// first) with the tile's rows: the mask of this lane's particle.
+__device__ __forceinline__ uint32_t filter_signs(const TileFilter& f, const float (&c)[4], uint32_t at) {
   const int t = threadIdx.x & 3;
-  const uint32_t xy = pack_half(fmaf(x, f.s, f.ox), fmaf(y, f.s, f.oy)), zz = pack_half(fmaf(z, f.s, f.oz), 0.f);
-  const float2 hxy = unpack_half(xy), hz = unpack_half(zz);
-  const float n = fmaf(hxy.x, hxy.x, fmaf(hxy.y, hxy.y, hz.x * hz.x));
-  const uint32_t zn = pack_half(hz.x, n), rest = pack_half(n - unpack_half(zn).y, 0.f);
-  __syncwarp();
-  asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(f.wr), "r"(xy), "r"(zn), "r"(rest), "r"(0u) : "memory");
-  __syncwarp();
   float d[2][4][4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     uint32_t b;
-    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(b) : "r"(f.rd[k]) : "memory");
-    mma_16n8k8(d[0][k], f.a[0], f.a[1], b, f.c[0], f.c[1]);
-    mma_16n8k8(d[1][k], f.a[2], f.a[3], b, f.c[2], f.c[3]);
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(b) : "r"(f.rd[k] + at) : "memory");
+    mma_16n8k8(d[0][k], f.a[0], f.a[1], b, c[0], c[1]);
+    mma_16n8k8(d[1][k], f.a[2], f.a[3], b, c[2], c[3]);
   }
   // the signs of rows g, g + 8 and of rows g + 16, g + 24, in two chains
   uint32_t h[2] = {0u, 0u};
@@ -203,6 +216,28 @@ __device__ __forceinline__ uint32_t filter_group(TileFilter& f, float x, float y
   m = __byte_perm(m, p, t & 1 ? 0x6240 : 0x3715);
   p = __shfl_xor_sync(0xffffffffu, m, 2);
   return __byte_perm(m, p, t & 2 ? 0x5410 : 0x3276);
+}
+
+__device__ __forceinline__ void filter_store(uint32_t at, uint32_t xy, float z, float n) {
+  const uint32_t zn = pack_half(z, n), rest = pack_half(n - unpack_half(zn).y, 0.f);
+  asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(xy), "r"(zn), "r"(rest), "r"(0u) : "memory");
+}
+
+// One group of 32 candidates, candidate `lane` at (x, y, z): the mask of this
+// lane's particle, bit 31 - k for candidate k.  TWO: also the candidates whose own
+// cutoff rc reaches the particle, by a second product with |x_j|^2 - rc_j^2.
+template <bool TWO>
+__device__ __forceinline__ uint32_t filter_group(const TileFilter& f, float x, float y, float z, float rc) {
+  const uint32_t xy = pack_half(fmaf(x, f.s, f.ox), fmaf(y, f.s, f.oy)), zz = pack_half(fmaf(z, f.s, f.oz), 0.f);
+  const float2 hxy = unpack_half(xy), hz = unpack_half(zz);
+  const float n = fmaf(hxy.x, hxy.x, fmaf(hxy.y, hxy.y, hz.x * hz.x));
+  __syncwarp();
+  filter_store(f.wr, xy, hz.x, n);
+  if constexpr (TWO) filter_store(f.wr + 512u, xy, hz.x, n - (rc * f.s) * (rc * f.s));
+  __syncwarp();
+  uint32_t m = filter_signs(f, f.c, 0u);
+  if constexpr (TWO) m |= filter_signs(f, f.c2, 512u);
+  return m;
 }
 
 // Append a mask and its group's address to a lane's list if any bit is set.
@@ -240,12 +275,15 @@ __device__ __forceinline__ int warp_incl_sum(int v) {
 //   i      the lane's particle (ignored where !active), xi its position (out:
 //          in the tile's frame), ri its cutoff (clamped)
 //   ahead  called once, when the tile's own loads are done with
-template <typename R, typename A, typename F>
-__device__ __forceinline__ bool tile_candidates(TileSmem<R>& sm, const typename RT<R>::R4* __restrict__ pos,
+//   reach  radius within which the lane may need candidates: ri, or more where
+//          own_cutoff(candidate) gives the candidates a cutoff of their own, which
+//          then counts too (NoCutoff: it does not)
+struct NoCutoff {};
+template <typename R, typename E, typename Own, typename A, typename F>
+__device__ __forceinline__ bool tile_candidates(TileSmem<E>& sm, const E* __restrict__ pos,
                                                 const int32_t* __restrict__ start, const Grid<R>& g,
                                                 const TileCfg& cfg, bool active, int i, R (&xi)[3], float ri,
-                                                A&& ahead, F&& consume) {
-  using R4 = typename RT<R>::R4;
+                                                float reach, Own own_cutoff, A&& ahead, F&& consume) {
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const float Lf[3] = {(float)g.L[0], (float)g.L[1], (float)g.L[2]};
@@ -261,7 +299,8 @@ __device__ __forceinline__ bool tile_candidates(TileSmem<R>& sm, const typename 
     lo[d] = warp_min_nonneg(lo[d]);
     hi[d] = warp_max_nonneg(hi[d]);
   }
-  const float rmax = warp_max_nonneg(active ? ri : 0.f);
+  const float rmax = warp_max_nonneg(active ? reach : 0.f);
+  const bool two = __any_sync(full, active && reach > ri);
   // cells that the spheres can reach, unwrapped, with the row walk's slack;
   // FP64 coordinates are rounded to FP32 here, a few 1e-7 of the box
   const float ed[3] = {(float)g.edge_x, (float)g.edge, (float)g.edge};
@@ -311,9 +350,10 @@ __device__ __forceinline__ bool tile_candidates(TileSmem<R>& sm, const typename 
   // a place that no particle of the tile reaches
   const R pad[3] = {(R)(-f.ox / f.s), (R)((kPadAt - f.oy) / f.s), (R)(-f.oz / f.s)};
   if (lane < kTileEnd) {
-    R4 far;  // what lists may be read past their end
-    far.x = (R)1e15f;
-    far.y = far.z = far.w = (R)0;
+    E far{};  // what lists may be read past their end
+    far.x = pad[0];
+    far.y = pad[1];
+    far.z = pad[2];
     sm.pos[kTileCand + lane] = far;
   }
   ahead();
@@ -387,13 +427,13 @@ __device__ __forceinline__ bool tile_candidates(TileSmem<R>& sm, const typename 
         if (!(held >> r & 15u)) continue;
         const int src = r + (lane >> 3);
         const int nn = __shfl_sync(full, len, src) - sub, jj = __shfl_sync(full, from, src) + sub;
-        const uint32_t dst = pos_s + (uint32_t)((__shfl_sync(full, to, src) + sub) * (int)sizeof(R4));
-        const R4* p = pos + jj;
-        copy_if<sizeof(R4), 0>(dst, p, nn);
-        copy_if<sizeof(R4), 8>(dst, p, nn);
-        copy_if<sizeof(R4), 16>(dst, p, nn);
+        const uint32_t dst = pos_s + (uint32_t)((__shfl_sync(full, to, src) + sub) * (int)sizeof(E));
+        const E* p = pos + jj;
+        copy_if<sizeof(E), 0>(dst, p, nn);
+        copy_if<sizeof(E), 8>(dst, p, nn);
+        copy_if<sizeof(E), 16>(dst, p, nn);
         if (most > 24)
-          for (int q = 24; q < most; q += 8) copy_if<sizeof(R4), 0>(dst + (uint32_t)(q * sizeof(R4)), p + q, nn - q);
+          for (int q = 24; q < most; q += 8) copy_if<sizeof(E), 0>(dst + (uint32_t)(q * sizeof(E)), p + q, nn - q);
       }
       if (images) {  // shift the image rows in place
         copy_async_wait();
@@ -403,7 +443,7 @@ __device__ __forceinline__ bool tile_candidates(TileSmem<R>& sm, const typename 
           const int nn = __shfl_sync(full, len, src), tt = __shfl_sync(full, to, src);
           const uint32_t code = __shfl_sync(full, im, src);
           for (int q = lane; q < nn; q += 32) {
-            R4 p = sm.pos[tt + q];
+            E p = sm.pos[tt + q];
             if (code & 1u) p.x -= g.L[0];
             if (code & 2u) p.y -= g.L[1];
             if (code & 4u) p.z -= g.L[2];
@@ -417,27 +457,32 @@ __device__ __forceinline__ bool tile_candidates(TileSmem<R>& sm, const typename 
       // a chunk is full, or ends with its half where the other one would not fit
       if (staged == kTileCand || (staged && done == total && (final || (end_half && 2 * staged > kTileCand)))) {
         if (staged + lane < (staged + 31 & ~31)) {  // fill the last group up
-          R4 p;
+          E p{};
           p.x = pad[0];
           p.y = pad[1];
           p.z = pad[2];
-          p.w = (R)0;
           sm.pos[staged + lane] = p;
         }
         copy_async_wait();
         __syncwarp();
         uint32_t ls = list_s, ad = pos_s;
-        const uint32_t end = pos_s + (uint32_t)(staged * (int)sizeof(R4));
-        const uint32_t own_ad = pos_s + (uint32_t)((selfcol & ~31) * (int)sizeof(R4)), own_bit = ~(0x80000000u >> (selfcol & 31));
+        const uint32_t end = pos_s + (uint32_t)(staged * (int)sizeof(E));
+        const uint32_t own_ad = pos_s + (uint32_t)((selfcol & ~31) * (int)sizeof(E)), own_bit = ~(0x80000000u >> (selfcol & 31));
         do {
-          const R4 p = *reinterpret_cast<const R4*>(reinterpret_cast<const char*>(sm.pos) + (ad - pos_s) + lane * sizeof(R4));
-          uint32_t m = filter_group(f, (float)p.x, (float)p.y, (float)p.z);
+          const E p = *reinterpret_cast<const E*>(reinterpret_cast<const char*>(sm.pos) + (ad - pos_s) + lane * sizeof(E));
+          uint32_t m;
+          if constexpr (std::is_same_v<Own, NoCutoff>) {
+            m = filter_group<false>(f, (float)p.x, (float)p.y, (float)p.z, 0.f);
+          } else {
+            m = two ? filter_group<true>(f, (float)p.x, (float)p.y, (float)p.z, own_cutoff(p))
+                    : filter_group<false>(f, (float)p.x, (float)p.y, (float)p.z, 0.f);
+          }
           if (ad == own_ad) m &= own_bit;
           list_push(ls, m, ad);
-          ad += 32u * (uint32_t)sizeof(R4);
+          ad += 32u * (uint32_t)sizeof(E);
         } while (ad < end);
         const int last = (int)(ls - list_s) >> 8;
-        sm.list[last][lane] = make_uint2(0xf0000000u, pos_s + kTileCand * (uint32_t)sizeof(R4));
+        sm.list[last][lane] = make_uint2(0xf0000000u, pos_s + kTileCand * (uint32_t)sizeof(E));
         consume(last);
         __syncwarp();
         staged = 0;
