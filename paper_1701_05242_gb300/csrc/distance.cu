@@ -152,6 +152,59 @@ __global__ void __launch_bounds__(256) k_dist_first(const uint8_t* __restrict__ 
   }
 }
 
+// Four boxes of a row per thread (nx a multiple of 4, flags 4-byte and
+// distances 16-byte aligned): the flags of a box and its row neighbours come
+// with one word and two bytes.
+__device__ __forceinline__ uint32_t zero_bytes(uint32_t s, uint32_t f) {  // 0xff where s == 0 or f != 0
+  return __vcmpeq4(s, 0u) | __vcmpne4(f, 0u);
+}
+__global__ void __launch_bounds__(256) k_dist_first4(const uint8_t* __restrict__ s, const uint8_t* __restrict__ iface,
+                                                     float* __restrict__ D0, float* __restrict__ D1, int nx, int ny,
+                                                     int nz, int zc, float h, float r_grid,
+                                                     uint8_t* __restrict__ fixed0) {
+  const int x = 4 * (blockIdx.x * 32 + (threadIdx.x & 31)), y = blockIdx.y * 8 + (threadIdx.x >> 5);
+  if (x >= nx || y >= ny) return;
+  const int z0 = blockIdx.z * zc, z1 = min(z0 + zc, nz);
+  const int nxy = nx * ny, col = x + nx * y;
+  auto word = [&](int b) {
+    return zero_bytes(__ldg(reinterpret_cast<const uint32_t*>(s + b)), __ldg(reinterpret_cast<const uint32_t*>(iface + b)));
+  };
+  auto zero = [&](int b) { return __ldg(s + b) == 0 || __ldg(iface + b) != 0; };
+  const int xm = x == 0 ? nx - 1 : -1, xp = x == nx - 4 ? 4 - nx : 4;
+  const int ym = y == 0 ? (ny - 1) * nx : -nx, yp = y == ny - 1 ? -(ny - 1) * nx : nx;
+  const float inf = RT<float>::inf();
+  // sweep 0 knows three values per axis pair: 0 or +inf
+  uint32_t below = word(col + nxy * (z0 == 0 ? nz - 1 : z0 - 1)), here = word(col + nxy * z0);
+  for (int z = z0; z < z1; ++z) {
+    const int b = col + nxy * z;
+    const uint32_t above = word(col + nxy * (z == nz - 1 ? 0 : z + 1));
+    float4 cur, v;
+    if (here == 0xffffffffu) {
+      cur = v = make_float4(0.f, 0.f, 0.f, 0.f);
+    } else {
+      const uint32_t ax = (here << 8 | (zero(b + xm) ? 0xffu : 0u)) | (here >> 8 | (zero(b + xp) ? 0xff000000u : 0u));
+      const uint32_t ay = word(b + ym) | word(b + yp), az = below | above;
+      float* pc = &cur.x;
+      float* pv = &v.x;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint32_t bit = 1u << (8 * q);
+        pc[q] = here & bit ? 0.f : inf;
+        pv[q] = pc[q];
+        if (!(here & bit)) {
+          const float d = godunov3<float>(ax & bit ? 0.f : inf, ay & bit ? 0.f : inf, az & bit ? 0.f : inf, h);
+          pv[q] = d < inf && d <= r_grid ? d : inf;
+        }
+      }
+    }
+    *reinterpret_cast<float4*>(D0 + b) = cur;
+    *reinterpret_cast<float4*>(D1 + b) = v;
+    *reinterpret_cast<uint32_t*>(fixed0 + b) = here & 0x01010101u;
+    below = here;
+    here = above;
+  }
+}
+
 // The queue of sweep 1: the boxes that sweep 0 changed and their neighbours.
 // Apart from the pass above, whose warps it would hold up at every front box.
 template <typename R>
@@ -171,13 +224,16 @@ __global__ void __launch_bounds__(256) k_dist_queue0(const R* __restrict__ D1, i
   }
 }
 
+// One large block per SM: the barrier between sweeps costs by the block.
+constexpr int kCoopBlock = 1024;
+
 // The sweeps after sweep 0 in one cooperative launch (every block resident):
 // each over its queue, a bounded grid barrier after it, until a sweep changes
 // nothing or `budget` sweeps have run.  The loop needs no host check and
 // launches nothing per sweep.  A barrier wait that runs past budget_ns records
 // DCM_ERR_TIMEOUT and ends the launch.
 template <typename R>
-__global__ void __launch_bounds__(256) k_dist_coop(R* D0, R* D1, int nx, int ny, int nz, R h, R r_grid,
+__global__ void __launch_bounds__(kCoopBlock) k_dist_coop(R* D0, R* D1, int nx, int ny, int nz, R h, R r_grid,
                                                    const uint8_t* __restrict__ fixed0, int32_t* stamp, int32_t* q0,
                                                    int32_t* q1, int32_t* qlen, int32_t* flags, int budget,
                                                    uint32_t* sync, int64_t budget_ns, int32_t* status) {
@@ -248,20 +304,31 @@ int distance_sweeps(dcm_ctx* ctx, const uint8_t* s, const uint8_t* iface, R* D, 
   const int zc = (int)std::max<int64_t>(1, std::min<int64_t>(64, (int64_t)nz * cols / (152 * 8)));
   if ((ny + 7) / 8 > 65535 || (nz + zc - 1) / zc > 65535)
     return set_error(ctx, DCM_ERR_CAPACITY, "distance sweeps: density grid too long");
-  DCM_LAUNCH(ctx, k_dist_first<R>, dim3((nx + 31) / 32, (ny + 7) / 8, (nz + zc - 1) / zc), 256, 0, st, s, iface, buf[0],
-             buf[1], nx, ny, nz, zc, h, rg, ctx->dfixed);
+  bool four = false;
+  if constexpr (sizeof(R) == 4) {
+    four = nx % 4 == 0 && (((uintptr_t)s | (uintptr_t)iface) & 3) == 0 && ((uintptr_t)D & 15) == 0;
+    if (four) {
+      const int64_t cols4 = (int64_t)((nx / 4 + 31) / 32) * ((ny + 7) / 8);
+      const int zc4 = (int)std::max<int64_t>(1, std::min<int64_t>(64, (int64_t)nz * cols4 / (152 * 8)));
+      DCM_LAUNCH(ctx, k_dist_first4, dim3((nx / 4 + 31) / 32, (ny + 7) / 8, (nz + zc4 - 1) / zc4), 256, 0, st, s, iface,
+                 buf[0], buf[1], nx, ny, nz, zc4, h, rg, ctx->dfixed);
+    }
+  }
+  if (!four)
+    DCM_LAUNCH(ctx, k_dist_first<R>, dim3((nx + 31) / 32, (ny + 7) / 8, (nz + zc - 1) / zc), 256, 0, st, s, iface,
+               buf[0], buf[1], nx, ny, nz, zc, h, rg, ctx->dfixed);
   DCM_LAUNCH(ctx, k_dist_queue0<R>, (unsigned)std::min<int64_t>((nbox + 255) / 256, 152 * 8), 256, 0, st, buf[1], nbox,
              nx, ny, nz, ctx->dfixed, ctx->dstamp, q[1], ctx->dqlen, ctx->flags);
   auto kern = k_dist_coop<R>;
   int per_sm = 0, sms = 0, dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, 0) != cudaSuccess || per_sm < 1)
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kCoopBlock, 0) != cudaSuccess || per_sm < 1)
     return set_error(ctx, DCM_ERR_CUDA, "distance sweeps: occupancy query failed");
   cudaLaunchConfig_t cfg = {};
-  // no more blocks than boxes to sweep: the barrier costs by the block
-  cfg.gridDim = dim3((unsigned)std::min<int64_t>((nbox + 255) / 256, std::min(per_sm, 4) * sms));
-  cfg.blockDim = dim3(256);
+  // no more blocks than boxes to sweep
+  cfg.gridDim = dim3((unsigned)std::min<int64_t>((nbox + kCoopBlock - 1) / kCoopBlock, sms));
+  cfg.blockDim = dim3(kCoopBlock);
   cfg.dynamicSmemBytes = 0;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];

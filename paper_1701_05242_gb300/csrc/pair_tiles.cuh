@@ -49,16 +49,19 @@
 
 namespace dcm {
 
-constexpr int kTileCand = 384;               // candidates staged at a time: half of those a bulk tile at rc = 3 meets
-constexpr int kTileGroups = kTileCand / 32;  // mask words per lane
+// Candidates staged at a time (a bulk tile at rc = 3 meets about 640): 16 warps
+// of 16-byte positions, or 12 of 32-byte records, fit an SM.
+template <typename E>
+constexpr int tile_cand() { return sizeof(E) == 16 ? 512 : 384; }
 constexpr int kTileEnd = 4;                  // candidates a list may be read past its end
 
 // Shared memory of one warp.  E: what is staged per candidate, a position
 // (x, y, z first) with whatever else the caller's pairs need.
 template <typename E>
 struct TileSmem {
-  E pos[kTileCand + kTileEnd];  // staged candidates; the last ones are far away and never accepted
-  uint2 list[kTileGroups + 2][32];  // per lane: mask of a group, shared address of its first candidate
+  static constexpr int kCand = tile_cand<E>();
+  E pos[kCand + kTileEnd];          // staged candidates; the last ones are far away and never accepted
+  uint2 list[kCand / 32 + 2][32];     // per lane: mask of a group, shared address of its first candidate
   uint4 frag[32 * (sizeof(E) == sizeof(float4) ? 1 : 2)];  // the filter's operands of the group at work
 };
 
@@ -284,6 +287,7 @@ __device__ __forceinline__ bool tile_candidates(TileSmem<E>& sm, const E* __rest
                                                 const int32_t* __restrict__ start, const Grid<R>& g,
                                                 const TileCfg& cfg, bool active, int i, R (&xi)[3], float ri,
                                                 float reach, Own own_cutoff, A&& ahead, F&& consume) {
+  constexpr int kTileCand = TileSmem<E>::kCand;
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const float Lf[3] = {(float)g.L[0], (float)g.L[1], (float)g.L[2]};

@@ -2,7 +2,7 @@
 //
 //   kick-drift-count:  v += dt/2 F;  x += dt v (wrapped);  cell and provisional
 //                      rank of every particle (atomic count)        [fused]
-//   scan, scatter, per-cell stable sort, gather into the other buffer
+//   scan, scatter, placement in the stable order of the other buffer
 //   every K steps:     box counts -> interface -> distances -> cutoffs
 //   forces;  kick:     v += dt/2 F with the kinetic energy reduced in FP64
 #include <algorithm>
@@ -74,19 +74,25 @@ __global__ void k_kick_ke(int64_t n, typename RT<R>::R4* __restrict__ vel, const
   if ((threadIdx.x & 31) == 0) part[i >> 5] = (double)ke;
 }
 
-// One pass over perm for the whole particle payload.
+// Every particle finds its place in the stable order (perm: the provisional
+// one) and writes its whole payload there; reads are coalesced, writes nearly
+// so (a particle moves a few cells per step).
 template <typename R>
-__global__ void k_gather_state(int64_t n, const int32_t* __restrict__ perm, const typename RT<R>::R4* __restrict__ p0,
-                               typename RT<R>::R4* __restrict__ p1, const typename RT<R>::R4* __restrict__ v0,
-                               typename RT<R>::R4* __restrict__ v1, const R* __restrict__ r0, R* __restrict__ r1,
-                               const int32_t* __restrict__ id0, int32_t* __restrict__ id1) {
-  int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n) return;
-  int src = perm[k];
-  p1[k] = p0[src];
-  v1[k] = v0[src];
-  r1[k] = r0[src];
-  if (id0) id1[k] = id0[src];
+__global__ void __launch_bounds__(256) k_place_state(
+    int64_t n, const int32_t* __restrict__ cell, const int32_t* __restrict__ start, const int32_t* __restrict__ perm,
+    const typename RT<R>::R4* __restrict__ p0, typename RT<R>::R4* __restrict__ p1,
+    const typename RT<R>::R4* __restrict__ v0, typename RT<R>::R4* __restrict__ v1, const R* __restrict__ r0,
+    R* __restrict__ r1, const int32_t* __restrict__ id0, int32_t* __restrict__ id1) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const auto p = p0[i], v = v0[i];
+  const R r = r0[i];
+  const int32_t id = id0 ? id0[i] : 0;
+  const int k = stable_place((int)i, cell, start, perm);
+  p1[k] = p;
+  v1[k] = v;
+  r1[k] = r;
+  if (id0) id1[k] = id;
 }
 
 __global__ void k_thermo(const double* totals, double* thermo) {
@@ -138,15 +144,15 @@ static int finish_thermo(dcm_ctx* ctx, int64_t n, typename RT<R>::R4* vel, const
 }
 
 template <typename R>
-static int gather_state(dcm_ctx* ctx, dcm_state* st, int64_t n, cudaStream_t s) {
+static int place_state(dcm_ctx* ctx, dcm_state* st, int64_t n, cudaStream_t s) {
   using R4 = typename RT<R>::R4;
   int c = st->cur, o = 1 - st->cur;
   bool ids = st->id[c] && st->id[o];
   if (n > 0)
-    DCM_LAUNCH(ctx, k_gather_state<R>, (unsigned)((n + 255) / 256), 256, 0, s, n, ctx->perm, (const R4*)st->pos[c],
-               (R4*)st->pos[o], (const R4*)st->vel[c], (R4*)st->vel[o], (const R*)st->rc[c], (R*)st->rc[o],
-               ids ? st->id[c] : nullptr, ids ? st->id[o] : nullptr);
-  return check_launch(ctx, "gather_state");
+    DCM_LAUNCH(ctx, k_place_state<R>, (unsigned)((n + 255) / 256), 256, 0, s, n, ctx->cell, ctx->cell_start, ctx->perm,
+               (const R4*)st->pos[c], (R4*)st->pos[o], (const R4*)st->vel[c], (R4*)st->vel[o], (const R*)st->rc[c],
+               (R*)st->rc[o], ids ? st->id[c] : nullptr, ids ? st->id[o] : nullptr);
+  return check_launch(ctx, "place_state");
 }
 
 template <typename R>
@@ -154,9 +160,9 @@ int step_init(dcm_ctx* ctx, dcm_state* st, int64_t n, cudaStream_t s) {
   using R4 = typename RT<R>::R4;
   int o = 1 - st->cur;
   Grid<R> g = cell_grid<R>(ctx);
-  int r = bin_particles<R>(ctx, n, (const R4*)st->pos[st->cur], g, ctx->cell, ctx->cell_start, ctx->perm, nullptr, s);
+  int r = bin_particles<R>(ctx, n, (const R4*)st->pos[st->cur], g, ctx->cell, ctx->cell_start, nullptr, nullptr, s);
   if (r) return r;
-  if ((r = gather_state<R>(ctx, st, n, s))) return r;
+  if ((r = place_state<R>(ctx, st, n, s))) return r;
   if ((r = recompute_cutoffs<R>(ctx, n, (const R4*)st->pos[o], (R*)st->rc[o], s))) return r;
   if (ctx->p.skin > 0.0) {
     if ((r = list_build<R>(ctx, n, (const R4*)st->pos[o], (const R*)st->rc[o], s))) return r;
@@ -204,8 +210,8 @@ static int step_run_lists(dcm_ctx* ctx, dcm_state* st, int64_t n, double dt, int
       int o = 1 - st->cur;
       stage_begin(ctx, DCM_STAGE_BIN, s);
       if ((r = exclusive_scan(ctx, ctx->cell_count, ctx->cell_start, ctx->ncell, s))) return r;
-      if ((r = scatter_sort(ctx, n, ctx->cell, ctx->slot, ctx->cell_start, ctx->ncell, ctx->perm, s))) return r;
-      if ((r = gather_state<R>(ctx, st, n, s))) return r;
+      if ((r = scatter_slots(ctx, n, ctx->cell, ctx->slot, ctx->cell_start, ctx->perm, s))) return r;
+      if ((r = place_state<R>(ctx, st, n, s))) return r;
       stage_end(ctx, DCM_STAGE_BIN, s);
       if (recompute)
         if ((r = recompute_cutoffs<R>(ctx, n, (const R4*)st->pos[o], (R*)st->rc[o], s))) return r;
@@ -247,8 +253,8 @@ int step_run(dcm_ctx* ctx, dcm_state* st, int64_t n, double dt, int nsteps, cuda
     stage_begin(ctx, DCM_STAGE_BIN, s);
     int r = exclusive_scan(ctx, ctx->cell_count, ctx->cell_start, ctx->ncell, s);
     if (r) return r;
-    if ((r = scatter_sort(ctx, n, ctx->cell, ctx->slot, ctx->cell_start, ctx->ncell, ctx->perm, s))) return r;
-    if ((r = gather_state<R>(ctx, st, n, s))) return r;
+    if ((r = scatter_slots(ctx, n, ctx->cell, ctx->slot, ctx->cell_start, ctx->perm, s))) return r;
+    if ((r = place_state<R>(ctx, st, n, s))) return r;
     stage_end(ctx, DCM_STAGE_BIN, s);
     st->t += 1;
     if (st->t % K == 0)
