@@ -9,9 +9,9 @@
 // (symmetric) Jacobian, g = 24 eps [2 s12 - s6] / r^2 and
 // g'/r = 24 eps [-28 s12 + 8 s6] / r^4 with s6 = (sigma/r)^6, s12 = s6^2.
 // Because the cutoffs differ per particle the second (reverse) sum runs over
-// the j whose own cutoff reaches k: one thread per k walks the stencil of a
-// radius that bounds every such rc_j, and every candidate is tested against
-// both rc_k (forward pair) and rc_j (reverse pair).  The bound is the largest
+// the j whose own cutoff reaches k: k searches the radius that bounds every
+// such rc_j (over tiles of 32 particles, with a warp of its own in a small
+// system, else by one thread), and every candidate is tested against both rc_k (forward pair) and rc_j (reverse pair).  The bound is the largest
 // cutoff in the 27 blocks around k, blocks of edge at least 1.001 rc_max
 // (a j with |r_kj| < rc_j <= rc_max lies in one of them), so away from the
 // interfaces, where every cutoff is rc_min, the walk covers the rc_min
@@ -625,7 +625,11 @@ __global__ void k_block_reach(const int32_t* __restrict__ bmax, BlockGrid bg, in
   reach[b] = m;
 }
 
-constexpr int kAdjTileWarps = 12;  // three per scheduler: the pair step wants up to 168 registers
+// Bound by instruction issue like the tiled forces; 260K particles of two types:
+// 650 us (the row walk, one thread per particle) -> 338 us.  Three warps per
+// scheduler: the pair step wants up to 168 registers, and twelve warps of 384
+// records of 32 bytes fill the shared memory.
+constexpr int kAdjTileWarps = 12;
 
 __global__ void __launch_bounds__(32 * kAdjTileWarps, 1) k_adjoint_tiles(
     const AdjRec* __restrict__ rec, const int32_t* __restrict__ start, const __grid_constant__ ForceArgs<float> a,
@@ -710,8 +714,8 @@ __global__ void __launch_bounds__(64) k_adjoint_rest(const float4* __restrict__ 
 // The packed adjoint of a small system, one warp per particle: the lanes
 // take the rows of the walk (radius `reach`), write their candidates into a
 // list in shared memory and then share the list, two candidates per lane and
-// step.  A launch of 2,000 particles lasts as long as one particle's walk: 435 us
-// with one thread per particle.  The sums of the lanes are added in a fixed tree.
+// step.  A launch of 2,000 particles lasts as long as one particle's walk: 444 us
+// for 1,935 particles with one thread each, 29 us so (30,000: 490 -> 171 us).  The sums of the lanes are added in a fixed tree.
 constexpr int kAdjWarps = 4, kAdjList = 1024;  // particles per block; candidates listed at a time
 
 __global__ void __launch_bounds__(32 * kAdjWarps) k_adjoint_warp(

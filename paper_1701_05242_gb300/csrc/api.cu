@@ -310,6 +310,10 @@ static ScratchPlan plan_of(const dcm_params* p) {
   s.ms_outer = p->ms_outer;
   const TilePlan tp = tile_plan(*p, nc, s.n_max);
   s.tile_cap = tp.usable ? tp.slots : 0;
+  if (s.skin > 0) {  // the lists' tiles use the same table
+    const TilePlan lp = list_tile_plan(*p, nc, s.n_max);
+    if (lp.usable && s.rsize == 4 && lp.slots > s.tile_cap) s.tile_cap = lp.slots;
+  }
   s.nblk = adjoint_blocks(p, 0) * adjoint_blocks(p, 1) * adjoint_blocks(p, 2);
   return s;
 }

@@ -288,6 +288,12 @@ struct TilePlan {
   bool usable;
 };
 TilePlan tile_plan(const dcm_params& p, const int64_t* nc, int64_t n);
+// The same for neighbour lists, whose spheres reach rc_max + skin.
+inline TilePlan list_tile_plan(dcm_params p, const int64_t* nc, int64_t n) {
+  p.rc_max += p.skin;
+  return tile_plan(p, nc, n);
+}
+constexpr int64_t kListTilesMinN = 4000;  // below: the row walk
 constexpr int64_t tile_ints(int64_t slots) { return 8 + 34 * slots; }
 bool tiles_serve(const dcm_ctx* ctx, int64_t n);  // whether lj_forces runs over tiles
 template <typename R>

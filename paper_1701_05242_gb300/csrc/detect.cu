@@ -4,8 +4,8 @@
 // interface boxes.
 //
 // All integer arithmetic, so the result is bit-identical to any correct
-// evaluation: the (2w+1)^3 box sum is computed as three separable 1-D periodic
-// sums, and the 2-means iteration runs on a histogram of the box sums (same
+// evaluation: the (2w+1)^3 box sum is separable, three 1-D periodic sums taken
+// in one pass over the counts (half widths above 4: three passes), and the 2-means iteration runs on a histogram of the box sums (same
 // counts and sums as scanning the volume, in one pass instead of one per
 // iteration).
 #include <algorithm>
@@ -42,8 +42,10 @@ __global__ void k_box_sum_axis(const int32_t* __restrict__ in, int32_t* __restri
 // then along y in shared memory, and enters a running sum of the last 2 W + 1
 // planes.  The counts are read once (1.7 times with the halos, which hit L2) and
 // the sums written once, where the three separate passes moved six arrays and
-// paid three integer divisions per box: 333 -> 45 us for 16.4M boxes (kernel
-// times), HBM-bound at 131 MB.  Also reduces the smallest and largest sum
+// paid three integer divisions per box: 333 -> 72 us for 16.4M boxes (kernel
+// times; the 131 MB alone would be 19 us, the rest is the chain of loads, sums
+// and barriers per plane).  Half widths above 4 keep the three passes: their
+// halos and the register window of 2 W + 1 planes outgrow the block.  Also reduces the smallest and largest sum
 // into thr[0], thr[1] if thr is given.
 template <int W>
 __global__ void __launch_bounds__(256) k_box_sum3(const int32_t* __restrict__ in, int32_t* __restrict__ out, int nx,
@@ -191,7 +193,7 @@ __device__ __forceinline__ void block_scan_ll(long long& n, long long& s, long l
 // One empty class: T = gmax + 1 (no interface).  fixed >= 0 bypasses it.
 // Every thread holds a run of bins and the counts and sums before it, so an
 // iteration is a look-up by the one thread whose run holds T (it was four sums
-// over the histogram, eight barriers each: 24 -> 6 us).
+// over the histogram, eight barriers each: 24 -> 7 us).
 __global__ void __launch_bounds__(1024) k_two_means(const int32_t* __restrict__ hist, int32_t* thr, int max_iter,
                                                     int fixed, int32_t* t_out) {
   __shared__ long long sh[64], low[2], all[2];
@@ -252,7 +254,7 @@ __global__ void __launch_bounds__(1024) k_two_means(const int32_t* __restrict__ 
 
 // s = (g >= T); interface = s and some face neighbour below T (periodic).
 // A block of 32 x 8 columns marches along z with the planes below and above
-// in registers (85 -> 25 us for 16.4M boxes against a thread per box, which
+// in registers (85 -> 37 us for 16.4M boxes, 98 MB, against a thread per box, which
 // divided its index and read seven values).
 __global__ void __launch_bounds__(256) k_segment(const int32_t* __restrict__ g, int nx, int ny, int nz, int zc,
                                                  const int32_t* thr, uint8_t* __restrict__ s,

@@ -120,7 +120,8 @@ __device__ __forceinline__ bool dist_update(const R* Din, R* Dout, int64_t b, in
 // Initial values and sweep 0 in one pass: before sweep 0 a box is 0 (low
 // density or interface) or +inf, so the sweep reads the bytes of s and iface
 // instead of the first iterate.  A thread marches along z.  HBM-bound: 33 MB read,
-// 211 MB written for 16.4M boxes (60 + 122 us as two passes).
+// 148 MB written for 16.4M boxes, 104 us (60 + 122 us as two passes); taken where
+// rows are no multiple of four boxes, k_dist_first4 (43 us) where they are.
 template <typename R>
 __global__ void __launch_bounds__(256) k_dist_first(const uint8_t* __restrict__ s, const uint8_t* __restrict__ iface,
                                                     R* __restrict__ D0, R* __restrict__ D1, int nx, int ny, int nz,

@@ -94,8 +94,8 @@ __global__ void __launch_bounds__(kX2Block, x2_min_blocks<M>()) k_forces_x2(int6
 // planes' partial sums are then added in the order of the planes with the
 // compensation of the plane-Kahan form, so the results are bit for bit those of
 // k_forces_x2.  A launch of 2,000 particles has 61 warps in the one-thread form,
-// and lasts as long as one particle's walk (150 us at rc = 6); this one has 968
-// and lasts about as long as one plane.
+// and lasts as long as one particle's walk; this one has 968 and lasts about as
+// long as one plane: 193 -> 41 us for 1,935 particles, 219 -> 97 us for 30,000.
 template <bool TYPED, bool EW>
 __global__ void __launch_bounds__(kPlaneBlock) k_forces_planes(int64_t n, const float4* __restrict__ pos,
                                                                const float* __restrict__ rc,

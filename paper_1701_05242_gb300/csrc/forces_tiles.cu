@@ -6,6 +6,13 @@
 // keeps a fixed number of warps per SM, each of which takes tile after tile from
 // a device queue.  Warps share nothing, so a long tile (at an interface the
 // spheres hold eight times the bulk's volume) holds up one warp only.
+//
+// Bound by instruction issue: 65% of the issue slots at 16 warps per SM, the
+// tensor pipe under 10% busy, HBM nearly idle.  Sixteen warps of 512 staged
+// candidates fill the SM's shared memory; 13 of 640 and 20 of 384 (at 96
+// registers) were slower.  Kernel times against the row walk, energies included:
+// 16.7M particles 6140 -> 4525 us, 1.1M 525 -> 426, 260K of two types 255 -> 180,
+// 260K in FP64 6000 -> 1725.
 #include <algorithm>
 #include <climits>
 #include <cmath>
@@ -359,7 +366,8 @@ __global__ void __launch_bounds__(64) k_forces_rest(const typename RT<R>::R4* __
   const int nfirst = __ldg(counters + kTileFirst), lane = threadIdx.x & 31;
   const int n = all ? nfirst + __ldg(counters + kTileLater) : __ldg(counters + kTileRest);
   for (int k = blockIdx.x * 2 + (threadIdx.x >> 5); k < n; k += gridDim.x * 2) {
-    const int slot = __ldg(!all ? rest + k : (k < nfirst ? list + k : list + (nslot - 1 - (k - nfirst)))), i = __ldg(idx + 32 * (int64_t)slot + lane);
+    const int slot = __ldg(!all ? rest + k : (k < nfirst ? list + k : list + (nslot - 1 - (k - nfirst))));
+    const int i = __ldg(idx + 32 * (int64_t)slot + lane);
     double e = 0, w = 0;
     int np = 0;
     if (i >= 0)
@@ -403,13 +411,14 @@ TilePlan tile_plan(const dcm_params& p, const int64_t* nc, int64_t n) {
   return t;
 }
 
-// Launches below this many particles keep the row walk.
+// Launches below this many particles keep the row walk: that few leave most
+// SMs without a tile, and a launch lasts as long as its longest tile (FP64;
+// the mixed form takes 16 lanes per particle up to kPlanesMaxN).
 constexpr int64_t kTilesMinN = 4000;
 
 bool tiles_serve(const dcm_ctx* ctx, int64_t n) {
   return ctx->tiles && n >= kTilesMinN && tile_plan(ctx->p, ctx->nc, n).usable;
 }
-
 
 template <typename R>
 int tile_cut(dcm_ctx* ctx, const TilePlan& tp, const typename RT<R>::R4* pos, const R* rc, const int32_t* cell_start,
@@ -447,8 +456,7 @@ int tile_forces(dcm_ctx* ctx, bool typed, bool ew, int64_t n, const typename RT<
   DCM_CUDA_TRY(ctx, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
   const unsigned grid = (unsigned)std::min<int64_t>((tp.slots + warps - 1) / warps, sms);
   DCM_LAUNCH(ctx, k, grid, 32 * warps, smem, st, pos, rc, cell_start, a, tp.cfg, t.idx, t.list, t.rest,
-             t.counters, force,
-             part, tp.slots);
+             t.counters, force, part, tp.slots);
   DCM_LAUNCH(ctx, kr, (unsigned)std::min<int64_t>((tp.slots + 1) / 2, 8 * sms), 64, 0, st, pos, rc, cell_start, a,
              t.idx, t.list, t.rest, t.counters, force, part, tp.slots);
   return check_launch(ctx, "tile_forces");

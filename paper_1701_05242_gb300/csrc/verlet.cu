@@ -4,11 +4,14 @@
 // (the Newton's third law variant Section 4.2 points to).
 //
 // Build (at a rebuild): for every particle i, the j != i with
-// |r_ij| < rc_i + skin, found by the same culled cell-row walk as the
-// cell-list force kernel.  The lists of the 32 particles of a warp share one
-// interleaved region (entry k of lane l at base + 32 k + l, base = 32 x the
-// sum of the earlier warps' capacities) so that the force loop reads them
-// coalesced.  Same-image neighbours are stored from the front of a lane's
+// |r_ij| < rc_i + skin, found over tiles with the tensor-core filter
+// (pair_tiles.cuh) or by the culled cell-row walk.  The lists of the 32 particles
+// of a warp share one interleaved region, in quads: entries 4 q .. 4 q + 3 of
+// lane l at base + 128 q + 4 l (base = 32 x the sum of the earlier warps'
+// capacities, which are multiples of 4), so that the force loop reads four entries
+// of every lane from 512 consecutive bytes, and the build writes four by one store:
+// its lanes are at different entries, so a store instruction meets 32 lines
+// whatever its width.  Same-image neighbours are stored from the front of a lane's
 // column as plain indices j; neighbours across the periodic boundary from the
 // back as j | image code << 26, the code per dimension 0 = same image, 1 = j
 // taken at x_j - L, 2 = i taken at x_i - L, so that every r_ij is formed
@@ -24,6 +27,7 @@
 #include <algorithm>
 
 #include "forces_core.cuh"
+#include "pair_tiles.cuh"
 
 namespace dcm {
 
@@ -135,22 +139,56 @@ struct CountVisitor {
   }
 };
 
-// Predicated 32-bit store (no branch around it in the candidate loop).
-__device__ __forceinline__ void store_if(bool p, uint32_t* addr, uint32_t v) {
-  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q st.global.u32 [%0], %1;\n\t}" ::"l"(addr), "r"(v),
-               "r"((uint32_t)p));  // no memory clobber: nothing in the build reads the lists back
+// Where entry k of a lane's column (which starts at lane_column) is.
+__device__ __forceinline__ int64_t entry_at(int k) { return (int64_t)(k & ~3) * 32 + (k & 3); }
+template <typename T>
+__device__ __forceinline__ T* lane_column(T* list, const int32_t* __restrict__ offw, int64_t i) {
+  return list + (int64_t)__ldg(offw + (i >> 5)) * 32 + 4 * (i & 31);
 }
+
+// A lane's column being filled: plain entries from the front, collected in
+// registers and stored four at a time (predicated: no branch in the candidate
+// loop), image entries from the back, nothing written past the capacity.
+struct ListColumn {
+  uint32_t* out;
+  int cap, kf, kb;
+  uint32_t b[4];  // the last four plain entries
+  __device__ __forceinline__ void plain(bool take, uint32_t j) {
+    b[0] = take ? b[1] : b[0];
+    b[1] = take ? b[2] : b[1];
+    b[2] = take ? b[3] : b[2];
+    b[3] = take ? j : b[3];
+    const bool full = take && (kf & 3) == 3 && kf < cap - kb;
+    // no memory clobber: nothing in the build reads the lists back
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %5, 0;\n\t@q st.global.v4.u32 [%0], {%1, %2, %3, %4};\n\t}" ::"l"(
+                     out + (int64_t)(kf & ~3) * 32),
+                 "r"(b[0]), "r"(b[1]), "r"(b[2]), "r"(b[3]), "r"((uint32_t)full));
+    kf += take ? 1 : 0;
+  }
+  __device__ __forceinline__ void image(uint32_t j, uint32_t code) {
+    if (kf + kb < cap) out[entry_at(cap - 1 - kb)] = j | (code << kIdxBits);
+    ++kb;
+  }
+  // the last, incomplete quad; whether all entries fit
+  __device__ __forceinline__ bool finish() {
+    const int k0 = kf & ~3, lim = cap - kb;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const int left = kf & 3;  // entries b[4 - left .. 3]
+      const uint32_t e = left == 1 ? b[3] : (left == 2 ? b[2 + (q & 1)] : b[1 + q]);
+      if (q < left && k0 + q < lim) out[entry_at(k0 + q)] = e;
+    }
+    return kf + kb <= cap;
+  }
+};
 
 template <typename R>
 struct FillVisitor {
   const typename RT<R>::R4* __restrict__ pos;
-  uint32_t* __restrict__ out;  // the lane's column: entry k at out[32 k]
   R rl2;
-  int cap, kf, kb;
+  ListColumn col;
   Owner<R> own;
   __device__ __forceinline__ void plain(int j0, int j1, R xi, R yi, R zi) {
-    const int lim = cap - kb;
-    int k = kf;
     int j = j0;
     if constexpr (sizeof(R) == 4) {  // two candidates per packed r^2 (the same roundings as one at a time)
       // four position loads in flight: the walk does little arithmetic per
@@ -163,46 +201,23 @@ struct FillVisitor {
                      ez = make_float2(zi - p2.z, zi - p3.z);
         const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
         const float2 s2 = __ffma2_rn(ex, ex, __ffma2_rn(ey, ey, __fmul2_rn(ez, ez)));
-        const bool a0 = r2.x < rl2 && own.keeps(j), a1 = r2.y < rl2 && own.keeps(j + 1),
-                   a2 = s2.x < rl2 && own.keeps(j + 2), a3 = s2.y < rl2 && own.keeps(j + 3);
-        store_if(a0 && k < lim, out + (int64_t)k * 32, (uint32_t)j);
-        k += a0 ? 1 : 0;
-        store_if(a1 && k < lim, out + (int64_t)k * 32, (uint32_t)(j + 1));
-        k += a1 ? 1 : 0;
-        store_if(a2 && k < lim, out + (int64_t)k * 32, (uint32_t)(j + 2));
-        k += a2 ? 1 : 0;
-        store_if(a3 && k < lim, out + (int64_t)k * 32, (uint32_t)(j + 3));
-        k += a3 ? 1 : 0;
-      }
-      for (; j + 1 < j1; j += 2) {
-        const float4 p0 = __ldg(pos + j), p1 = __ldg(pos + j + 1);
-        const float2 dx = make_float2(xi - p0.x, xi - p1.x), dy = make_float2(yi - p0.y, yi - p1.y),
-                     dz = make_float2(zi - p0.z, zi - p1.z);
-        const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
-        const bool a0 = r2.x < rl2 && own.keeps(j), a1 = r2.y < rl2 && own.keeps(j + 1);
-        store_if(a0 && k < lim, out + (int64_t)k * 32, (uint32_t)j);
-        k += a0 ? 1 : 0;
-        store_if(a1 && k < lim, out + (int64_t)k * 32, (uint32_t)(j + 1));
-        k += a1 ? 1 : 0;
+        col.plain(r2.x < rl2 && own.keeps(j), (uint32_t)j);
+        col.plain(r2.y < rl2 && own.keeps(j + 1), (uint32_t)(j + 1));
+        col.plain(s2.x < rl2 && own.keeps(j + 2), (uint32_t)(j + 2));
+        col.plain(s2.y < rl2 && own.keeps(j + 3), (uint32_t)(j + 3));
       }
     }
     for (; j < j1; ++j) {
       auto pj = ldg4(pos + j);
       R dx = xi - pj.x, dy = yi - pj.y, dz = zi - pj.z;
-      const bool acc = fma(dx, dx, fma(dy, dy, dz * dz)) < rl2 && own.keeps(j);
-      store_if(acc && k < lim, out + (int64_t)k * 32, (uint32_t)j);
-      k += acc ? 1 : 0;
+      col.plain(fma(dx, dx, fma(dy, dy, dz * dz)) < rl2 && own.keeps(j), (uint32_t)j);
     }
-    kf = k;
   }
   __device__ __forceinline__ void image(int j0, int j1, R xi, R yi, R zi, R shx, R shy, R shz, uint32_t code) {
     for (int j = j0; j < j1; ++j) {
       auto pj = ldg4(pos + j);
       R dx = xi - (pj.x + shx), dy = yi - (pj.y + shy), dz = zi - (pj.z + shz);
-      if (fma(dx, dx, fma(dy, dy, dz * dz)) < rl2 && own.keeps(j)) {
-        if (kf + kb < cap) out[(int64_t)(cap - 1 - kb) * 32] = (uint32_t)j | (code << kIdxBits);
-        ++kb;
-      }
+      if (fma(dx, dx, fma(dy, dy, dz * dz)) < rl2 && own.keeps(j)) col.image((uint32_t)j, code);
     }
   }
 };
@@ -230,7 +245,24 @@ __global__ void __launch_bounds__(128) k_list_count(int64_t n, const typename RT
   }
   int m = cnt;
   for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) capw[i >> 5] = m;
+  if ((threadIdx.x & 31) == 0) capw[i >> 5] = (m + 3) & ~3;
+}
+
+// The list of particle i by the row walk.
+template <typename R>
+__device__ __forceinline__ bool fill_one(int i, const typename RT<R>::R4* __restrict__ pos, const R* __restrict__ rc,
+                                         const int32_t* __restrict__ start, const Grid<R>& g, R rc_max, R skin, int n3,
+                                         const int32_t* __restrict__ capw, const int32_t* __restrict__ offw,
+                                         uint32_t* __restrict__ list, int32_t* __restrict__ nnb,
+                                         int32_t* __restrict__ nimg) {
+  auto pi = ldg4(pos + i);
+  R rl = list_radius<R>(rc[i], rc_max, skin);
+  FillVisitor<R> v{pos, rl * rl, ListColumn{lane_column(list, offw, i), capw[i >> 5], 0, 0, {0, 0, 0, 0}},
+                   Owner<R>{rc, clamp_cutoff<R>(rc[i], rc_max), rc_max, i, n3}};
+  walk_segments<R>(start, g, i, pi, rl, v);
+  nnb[i] = v.col.kf;
+  nimg[i] = v.col.kb;
+  return v.col.finish();
 }
 
 // Fill lane columns of capacity capw[warp]: plain entries from the front,
@@ -246,14 +278,114 @@ __global__ void __maxnreg__(80) k_list_fill(int64_t n, const typename RT<R>::R4*
                                                    int32_t* __restrict__ flag) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  auto pi = ldg4(pos + i);
-  R rl = list_radius<R>(rc[i], rc_max, skin);
-  FillVisitor<R> v{pos, list + (int64_t)offw[i >> 5] * 32 + (threadIdx.x & 31), rl * rl, capw[i >> 5], 0, 0,
-                   Owner<R>{rc, clamp_cutoff<R>(rc[i], rc_max), rc_max, (int)i, n3}};
-  walk_segments<R>(start, g, (int)i, pi, rl, v);
-  nnb[i] = v.kf;
-  nimg[i] = v.kb;
-  if (v.kf + v.kb > v.cap) atomicExch(flag, 1);
+  if (!fill_one<R>((int)i, pos, rc, start, g, rc_max, skin, n3, capw, offw, list, nnb, nimg)) atomicExch(flag, 1);
+}
+
+// What the tiles stage: position and index (-0 becomes +0, so that a sign bit
+// means an image).
+__global__ void k_list_records(int64_t n, const float4* __restrict__ pos, float4* __restrict__ rec) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const float4 p = __ldg(pos + i);
+  rec[i] = make_float4(p.x + 0.f, p.y + 0.f, p.z + 0.f, __int_as_float((int)i));
+}
+
+constexpr int kListTileWarps = 16;  // as the tiled forces: as many as the SM's shared memory holds
+
+// The lists over tiles of 32 particles (pair_tiles.cuh): the same r^2 of the same
+// coordinates as the row walk, so the same entries, in another order.  In a
+// tile's frame a coordinate below zero is taken at x - L; an entry is plain where
+// both particles or neither are.  Issue-bound like the tiled forces, with the
+// scattered stores behind it: 1.1M particles at skin 0.5 took 1069 us by the row
+// walk (1170 with quads), 914 over tiles with one 4-byte store per entry, 736 with
+// pairs of entries, 662 with quads; 16.7M particles 13.3 -> 8.7 ms with all else
+// that a build does.
+template <bool N3>
+__global__ void __launch_bounds__(32 * kListTileWarps, 1) k_list_tiles(
+    const float4* __restrict__ rec, const float* __restrict__ rc, const int32_t* __restrict__ start,
+    const __grid_constant__ Grid<float> g, TileCfg cfg, TileTable t, int64_t nslot, float rc_max, float skin,
+    const int32_t* __restrict__ capw, const int32_t* __restrict__ offw, uint32_t* __restrict__ list,
+    int32_t* __restrict__ nnb, int32_t* __restrict__ nimg, int32_t* __restrict__ flag) {
+  const unsigned full = 0xffffffffu;
+  extern __shared__ __align__(32) unsigned char smem_raw[];
+  TileSmem<float4>& sm = reinterpret_cast<TileSmem<float4>*>(smem_raw)[threadIdx.x >> 5];
+  const int lane = threadIdx.x & 31;
+  const int nfirst = __ldg(t.counters + kTileFirst), ntile = nfirst + __ldg(t.counters + kTileLater);
+  if (__ldg(t.counters + kTileOutside)) return;  // all tiles go to the row walk
+  for (;;) {
+    int k = 0;
+    if (lane == 0) k = atomicAdd(t.counters + kTileQueue, 1);
+    k = __shfl_sync(full, k, 0);
+    if (k >= ntile) break;
+    const int slot = __ldg(k < nfirst ? t.list + k : t.list + (nslot - 1 - (k - nfirst)));
+    const int i = __ldg(t.idx + 32 * (int64_t)slot + lane);
+    const bool active = i >= 0;
+    const float4 pi = __ldg(rec + max(i, 0));
+    const float ri = rc[max(i, 0)], rci = clamp_cutoff<float>(ri, rc_max), rl = list_radius<float>(ri, rc_max, skin);
+    const float rl2 = active ? rl * rl : 0.f;
+    float xi[3] = {pi.x, pi.y, pi.z};
+    ListColumn col{list, 0, 0, 0, {0, 0, 0, 0}};
+    if (active) {
+      col.out = lane_column(list, offw, i);
+      col.cap = __ldg(capw + (i >> 5));
+    }
+    const bool done = tile_candidates<float, float4>(
+        sm, rec, start, g, cfg, active, i, xi, rl, rl, NoCutoff{}, []() {}, [&](int last) {
+          ListWalk l;
+          l.begin(shared_addr(&sm.list[0][lane]), last);
+          while (l.more()) {
+            float4 p[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) p[q] = lds4(l.next(4));
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const float dx = xi[0] - p[q].x, dy = xi[1] - p[q].y, dz = xi[2] - p[q].z;
+              bool take = fmaf(dx, dx, fmaf(dy, dy, dz * dz)) < rl2;
+              const int j = __float_as_int(p[q].w);
+              if constexpr (N3) {
+                if (take) {
+                  const float rcj = clamp_cutoff<float>(__ldg(rc + j), rc_max);
+                  take = rci > rcj || (rci == rcj && i < j);
+                }
+              }
+              const uint32_t sx = __float_as_uint(p[q].x), sy = __float_as_uint(p[q].y), sz = __float_as_uint(p[q].z);
+              const uint32_t mx = __float_as_uint(xi[0]), my = __float_as_uint(xi[1]), mz = __float_as_uint(xi[2]);
+              const bool image = (int)((sx ^ mx) | (sy ^ my) | (sz ^ mz)) < 0;
+              if (take && image) {  // per dimension 1: j at x - L and i not, 2: i at x - L and j not
+                auto code = [](uint32_t j_at, uint32_t i_at) { return (j_at & ~i_at) >> 31 | ((i_at & ~j_at) >> 31) << 1; };
+                col.image((uint32_t)j, code(sx, mx) | code(sy, my) << 2 | code(sz, mz) << 4);
+              }
+              col.plain(take && !image, (uint32_t)j);
+            }
+          }
+        });
+    if (!done) {
+      if (lane == 0) t.rest[atomicAdd(t.counters + kTileRest, 1)] = slot;
+    } else if (active) {
+      nnb[i] = col.kf;
+      nimg[i] = col.kb;
+      if (!col.finish()) atomicExch(flag, 1);
+    }
+  }
+}
+
+// The tiles that the filter does not serve, by the row walk: those left over,
+// or all of them if a coordinate lies outside the box.
+__global__ void __launch_bounds__(64) k_list_rest(const float4* __restrict__ pos, const float* __restrict__ rc,
+                                                  const int32_t* __restrict__ start, Grid<float> g, TileTable t,
+                                                  int64_t nslot, float rc_max, float skin, int n3,
+                                                  const int32_t* __restrict__ capw, const int32_t* __restrict__ offw,
+                                                  uint32_t* __restrict__ list, int32_t* __restrict__ nnb,
+                                                  int32_t* __restrict__ nimg, int32_t* __restrict__ flag) {
+  const bool all = __ldg(t.counters + kTileOutside) != 0;
+  const int nfirst = __ldg(t.counters + kTileFirst), lane = threadIdx.x & 31;
+  const int n = all ? nfirst + __ldg(t.counters + kTileLater) : __ldg(t.counters + kTileRest);
+  for (int k = blockIdx.x * 2 + (threadIdx.x >> 5); k < n; k += gridDim.x * 2) {
+    const int slot = __ldg(!all ? t.rest + k : (k < nfirst ? t.list + k : t.list + (nslot - 1 - (k - nfirst))));
+    const int i = __ldg(t.idx + 32 * (int64_t)slot + lane);
+    if (i >= 0 && !fill_one<float>(i, pos, rc, start, g, rc_max, skin, n3, capw, offw, list, nnb, nimg))
+      atomicExch(flag, 1);
+  }
 }
 
 // Capacity bound of a list of radius R: the particles a sphere of radius R can
@@ -270,7 +402,7 @@ __global__ void k_list_caps(int64_t n, const R* __restrict__ rc, R rc_max, R ski
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   int cap = i < n ? list_cap_bound<R>(list_radius<R>(rc[i], rc_max, skin)) : 0;
   for (int o = 16; o > 0; o >>= 1) cap = max(cap, __shfl_xor_sync(0xffffffffu, cap, o));
-  if ((threadIdx.x & 31) == 0) capw[i >> 5] = cap;
+  if ((threadIdx.x & 31) == 0) capw[i >> 5] = (cap + 3) & ~3;
 }
 
 // Per-warp partials (E, W, pairs) as in the cell-list kernel.
@@ -385,16 +517,16 @@ __global__ void __launch_bounds__(128) k_forces_list(int64_t n, const typename R
         ushift[t] = (TYPED ? a.eps4[tp] : (R)4) * s6 * (s6 - (R)1);
       }
     }
-    const uint32_t* lp = list + (int64_t)offw[i >> 5] * 32 + (threadIdx.x & 31);
+    const uint32_t* lp = lane_column(list, offw, i);
     const int m = nnb[i], cap = capw[i >> 5], mb = nimg[i];
 #pragma unroll 2
     for (int k = 0; k < m; ++k) {
-      int j = (int)__ldg(lp + (int64_t)k * 32);
+      int j = (int)__ldg(lp + entry_at(k));
       auto pj = ldg4(pos + j);
       list_pair<R, TYPED>(pi.x - pj.x, pi.y - pj.y, pi.z - pj.z, rc2, ti, pj.w, a, ushift, c);
     }
     for (int k = cap - mb; k < cap; ++k) {
-      uint32_t e = __ldg(lp + (int64_t)k * 32);
+      uint32_t e = __ldg(lp + entry_at(k));
       auto pj = ldg4(pos + (e & kIdxMask));
       R dx, dy, dz;
       image_delta<R>(e >> kIdxBits, pi, pj, a.g, dx, dy, dz);
@@ -466,32 +598,32 @@ __global__ void __launch_bounds__(128) k_forces_list_x2(int64_t n, const float4*
     if (!(rci <= a.rc_max)) rci = a.rc_max;
     if (!(rci > 0.f)) rci = 0.f;
     const float rc2 = rci * rci;
-    const uint32_t* lp = list + (int64_t)offw[i >> 5] * 32 + (threadIdx.x & 31);
+    const uint32_t* lp = lane_column(list, offw, i);
     const int m = nnb[i], cap = capw[i >> 5], mb = nimg[i];
     PackedAcc pc;
     pc.fx = pc.fy = pc.fz = pc.en = pc.vir = f2(0.f, 0.f);
     pc.np = 0;
     int k = 0;
-    // four entries per iteration; the next four indices are requested before
-    // this iteration's arithmetic (the list streams from DRAM once, so its
-    // loads bypass L1 and leave it to the positions)
+    // a quad of entries per iteration; the next quad is requested before this
+    // iteration's arithmetic (the list streams from DRAM once, so its loads
+    // bypass L1 and leave it to the positions).  Two 8-byte loads: 357 us for 1.1M
+    // particles, 394 us with one of 16 bytes
     if (k + 3 < m) {
-      int e0 = (int)__ldcs(lp), e1 = (int)__ldcs(lp + 32), e2 = (int)__ldcs(lp + 64), e3 = (int)__ldcs(lp + 96);
+      const uint2* q = reinterpret_cast<const uint2*>(lp);
+      uint2 e0 = __ldcs(q), e1 = __ldcs(q + 1);
       for (; k + 3 < m; k += 4) {
-        const float4 p0 = __ldg(pos + e0), p1 = __ldg(pos + e1), p2 = __ldg(pos + e2), p3 = __ldg(pos + e3);
+        const float4 p0 = __ldg(pos + e0.x), p1 = __ldg(pos + e0.y), p2 = __ldg(pos + e1.x), p3 = __ldg(pos + e1.y);
+        q += 64;
         if (k + 7 < m) {
-          const uint32_t* q = lp + (int64_t)(k + 4) * 32;
-          e0 = (int)__ldcs(q);
-          e1 = (int)__ldcs(q + 32);
-          e2 = (int)__ldcs(q + 64);
-          e3 = (int)__ldcs(q + 96);
+          e0 = __ldcs(q);
+          e1 = __ldcs(q + 1);
         }
         packed_pair(pi, p0, p1, rc2, pc);
         packed_pair(pi, p2, p3, rc2, pc);
       }
     }
     if (k + 1 < m) {
-      const int j0 = (int)__ldg(lp + (int64_t)k * 32), j1 = (int)__ldg(lp + (int64_t)(k + 1) * 32);
+      const int j0 = (int)__ldg(lp + entry_at(k)), j1 = (int)__ldg(lp + entry_at(k + 1));
       packed_pair(pi, __ldg(pos + j0), __ldg(pos + j1), rc2, pc);
       k += 2;
     }
@@ -506,12 +638,12 @@ __global__ void __launch_bounds__(128) k_forces_list_x2(int64_t n, const float4*
     c.np = np;
     const float ushift0 = 0.f;
     if (k < m) {
-      const int j = (int)__ldg(lp + (int64_t)k * 32);
+      const int j = (int)__ldg(lp + entry_at(k));
       const float4 pj = __ldg(pos + j);
       list_pair<float, false>(pi.x - pj.x, pi.y - pj.y, pi.z - pj.z, rc2, 0, pj.w, a, &ushift0, c);
     }
     for (int kk = cap - mb; kk < cap; ++kk) {
-      const uint32_t e = __ldg(lp + (int64_t)kk * 32);
+      const uint32_t e = __ldg(lp + entry_at(kk));
       const float4 pj = __ldg(pos + (e & kIdxMask));
       float dx, dy, dz;
       image_delta<float>(e >> kIdxBits, pi, pj, a.g, dx, dy, dz);
@@ -639,7 +771,7 @@ __global__ void __launch_bounds__(128) k_forces_list_n3(int64_t n, const typenam
       return a.eps4[tp] * s6 * (s6 - (R)1);
     };
     R fx = 0, fy = 0, fz = 0, ei = 0;
-    const uint32_t* lp = list + (int64_t)offw[i >> 5] * 32 + (threadIdx.x & 31);
+    const uint32_t* lp = lane_column(list, offw, i);
     const int m = nnb[i], cap = capw[i >> 5], mb = nimg[i];
     auto pair = [&](uint32_t e, bool image) {
       const int j = (int)(e & kIdxMask);
@@ -680,8 +812,8 @@ __global__ void __launch_bounds__(128) k_forces_list_n3(int64_t n, const typenam
         ++np;
       }
     };
-    for (int k = 0; k < m; ++k) pair(__ldg(lp + (int64_t)k * 32), false);
-    for (int k = cap - mb; k < cap; ++k) pair(__ldg(lp + (int64_t)k * 32), true);
+    for (int k = 0; k < m; ++k) pair(__ldg(lp + entry_at(k)), false);
+    for (int k = cap - mb; k < cap; ++k) pair(__ldg(lp + entry_at(k)), true);
     ei *= (R)0.5;
     E += (double)ei;
     add_force4<R>(force + i, fx, fy, fz, ei);
@@ -732,13 +864,14 @@ __global__ void __launch_bounds__(128) k_forces_list_n3_x2(int64_t n, const floa
       return 4.f * s6 * (s6 - 1.f);
     };
     const float usi = ushift(rc2);
-    const uint32_t* lp = list + (int64_t)offw[i >> 5] * 32 + (threadIdx.x & 31);
+    const uint32_t* lp = lane_column(list, offw, i);
     const int m = nnb[i], cap = capw[i >> 5], mb = nimg[i];
     float2 fx = f2(0.f, 0.f), fy = f2(0.f, 0.f), fz = f2(0.f, 0.f);
     const float2 two = f2(2.f, 2.f), m1 = f2(-1.f, -1.f);
     int k = 0;
     for (; k + 1 < m; k += 2) {
-      const int j0 = (int)__ldcs(lp + (int64_t)k * 32), j1 = (int)__ldcs(lp + (int64_t)(k + 1) * 32);
+      const uint2 e = __ldcs(reinterpret_cast<const uint2*>(lp + entry_at(k)));
+      const int j0 = (int)e.x, j1 = (int)e.y;
       const float4 p0 = __ldg(pos + j0), p1 = __ldg(pos + j1);
       const float rj0 = clamp_cutoff<float>(__ldg(rc + j0), a.rc_max), rj1 = clamp_cutoff<float>(__ldg(rc + j1), a.rc_max);
       const float2 dx = f2(pi.x - p0.x, pi.x - p1.x), dy = f2(pi.y - p0.y, pi.y - p1.y), dz = f2(pi.z - p0.z, pi.z - p1.z);
@@ -815,8 +948,8 @@ __global__ void __launch_bounds__(128) k_forces_list_n3_x2(int64_t n, const floa
         ++np;
       }
     };
-    if (k < m) pair(__ldg(lp + (int64_t)k * 32), false);
-    for (int kk = cap - mb; kk < cap; ++kk) pair(__ldg(lp + (int64_t)kk * 32), true);
+    if (k < m) pair(__ldg(lp + entry_at(k)), false);
+    for (int kk = cap - mb; kk < cap; ++kk) pair(__ldg(lp + entry_at(kk)), true);
     ei = 0.5f * (ei + sei);
     add_force4<float>(force + i, (fx.x + fx.y) + sfx, (fy.x + fy.y) + sfy, (fz.x + fz.y) + sfz, ei);
   }
@@ -852,6 +985,45 @@ static int ensure_list_capacity(dcm_ctx* ctx, int64_t need) {
   return DCM_OK;
 }
 
+// Fill the columns of the capacities capw, over tiles where they serve (mixed
+// form).  Leaves the positions of the build in xbuild (the tiles stage them from
+// there; w then holds the index, which nothing else reads).
+template <typename R>
+static int list_fill(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, const R* rc, cudaStream_t st) {
+  const Grid<R> g = cell_grid<R>(ctx);
+  const R skin = (R)ctx->p.skin, rcm = (R)ctx->p.rc_max;
+  const int n3 = ctx->p.newton3;
+  const unsigned nblk = (unsigned)((n + 127) / 128);
+  if constexpr (sizeof(R) == 4) {
+    const TilePlan tp = list_tile_plan(ctx->p, ctx->nc, n);
+    if (ctx->tiles && tp.usable && n >= kListTilesMinN) {
+      float4* rec = (float4*)ctx->xbuild;
+      TileTable t;
+      int r = tile_cut<float>(ctx, tp, pos, rc, ctx->cell_start, g, t, st);
+      if (r) return r;
+      auto k = n3 ? k_list_tiles<true> : k_list_tiles<false>;
+      constexpr int smem = kListTileWarps * (int)sizeof(TileSmem<float4>);
+      static_assert(smem <= 227 * 1024, "one block per SM");
+      DCM_CUDA_TRY(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+      int sms = 0;
+      DCM_CUDA_TRY(ctx, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
+      DCM_LAUNCH(ctx, k_list_records, (unsigned)((n + 255) / 256), 256, 0, st, n, pos, rec);
+      DCM_LAUNCH(ctx, k, (unsigned)std::min<int64_t>((tp.slots + kListTileWarps - 1) / kListTileWarps, sms),
+                 32 * kListTileWarps, smem, st, rec, rc, ctx->cell_start, g, tp.cfg, t, tp.slots, rcm, skin, ctx->capw,
+                 ctx->offw, ctx->list, ctx->nnb, ctx->nimg, ctx->lflag);
+      DCM_LAUNCH(ctx, k_list_rest, (unsigned)std::min<int64_t>((tp.slots + 1) / 2, 8 * sms), 64, 0, st, pos, rc,
+                 ctx->cell_start, g, t, tp.slots, rcm, skin, n3, ctx->capw, ctx->offw, ctx->list, ctx->nnb, ctx->nimg,
+                 ctx->lflag);
+      return DCM_OK;
+    }
+  }
+  if (n > 0)
+    DCM_LAUNCH(ctx, k_list_fill<R>, nblk, 128, 0, st, n, pos, rc, ctx->cell_start, g, rcm, skin, n3, ctx->capw,
+               ctx->offw, ctx->list, ctx->nnb, ctx->nimg, ctx->lflag);
+  DCM_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->xbuild, pos, sizeof(typename RT<R>::R4) * n, cudaMemcpyDeviceToDevice, st));
+  return DCM_OK;
+}
+
 // Build: bounded capacities -> one walk; on overflow, exact count + fill.
 template <typename R>
 int list_build(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, const R* rc, cudaStream_t st) {
@@ -867,9 +1039,7 @@ int list_build(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, const R* 
   DCM_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->host_status + 1, ctx->offw + nw, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
   DCM_CUDA_TRY(ctx, cudaStreamSynchronize(st));
   if ((r = ensure_list_capacity(ctx, (int64_t)ctx->host_status[1] * 32))) return r;
-  if (n > 0)
-    DCM_LAUNCH(ctx, k_list_fill<R>, (unsigned)nblk, 128, 0, st, n, pos, rc, ctx->cell_start, g, rcm, skin, n3,
-               ctx->capw, ctx->offw, ctx->list, ctx->nnb, ctx->nimg, ctx->lflag);
+  if ((r = list_fill<R>(ctx, n, pos, rc, st))) return r;
   DCM_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->host_status + 3, ctx->lflag, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
   DCM_CUDA_TRY(ctx, cudaStreamSynchronize(st));
   if (ctx->host_status[3]) {
@@ -882,11 +1052,8 @@ int list_build(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, const R* 
     DCM_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->host_status + 1, ctx->offw + nw, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     DCM_CUDA_TRY(ctx, cudaStreamSynchronize(st));
     if ((r = ensure_list_capacity(ctx, (int64_t)ctx->host_status[1] * 32))) return r;
-    if (n > 0)
-      DCM_LAUNCH(ctx, k_list_fill<R>, (unsigned)nblk, 128, 0, st, n, pos, rc, ctx->cell_start, g, rcm, skin, n3,
-                 ctx->capw, ctx->offw, ctx->list, ctx->nnb, ctx->nimg, ctx->lflag);
+    if ((r = list_fill<R>(ctx, n, pos, rc, st))) return r;
   }
-  DCM_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->xbuild, pos, sizeof(typename RT<R>::R4) * n, cudaMemcpyDeviceToDevice, st));
   stage_end(ctx, DCM_STAGE_LISTS, st);
   ctx->list_valid = 1;
   return check_launch(ctx, "list_build");

@@ -147,3 +147,120 @@ def test_tiles_coordinates_outside_the_box(D, bad):
     assert np.sqrt(((F1 - F0)[ok, :3] ** 2).mean()) <= MIXED_RMS * rms
     if np.isfinite(t0).all():
         assert t1[2] == t0[2]
+
+
+def by_input(D, box, pos, rc, types, upstream=None, **kw):
+    """Forces (or, with upstream gradients, the adjoint) in input order."""
+    n = len(pos)
+    fp64 = kw.get("precision") == D.DCM_PREC_FP64
+    real = torch.float64 if fp64 else torch.float32
+    ctx = D.Context(D.make_params(box, n_max=n, ntypes=2, eps=(1.0, 0.8), sigma=(1.0, 1.1), **kw))
+    p4 = D.to_real4(torch.from_numpy(pos), torch.from_numpy(types), real)
+    dev = dict(dtype=torch.int32, device="cuda")
+    cell, start, perm = torch.empty(n, **dev), torch.empty(ctx.ncell + 1, **dev), torch.empty(n, **dev)
+    ps = torch.empty_like(p4)
+    D.dcm_bin(ctx, n, p4, cell, start, perm, ps)
+    perm = perm.long()
+    rcs = torch.from_numpy(rc).to(real).cuda()[perm].contiguous()
+    out = torch.empty_like(ps)
+    dpar = torch.zeros(4, dtype=torch.float64, device="cuda")
+    if upstream is None:
+        D.dcm_forces(ctx, n, ps, rcs, start, out)
+    else:
+        A = torch.from_numpy(upstream).to(real).cuda()[perm].contiguous()
+        D.dcm_forces_backward(ctx, n, ps, rcs, start, A, 0.7, out, dpar)
+    res = torch.empty_like(out)
+    res[perm] = out
+    assert D.dcm_status(ctx) == D.DCM_OK
+    ctx.close()
+    return res.double().cpu().numpy(), dpar.cpu().numpy()
+
+
+def crossing(n_small, seed):
+    """n_small particles, and the same with one more, alone in the vapor
+    beyond everybody's cutoff."""
+    box = (63.0, 61.5, 72.0)
+    pos = lattice(box, seed)
+    pos = pos[np.abs(pos[:, 2] - 36.0) < 18.0]
+    rng = np.random.default_rng(seed)
+    pos = pos[rng.permutation(len(pos))]
+    assert len(pos) > n_small
+    pos = pos[:n_small]
+    rc = np.clip(6.0 - (18.0 - np.abs(pos[:, 2] - 36.0)), 3.0, 6.0)
+    types = rng.integers(0, 2, n_small + 1).astype(np.float32)
+    lone = np.array([[30.0, 30.0, 1.0]], np.float32)
+    return box, np.concatenate([pos, lone]), np.append(rc, 6.0), types, rng
+
+
+@pytest.mark.parametrize("lx", [0.0, 0.5])
+def test_forces_on_both_sides_of_the_switch_to_tiles(D, lx):
+    """32,768 particles run 16 lanes per particle, one more runs tiles."""
+    n = 32768
+    box, pos, rc, types, _ = crossing(n, 21)
+    F0, _ = by_input(D, box, pos[:n], rc[:n], types[:n], lx=lx)
+    F1, _ = by_input(D, box, pos, rc, types, lx=lx)
+    assert np.all(F1[n] == 0.0)
+    rms = np.sqrt((F0[:, :3] ** 2).mean())
+    assert np.sqrt(((F1[:n] - F0)[:, :3] ** 2).mean()) <= MIXED_RMS * rms
+
+
+@pytest.mark.parametrize("n,lx", [(3000, 0.0), (49152, 0.5), (49153, 0.5), (49153, 0.0)])
+def test_adjoint_forms_against_fp64(D, n, lx):
+    """A warp per particle (up to 49,152) and tiles (above) against the FP64
+    row walk.  A pair term g'/r d d.A carries about 20 roundings, amplified by the
+    powers of 1/r^2 (14 at most): 20 x 14 x 2^-24 = 1.7e-5 at worst, random over
+    the pairs: RMS 5e-6; parameter sums over all pairs likewise."""
+    box, pos, rc, types, rng = crossing(n - 1, 31)
+    A = np.concatenate([rng.normal(size=(n, 3)), np.zeros((n, 1))], 1).astype(np.float32)
+    # pairs whose distance is within FP32 rounding of a cutoff may fall on either side: their terms are of the
+    # size of the forces at the cutoff, 1e-3 of the RMS gradient, and rare
+    G0, d0 = by_input(D, box, pos, rc.astype(np.float32).astype(np.float64), types, A, lx=lx, shift_energy=1,
+                      precision=D.DCM_PREC_FP64)
+    G1, d1 = by_input(D, box, pos, rc.astype(np.float32).astype(np.float64), types, A, lx=lx, shift_energy=1)
+    rms = np.sqrt((G0[:, :3] ** 2).mean())
+    assert np.sqrt(((G1 - G0)[:, :3] ** 2).mean()) <= 5e-6 * rms
+    assert np.all(G1[:, 3] == 0.0)
+    assert np.all(np.abs(d1 - d0) <= 5e-6 * np.abs(d0).max())
+
+
+@pytest.mark.parametrize("box,n,spacing,typed,kw", [
+    ((42.0, 45.0, 51.0), None, 1.12, False, dict(lx=0.5)),              # tiles across every boundary
+    ((27.0, 30.0, 40.5), None, 1.12, True, dict()),                     # most tiles at a boundary, two types
+    ((42.0, 45.0, 51.0), None, 1.12, False, dict(newton3=1)),           # half lists
+    ((27.0, 30.0, 40.5), None, 1.12, True, dict(newton3=1, lx=0.75)),
+    ((27.0, 30.0, 40.5), None, 0.8, False, dict(lx=0.5)),               # denser than the capacity bound: two fills
+    ((42.0, 45.0, 51.0), 4000, 1.12, False, dict(shift_energy=1)),      # the switch to tiles
+    ((42.0, 45.0, 51.0), 3999, 1.12, False, dict(shift_energy=1)),
+])
+def test_lists_over_tiles(D, box, n, spacing, typed, kw):
+    """Neighbour lists built over tiles against the cell path: the same pairs
+    exactly; forces to 1e-5 (sums of up to 500 FP32 terms in one chain: 2^-24
+    sqrt(500) = 1.3e-6 of partial sums a few times the force)."""
+    pos = lattice(box, 41, spacing, 0.2 * spacing / 1.12)
+    rng = np.random.default_rng(41)
+    if n:
+        pos = pos[rng.permutation(len(pos))[:n]]
+    types = rng.integers(0, 2, len(pos)).astype(np.float32) if typed else None
+    if typed:
+        kw = dict(kw, ntypes=2, eps=(1.0, 0.8), sigma=(1.0, 1.1))
+    res = []
+    for skin in (0.5, 0.0):
+        k = dict(kw) if skin else {a: b for a, b in kw.items() if a != "newton3"}
+        ctx = D.Context(D.make_params(box, n_max=len(pos), recompute_every=4, skin=skin, **k))
+        st = D.State(ctx, D.to_real4(torch.from_numpy(pos), None if types is None else torch.from_numpy(types)),
+                     torch.zeros(len(pos), 4))
+        D.dcm_step_init(ctx, st)
+        for _ in range(2):  # a step so short that nothing moves
+            D.dcm_step(ctx, st, 1e-12, 1)
+        assert D.dcm_status(ctx) == D.DCM_OK
+        _, _, rc, ids = st.current()
+        F, r = np.empty((len(pos), 3)), np.empty(len(pos))
+        ids = ids.cpu().numpy()
+        F[ids], r[ids] = st.force.double().cpu().numpy()[:, :3], rc.double().cpu().numpy()
+        res.append((F, r, st.thermo.cpu().numpy()))
+        ctx.close()
+    (F0, r0, t0), (F1, r1, t1) = res
+    assert np.array_equal(r0, r1)
+    assert t0[3] == t1[3]
+    assert np.sqrt(((F0 - F1) ** 2).mean()) <= 1e-5 * np.sqrt((F1 ** 2).mean())
+    assert abs(t0[0] - t1[0]) <= 1e-5 * abs(t1[0]) and abs(t0[1] - t1[1]) <= 1e-5 * abs(t1[1])
