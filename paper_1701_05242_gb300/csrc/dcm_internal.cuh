@@ -264,12 +264,16 @@ int lj_forces(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, const R* r
 
 // Systems of at most kPlanesMaxN particles (mixed form, default accumulation)
 // take 16 lanes per particle in the forces (k_forces_planes), whose blocks of 8
-// particles each leave one partial sum.
+// particles each leave one partial sum.  With energies, 16 lanes / one thread per
+// particle / tiles: 41 / 193 / - us for 1,935 particles, 97 / 219 / - for 30,240,
+// - / 238 / 106 for 39,191.
 constexpr int64_t kPlanesMaxN = 32768;
 constexpr int kPlaneLanes = 16, kPlaneBlock = 128;  // lanes per particle, threads per block
 constexpr int64_t plane_slots(int64_t n) { return (n + 7) / 8; }
 // Systems of at most kAdjWarpMaxN particles take a warp per particle in the
-// packed adjoint (k_adjoint_warp, blocks of 4 particles).
+// packed adjoint (k_adjoint_warp, blocks of 4 particles): the whole call takes
+// 249 us for 41,368 particles so and 199 for 51,106 over tiles; 171 for 30,240
+// (one thread each: 490).
 constexpr int64_t kAdjWarpMaxN = 49152;
 constexpr int64_t adj_warp_slots(int64_t n) { return (n + 3) / 4; }
 
@@ -288,12 +292,20 @@ struct TilePlan {
   bool usable;
 };
 TilePlan tile_plan(const dcm_params& p, const int64_t* nc, int64_t n);
-// The same for neighbour lists, whose spheres reach rc_max + skin.
+// The same for neighbour lists, whose spheres reach R = rc_max + skin.  Boxes of
+// at least 5 R: in smaller ones too many tiles reach past a boundary from the
+// other half of the box and are left to a second kernel (a step with a build, row
+// walk / tiles: 568 / 641 us for 18,371 particles in a box of 4.15 R, 690 / 737
+// for 15,120 in 4.6 R, 632 / 445 for 10,062 in 5.1 R, 659 / 440 for 48,989 in 5.5 R).
 inline TilePlan list_tile_plan(dcm_params p, const int64_t* nc, int64_t n) {
   p.rc_max += p.skin;
-  return tile_plan(p, nc, n);
+  TilePlan t = tile_plan(p, nc, n);
+  const double lx = p.lx > 0.0 ? p.lx : p.l;
+  const double a = (double)nc[0] * lx, b = (double)nc[1] * p.l, c = (double)nc[2] * p.l;
+  t.usable = t.usable && a >= 5.0 * p.rc_max && b >= 5.0 * p.rc_max && c >= 5.0 * p.rc_max;
+  return t;
 }
-constexpr int64_t kListTilesMinN = 4000;  // below: the row walk
+constexpr int64_t kListTilesMinN = 4000;  // below: the row walk, as the forces (kTilesMinN)
 constexpr int64_t tile_ints(int64_t slots) { return 8 + 34 * slots; }
 bool tiles_serve(const dcm_ctx* ctx, int64_t n);  // whether lj_forces runs over tiles
 template <typename R>

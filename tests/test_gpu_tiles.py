@@ -225,10 +225,10 @@ def test_adjoint_forms_against_fp64(D, n, lx):
 
 @pytest.mark.parametrize("box,n,spacing,typed,kw", [
     ((42.0, 45.0, 51.0), None, 1.12, False, dict(lx=0.5)),              # tiles across every boundary
-    ((27.0, 30.0, 40.5), None, 1.12, True, dict()),                     # most tiles at a boundary, two types
+    ((33.0, 34.5, 40.5), None, 1.12, True, dict()),                     # most tiles at a boundary, two types
     ((42.0, 45.0, 51.0), None, 1.12, False, dict(newton3=1)),           # half lists
-    ((27.0, 30.0, 40.5), None, 1.12, True, dict(newton3=1, lx=0.75)),
-    ((27.0, 30.0, 40.5), None, 0.8, False, dict(lx=0.5)),               # denser than the capacity bound: two fills
+    ((33.0, 34.5, 40.5), None, 1.12, True, dict(newton3=1, lx=0.75)),
+    ((33.0, 34.5, 40.5), None, 0.8, False, dict(lx=0.5)),               # denser than the capacity bound: two fills
     ((42.0, 45.0, 51.0), 4000, 1.12, False, dict(shift_energy=1)),      # the switch to tiles
     ((42.0, 45.0, 51.0), 3999, 1.12, False, dict(shift_energy=1)),
 ])
