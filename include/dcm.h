@@ -70,12 +70,17 @@ enum dcm_status_code {
   DCM_ERR_TIMEOUT = 7        /* a device-side wait ran past its budget (a grid barrier, the cell-count scan) */
 };
 
-/* Cell-list force kernels (both walk the same culled cell rows and accept the
- * same pairs; they differ in how the pair arithmetic is issued).  The packed
+/* Cell-list force kernels (all accept the same pairs; they differ in how the
+ * candidates are found and the pair arithmetic is issued).  The packed
  * kernel serves FP32 runs (DCM_PREC_MIXED) of one or two types; otherwise
- * kernel 1 runs.  Values 2, 4 and 5 are not used (invalid). */
+ * kernel 1 runs.  AUTO finds the candidates over tiles of 32 particles with a
+ * tensor-core filter where that is faster: boxes of at least 4 rc_max, the
+ * default accumulation, more than 32,768 particles in the mixed form and 4,000
+ * in the FP64 form.  Smaller systems of the mixed form take 16 lanes per
+ * particle (AUTO and PACKED; the same sums bit for bit as one thread each).
+ * Values 2, 4 and 5 are not used (invalid). */
 enum {
-  DCM_FORCE_AUTO = 0,        /* kernel 3 where it applies, else kernel 1 */
+  DCM_FORCE_AUTO = 0,        /* tiles where they serve, else kernel 3 where it applies, else kernel 1 */
   DCM_FORCE_THREAD = 1,      /* one thread per particle i, one candidate per instruction */
   DCM_FORCE_PACKED = 3       /* one thread per particle i, two candidates per FP32x2 instruction */
 };
@@ -93,7 +98,9 @@ enum {
  *   DCM_ACC_PAIR_FP64  every pair term added in FP64
  *   DCM_ACC_PLANE_FP64 FP32 sum per z-plane of the stencil (its rows: up to
  *                      five at rc = 3), plane sums added in FP64
- *   DCM_ACC_PLANE_KAHAN the same, plane sums Kahan-compensated in FP32
+ *   DCM_ACC_PLANE_KAHAN the same, plane sums Kahan-compensated in FP32 (over
+ *                      tiles: runs of at most 32 pairs, two partial sums each,
+ *                      in place of the planes)
  *   DCM_ACC_AUTO (0)   DCM_ACC_PLANE_KAHAN, the cheapest of the compensated
  *                      forms at the accuracy of the FP64 ones (measured)
  * The pair forms run on the packed kernel; the scalar FP32 kernel (three or
@@ -283,7 +290,8 @@ int dcm_remove_small_components(dcm_ctx* ctx, const uint8_t* s_in, uint8_t* s_ou
 /* Box-interface distances, Section 2.2 and Algorithm 2.1.  D = 0 on boxes
  * with s = 0 or iface = 1, +inf elsewhere; then Godunov fast-sweeping updates
  * d = min(d, solve(neighbours)) accepted only if <= r_grid, iterated (Jacobi)
- * until no box changes.  Boxes farther than r_grid stay +inf.
+ * until no box changes, in one cooperative launch.  Boxes farther than r_grid
+ * stay +inf.
  *   D real[nboxes] out;  iters int32[1] out (device, nullable): sweeps used.
  * SYNCHRONOUS: returns DCM_ERR_NOT_CONVERGED if iter_max sweeps did not
  * converge (D then holds the last iterate). */
@@ -482,7 +490,7 @@ int dcm_batch_launch_count(dcm_batch* b, int64_t* count, int32_t reset);
 /* Stages of dcm_step whose GPU time can be measured. */
 enum dcm_stage {
   DCM_STAGE_KICK_DRIFT = 0, /* half kick, drift, cell count */
-  DCM_STAGE_BIN = 1,        /* scan, scatter, per-cell sort, gather of the state */
+  DCM_STAGE_BIN = 1,        /* scan, placement in the stable order, gather of the state */
   DCM_STAGE_DETECT = 2,     /* dcm_detect_interface */
   DCM_STAGE_DISTANCE = 3,   /* dcm_distance sweeps */
   DCM_STAGE_CUTOFFS = 4,    /* dcm_cutoffs */
@@ -509,9 +517,9 @@ int dcm_stage_times(dcm_ctx* ctx, double* ms, int64_t* count);
 /* Number of CUDA kernels this context has launched; reset if reset != 0. */
 int dcm_launch_count(dcm_ctx* ctx, int64_t* count, int32_t reset);
 
-/* The DCM_FORCE_* kernel that dcm_forces and dcm_step run on the cell lists
- * for this context's parameters (params.force_kernel with AUTO and the
- * kernels' limits resolved), written to *kernel.  Host only. */
+/* The DCM_FORCE_* kernel whose pair arithmetic dcm_forces and dcm_step run on
+ * the cell lists for this context's parameters (params.force_kernel with AUTO
+ * and the kernels' limits resolved; the same over tiles), written to *kernel.  Host only. */
 int dcm_force_kernel(const dcm_ctx* ctx, int32_t* kernel);
 
 /* The DCM_ACC_* form in which this context's force launches sum each

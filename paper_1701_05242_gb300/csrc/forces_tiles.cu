@@ -7,11 +7,11 @@
 // a device queue.  Warps share nothing, so a long tile (at an interface the
 // spheres hold eight times the bulk's volume) holds up one warp only.
 //
-// Bound by instruction issue: 65% of the issue slots at 16 warps per SM, the
-// tensor pipe under 10% busy, HBM nearly idle.  Sixteen warps of 512 staged
+// Bound by instruction issue: 64% of the issue slots at 16 warps per SM, the
+// tensor pipe 11% busy, HBM nearly idle.  Sixteen warps of 512 staged
 // candidates fill the SM's shared memory; 13 of 640 and 20 of 384 (at 96
 // registers) were slower.  Kernel times against the row walk, energies included:
-// 16.7M particles 6140 -> 4525 us, 1.1M 525 -> 426, 260K of two types 255 -> 180,
+// 15.5M particles 6140 -> 4525 us, 1.0M 525 -> 426, 260K of two types 255 -> 180,
 // 260K in FP64 6000 -> 1725.
 #include <algorithm>
 #include <climits>
@@ -412,8 +412,9 @@ TilePlan tile_plan(const dcm_params& p, const int64_t* nc, int64_t n) {
 }
 
 // Launches below this many particles keep the row walk: that few leave most
-// SMs without a tile, and a launch lasts as long as its longest tile (FP64;
-// the mixed form takes 16 lanes per particle up to kPlanesMaxN).
+// SMs without a tile, and a launch lasts as long as its longest tile (FP64:
+// 4,838 particles 1594 us by the row walk, 618 over tiles; the mixed form takes
+// 16 lanes per particle up to kPlanesMaxN).
 constexpr int64_t kTilesMinN = 4000;
 
 bool tiles_serve(const dcm_ctx* ctx, int64_t n) {

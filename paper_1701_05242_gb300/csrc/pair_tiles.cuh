@@ -30,7 +30,7 @@
 // Why warp-wide products: the filter's product is private to 32 particles.  A
 // tcgen05 product has at least 64 rows for one set of columns (128 to use every
 // lane of the tensor memory), so the candidate columns per row would double, and
-// the shifts that read the signs, not the products (under a tenth of the
+// the shifts that read the signs, not the products (a ninth of the
 // tensor pipe), are what the filter costs.
 //
 // Periodic images keep the exact arithmetic of the row walk: an image at -L is

@@ -296,9 +296,9 @@ constexpr int kListTileWarps = 16;  // as the tiled forces: as many as the SM's 
 // coordinates as the row walk, so the same entries, in another order.  In a
 // tile's frame a coordinate below zero is taken at x - L; an entry is plain where
 // both particles or neither are.  Issue-bound like the tiled forces, with the
-// scattered stores behind it: 1.1M particles at skin 0.5 took 1069 us by the row
+// scattered stores behind it: 1.0M particles at skin 0.5 took 1069 us by the row
 // walk (1170 with quads), 914 over tiles with one 4-byte store per entry, 736 with
-// pairs of entries, 662 with quads; 16.7M particles 13.3 -> 8.7 ms with all else
+// pairs of entries, 662 with quads; 15.5M particles 13.3 -> 8.7 ms with all else
 // that a build does.
 template <bool N3>
 __global__ void __launch_bounds__(32 * kListTileWarps, 1) k_list_tiles(
@@ -606,7 +606,7 @@ __global__ void __launch_bounds__(128) k_forces_list_x2(int64_t n, const float4*
     int k = 0;
     // a quad of entries per iteration; the next quad is requested before this
     // iteration's arithmetic (the list streams from DRAM once, so its loads
-    // bypass L1 and leave it to the positions).  Two 8-byte loads: 357 us for 1.1M
+    // bypass L1 and leave it to the positions).  Two 8-byte loads: 357 us for 1.0M
     // particles, 394 us with one of 16 bytes
     if (k + 3 < m) {
       const uint2* q = reinterpret_cast<const uint2*>(lp);
