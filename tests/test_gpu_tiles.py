@@ -264,3 +264,71 @@ def test_lists_over_tiles(D, box, n, spacing, typed, kw):
     assert t0[3] == t1[3]
     assert np.sqrt(((F0 - F1) ** 2).mean()) <= 1e-5 * np.sqrt((F1 ** 2).mean())
     assert abs(t0[0] - t1[0]) <= 1e-5 * abs(t1[0]) and abs(t0[1] - t1[1]) <= 1e-5 * abs(t1[1])
+
+
+def with_negative_zeros(box, seed):
+    """The lattice with some coordinates of -0.0 per axis (particles next to
+    the boundary moved onto it, and those alone: nobody else within 0.9)."""
+    pos = lattice(box, seed)
+    rng = np.random.default_rng(seed)
+    L = np.array(box, np.float32)
+    keep = np.ones(len(pos), bool)
+    on = []
+    for d in range(3):
+        near = np.flatnonzero(keep & (pos[:, d] < 0.9))
+        for k in rng.choice(near, min(40, len(near)), replace=False):
+            if keep[k]:
+                pos[k, d] = -0.0
+                dist = np.abs(pos - pos[k])
+                dist = np.minimum(dist, L - dist)
+                close = (dist ** 2).sum(1) < 0.81
+                close[k] = False
+                keep &= ~close
+                on.append((k, d))
+    on = [(k, d) for k, d in on if keep[k]]
+    for d in range(3):
+        assert sum(e == d for _, e in on) >= 10
+    pos = pos[keep]
+    assert (np.signbit(pos) & (pos == 0)).sum() >= 30
+    return pos
+
+
+@pytest.mark.parametrize("form", ["mixed", "fp64", "adjoint", "lists"])
+@pytest.mark.parametrize("lx", [0.0, 0.5])
+def test_coordinates_of_negative_zero(D, form, lx):
+    """-0.0 lies in [0, L): the tiles that hold it reach as far as with +0.0."""
+    box = (48.0, 60.0, 72.0)
+    pos = with_negative_zeros(box, 71)
+    rng = np.random.default_rng(72)
+    rc = cutoffs(pos, box, "ramp", rng)
+    assert len(pos) > 49152
+    if form in ("mixed", "fp64"):
+        walk = D.DCM_FORCE_PACKED if form == "mixed" else D.DCM_FORCE_THREAD
+        F0, t0 = forces(D, box, pos, rc, prec=form, force_kernel=walk, lx=lx)
+        F1, t1 = forces(D, box, pos, rc, prec=form, lx=lx)
+        assert t1[2] == t0[2]
+        tol = MIXED_RMS if form == "mixed" else FP64_RMS
+        assert np.sqrt(((F1 - F0)[:, :3] ** 2).mean()) <= tol * np.sqrt((F0[:, :3] ** 2).mean())
+    elif form == "adjoint":  # bounds as in test_adjoint_forms_against_fp64
+        types = rng.integers(0, 2, len(pos)).astype(np.float32)
+        A = np.concatenate([rng.normal(size=(len(pos), 3)), np.zeros((len(pos), 1))], 1).astype(np.float32)
+        rc = rc.astype(np.float32).astype(np.float64)
+        G0, d0 = by_input(D, box, pos, rc, types, A, lx=lx, precision=D.DCM_PREC_FP64)
+        G1, d1 = by_input(D, box, pos, rc, types, A, lx=lx)
+        assert np.sqrt(((G1 - G0)[:, :3] ** 2).mean()) <= 5e-6 * np.sqrt((G0[:, :3] ** 2).mean())
+        assert np.all(np.abs(d1 - d0) <= 5e-6 * np.abs(d0).max())
+    else:
+        res = []
+        for skin in (0.5, 0.0):
+            ctx = D.Context(D.make_params(box, n_max=len(pos), skin=skin, lx=lx))
+            st = D.State(ctx, D.to_real4(torch.from_numpy(pos)), torch.zeros(len(pos), 4))
+            D.dcm_step_init(ctx, st)
+            assert D.dcm_status(ctx) == D.DCM_OK
+            ids = st.current()[3].cpu().numpy()
+            F = np.empty((len(pos), 3))
+            F[ids] = st.force.double().cpu().numpy()[:, :3]
+            res.append((F, st.thermo.cpu().numpy()))
+            ctx.close()
+        (F0, t0), (F1, t1) = res
+        assert t0[3] == t1[3]
+        assert np.sqrt(((F0 - F1) ** 2).mean()) <= 1e-5 * np.sqrt((F1 ** 2).mean())
