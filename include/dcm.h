@@ -234,8 +234,13 @@ const char* dcm_last_error(const dcm_ctx* ctx);
 
 /* Synchronise `stream`, read and clear the device status word of ctx.
  * Returns DCM_OK or the first device-side error recorded since the last call
- * (DCM_ERR_NOT_CONVERGED, DCM_ERR_CAPACITY). */
+ * (DCM_ERR_NOT_CONVERGED, DCM_ERR_CAPACITY, DCM_ERR_TIMEOUT). */
 int dcm_status(dcm_ctx* ctx, dcm_stream_t stream);
+
+/* Longest time, in nanoseconds (>= 1000), that a block of the distance sweeps
+ * waits at a grid barrier before it gives up with DCM_ERR_TIMEOUT.  Default
+ * 2 s.  Host only; takes effect for later calls (a captured one keeps its own). */
+int dcm_set_wait_budget(dcm_ctx* ctx, int64_t ns);
 
 /* Self-test of the failure path of the cell-count scan (the single-pass scan
  * with decoupled look-back that every binning runs): scans two tiles with the
@@ -294,7 +299,9 @@ int dcm_remove_small_components(dcm_ctx* ctx, const uint8_t* s_in, uint8_t* s_ou
  * stay +inf.
  *   D real[nboxes] out;  iters int32[1] out (device, nullable): sweeps used.
  * SYNCHRONOUS: returns DCM_ERR_NOT_CONVERGED if iter_max sweeps did not
- * converge (D then holds the last iterate). */
+ * converge (D then holds the last iterate), and DCM_ERR_TIMEOUT if a wait at the
+ * launch's barriers ran out (dcm_set_wait_budget; D is then unfinished).  Both
+ * leave iters = -1 and the same code in the device status. */
 int dcm_distance(dcm_ctx* ctx, const uint8_t* s, const uint8_t* iface, void* D, int32_t* iters,
                  dcm_stream_t stream);
 

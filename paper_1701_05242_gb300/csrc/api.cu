@@ -361,6 +361,7 @@ extern "C" int dcm_create(const dcm_params* p, dcm_ctx** out) {
   memset(ctx, 0, sizeof(*ctx));
   ctx->p = resolved(p);
   ctx->precision = p->precision;
+  ctx->wait_budget = (int64_t)2000000000;  // 2 s
   for (int d = 0; d < 3; ++d) {
     grid_of(p->box[d], cell_edge(p, d), ctx->nc + d);
     grid_of(p->box[d], p->h, ctx->nh + d);
@@ -469,6 +470,12 @@ extern "C" int dcm_status(dcm_ctx* ctx, dcm_stream_t stream) {
   DCM_CUDA_TRY(ctx, cudaMemsetAsync(ctx->status, 0, sizeof(int32_t), st));
   if (code) set_error(ctx, code, "device status %d", code);
   return code;
+}
+
+extern "C" int dcm_set_wait_budget(dcm_ctx* ctx, int64_t ns) {
+  if (!ctx || ns < 1000) return DCM_ERR_INVALID_ARG;
+  ctx->wait_budget = ns;
+  return DCM_OK;
 }
 
 extern "C" int dcm_scan_wait_selftest(dcm_ctx* ctx, dcm_stream_t stream) {

@@ -270,19 +270,24 @@ __global__ void __launch_bounds__(kCoopBlock) k_dist_coop(R* D0, R* D1, int nx, 
 
 // iters = 1 + index of the first sweep that changed nothing (or -1), and a
 // device status if the budget ran out.  One warp; result (device, nullable)
-// gets the same number as iters.
-__global__ void k_dist_finish(const int32_t* flags, int sweeps, int32_t* iters, int32_t* result, int32_t* status) {
+// gets the same number as iters, or kSweepsAborted where a barrier wait ran out
+// (sync[2], with DCM_ERR_TIMEOUT in the status already): the flags of the
+// sweeps that did not run are zero then too, and mean nothing.
+constexpr int kSweepsAborted = -2;
+__global__ void k_dist_finish(const int32_t* flags, int sweeps, const uint32_t* sync, int32_t* iters, int32_t* result,
+                              int32_t* status) {
   const int lane = threadIdx.x;
+  const bool aborted = sync[2] != 0;
   int first = -1;
   for (int k0 = 0; k0 < sweeps && first < 0; k0 += 32) {
     const unsigned m = __ballot_sync(0xffffffffu, k0 + lane < sweeps && flags[k0 + lane] == 0);
     if (m) first = k0 + __ffs(m) - 1;
   }
   if (lane == 0) {
-    const int v = first >= 0 ? first + 1 : -1;
+    const int v = first >= 0 && !aborted ? first + 1 : -1;
     if (iters) *iters = v;
-    if (result) *result = v;
-    if (first < 0) raise_status(status, DCM_ERR_NOT_CONVERGED);
+    if (result) *result = aborted ? kSweepsAborted : v;
+    if (first < 0 && !aborted) raise_status(status, DCM_ERR_NOT_CONVERGED);
   }
 }
 
@@ -341,13 +346,15 @@ int distance_sweeps(dcm_ctx* ctx, const uint8_t* s, const uint8_t* iface, R* D, 
   ++ctx->launches;
   cudaError_t e = cudaLaunchKernelEx(&cfg, kern, buf[0], buf[1], nx, ny, nz, h, rg, (const uint8_t*)ctx->dfixed,
                                      ctx->dstamp, q[0], q[1], ctx->dqlen, ctx->flags, budget, ctx->coop_sync,
-                                     (int64_t)2000000000, ctx->status);
+                                     ctx->wait_budget, ctx->status);
   if (e != cudaSuccess) return set_error(ctx, DCM_ERR_CUDA, "distance sweeps: %s", cudaGetErrorString(e));
-  DCM_LAUNCH(ctx, k_dist_finish, 1, 32, 0, st, ctx->flags, budget, iters, host_check ? ctx->thr + 3 : nullptr,
-             ctx->status);
+  DCM_LAUNCH(ctx, k_dist_finish, 1, 32, 0, st, ctx->flags, budget, (const uint32_t*)ctx->coop_sync, iters,
+             host_check ? ctx->thr + 3 : nullptr, ctx->status);
   if (host_check) {
     DCM_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->host_status, ctx->thr + 3, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     DCM_CUDA_TRY(ctx, cudaStreamSynchronize(st));
+    if (ctx->host_status[0] == kSweepsAborted)
+      return set_error(ctx, DCM_ERR_TIMEOUT, "distance sweeps: a grid barrier's wait ran out");
     if (ctx->host_status[0] < 0) {
       if (iter_max & 1) DCM_CUDA_TRY(ctx, cudaMemcpyAsync(D, buf[1], sizeof(R) * nbox, cudaMemcpyDeviceToDevice, st));
       check_launch(ctx, "distance_sweeps");

@@ -85,6 +85,7 @@ _SIGS = {
     "dcm_destroy": (None, [_vp]),
     "dcm_last_error": (ctypes.c_char_p, [_vp]),
     "dcm_status": (_i32, [_vp, _vp]),
+    "dcm_set_wait_budget": (_i32, [_vp, _i64]),
     "dcm_bin": (_i32, [_vp, _i64, _vp, _vp, _vp, _vp, _vp, _vp]),
     "dcm_box_counts": (_i32, [_vp, _i64, _vp, _vp, _vp]),
     "dcm_detect_interface": (_i32, [_vp, _vp, _vp, _vp, _vp, _vp, _vp]),
@@ -450,6 +451,10 @@ def dcm_batch_barrier_selftest(b: Batch, phantom: int, budget_ns: int, stream=No
     """Runs the persistent grid's barrier against `phantom` missing blocks;
     returns the device status (DCM_ERR_TIMEOUT when the bounded waits ran out)."""
     return lib.dcm_batch_barrier_selftest(b.handle, int(phantom), int(budget_ns), _stream(stream))
+
+
+def dcm_set_wait_budget(ctx: Context, ns: int):
+    ctx.check(lib.dcm_set_wait_budget(ctx.handle, int(ns)))
 
 
 def dcm_scan_wait_selftest(ctx: Context, stream=None) -> int:

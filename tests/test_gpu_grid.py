@@ -83,3 +83,39 @@ def test_placement_of_crowded_cells(D, n):
     assert np.array_equal(cell.cpu().numpy(), oc) and np.array_equal(start.cpu().numpy(), ostart)
     assert np.array_equal(perm.cpu().numpy(), operm)
     assert np.array_equal(ps.cpu().numpy(), p4.cpu().numpy()[operm])
+
+
+def test_distances_with_an_exhausted_wait_budget(D):
+    """A wait budget of 1 microsecond, below the time between the first and the
+    last block of a sweep: the launch ends, and the call says so instead of
+    returning unfinished distances; with the budget restored it gives what a fresh
+    context gives."""
+    nh = (96, 96, 96)
+    nb = int(np.prod(nh))
+    rng = np.random.default_rng(1)
+    s = torch.ones(nb, dtype=torch.uint8, device="cuda")
+    iface = torch.from_numpy((rng.random(nb) < 0.002).astype(np.uint8)).cuda()
+    i32 = dict(dtype=torch.int32, device="cuda")
+
+    def run(ctx):
+        d, it = torch.empty(nb, device="cuda"), torch.full((1,), 77, **i32)
+        try:
+            D.dcm_distance(ctx, s, iface, d, it)
+            code = D.DCM_OK
+        except D.DcmError as e:
+            code = e.code
+        return code, d, int(it.item())
+
+    ctx, fresh = context(D, nh, r_grid=12.0), context(D, nh, r_grid=12.0)
+    code, d0, it0 = run(fresh)
+    assert code == D.DCM_OK and it0 > 5
+    with pytest.raises(D.DcmError):
+        D.dcm_set_wait_budget(ctx, 999)
+    D.dcm_set_wait_budget(ctx, 1000)
+    code, _, it = run(ctx)
+    assert code == D.DCM_ERR_TIMEOUT and it == -1
+    assert D.dcm_status(ctx) == D.DCM_ERR_TIMEOUT
+    D.dcm_set_wait_budget(ctx, 2_000_000_000)
+    code, d, it = run(ctx)
+    assert code == D.DCM_OK and it == it0 and torch.equal(d, d0)
+    assert D.dcm_status(ctx) == D.DCM_OK
