@@ -294,8 +294,8 @@ __device__ __forceinline__ bool tile_candidates(TileSmem<E>& sm, const E* __rest
   float lo[3], hi[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    // without the sign: -0 lies in the box, and its bits are the largest of all
-    const float v = fabsf((float)xi[d]);
+    // -0 becomes +0: it lies in the box, and its bits are the largest of all
+    const float v = (float)xi[d] + 0.f;
     lo[d] = active ? v : Lf[d];
     hi[d] = active ? v : 0.f;
   }
