@@ -633,14 +633,14 @@ constexpr int kAdjTileWarps = 12;
 
 __global__ void __launch_bounds__(32 * kAdjTileWarps, 1) k_adjoint_tiles(
     const AdjRec* __restrict__ rec, const int32_t* __restrict__ start, const __grid_constant__ ForceArgs<float> a,
-    TileCfg cfg, TileTable t, float half_dlde, BlockGrid bg, const int32_t* __restrict__ block_reach,
+    TileCfg cfg, const __grid_constant__ TileTable t, float half_dlde, BlockGrid bg, const int32_t* __restrict__ block_reach,
     float4* __restrict__ G, double* __restrict__ part, int64_t nslot) {
   const unsigned full = 0xffffffffu;
   extern __shared__ __align__(32) unsigned char smem_raw[];
   TileSmem<AdjRec>& sm = reinterpret_cast<TileSmem<AdjRec>*>(smem_raw)[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
   const int nfirst = __ldg(t.counters + kTileFirst), ntile = nfirst + __ldg(t.counters + kTileLater);
-  if (__ldg(t.counters + kTileOutside)) return;  // all tiles go to the row walk
+  const bool outside = __ldg(t.counters + kTileOutside) != 0;
   auto take = [&]() {
     int q = 0;
     if (lane == 0) q = atomicAdd(t.counters + kTileQueue, 1);
@@ -666,7 +666,8 @@ __global__ void __launch_bounds__(32 * kAdjTileWarps, 1) k_adjoint_tiles(
     const AdjRow k = adj_row(a, tk, rck2);
     AdjAcc2 c;
     float xi[3] = {pi.x, pi.y, pi.z};
-    const bool done = tile_candidates<float, AdjRec>(sm, rec, start, a.g, cfg, active, i, xi, rck, reach,
+    const bool met = outside && tile_meets_outside<float>(cfg, t.outside, a.g, active, pi.y, pi.z, reach);
+    const bool done = !met && tile_candidates<float, AdjRec>(sm, rec, start, a.g, cfg, active, i, xi, rck, reach,
                                                           [](const AdjRec& q) { return q.rc; }, []() {}, [&](int last) {
       ListWalk l;
       l.begin(shared_addr(&sm.list[0][lane]), last);
@@ -688,168 +689,205 @@ __global__ void __launch_bounds__(32 * kAdjTileWarps, 1) k_adjoint_tiles(
   }
 }
 
-// The tiles that the filter does not serve, by the row walk.
-__global__ void __launch_bounds__(64) k_adjoint_rest(const float4* __restrict__ pos, const float* __restrict__ rc,
-                                                     const int32_t* __restrict__ start, ForceArgs<float> a, TileTable t,
-                                                     const float4* __restrict__ A, float half_dlde,
-                                                     float4* __restrict__ G, double* __restrict__ part, int64_t nslot,
-                                                     BlockGrid bg, const int32_t* __restrict__ bmax) {
-  const bool all = __ldg(t.counters + kTileOutside) != 0;
-  const int nfirst = __ldg(t.counters + kTileFirst), lane = threadIdx.x & 31;
-  const int n = all ? nfirst + __ldg(t.counters + kTileLater) : __ldg(t.counters + kTileRest);
-  for (int q = blockIdx.x * 2 + (threadIdx.x >> 5); q < n; q += gridDim.x * 2) {
-    const int slot = __ldg(!all ? t.rest + q : (q < nfirst ? t.list + q : t.list + (nslot - 1 - (q - nfirst))));
-    const int i = __ldg(t.idx + 32 * (int64_t)slot + lane);
-    AdjAcc2 c;
-    int tk = 0;
-    if (i >= 0) {
-      tk = adj_one_x2(pos, rc, start, a, A, half_dlde, bg, bmax, i, c);
-      G[i] = make_float4(c.gx.x + c.gx.y, c.gy.x + c.gy.y, c.gz.x + c.gz.y, 0.f);
+// The packed adjoint of particle i by a warp: the lanes take the rows of the
+// walk (radius `reach`), write their candidates into a list in shared memory
+// (kAdjList entries, visited whenever it is full) and then share the list, two
+// candidates per lane and step.  The sums of the lanes are added in a fixed tree:
+// G in v[0 .. 2], the parameter sums of the forward pairs by partner type in v[3], v[4]
+// (eps) and v[5], v[6] (sigma).  Returns the particle's type.
+constexpr int kAdjList = 1024;
+
+__device__ __forceinline__ int adj_warp_one(uint32_t* list, uint8_t* codes, const float4* __restrict__ pos,
+                                            const float* __restrict__ rc, const int32_t* __restrict__ start,
+                                            const ForceArgs<float>& a, const float4* __restrict__ A, float half_dlde,
+                                            const BlockGrid& bg, const int32_t* __restrict__ bmax, int i,
+                                            float (&v)[7]) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const Grid<float>& g = a.g;
+  AdjAcc2 c;
+  const float4 pi = __ldg(pos + i), ak = __ldg(A + i);
+  const float rck = clamp_cutoff<float>(__ldg(rc + i), a.rc_max), rck2 = rck * rck;
+  // the largest cutoff of the 27 blocks around (reverse_reach), one block per lane
+  float m = 0.f;
+  if (lane < 27) {
+    const int b0 = block_coord(pi.x, bg.inv_be[0], bg.nb[0]) + lane % 3 - 1,
+              b1 = block_coord(pi.y, bg.inv_be[1], bg.nb[1]) + lane / 3 % 3 - 1,
+              b2 = block_coord(pi.z, bg.inv_be[2], bg.nb[2]) + lane / 9 - 1;
+    const int xx = (b0 + bg.nb[0]) % bg.nb[0], yy = (b1 + bg.nb[1]) % bg.nb[1], zz = (b2 + bg.nb[2]) % bg.nb[2];
+    m = __int_as_float(__ldg(bmax + xx + bg.nb[0] * (yy + bg.nb[1] * zz)));
+  }
+  m = __int_as_float(__reduce_max_sync(full, __float_as_int(m)));  // cutoffs are not negative
+  const float reach = fmaxf(fminf(m, a.rc_max), rck);
+  const float reach2s = reach * reach * 1.000004f;
+  const int tk = type_of(pi.w, a.ntypes);
+  const AdjRow k = adj_row(a, tk, rck2);
+  const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
+  const float l = g.edge, il = g.inv_edge, ilx = g.inv_edge_x;
+  const int cx = cell_coord<float>(pi.x, g.edge_x, ilx, nx), cy = cell_coord<float>(pi.y, l, il, ny),
+            cz = cell_coord<float>(pi.z, l, il, nz);
+  const int H = (int)ceilf(reach * il), Hx = (int)ceilf(reach * ilx), side = 2 * H + 1;
+  int listed = 0;
+  auto visit = [&]() {
+    __syncwarp();
+    for (int q = 2 * lane; q < listed; q += 64) {
+      const bool has1 = q + 1 < listed;
+      const int q1 = has1 ? q + 1 : q;
+      const int j0 = (int)list[q], j1 = (int)list[q1];
+      const uint32_t e0 = codes[q], e1 = codes[q1];
+      const float4 p0 = __ldg(pos + j0), p1 = __ldg(pos + j1), a0 = __ldg(A + j0), a1 = __ldg(A + j1);
+      const float rc0 = clamp_cutoff<float>(__ldg(rc + j0), a.rc_max), rc1 = clamp_cutoff<float>(__ldg(rc + j1), a.rc_max);
+      // an image at -L shifts j, one at +L shifts the particle itself
+      auto diff = [&](float pj, float pk, float L, uint32_t e) {
+        return (e & 1u ? pj - L : pj) - (e & 2u ? pk - L : pk);
+      };
+      const float2 dx = make_float2(diff(p0.x, pi.x, g.L[0], e0), diff(p1.x, pi.x, g.L[0], e1)),
+                   dy = make_float2(diff(p0.y, pi.y, g.L[1], e0 >> 2), diff(p1.y, pi.y, g.L[1], e1 >> 2)),
+                   dz = make_float2(diff(p0.z, pi.z, g.L[2], e0 >> 4), diff(p1.z, pi.z, g.L[2], e1 >> 4));
+      adj_pair_x2(dx, dy, dz, !(j0 == i && e0 == 0), has1 && !(j1 == i && e1 == 0), rc0, rc1, p0.w, p1.w, a0, a1,
+                  rck2, ak, half_dlde, k, c);
     }
     __syncwarp();
-    if (part) adj_warp_partials(a, i >= 0, tk, c, part, nslot, slot);
+    listed = 0;
+  };
+  // the rows, each in up to three pieces along x (image at -L, the box, image at +L)
+  const int nitem = 3 * side * side;
+  for (int it0 = 0; it0 < nitem; it0 += 32) {
+    const int it = it0 + lane;
+    int j0 = 0, cnt = 0;
+    uint32_t code = 0;
+    if (it < nitem) {
+      const int piece = it % 3, row = it / 3, uy = cy - H + row % side, uz = cz - H + row / side;
+      const float gz = uz > cz ? (float)uz * l - pi.z : (uz < cz ? pi.z - (float)(uz + 1) * l : 0.f);
+      const float gy = uy > cy ? (float)uy * l - pi.y : (uy < cy ? pi.y - (float)(uy + 1) * l : 0.f);
+      const float g2 = gz * gz + gy * gy;
+      if (g2 < reach2s) {
+        const float wx = sqrtf(reach2s - g2);
+        const int ulo = max(ufloor<float>((pi.x - wx) * ilx - 5e-4f), cx - Hx);
+        const int uhi = min(ufloor<float>((pi.x + wx) * ilx + 5e-4f), cx + Hx);
+        // a coordinate outside [0, L): no window
+        const int lo = piece == 0 ? ulo : (piece == 1 ? max(ulo, 0) : max(ulo, nx));
+        const int hi = piece == 0 ? min(uhi, -1) : (piece == 1 ? min(uhi, nx - 1) : uhi);
+        if (lo <= hi) {
+          const int wy = uy < 0 ? uy + ny : (uy >= ny ? uy - ny : uy), wz = uz < 0 ? uz + nz : (uz >= nz ? uz - nz : uz);
+          const int base = nx * (wy + ny * wz) + (piece == 0 ? nx : (piece == 2 ? -nx : 0));
+          j0 = __ldg(start + base + lo);
+          cnt = max(__ldg(start + base + hi + 1) - j0, 0);
+          code = (piece == 0 ? 1u : (piece == 2 ? 2u : 0u)) | (uy < 0 ? 4u : (uy >= ny ? 8u : 0u)) |
+                 (uz < 0 ? 16u : (uz >= nz ? 32u : 0u));
+        }
+      }
+    }
+    int incl = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(full, incl, o);
+      if (lane >= o) incl += u;
+    }
+    const int off = incl - cnt, total = __shfl_sync(full, incl, 31);
+    for (int done = 0; done < total;) {
+      const int take = min(total - done, kAdjList - listed);
+      for (int q = max(done - off, 0); q < min(done + take - off, cnt); ++q) {
+        list[listed + off + q - done] = (uint32_t)(j0 + q);
+        codes[listed + off + q - done] = (uint8_t)code;
+      }
+      listed += take;
+      done += take;
+      if (listed == kAdjList) visit();
+    }
+  }
+  visit();
+  v[0] = c.gx.x + c.gx.y;
+  v[1] = c.gy.x + c.gy.y;
+  v[2] = c.gz.x + c.gz.y;
+  v[3] = c.de[0].x + c.de[0].y;
+  v[4] = c.de[1].x + c.de[1].y;
+  v[5] = c.ds[0].x + c.ds[0].y;
+  v[6] = c.ds[1].x + c.ds[1].y;
+#pragma unroll
+  for (int q = 0; q < 7; ++q)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(full, v[q], o);
+  return tk;
+}
+
+// Lane p + 4 q of a warp: the share of a particle of type tk in the sum of type
+// pair p, eps (q = 0) or sigma (q = 1), in FP64.
+__device__ __forceinline__ double adj_warp_term(const ForceArgs<float>& a, int tk, const float (&v)[7]) {
+  const int lane = threadIdx.x & 31, p = lane & 3, q = lane >> 2, nt = a.ntypes;
+  if (lane >= 8 || p >= nt * nt || tk != p / nt) return 0.0;
+  const bool t1 = p % nt == 1;
+  return q ? (double)(t1 ? v[6] : v[5]) * 0.25 * (double)a.eps4[p] / sqrt((double)a.sig2[p])  // eps_p / sigma_p
+           : (double)(t1 ? v[4] : v[3]);
+}
+
+// A block's sums (sum: per warp, as adj_warp_term) into a slot of the partials, in the order of the warps.
+template <int WARPS>
+__device__ __forceinline__ void adj_block_partials(const double (&sum)[WARPS][8], int nt, double* __restrict__ part,
+                                                   int64_t nslot, int64_t slot) {
+  __syncthreads();
+  if (threadIdx.x < 8 && (threadIdx.x & 3) < nt * nt) {
+    double t = 0.0;
+    for (int w = 0; w < WARPS; ++w) t += sum[w][threadIdx.x];
+    part[(int64_t)(nt * nt * (threadIdx.x >> 2) + (threadIdx.x & 3)) * nslot + slot] = t;
   }
 }
 
-// The packed adjoint of a small system, one warp per particle: the lanes
-// take the rows of the walk (radius `reach`), write their candidates into a
-// list in shared memory and then share the list, two candidates per lane and
-// step.  A launch of 2,000 particles lasts as long as one particle's walk: 444 us
-// for 1,935 particles with one thread each, 29 us so (30,000: 490 -> 171 us).  The sums of the lanes are added in a fixed tree.
-constexpr int kAdjWarps = 4, kAdjList = 1024;  // particles per block; candidates listed at a time
+// A small system, one warp per particle.  A launch of 2,000 particles lasts as
+// long as one particle's walk: 444 us for 1,935 particles with one thread each, 29
+// us so (30,000: 490 -> 171 us).
+constexpr int kAdjWarps = 4;  // particles per block
 
 __global__ void __launch_bounds__(32 * kAdjWarps) k_adjoint_warp(
     int64_t n, const float4* __restrict__ pos, const float* __restrict__ rc, const int32_t* __restrict__ start,
     ForceArgs<float> a, const float4* __restrict__ A, float half_dlde, float4* __restrict__ G,
     double* __restrict__ part, int64_t nslot, BlockGrid bg, const int32_t* __restrict__ bmax) {
-  __shared__ uint32_t list_sh[kAdjWarps][kAdjList];  // particle, and its image along x, y, z (adjoint code) per entry
-  __shared__ uint8_t code_sh[kAdjWarps][kAdjList];
+  __shared__ uint32_t list_sh[kAdjWarps][kAdjList];
+  __shared__ uint8_t code_sh[kAdjWarps][kAdjList];  // the entry's image along x, y, z (adjoint code)
   __shared__ double sum_sh[kAdjWarps][8];
-  const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  uint32_t* list = list_sh[wid];
-  uint8_t* codes = code_sh[wid];
   const int64_t i = (int64_t)blockIdx.x * kAdjWarps + wid;
-  const int nt = a.ntypes;
-  const Grid<float>& g = a.g;
-  AdjAcc2 c;
-  int tk = 0;
+  double term = 0.0;
   if (i < n) {
-    const float4 pi = __ldg(pos + i), ak = __ldg(A + i);
-    const float rck = clamp_cutoff<float>(__ldg(rc + i), a.rc_max), rck2 = rck * rck;
-    // the largest cutoff of the 27 blocks around (reverse_reach), one block per lane
-    float m = 0.f;
-    if (lane < 27) {
-      const int b0 = block_coord(pi.x, bg.inv_be[0], bg.nb[0]) + lane % 3 - 1,
-                b1 = block_coord(pi.y, bg.inv_be[1], bg.nb[1]) + lane / 3 % 3 - 1,
-                b2 = block_coord(pi.z, bg.inv_be[2], bg.nb[2]) + lane / 9 - 1;
-      const int xx = (b0 + bg.nb[0]) % bg.nb[0], yy = (b1 + bg.nb[1]) % bg.nb[1], zz = (b2 + bg.nb[2]) % bg.nb[2];
-      m = __int_as_float(__ldg(bmax + xx + bg.nb[0] * (yy + bg.nb[1] * zz)));
-    }
-    m = __int_as_float(__reduce_max_sync(full, __float_as_int(m)));  // cutoffs are not negative
-    const float reach = fmaxf(fminf(m, a.rc_max), rck);
-    const float reach2s = reach * reach * 1.000004f;
-    tk = type_of(pi.w, nt);
-    const AdjRow k = adj_row(a, tk, rck2);
-    const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
-    const float l = g.edge, il = g.inv_edge, ilx = g.inv_edge_x;
-    const int cx = cell_coord<float>(pi.x, g.edge_x, ilx, nx), cy = cell_coord<float>(pi.y, l, il, ny),
-              cz = cell_coord<float>(pi.z, l, il, nz);
-    const int H = (int)ceilf(reach * il), Hx = (int)ceilf(reach * ilx), side = 2 * H + 1;
-    int listed = 0;
-    auto visit = [&]() {
-      __syncwarp();
-      for (int q = 2 * lane; q < listed; q += 64) {
-        const bool has1 = q + 1 < listed;
-        const int q1 = has1 ? q + 1 : q;
-        const int j0 = (int)list[q], j1 = (int)list[q1];
-        const uint32_t e0 = codes[q], e1 = codes[q1];
-        const float4 p0 = __ldg(pos + j0), p1 = __ldg(pos + j1), a0 = __ldg(A + j0), a1 = __ldg(A + j1);
-        const float rc0 = clamp_cutoff<float>(__ldg(rc + j0), a.rc_max), rc1 = clamp_cutoff<float>(__ldg(rc + j1), a.rc_max);
-        // an image at -L shifts j, one at +L shifts the particle itself
-        auto diff = [&](float pj, float pk, float L, uint32_t e) {
-          return (e & 1u ? pj - L : pj) - (e & 2u ? pk - L : pk);
-        };
-        const float2 dx = make_float2(diff(p0.x, pi.x, g.L[0], e0), diff(p1.x, pi.x, g.L[0], e1)),
-                     dy = make_float2(diff(p0.y, pi.y, g.L[1], e0 >> 2), diff(p1.y, pi.y, g.L[1], e1 >> 2)),
-                     dz = make_float2(diff(p0.z, pi.z, g.L[2], e0 >> 4), diff(p1.z, pi.z, g.L[2], e1 >> 4));
-        adj_pair_x2(dx, dy, dz, !(j0 == i && e0 == 0), has1 && !(j1 == i && e1 == 0), rc0, rc1, p0.w, p1.w, a0, a1,
-                    rck2, ak, half_dlde, k, c);
-      }
-      __syncwarp();
-      listed = 0;
-    };
-    // the rows, each in up to three pieces along x (image at -L, the box, image at +L)
-    const int nitem = 3 * side * side;
-    for (int it0 = 0; it0 < nitem; it0 += 32) {
-      const int it = it0 + lane;
-      int j0 = 0, cnt = 0;
-      uint32_t code = 0;
-      if (it < nitem) {
-        const int piece = it % 3, row = it / 3, uy = cy - H + row % side, uz = cz - H + row / side;
-        const float gz = uz > cz ? (float)uz * l - pi.z : (uz < cz ? pi.z - (float)(uz + 1) * l : 0.f);
-        const float gy = uy > cy ? (float)uy * l - pi.y : (uy < cy ? pi.y - (float)(uy + 1) * l : 0.f);
-        const float g2 = gz * gz + gy * gy;
-        if (g2 < reach2s) {
-          const float wx = sqrtf(reach2s - g2);
-          const int ulo = max(ufloor<float>((pi.x - wx) * ilx - 5e-4f), cx - Hx);
-          const int uhi = min(ufloor<float>((pi.x + wx) * ilx + 5e-4f), cx + Hx);
-          // a coordinate outside [0, L): no window
-          const int lo = piece == 0 ? ulo : (piece == 1 ? max(ulo, 0) : max(ulo, nx));
-          const int hi = piece == 0 ? min(uhi, -1) : (piece == 1 ? min(uhi, nx - 1) : uhi);
-          if (lo <= hi) {
-            const int wy = uy < 0 ? uy + ny : (uy >= ny ? uy - ny : uy), wz = uz < 0 ? uz + nz : (uz >= nz ? uz - nz : uz);
-            const int base = nx * (wy + ny * wz) + (piece == 0 ? nx : (piece == 2 ? -nx : 0));
-            j0 = __ldg(start + base + lo);
-            cnt = max(__ldg(start + base + hi + 1) - j0, 0);
-            code = (piece == 0 ? 1u : (piece == 2 ? 2u : 0u)) | (uy < 0 ? 4u : (uy >= ny ? 8u : 0u)) |
-                   (uz < 0 ? 16u : (uz >= nz ? 32u : 0u));
-          }
-        }
-      }
-      int incl = cnt;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int u = __shfl_up_sync(full, incl, o);
-        if (lane >= o) incl += u;
-      }
-      const int off = incl - cnt, total = __shfl_sync(full, incl, 31);
-      for (int done = 0; done < total;) {
-        const int take = min(total - done, kAdjList - listed);
-        for (int q = max(done - off, 0); q < min(done + take - off, cnt); ++q) {
-          list[listed + off + q - done] = (uint32_t)(j0 + q);
-          codes[listed + off + q - done] = (uint8_t)code;
-        }
-        listed += take;
-        done += take;
-        if (listed == kAdjList) visit();
-      }
-    }
-    visit();
+    float v[7];
+    const int tk = adj_warp_one(list_sh[wid], code_sh[wid], pos, rc, start, a, A, half_dlde, bg, bmax, (int)i, v);
+    if (lane == 0) G[i] = make_float4(v[0], v[1], v[2], 0.f);
+    term = adj_warp_term(a, tk, v);
   }
-  float v[7] = {c.gx.x + c.gx.y, c.gy.x + c.gy.y, c.gz.x + c.gz.y, c.de[0].x + c.de[0].y, c.de[1].x + c.de[1].y,
-                c.ds[0].x + c.ds[0].y, c.ds[1].x + c.ds[1].y};
-#pragma unroll
-  for (int q = 0; q < 7; ++q)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(full, v[q], o);
-  if (i < n && lane == 0) G[i] = make_float4(v[0], v[1], v[2], 0.f);
   if (part) {  // per block, in FP64, in the order of the particles
-    if (lane < 8) {
-      const int p = lane & 3, q = lane >> 2;  // type pair, eps or sigma
-      double t = 0.0;
-      if (p < nt * nt && i < n && tk == p / nt) {
-        const bool t1 = p % nt == 1;
-        t = q ? (double)(t1 ? v[6] : v[5]) * 0.25 * (double)a.eps4[p] / sqrt((double)a.sig2[p])  // eps_p / sigma_p
-              : (double)(t1 ? v[4] : v[3]);
-      }
-      sum_sh[wid][lane] = t;
+    if (lane < 8) sum_sh[wid][lane] = term;
+    adj_block_partials(sum_sh, a.ntypes, part, nslot, blockIdx.x);
+  }
+}
+
+// The tiles that the filter does not serve: a block per tile, a warp per
+// particle.  There are few of them, so the launch lasts as long as its longest
+// walks (a thread per particle: 1363 us for all of 260K particles of two types).
+constexpr int kAdjRestWarps = 8;
+
+__global__ void __launch_bounds__(32 * kAdjRestWarps) k_adjoint_rest(
+    const float4* __restrict__ pos, const float* __restrict__ rc, const int32_t* __restrict__ start, ForceArgs<float> a,
+    TileTable t, const float4* __restrict__ A, float half_dlde, float4* __restrict__ G, double* __restrict__ part,
+    int64_t nslot, BlockGrid bg, const int32_t* __restrict__ bmax) {
+  __shared__ uint32_t list_sh[kAdjRestWarps][kAdjList];
+  __shared__ uint8_t code_sh[kAdjRestWarps][kAdjList];
+  __shared__ double sum_sh[kAdjRestWarps][8];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, n = __ldg(t.counters + kTileRest);
+  for (int q = blockIdx.x; q < n; q += gridDim.x) {
+    const int slot = __ldg(t.rest + q);
+    double term = 0.0;
+    for (int k = wid; k < 32; k += kAdjRestWarps) {
+      const int i = __ldg(t.idx + 32 * (int64_t)slot + k);
+      if (i < 0) continue;
+      float v[7];
+      const int tk = adj_warp_one(list_sh[wid], code_sh[wid], pos, rc, start, a, A, half_dlde, bg, bmax, i, v);
+      if (lane == 0) G[i] = make_float4(v[0], v[1], v[2], 0.f);
+      term += adj_warp_term(a, tk, v);
     }
-    __syncthreads();
-    if (threadIdx.x < 8 && (threadIdx.x & 3) < nt * nt) {
-      double t = 0.0;
-      for (int w = 0; w < kAdjWarps; ++w) t += sum_sh[w][threadIdx.x];
-      part[(int64_t)(nt * nt * (threadIdx.x >> 2) + (threadIdx.x & 3)) * nslot + blockIdx.x] = t;
+    if (part) {
+      __syncthreads();  // the tile before is summed
+      if (lane < 8) sum_sh[wid][lane] = term;
+      adj_block_partials(sum_sh, a.ntypes, part, nslot, slot);
     }
   }
 }
@@ -962,8 +1000,8 @@ int lj_adjoint(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, const R* 
       DCM_LAUNCH(ctx, k_adjoint_tiles, (unsigned)std::min<int64_t>((nwarp + kAdjTileWarps - 1) / kAdjTileWarps, sms),
                  32 * kAdjTileWarps, smem, st, rec, cell_start, a, tp.cfg, tt, (float)(0.5 * dlde), bg,
                  (const int32_t*)(ctx->blk_max + ctx->nblk), G, part, nwarp);
-      DCM_LAUNCH(ctx, k_adjoint_rest, 8 * sms, 64, 0, st, pos, rc, cell_start, a, tt, A, (float)(0.5 * dlde), G, part,
-                 nwarp, bg, (const int32_t*)ctx->blk_max);
+      DCM_LAUNCH(ctx, k_adjoint_rest, (unsigned)std::min<int64_t>(nwarp, 4 * sms), 32 * kAdjRestWarps, 0, st, pos, rc,
+                 cell_start, a, tt, A, (float)(0.5 * dlde), G, part, nwarp, bg, (const int32_t*)ctx->blk_max);
     }
   }
   // launch order of the tiles, the widest walks first, where that pays

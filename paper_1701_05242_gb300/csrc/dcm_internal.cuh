@@ -121,7 +121,8 @@ struct dcm_ctx {
   int64_t red_cap;          // number of partial slots in red (per quantity)
   int32_t* blk_max;         // 2 nblk: largest cutoff (float bits) per adjoint block, and of the 27 around it
   int32_t* tile_scratch;    // tile_scratch_ints(n_max): launch order of the force and adjoint tiles
-  int32_t* tiles;           // tile_ints(tile_cap): counters, slots in use, slots left to the row walk, particles of the slots
+  int32_t* tiles;           // tile_ints(tile_cap): counters, slots in use, slots left to the row walk, flags of the
+                            // bundles, particles of the slots
   int64_t tile_cap;         // pair tile slots (0: tiles not served)
   int nblk3[3];             // adjoint blocks per dimension (edge >= 1.001 rc_max)
   int64_t nblk;
@@ -307,7 +308,7 @@ inline TilePlan list_tile_plan(dcm_params p, const int64_t* nc, int64_t n) {
   return t;
 }
 constexpr int64_t kListTilesMinN = 4000;  // below: the row walk, as the forces (kTilesMinN)
-constexpr int64_t tile_ints(int64_t slots) { return 8 + 34 * slots; }
+constexpr int64_t tile_ints(int64_t slots) { return 8 + 35 * slots; }
 bool tiles_serve(const dcm_ctx* ctx, int64_t n);  // whether lj_forces runs over tiles
 template <typename R>
 struct ForceArgs;

@@ -89,59 +89,25 @@ __global__ void __launch_bounds__(kX2Block, x2_min_blocks<M>()) k_forces_x2(int6
   if (part) warp_partials3(e_out, w_out, np, part, nwarp, i >> 5);
 }
 
-// The packed walk of a small system, 16 lanes per particle: each lane walks
-// one z-plane of the stencil (or every 16th, where the cells are fine), and the
-// planes' partial sums are then added in the order of the planes with the
-// compensation of the plane-Kahan form, so the results are bit for bit those of
-// k_forces_x2.  A launch of 2,000 particles has 61 warps in the one-thread form,
-// and lasts as long as one particle's walk; this one has 968 and lasts about as
-// long as one plane: 193 -> 41 us for 1,935 particles, 219 -> 97 us for 30,000.
+// A small system, 16 lanes per particle (force_planes): the results are bit for
+// bit those of k_forces_x2.  A launch of 2,000 particles has 61 warps in the
+// one-thread form, and lasts as long as one particle's walk; this one has 968 and
+// lasts about as long as one plane: 193 -> 41 us for 1,935 particles, 219 -> 97 us
+// for 30,000.
 template <bool TYPED, bool EW>
 __global__ void __launch_bounds__(kPlaneBlock) k_forces_planes(int64_t n, const float4* __restrict__ pos,
                                                                const float* __restrict__ rc,
                                                                const int32_t* __restrict__ start, ForceArgs<float> a,
                                                                float4* __restrict__ force, double* __restrict__ part,
                                                                int64_t nslot) {
-  constexpr Accum M = Accum::kPlaneKahan;
   constexpr int kPer = kPlaneBlock / kPlaneLanes;
-  const unsigned full = 0xffffffffu;
   const int sub = threadIdx.x % kPlaneLanes, grp = threadIdx.x / kPlaneLanes;
   const int64_t i = (int64_t)blockIdx.x * kPer + grp;
   const bool in = i < n;
-  const float4 pi = __ldg(pos + (in ? i : 0));
-  const float rci = in ? clamp_cutoff<float>(__ldg(rc + i), a.rc_max) : 0.f;
-  const Walker<float> wk(a.g, pi, rci);
-  const int ti = TYPED ? type_of(pi.w, a.ntypes) : 0;
-  float k8[8];
-  row_constants<float, TYPED, true>(a, ti, wk.rc2, k8);
-  const int np = in ? 2 * wk.H + 1 : 0, most = __reduce_max_sync(full, np);
-  Acc<float> c;
-  Acc2 c2;
-  Sums<M> S;
-  for (int q0 = 0; q0 < most; q0 += kPlaneLanes) {
-    const int q = q0 + sub;
-    c2.fx = c2.fy = c2.fz = c2.en = c2.vir = make_float2(0.f, 0.f);
-    const bool reached = q < np && walk_plane<float, TYPED, true, M, true, Walk::kAll, EW>(
-                                       pos, start, a.g, a, (int)i, pi, wk, wk.cz - wk.H + q, ti, k8, c, c2, S);
-    __syncwarp();
-    const float v[5] = {c2.fx.x + c2.fx.y, c2.fy.x + c2.fy.y, c2.fz.x + c2.fz.y, c2.en.x + c2.en.y,
-                        c2.vir.x + c2.vir.y};
-    const unsigned mask = __ballot_sync(full, reached) >> (threadIdx.x & 16);
-    for (int k = 0; k < min(kPlaneLanes, most - q0); ++k) {
-#pragma unroll
-      for (int m = 0; m < (EW ? 5 : 3); ++m) {
-        const float x = __shfl_sync(full, v[m], k, kPlaneLanes);
-        if (mask >> k & 1u) kahan_add(S.s[m], S.k[m], x);
-      }
-    }
-  }
-  for (int o = kPlaneLanes / 2; o > 0; o >>= 1) c2.np += __shfl_xor_sync(full, c2.np, o);
   double e = 0, w = 0;
   int pairs = 0;
-  if (in) {
-    const float4 f = finish_sums<float, TYPED, true, M, EW>(c, c2, S, k8, e, w, pairs);
-    if (sub == 0) force[i] = f;
-  }
+  const float4 f = force_planes<float, TYPED, EW>(pos, start, a, in, in ? (int)i : 0, rc, e, w, pairs);
+  if (in && sub == 0) force[i] = f;
   if (EW && part) {  // one partial per block, summed in the order of the particles
     __shared__ double sh[3][kPer];
     if (sub == 0) {

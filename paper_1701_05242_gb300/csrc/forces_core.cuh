@@ -701,4 +701,73 @@ __device__ __forceinline__ typename RT<R>::R4 force_one(const typename RT<R>::R4
   return finish_sums<R, TYPED, X2, M, EW>(c, c2, S, ushift, e_out, w_out, np_out);
 }
 
+// Force, energy and virial of particle i (in: whether there is one) with 16
+// lanes, by a whole warp for its two half-warps' particles: each lane walks one
+// z-plane of the stencil (or every 16th, where the cells are fine).  FP32: the
+// planes' partial sums are then added in the order of the planes with the
+// compensation of the plane-Kahan form, so the results are bit for bit those of
+// force_one in that form; FP64: the lanes' sums are added in a fixed tree.  All 16
+// lanes return the results.
+template <typename R, bool TYPED, bool EW>
+__device__ __forceinline__ typename RT<R>::R4 force_planes(const typename RT<R>::R4* __restrict__ pos,
+                                                           const int32_t* __restrict__ start, const ForceArgs<R>& a,
+                                                           bool in, int i, const R* __restrict__ rc, double& e,
+                                                           double& w, int& pairs) {
+  constexpr bool kX2 = sizeof(R) == 4;
+  constexpr Accum M = kX2 ? Accum::kPlaneKahan : Accum::kPlain;
+  static_assert(EW || kX2, "the scalar loop always sums energy and virial");
+  const unsigned full = 0xffffffffu;
+  const int sub = threadIdx.x % kPlaneLanes;
+  const auto pi = ldg4(pos + i);
+  const R rci = in ? clamp_cutoff<R>(rc[i], a.rc_max) : (R)0;
+  const Walker<R> wk(a.g, pi, rci);
+  const int ti = TYPED ? type_of(pi.w, a.ntypes) : 0;
+  R k8[8];
+  row_constants<R, TYPED, kX2>(a, ti, wk.rc2, k8);
+  const int np = in ? 2 * wk.H + 1 : 0;
+  Acc<R> c;
+  Acc2 c2;
+  Sums<M> S;
+  if constexpr (kX2) {
+    const int most = __reduce_max_sync(full, np);
+    for (int q0 = 0; q0 < most; q0 += kPlaneLanes) {
+      const int q = q0 + sub;
+      c2.fx = c2.fy = c2.fz = c2.en = c2.vir = make_float2(0.f, 0.f);
+      const bool reached = q < np && walk_plane<R, TYPED, true, M, true, Walk::kAll, EW>(
+                                         pos, start, a.g, a, i, pi, wk, wk.cz - wk.H + q, ti, k8, c, c2, S);
+      __syncwarp();
+      const float v[5] = {c2.fx.x + c2.fx.y, c2.fy.x + c2.fy.y, c2.fz.x + c2.fz.y, c2.en.x + c2.en.y,
+                          c2.vir.x + c2.vir.y};
+      const unsigned mask = __ballot_sync(full, reached) >> (threadIdx.x & 16);
+      for (int k = 0; k < min(kPlaneLanes, most - q0); ++k) {
+#pragma unroll
+        for (int m = 0; m < (EW ? 5 : 3); ++m) {
+          const float x = __shfl_sync(full, v[m], k, kPlaneLanes);
+          if (mask >> k & 1u) kahan_add(S.s[m], S.k[m], x);
+        }
+      }
+    }
+    for (int o = kPlaneLanes / 2; o > 0; o >>= 1) c2.np += __shfl_xor_sync(full, c2.np, o);
+  } else {
+    for (int q = sub; q < np; q += kPlaneLanes)
+      walk_plane<R, TYPED, false, M, true, Walk::kAll, true>(pos, start, a.g, a, i, pi, wk, wk.cz - wk.H + q, ti, k8, c,
+                                                            c2, S);
+    __syncwarp();
+#pragma unroll
+    for (int o = kPlaneLanes / 2; o > 0; o >>= 1) {
+      c.fx += __shfl_xor_sync(full, c.fx, o);
+      c.fy += __shfl_xor_sync(full, c.fy, o);
+      c.fz += __shfl_xor_sync(full, c.fz, o);
+      c.en += __shfl_xor_sync(full, c.en, o);
+      c.vir += __shfl_xor_sync(full, c.vir, o);
+      c.np += __shfl_xor_sync(full, c.np, o);
+    }
+  }
+  e = w = 0;
+  pairs = 0;
+  typename RT<R>::R4 f{};
+  if (in) f = finish_sums<R, TYPED, kX2, M, EW>(c, c2, S, k8, e, w, pairs);
+  return f;
+}
+
 }  // namespace dcm

@@ -37,14 +37,15 @@ namespace dcm {
 // of few tiles per warp does not end on them (300K particles, a cylinder of
 // liquid: 259 -> 246 us against full tiles alone first).  Coordinates
 // outside the box are looked for in the boundary cells, the only ones that may
-// hold them.  NR: cell rows of a bundle, at most; the starts of the next 32
+// hold them; the bundle's flag says whether there are any.  NR: cell rows of a bundle, at most; the starts of the next 32
 // steps are loaded while these are dealt.
 template <typename R, int NR>
 __global__ void __launch_bounds__(128) k_tile_cut(const int32_t* __restrict__ start,
                                                   const typename RT<R>::R4* __restrict__ pos,
                                                   const R* __restrict__ rc, R wide, Grid<R> g, TileCfg cfg,
                                                   int32_t* __restrict__ idx, int32_t* __restrict__ list,
-                                                  int32_t* __restrict__ counters, int64_t nslot) {
+                                                  int32_t* __restrict__ counters, int32_t* __restrict__ flag,
+                                                  int64_t nslot) {
   const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
@@ -125,7 +126,11 @@ __global__ void __launch_bounds__(128) k_tile_cut(const int32_t* __restrict__ st
         }
       }
   }
-  if (outside) counters[kTileOutside] = 1;
+  outside = __any_sync(full, outside);
+  if (lane == 0) {
+    flag[b] = outside;
+    if (outside) counters[kTileOutside] = 1;
+  }
   if (S + lane < B && S + lane < lim) idx[S + lane] = -1;
   __syncwarp();
   const int nt = min(B, lim) >> 5;
@@ -269,8 +274,7 @@ constexpr int tile_warps() {
 template <typename R, bool TYPED, bool EW>
 __global__ void __launch_bounds__(32 * tile_warps<R>(), 1) k_forces_tiles(
     const typename RT<R>::R4* __restrict__ pos, const R* __restrict__ rc, const int32_t* __restrict__ start,
-    const __grid_constant__ ForceArgs<R> a, TileCfg cfg, const int32_t* __restrict__ idx,
-    const int32_t* __restrict__ list, int32_t* __restrict__ rest, int32_t* __restrict__ counters,
+    const __grid_constant__ ForceArgs<R> a, TileCfg cfg, const __grid_constant__ TileTable tt,
     typename RT<R>::R4* __restrict__ force, double* __restrict__ part, int64_t nslot) {
   using R4 = typename RT<R>::R4;
   constexpr bool kX2 = sizeof(R) == 4;
@@ -280,8 +284,10 @@ __global__ void __launch_bounds__(32 * tile_warps<R>(), 1) k_forces_tiles(
   TileSmem<R4>& sm = reinterpret_cast<TileSmem<R4>*>(smem_raw)[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
   const Grid<R>& g = a.g;
+  const int32_t *idx = tt.idx, *list = tt.list;
+  int32_t* counters = tt.counters;
   const int nfirst = __ldg(counters + kTileFirst), ntile = nfirst + __ldg(counters + kTileLater);
-  if (__ldg(counters + kTileOutside)) return;  // all tiles go to the row walk
+  const bool outside = __ldg(counters + kTileOutside) != 0;
   auto take = [&]() {
     int t = 0;
     if (lane == 0) t = atomicAdd(counters + kTileQueue, 1);
@@ -319,7 +325,8 @@ __global__ void __launch_bounds__(32 * tile_warps<R>(), 1) k_forces_tiles(
     R xi[3] = {pi.x, pi.y, pi.z};
     // the FP64 cutoff rounded up
     const float rf = sizeof(R) == 4 ? (float)rci : __double2float_ru((double)rci);
-    const bool done = tile_candidates<R, R4>(sm, pos, start, g, cfg, active, i, xi, rf, rf, NoCutoff{}, ahead, [&](int last) {
+    const bool met = outside && tile_meets_outside<R>(cfg, tt.outside, g, active, pi.y, pi.z, rf);
+    const bool done = !met && tile_candidates<R, R4>(sm, pos, start, g, cfg, active, i, xi, rf, rf, NoCutoff{}, ahead, [&](int last) {
       ListWalk l;
       l.begin(shared_addr(&sm.list[0][lane]), last);
       if constexpr (kX2)
@@ -340,7 +347,7 @@ __global__ void __launch_bounds__(32 * tile_warps<R>(), 1) k_forces_tiles(
       if (active) force[i] = finish_sums<R, TYPED, kX2, M, EW || !kX2>(c, c2, S, k8, e, w, np);
       if (EW && part) tile_partials(e, w, np, part, nslot, (uint32_t)slot);
     } else {
-      if (lane == 0) rest[atomicAdd(counters + kTileRest, 1)] = slot;
+      if (lane == 0) tt.rest[atomicAdd(counters + kTileRest, 1)] = slot;
       ahead();
     }
     slot = slot1;
@@ -351,30 +358,64 @@ __global__ void __launch_bounds__(32 * tile_warps<R>(), 1) k_forces_tiles(
   }
 }
 
-// The tiles that the filter does not serve, by the row walk: those left over,
-// or all of them if a coordinate lies outside the box.
+// The tiles that the filter does not serve, by the row walk.  Few of them: a
+// block per tile, 16 lanes per particle (force_planes), because such a launch lasts
+// as long as its longest walk (FP64, a quarter of 7,738 particles: 1180 us with a
+// thread per particle, about 500 so).  Many of them (coordinates outside the box all
+// over it): a warp per tile, a thread per particle, which keeps more lanes busy (all
+// 8,900 tiles of 260K particles: 680 us with 16 lanes, 260 with one; FP64, 2,000
+// tiles: 4700 and 2000).
+constexpr int kRestBlock = 32 * kPlaneLanes;
+template <typename R>
+constexpr int rest_many() { return sizeof(R) == 4 ? 1500 : 600; }
+
 template <typename R, bool TYPED, bool EW>
-__global__ void __launch_bounds__(64) k_forces_rest(const typename RT<R>::R4* __restrict__ pos,
-                                                    const R* __restrict__ rc, const int32_t* __restrict__ start,
-                                                    ForceArgs<R> a, const int32_t* __restrict__ idx,
-                                                    const int32_t* __restrict__ list, const int32_t* __restrict__ rest,
-                                                    const int32_t* __restrict__ counters,
-                                                    typename RT<R>::R4* __restrict__ force, double* __restrict__ part,
-                                                    int64_t nslot) {
-  constexpr bool kX2 = sizeof(R) == 4;
-  const bool all = __ldg(counters + kTileOutside) != 0;
-  const int nfirst = __ldg(counters + kTileFirst), lane = threadIdx.x & 31;
-  const int n = all ? nfirst + __ldg(counters + kTileLater) : __ldg(counters + kTileRest);
-  for (int k = blockIdx.x * 2 + (threadIdx.x >> 5); k < n; k += gridDim.x * 2) {
-    const int slot = __ldg(!all ? rest + k : (k < nfirst ? list + k : list + (nslot - 1 - (k - nfirst))));
-    const int i = __ldg(idx + 32 * (int64_t)slot + lane);
+__global__ void __launch_bounds__(kRestBlock, sizeof(R) == 4 ? 2 : 1) k_forces_rest(const typename RT<R>::R4* __restrict__ pos,
+                                                               const R* __restrict__ rc,
+                                                               const int32_t* __restrict__ start, ForceArgs<R> a,
+                                                               TileTable t, typename RT<R>::R4* __restrict__ force,
+                                                               double* __restrict__ part, int64_t nslot) {
+  constexpr bool kX2 = sizeof(R) == 4, kEW = EW || !kX2;
+  __shared__ double sh[3][32];
+  const int n = __ldg(t.counters + kTileRest);
+  if (n >= rest_many<R>()) {
+    constexpr int kWarps = kRestBlock / 32;
+    for (int k = blockIdx.x * kWarps + (threadIdx.x >> 5); k < n; k += gridDim.x * kWarps) {
+      const int slot = __ldg(t.rest + k);
+      const int i = __ldg(t.idx + 32 * (int64_t)slot + (threadIdx.x & 31));
+      double e = 0, w = 0;
+      int np = 0;
+      if (i >= 0)
+        force[i] = force_one<R, TYPED, kX2, kX2 ? Accum::kPlaneKahan : Accum::kPlain, true, kEW>(
+            pos, start, a.g, a, i, ldg4(pos + i), rc[i], e, w, np);
+      __syncwarp();
+      if (EW && part) tile_partials(e, w, np, part, nslot, (uint32_t)slot);
+    }
+    return;
+  }
+  const int q = threadIdx.x / kPlaneLanes;
+  for (int k = blockIdx.x; k < n; k += gridDim.x) {
+    const int slot = __ldg(t.rest + k);
+    const int i = __ldg(t.idx + 32 * (int64_t)slot + q);
     double e = 0, w = 0;
     int np = 0;
-    if (i >= 0)
-      force[i] = force_one<R, TYPED, kX2, kX2 ? Accum::kPlaneKahan : Accum::kPlain, true, EW || !kX2>(
-          pos, start, a.g, a, i, ldg4(pos + i), rc[i], e, w, np);
-    __syncwarp();
-    if (EW && part) tile_partials(e, w, np, part, nslot, (uint32_t)slot);
+    const auto f = force_planes<R, TYPED, kEW>(pos, start, a, i >= 0, max(i, 0), rc, e, w, np);
+    const bool own = threadIdx.x % kPlaneLanes == 0;
+    if (own && i >= 0) force[i] = f;
+    if (EW && part) {  // summed in the order of the particles
+      __syncthreads();
+      if (own) {
+        sh[0][q] = e;
+        sh[1][q] = w;
+        sh[2][q] = (double)np;
+      }
+      __syncthreads();
+      if (threadIdx.x < 3) {
+        double v = 0;
+        for (int p = 0; p < 32; ++p) v += sh[threadIdx.x][p];
+        part[threadIdx.x * nslot + slot] = v;
+      }
+    }
   }
 }
 
@@ -427,12 +468,13 @@ int tile_cut(dcm_ctx* ctx, const TilePlan& tp, const typename RT<R>::R4* pos, co
   t.counters = ctx->tiles;
   t.list = t.counters + kTileCounters;
   t.rest = t.list + tp.slots;
-  t.idx = t.rest + tp.slots;
+  t.outside = t.rest + tp.slots;  // one per bundle, each of which has slots of its own
+  t.idx = t.outside + tp.slots;
   const int64_t nb = (int64_t)tp.cfg.nby * tp.cfg.nbz;
   DCM_CUDA_TRY(ctx, cudaMemsetAsync(t.counters, 0, kTileCounters * sizeof(int32_t), st));
   auto kc = tp.cfg.ry * tp.cfg.rz <= 4 ? k_tile_cut<R, 4> : k_tile_cut<R, 16>;
   DCM_LAUNCH(ctx, kc, (unsigned)((nb + 3) / 4), 128, 0, st, cell_start, pos, rc, (R)(1.2 * ctx->p.rc_min), g, tp.cfg,
-             t.idx, t.list, t.counters, tp.slots);
+             t.idx, t.list, t.counters, t.outside, tp.slots);
   return DCM_OK;
 }
 template int tile_cut<float>(dcm_ctx*, const TilePlan&, const float4*, const float*, const int32_t*,
@@ -456,10 +498,9 @@ int tile_forces(dcm_ctx* ctx, bool typed, bool ew, int64_t n, const typename RT<
   int sms = 0;
   DCM_CUDA_TRY(ctx, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
   const unsigned grid = (unsigned)std::min<int64_t>((tp.slots + warps - 1) / warps, sms);
-  DCM_LAUNCH(ctx, k, grid, 32 * warps, smem, st, pos, rc, cell_start, a, tp.cfg, t.idx, t.list, t.rest,
-             t.counters, force, part, tp.slots);
-  DCM_LAUNCH(ctx, kr, (unsigned)std::min<int64_t>((tp.slots + 1) / 2, 8 * sms), 64, 0, st, pos, rc, cell_start, a,
-             t.idx, t.list, t.rest, t.counters, force, part, tp.slots);
+  DCM_LAUNCH(ctx, k, grid, 32 * warps, smem, st, pos, rc, cell_start, a, tp.cfg, t, force, part, tp.slots);
+  DCM_LAUNCH(ctx, kr, (unsigned)std::min<int64_t>(tp.slots, 2 * sms), kRestBlock, 0, st, pos, rc, cell_start, a, t,
+             force, part, tp.slots);
   return check_launch(ctx, "tile_forces");
 }
 

@@ -38,9 +38,9 @@
 // -L (x_i - L and, inside the box, x_j - L, both exact because the tile and
 // everything within its cutoffs lie in the upper half).  A tile that reaches
 // past both ends of an axis is left to the per-particle row walk, and so is
-// every tile of a system in which a coordinate lies outside the box (or is
-// NaN): binning puts such particles into the boundary cells, where the kernel that
-// cuts the tiles looks for them.
+// every tile that may meet a coordinate outside the box (or a NaN): binning puts
+// such particles into the boundary cells, where the kernel that cuts the tiles
+// looks for them and marks their bundles.
 #pragma once
 
 #include <cuda_fp16.h>
@@ -71,9 +71,10 @@ enum { kTileFirst = 0, kTileLater = 1, kTileQueue = 2, kTileRest = 3, kTileOutsi
 // The tiles of a launch (forces_tiles.cu): the slots in use are list[0 ..
 // counters[kTileFirst]) and list[nslot - counters[kTileLater] .. nslot) from its
 // end, slot s holds particles idx[32 s .. 32 s + 31], rest takes the slots that a
-// kernel leaves to the row walk.
+// kernel leaves to the row walk, outside says which bundles hold a coordinate
+// outside the box (counters[kTileOutside]: whether any does).
 struct TileTable {
-  int32_t *counters, *list, *rest, *idx;
+  int32_t *counters, *list, *rest, *outside, *idx;
 };
 template <typename R>
 int tile_cut(dcm_ctx* ctx, const TilePlan& tp, const typename RT<R>::R4* pos, const R* rc, const int32_t* cell_start,
@@ -267,6 +268,26 @@ __device__ __forceinline__ int warp_incl_sum(int v) {
     if (lane >= o) v += u;
   }
   return v;
+}
+
+// Whether a tile may meet a coordinate outside the box: whether its own bundle
+// or one of those within its largest reach holds any (y, z, reach: of the lanes'
+// particles, which are one bundle's; lane 0 always holds one).  Called by whole warps,
+// and only where some bundle does.
+template <typename R>
+static __device__ __noinline__ bool tile_meets_outside(const TileCfg& cfg, const int32_t* __restrict__ outside,
+                                                       const Grid<R>& g, bool active, R y, R z, float reach) {
+  const float most = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(active ? reach : 0.f)));
+  const int h = (int)(most * (float)g.inv_edge + 0.05f) + 1, ny = g.n[1], nz = g.n[2];  // rows, with room for rounding
+  const int by = __shfl_sync(0xffffffffu, cell_coord<R>(y, g.edge, g.inv_edge, ny), 0) / cfg.ry,
+            bz = __shfl_sync(0xffffffffu, cell_coord<R>(z, g.edge, g.inv_edge, nz), 0) / cfg.rz;
+  const int ry = cfg.ry + 2 * h, n = ry * (cfg.rz + 2 * h);
+  bool any = false;
+  for (int k = threadIdx.x & 31; k < n; k += 32) {
+    const int v = ((by * cfg.ry - h + k % ry) % ny + ny) % ny, w = ((bz * cfg.rz - h + k / ry) % nz + nz) % nz;
+    any = any || __ldg(outside + v / cfg.ry + cfg.nby * (w / cfg.rz)) != 0;
+  }
+  return __any_sync(0xffffffffu, any);
 }
 
 // Visits the candidates of one pass of a tile (at most 32 particles): stages

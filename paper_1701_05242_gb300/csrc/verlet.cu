@@ -303,7 +303,7 @@ constexpr int kListTileWarps = 16;  // as the tiled forces: as many as the SM's 
 template <bool N3>
 __global__ void __launch_bounds__(32 * kListTileWarps, 1) k_list_tiles(
     const float4* __restrict__ rec, const float* __restrict__ rc, const int32_t* __restrict__ start,
-    const __grid_constant__ Grid<float> g, TileCfg cfg, TileTable t, int64_t nslot, float rc_max, float skin,
+    const __grid_constant__ Grid<float> g, TileCfg cfg, const __grid_constant__ TileTable t, int64_t nslot, float rc_max, float skin,
     const int32_t* __restrict__ capw, const int32_t* __restrict__ offw, uint32_t* __restrict__ list,
     int32_t* __restrict__ nnb, int32_t* __restrict__ nimg, int32_t* __restrict__ flag) {
   const unsigned full = 0xffffffffu;
@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(32 * kListTileWarps, 1) k_list_tiles(
   TileSmem<float4>& sm = reinterpret_cast<TileSmem<float4>*>(smem_raw)[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
   const int nfirst = __ldg(t.counters + kTileFirst), ntile = nfirst + __ldg(t.counters + kTileLater);
-  if (__ldg(t.counters + kTileOutside)) return;  // all tiles go to the row walk
+  const bool outside = __ldg(t.counters + kTileOutside) != 0;
   for (;;) {
     int k = 0;
     if (lane == 0) k = atomicAdd(t.counters + kTileQueue, 1);
@@ -329,7 +329,8 @@ __global__ void __launch_bounds__(32 * kListTileWarps, 1) k_list_tiles(
       col.out = lane_column(list, offw, i);
       col.cap = __ldg(capw + (i >> 5));
     }
-    const bool done = tile_candidates<float, float4>(
+    const bool met = outside && tile_meets_outside<float>(cfg, t.outside, g, active, pi.y, pi.z, rl);
+    const bool done = !met && tile_candidates<float, float4>(
         sm, rec, start, g, cfg, active, i, xi, rl, rl, NoCutoff{}, []() {}, [&](int last) {
           ListWalk l;
           l.begin(shared_addr(&sm.list[0][lane]), last);
@@ -369,19 +370,16 @@ __global__ void __launch_bounds__(32 * kListTileWarps, 1) k_list_tiles(
   }
 }
 
-// The tiles that the filter does not serve, by the row walk: those left over,
-// or all of them if a coordinate lies outside the box.
+// The tiles that the filter does not serve, by the row walk.
 __global__ void __launch_bounds__(64) k_list_rest(const float4* __restrict__ pos, const float* __restrict__ rc,
                                                   const int32_t* __restrict__ start, Grid<float> g, TileTable t,
-                                                  int64_t nslot, float rc_max, float skin, int n3,
+                                                  float rc_max, float skin, int n3,
                                                   const int32_t* __restrict__ capw, const int32_t* __restrict__ offw,
                                                   uint32_t* __restrict__ list, int32_t* __restrict__ nnb,
                                                   int32_t* __restrict__ nimg, int32_t* __restrict__ flag) {
-  const bool all = __ldg(t.counters + kTileOutside) != 0;
-  const int nfirst = __ldg(t.counters + kTileFirst), lane = threadIdx.x & 31;
-  const int n = all ? nfirst + __ldg(t.counters + kTileLater) : __ldg(t.counters + kTileRest);
+  const int lane = threadIdx.x & 31, n = __ldg(t.counters + kTileRest);
   for (int k = blockIdx.x * 2 + (threadIdx.x >> 5); k < n; k += gridDim.x * 2) {
-    const int slot = __ldg(!all ? t.rest + k : (k < nfirst ? t.list + k : t.list + (nslot - 1 - (k - nfirst))));
+    const int slot = __ldg(t.rest + k);
     const int i = __ldg(t.idx + 32 * (int64_t)slot + lane);
     if (i >= 0 && !fill_one<float>(i, pos, rc, start, g, rc_max, skin, n3, capw, offw, list, nnb, nimg))
       atomicExch(flag, 1);
@@ -1012,7 +1010,7 @@ static int list_fill(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, con
                  32 * kListTileWarps, smem, st, rec, rc, ctx->cell_start, g, tp.cfg, t, tp.slots, rcm, skin, ctx->capw,
                  ctx->offw, ctx->list, ctx->nnb, ctx->nimg, ctx->lflag);
       DCM_LAUNCH(ctx, k_list_rest, (unsigned)std::min<int64_t>((tp.slots + 1) / 2, 8 * sms), 64, 0, st, pos, rc,
-                 ctx->cell_start, g, t, tp.slots, rcm, skin, n3, ctx->capw, ctx->offw, ctx->list, ctx->nnb, ctx->nimg,
+                 ctx->cell_start, g, t, rcm, skin, n3, ctx->capw, ctx->offw, ctx->list, ctx->nnb, ctx->nimg,
                  ctx->lflag);
       return DCM_OK;
     }

@@ -332,3 +332,83 @@ def test_coordinates_of_negative_zero(D, form, lx):
         (F0, t0), (F1, t1) = res
         assert t0[3] == t1[3]
         assert np.sqrt(((F0 - F1) ** 2).mean()) <= 1e-5 * np.sqrt((F1 ** 2).mean())
+
+
+@pytest.mark.parametrize("prec,typed", [("mixed", False), ("mixed", True), ("fp64", False), ("fp64", True)])
+@pytest.mark.parametrize("box,outside", [
+    ((61.5, 25.5, 70.5), 0),    # tiles that reach past both ends of y
+    ((70.5, 61.5, 25.5), 0),    # of z
+    ((25.5, 25.5, 150.0), 0),   # of x and y
+    ((48.0, 45.0, 51.0), 1),    # one bundle with a coordinate outside the box
+    ((48.0, 45.0, 51.0), 60),   # most tiles next to one
+])
+def test_tiles_left_to_the_row_walk(D, box, outside, prec, typed):
+    """Tiles that the filter does not serve, a few or most of them."""
+    pos = lattice(box, 51)
+    rng = np.random.default_rng(52)
+    for k in rng.choice(len(pos), outside, replace=False):
+        d = rng.integers(0, 3)
+        pos[k, d] = rng.choice([-0.25, box[d], box[d] + 0.75])
+    rc = cutoffs(pos, box, "mixed" if typed else "ramp", rng)
+    assert len(pos) > 32768
+    kw, types = dict(shift_energy=1), None
+    if typed:
+        types = rng.integers(0, 2, len(pos)).astype(np.float32)
+        kw.update(ntypes=2, eps=(1.0, 0.8), sigma=(1.0, 1.1))
+    walk = D.DCM_FORCE_PACKED if prec == "mixed" else D.DCM_FORCE_THREAD
+    F0, t0 = forces(D, box, pos, rc, types, prec, force_kernel=walk, **kw)
+    F1, t1 = forces(D, box, pos, rc, types, prec, **kw)
+    assert t1[2] == t0[2]
+    tol = MIXED_RMS if prec == "mixed" else FP64_RMS
+    # one particle on top of another may outweigh all others: particle by particle, against the larger of its own
+    # force and the RMS without the largest
+    mag = np.sqrt((F0[:, :3] ** 2).sum(1))
+    rms = np.sqrt((np.sort(mag)[:-200] ** 2).mean())
+    err = np.sqrt(((F1 - F0)[:, :3] ** 2).sum(1)) / np.maximum(mag, rms)
+    assert np.sqrt((err ** 2).mean()) <= tol and err.max() <= 40 * tol
+    assert abs(t1[0] - t0[0]) <= 4 * tol * np.abs(F0[:, 3]).sum()
+
+
+@pytest.mark.parametrize("ntypes", [1, 2])
+@pytest.mark.parametrize("box,outside", [
+    ((63.0, 61.5, 72.0), 0),    # hardly any tile left over
+    ((64.5, 25.5, 102.0), 0),   # tiles that reach past both ends of y
+    ((63.0, 61.5, 72.0), 1),
+    ((63.0, 61.5, 72.0), 60),
+])
+def test_adjoint_tiles_left_to_the_row_walk(D, box, outside, ntypes):
+    """The tiled adjoint and the kernel for the tiles left over, whose
+    parameter sums share one table, against the FP64 row walk: bounds as in
+    test_adjoint_forms_against_fp64."""
+    pos = lattice(box, 61)
+    rng = np.random.default_rng(62)
+    rc = cutoffs(pos, box, "ramp", rng).astype(np.float32).astype(np.float64)
+    for k in rng.choice(np.flatnonzero(rc > 5.9), outside, replace=False):  # in the vapor: nobody on top of another
+        d = rng.integers(0, 2)
+        pos[k, d] = rng.choice([-0.25, box[d], box[d] + 0.75])
+    n = len(pos)
+    assert n > 49152
+    types = rng.integers(0, ntypes, n).astype(np.float32)
+    A = np.concatenate([rng.normal(size=(n, 3)), np.zeros((n, 1))], 1).astype(np.float32)
+    res = []
+    for prec, real in ((D.DCM_PREC_FP64, torch.float64), (D.DCM_PREC_MIXED, torch.float32)):
+        ctx = D.Context(D.make_params(box, n_max=n, ntypes=ntypes, eps=(1.0, 0.8)[:ntypes], sigma=(1.0, 1.1)[:ntypes],
+                                      shift_energy=1, precision=prec))
+        i32 = dict(dtype=torch.int32, device="cuda")
+        cell, start, perm = torch.empty(n, **i32), torch.empty(ctx.ncell + 1, **i32), torch.empty(n, **i32)
+        p4 = D.to_real4(torch.from_numpy(pos), torch.from_numpy(types), real)
+        ps = torch.empty_like(p4)
+        D.dcm_bin(ctx, n, p4, cell, start, perm, ps)
+        perm = perm.long()
+        G, dpar = torch.full_like(ps, 7.0), torch.full((2 * ntypes,), 7.0, dtype=torch.float64, device="cuda")
+        D.dcm_forces_backward(ctx, n, ps, torch.from_numpy(rc).to(real).cuda()[perm].contiguous(), start,
+                              torch.from_numpy(A).to(real).cuda()[perm].contiguous(), 0.7, G, dpar)
+        out = torch.empty_like(G)
+        out[perm] = G
+        assert D.dcm_status(ctx) == D.DCM_OK
+        res.append((out.double().cpu().numpy(), dpar.cpu().numpy()))
+        ctx.close()
+    (G0, d0), (G1, d1) = res
+    assert np.sqrt(((G1 - G0)[:, :3] ** 2).mean()) <= 5e-6 * np.sqrt((G0[:, :3] ** 2).mean())
+    assert np.all(G1[:, 3] == 0.0)
+    assert np.all(np.abs(d1 - d0) <= 5e-6 * np.abs(d0).max())
