@@ -75,14 +75,16 @@ enum dcm_status_code {
  * kernel serves FP32 runs (DCM_PREC_MIXED) of one or two types; otherwise
  * kernel 1 runs.  AUTO finds the candidates over tiles of 32 particles with a
  * tensor-core filter where that is faster: boxes of at least 4 rc_max, the
- * default accumulation, more than 32,768 particles in the mixed form and 4,000
- * in the FP64 form.  Smaller systems of the mixed form take 16 lanes per
- * particle (AUTO and PACKED; the same sums bit for bit as one thread each).
+ * default accumulation, more than 32,768 particles in the mixed form (20,480
+ * where the cells are no narrower than rc_min) and 4,000 in the FP64 form.  Smaller
+ * systems of the mixed form take 16 lanes per particle (AUTO and PACKED; the same
+ * sums bit for bit as one thread each; PACKED, and AUTO without tiles, up to 23,552
+ * there).
  * Values 2, 4 and 5 are not used (invalid). */
 enum {
   DCM_FORCE_AUTO = 0,        /* tiles where they serve, else kernel 3 where it applies, else kernel 1 */
   DCM_FORCE_THREAD = 1,      /* one thread per particle i, one candidate per instruction */
-  DCM_FORCE_PACKED = 3       /* one thread per particle i, two candidates per FP32x2 instruction */
+  DCM_FORCE_PACKED = 3       /* two candidates per FP32x2 instruction; one thread per particle i, in small systems 16 */
 };
 
 /* Per-particle accumulation of the mixed precision form (dcm_params.

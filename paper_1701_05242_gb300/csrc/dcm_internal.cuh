@@ -268,8 +268,16 @@ int lj_forces(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, const R* r
 // take 16 lanes per particle in the forces (k_forces_planes), whose blocks of 8
 // particles each leave one partial sum.  With energies, 16 lanes / one thread per
 // particle / tiles: 41 / 193 / - us for 1,935 particles, 97 / 219 / - for 30,240,
-// - / 238 / 106 for 39,191.
+// - / 238 / 106 for 39,191.  Where the cells are so wide that most cutoffs span
+// three planes (13 lanes idle) the line lies lower: with cells of 3 sigma and a
+// cutoff of 3, 16 lanes / one thread / tiles take 95 / 130 / 66 us for 15,483
+// particles, 126 / 142 / 72 for 22,045, 162 / 136 / 76 for 30,240; with cells of 6 and
+// two types 446 / 514 / 190 for 19,354, 560 / 517 / 187 for 24,192.  (tiles: whether
+// they take over above the line, else one thread per particle does.)
 constexpr int64_t kPlanesMaxN = 32768;
+inline int64_t planes_max_n(const dcm_params& p, bool tiles) {
+  return p.rc_min > p.l ? kPlanesMaxN : (tiles ? 20480 : 23552);
+}
 constexpr int kPlaneLanes = 16, kPlaneBlock = 128;  // lanes per particle, threads per block
 constexpr int64_t plane_slots(int64_t n) { return (n + 7) / 8; }
 // Systems of at most kAdjWarpMaxN particles take a warp per particle in the

@@ -224,8 +224,12 @@ int lj_forces(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, const R* r
   a.rc_max = (R)ctx->p.rc_max;
   const bool typed = lj_general(t);
   const int kind = resolve_force_kernel(ctx);
+  // the default accumulation of the packed pair loop; AUTO runs over tiles where
+  // they serve (their sums carried by the same Kahan compensation), or FP64
+  const bool kahan = kind == DCM_FORCE_PACKED && resolve_accumulation(ctx) == DCM_ACC_PLANE_KAHAN;
+  const bool tiles = ctx->p.force_kernel == DCM_FORCE_AUTO && (sizeof(R) == 8 || kahan) && tiles_serve(ctx, n);
   if constexpr (sizeof(R) == 4) {
-    if (kind == DCM_FORCE_PACKED && n <= kPlanesMaxN && resolve_accumulation(ctx) == DCM_ACC_PLANE_KAHAN) {
+    if (kahan && n <= planes_max_n(ctx->p, tiles)) {
       const bool ew = energies || totals;
       double* part = totals ? ctx->red : nullptr;
       const int64_t nblk = plane_slots(n);
@@ -240,10 +244,7 @@ int lj_forces(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, const R* r
       return DCM_OK;
     }
   }
-  // AUTO runs over tiles where they serve: the default accumulation (the
-  // packed pair loop, its sums carried by the same Kahan compensation), or FP64
-  if (ctx->p.force_kernel == DCM_FORCE_AUTO && tiles_serve(ctx, n) &&
-      (sizeof(R) == 8 || (kind == DCM_FORCE_PACKED && resolve_accumulation(ctx) == DCM_ACC_PLANE_KAHAN))) {
+  if (tiles) {
     double* part = totals ? ctx->red : nullptr;
     stage_begin(ctx, DCM_STAGE_FORCES, st);
     int r = tile_forces<R>(ctx, typed, energies || totals, n, pos, rc, cell_start, a, force, part, st);

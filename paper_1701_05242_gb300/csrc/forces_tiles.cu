@@ -455,7 +455,7 @@ TilePlan tile_plan(const dcm_params& p, const int64_t* nc, int64_t n) {
 // Launches below this many particles keep the row walk: that few leave most
 // SMs without a tile, and a launch lasts as long as its longest tile (FP64:
 // 4,838 particles 1594 us by the row walk, 618 over tiles; the mixed form takes
-// 16 lanes per particle up to kPlanesMaxN).
+// 16 lanes per particle up to planes_max_n).
 constexpr int64_t kTilesMinN = 4000;
 
 bool tiles_serve(const dcm_ctx* ctx, int64_t n) {

@@ -412,3 +412,32 @@ def test_adjoint_tiles_left_to_the_row_walk(D, box, outside, ntypes):
     assert np.sqrt(((G1 - G0)[:, :3] ** 2).mean()) <= 5e-6 * np.sqrt((G0[:, :3] ** 2).mean())
     assert np.all(G1[:, 3] == 0.0)
     assert np.all(np.abs(d1 - d0) <= 5e-6 * np.abs(d0).max())
+
+
+@pytest.mark.parametrize("l", [3.0, 6.0])
+@pytest.mark.parametrize("typed", [False, True])
+@pytest.mark.parametrize("n,kernel", [(20480, 0), (23552, 3)])
+def test_wide_cells_on_both_sides_of_the_switch(D, l, typed, n, kernel):
+    """With cells no narrower than rc_min, up to 20,480 particles run 16 lanes
+    per particle, one more runs tiles (AUTO); without tiles (PACKED) up to 23,552
+    do, and one more runs one thread per particle."""
+    box = (60.0, 48.0, 48.0)
+    pos = lattice(box, 81, spacing=1.3)
+    rng = np.random.default_rng(82)
+    pos = pos[np.abs(pos[:, 2] - 24.0) < 12.0]
+    pos = pos[rng.permutation(len(pos))]
+    assert len(pos) > n
+    pos = np.concatenate([pos[:n], [[30.0, 24.0, 1.0]]]).astype(np.float32)
+    rc = np.append(np.clip(6.0 - (12.0 - np.abs(pos[:n, 2] - 24.0)), 3.0, 6.0), 6.0)
+    types = rng.integers(0, 2 if typed else 1, n + 1).astype(np.float32)
+    F0, _ = by_input(D, box, pos[:n], rc[:n], types[:n], l=l, h=1.5, force_kernel=kernel)
+    F1, _ = by_input(D, box, pos, rc, types, l=l, h=1.5, force_kernel=kernel)
+    assert np.all(F1[n] == 0.0)
+    if kernel == D.DCM_FORCE_PACKED:
+        assert np.array_equal(F1[:n], F0)  # the same sums in the same order
+    assert np.sqrt(((F1[:n] - F0)[:, :3] ** 2).mean()) <= MIXED_RMS * np.sqrt((F0[:, :3] ** 2).mean())
+    F0n, t0 = forces(D, box, pos, rc, types if typed else None, force_kernel=D.DCM_FORCE_THREAD, l=l, h=1.5,
+                     **(dict(ntypes=2, eps=(1.0, 0.8), sigma=(1.0, 1.1)) if typed else {}))
+    F1n, t1 = forces(D, box, pos, rc, types if typed else None, l=l, h=1.5, force_kernel=kernel,
+                     **(dict(ntypes=2, eps=(1.0, 0.8), sigma=(1.0, 1.1)) if typed else {}))
+    assert t1[2] == t0[2]
