@@ -122,7 +122,7 @@ struct dcm_ctx {
   int32_t* blk_max;         // 2 nblk: largest cutoff (float bits) per adjoint block, and of the 27 around it
   int32_t* tile_scratch;    // tile_scratch_ints(n_max): launch order of the force and adjoint tiles
   int32_t* tiles;           // tile_ints(tile_cap): counters, slots in use, slots left to the row walk, flags of the
-                            // bundles, particles of the slots
+                            // bundles' pieces, particles of the slots
   int64_t tile_cap;         // pair tile slots (0: tiles not served)
   int nblk3[3];             // adjoint blocks per dimension (edge >= 1.001 rc_max)
   int64_t nblk;
@@ -292,8 +292,9 @@ constexpr int64_t adj_warp_slots(int64_t n) { return (n + 3) / 4; }
 struct TileCfg {
   int ry, rz;      // cell rows of a bundle along y and z
   int nby, nbz;    // bundles along y and z
+  int np, px;      // pieces of a bundle along x, and the cells of each (the last one may have fewer)
   int cap;         // longest tile, in cells along x
-  int cmax;        // spare tile slots per bundle (tiles that are not full)
+  int cmax;        // spare tile slots per piece (tiles that are not full)
   float scale;     // power of two that takes rc_max into [4, 8)
 };
 struct TilePlan {

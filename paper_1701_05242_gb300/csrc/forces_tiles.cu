@@ -25,19 +25,19 @@ namespace dcm {
 // tiles
 // ---------------------------------------------------------------------------
 
-// One warp per bundle: deals the bundle's particles, in the order of their
+// One warp per piece of a bundle: deals its particles, in the order of their
 // cell step along x, into tiles of 32 (a tile ends early only where it would
-// grow longer than cfg.cap cells, and at the bundle's end).  The particles of the
+// grow longer than cfg.cap cells, and at the piece's end).  The particles of the
 // tile in slot s are idx[32 s .. 32 s + 31] (-1: none).  Slots follow the
-// particles (those before the bundle / 32, plus cmax per bundle, which covers the
+// particles (those before the piece / 32, plus cmax per piece, which covers the
 // tiles that are not full), so sums kept per slot do not depend on timing; the
-// list of the slots in use does (bundles append to it as they finish).  Tiles
+// list of the slots in use does (pieces append to it as they finish).  Tiles
 // whose first or 16th particle has a cutoff above `wide` are listed from the
 // front, the others from the back: the costly ones start first, so that a launch
 // of few tiles per warp does not end on them (300K particles, a cylinder of
 // liquid: 259 -> 246 us against full tiles alone first).  Coordinates
 // outside the box are looked for in the boundary cells, the only ones that may
-// hold them; the bundle's flag says whether there are any.  NR: cell rows of a bundle, at most; the starts of the next 32
+// hold them; the piece's flag says whether there are any.  NR: cell rows of a bundle, at most; the starts of the next 32
 // steps are loaded while these are dealt.
 template <typename R, int NR>
 __global__ void __launch_bounds__(128) k_tile_cut(const int32_t* __restrict__ start,
@@ -49,16 +49,21 @@ __global__ void __launch_bounds__(128) k_tile_cut(const int32_t* __restrict__ st
   const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  const int b = blockIdx.x * 4 + (threadIdx.x >> 5);
+  const int piece = blockIdx.x * 4 + (threadIdx.x >> 5), b = piece / cfg.np;
   if (b >= cfg.nby * cfg.nbz) return;
   const int by = b % cfg.nby, bz = b / cfg.nby;
+  const int xs = (piece - b * cfg.np) * cfg.px, xe = min(xs + cfg.px, nx);
   const int y0 = by * cfg.ry, z0 = bz * cfg.rz, nr_y = min(cfg.ry, ny - y0), nr_z = min(cfg.rz, nz - z0);
   const int nr = nr_y * nr_z;
-  // particles in the bundles before this one
+  // particles in the bundles before this one, and in the pieces before in it
   int before = 0;
   if (lane < nr_z) {
     const int z = nx * ny * (z0 + lane);
     before = __ldg(start + z + nx * y0) - __ldg(start + z);
+  }
+  if (xs > 0 && lane < nr) {
+    const int c = nx * (y0 + lane % nr_y + ny * (z0 + lane / nr_y));
+    before += __ldg(start + c + xs) - __ldg(start + c);
   }
   const int plane = __ldg(start + nx * ny * z0);
   int row[NR];
@@ -74,18 +79,18 @@ __global__ void __launch_bounds__(128) k_tile_cut(const int32_t* __restrict__ st
   auto load = [&](int x) {
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
-      const bool in = r < nr && x < nx;
+      const bool in = r < nr && x < xe;
       from[r] = in ? __ldg(start + row[r] + x) : 0;
       to[r] = in ? __ldg(start + row[r] + x + 1) : 0;
     }
   };
-  load(lane);
+  load(xs + lane);
   before = __reduce_add_sync(full, before) + plane;
-  const int64_t slot0 = (before >> 5) + (int64_t)b * cfg.cmax;
+  const int64_t slot0 = (before >> 5) + (int64_t)piece * cfg.cmax;
   idx += 32 * slot0;
   const int lim = (int)min(32 * (nslot - slot0), (int64_t)INT_MAX);  // never reached (see above)
-  int S = 0, B = 0, x0 = 0;  // next place, end of the open tile, its first cell step
-  for (int xb = 0; xb < nx; xb += 32) {
+  int S = 0, B = 0, x0 = xs;  // next place, end of the open tile, its first cell step
+  for (int xb = xs; xb < xe; xb += 32) {
     const int x = xb + lane;
     int k0[NR], k1[NR], c = 0;
 #pragma unroll
@@ -94,7 +99,7 @@ __global__ void __launch_bounds__(128) k_tile_cut(const int32_t* __restrict__ st
       k1[r] = max(to[r], from[r]);
       c += k1[r] - k0[r];
     }
-    if (xb + 32 < nx) load(x + 32);
+    if (xb + 32 < xe) load(x + 32);
     const int s = warp_incl_sum(c);
     int place = S + s - c, at = 0;  // where the lane's particles go; lanes settled
     for (;;) {
@@ -128,7 +133,7 @@ __global__ void __launch_bounds__(128) k_tile_cut(const int32_t* __restrict__ st
   }
   outside = __any_sync(full, outside);
   if (lane == 0) {
-    flag[b] = outside;
+    flag[piece] = outside;
     if (outside) counters[kTileOutside] = 1;
   }
   if (S + lane < B && S + lane < lim) idx[S + lane] = -1;
@@ -436,19 +441,31 @@ TilePlan tile_plan(const dcm_params& p, const int64_t* nc, int64_t n) {
   const double lx = p.lx > 0.0 ? p.lx : p.l, Lx = (double)nc[0] * lx;
   const double cap = std::min(24.0 * p.rc_max, 0.5 * Lx - 2.0 * p.rc_max);
   t.cfg.cap = (int)std::max(1.0, std::min(std::floor(cap / lx), 65535.0));
-  t.cfg.cmax = 2 + (int)((nc[0] + t.cfg.cap - 1) / t.cfg.cap);
   int k;
   std::frexp(p.rc_max, &k);  // rc_max = f 2^k, f in [0.5, 1)
   t.cfg.scale = std::ldexp(1.0f, 3 - k);
   const int64_t nb = (int64_t)t.cfg.nby * t.cfg.nbz;
-  t.slots = n / 32 + nb * t.cfg.cmax + 1;
+  // Few bundles are cut into pieces along x, a warp each, because one warp takes
+  // about 1.2 us per 32 cell steps (a box of 4800 x 16 x 16 cells: 372 us in 64
+  // warps), and a launch of 8 warps per SM hides most of that.  Pieces of at least 16
+  // rc_max and of 8 tiles at the mean density (for n_max particles, so that the
+  // table of n never outgrows that of n_max): every piece ends on a tile that is not full.
+  const double dense = (double)p.n_max / ((double)nc[0] * (double)nc[1] * (double)nc[2]) * t.cfg.ry * t.cfg.rz;
+  const double least = std::max(16.0 * p.rc_max / lx, 8.0 * 32.0 / std::max(dense, 1e-9));  // cells
+  const int64_t most = (int64_t)std::max(1.0, std::min((double)nc[0] / least, 65536.0));
+  const int64_t pieces = std::max<int64_t>(1, std::min(most, (152 * 8 + nb - 1) / nb));
+  t.cfg.px = (int)((nc[0] + pieces - 1) / pieces);
+  t.cfg.np = (int)((nc[0] + t.cfg.px - 1) / t.cfg.px);
+  auto spare = [&](int64_t cells) { return 2 + (int)((cells + t.cfg.cap - 1) / t.cfg.cap); };
+  t.cfg.cmax = spare(t.cfg.px);
+  t.slots = n / 32 + nb * t.cfg.np * t.cfg.cmax + 1;
   // A box of at least 4 rc_max (in a smaller one most tiles at an interface
   // reach past both ends of an axis), cells no wider than the cutoff sphere
   // (FP16 range of the staged coordinates) and a table that stays in proportion
   // to the particles.
   const double Lmin = std::min(Lx, std::min((double)nc[1], (double)nc[2]) * p.l);
   t.usable = Lmin >= 4.0 * p.rc_max && p.l <= 2.0 * p.rc_max && lx <= 2.0 * p.rc_max &&
-             8 * nb * t.cfg.cmax <= n + 65536 && 32 * t.slots < (int64_t)1 << 31;
+             8 * nb * spare(nc[0]) <= n + 65536 && 32 * t.slots < (int64_t)1 << 31;
   return t;
 }
 
@@ -468,9 +485,9 @@ int tile_cut(dcm_ctx* ctx, const TilePlan& tp, const typename RT<R>::R4* pos, co
   t.counters = ctx->tiles;
   t.list = t.counters + kTileCounters;
   t.rest = t.list + tp.slots;
-  t.outside = t.rest + tp.slots;  // one per bundle, each of which has slots of its own
+  t.outside = t.rest + tp.slots;  // one per piece of a bundle, each of which has slots of its own
   t.idx = t.outside + tp.slots;
-  const int64_t nb = (int64_t)tp.cfg.nby * tp.cfg.nbz;
+  const int64_t nb = (int64_t)tp.cfg.nby * tp.cfg.nbz * tp.cfg.np;
   DCM_CUDA_TRY(ctx, cudaMemsetAsync(t.counters, 0, kTileCounters * sizeof(int32_t), st));
   auto kc = tp.cfg.ry * tp.cfg.rz <= 4 ? k_tile_cut<R, 4> : k_tile_cut<R, 16>;
   DCM_LAUNCH(ctx, kc, (unsigned)((nb + 3) / 4), 128, 0, st, cell_start, pos, rc, (R)(1.2 * ctx->p.rc_min), g, tp.cfg,

@@ -71,8 +71,8 @@ enum { kTileFirst = 0, kTileLater = 1, kTileQueue = 2, kTileRest = 3, kTileOutsi
 // The tiles of a launch (forces_tiles.cu): the slots in use are list[0 ..
 // counters[kTileFirst]) and list[nslot - counters[kTileLater] .. nslot) from its
 // end, slot s holds particles idx[32 s .. 32 s + 31], rest takes the slots that a
-// kernel leaves to the row walk, outside says which bundles hold a coordinate
-// outside the box (counters[kTileOutside]: whether any does).
+// kernel leaves to the row walk, outside says which bundles' pieces hold a
+// coordinate outside the box (counters[kTileOutside]: whether any does).
 struct TileTable {
   int32_t *counters, *list, *rest, *outside, *idx;
 };
@@ -285,7 +285,8 @@ static __device__ __noinline__ bool tile_meets_outside(const TileCfg& cfg, const
   bool any = false;
   for (int k = threadIdx.x & 31; k < n; k += 32) {
     const int v = ((by * cfg.ry - h + k % ry) % ny + ny) % ny, w = ((bz * cfg.rz - h + k / ry) % nz + nz) % nz;
-    any = any || __ldg(outside + v / cfg.ry + cfg.nby * (w / cfg.rz)) != 0;
+    for (int p = 0; p < cfg.np; ++p)
+      any = any || __ldg(outside + (v / cfg.ry + cfg.nby * (w / cfg.rz)) * cfg.np + p) != 0;
   }
   return __any_sync(0xffffffffu, any);
 }

@@ -441,3 +441,55 @@ def test_wide_cells_on_both_sides_of_the_switch(D, l, typed, n, kernel):
     F1n, t1 = forces(D, box, pos, rc, types if typed else None, l=l, h=1.5, force_kernel=kernel,
                      **(dict(ntypes=2, eps=(1.0, 0.8), sigma=(1.0, 1.1)) if typed else {}))
     assert t1[2] == t0[2]
+
+
+@pytest.mark.parametrize("prec", ["mixed", "fp64"])
+@pytest.mark.parametrize("box,lx,outside", [
+    ((480.0, 24.0, 27.0), 0.0, 0),
+    ((480.0, 24.0, 27.0), 0.5, 0),    # a last piece of fewer cells
+    ((480.0, 24.0, 27.0), 0.75, 1),   # one piece with a coordinate outside the box
+    ((600.0, 30.0, 33.0), 1.5, 3),
+])
+def test_tiles_of_long_bundles(D, box, lx, outside, prec):
+    """Few and long bundles of cell rows, which are cut into pieces."""
+    pos = lattice(box, 91)
+    rng = np.random.default_rng(92)
+    for k in rng.choice(np.flatnonzero(np.abs(pos[:, 2] - 0.5 * box[2]) > 0.3 * box[2]), outside, replace=False):
+        pos[k, 0] = rng.choice([-0.25, box[0]])
+    rc = cutoffs(pos, box, "ramp", rng)
+    assert len(pos) > 32768
+    walk = D.DCM_FORCE_PACKED if prec == "mixed" else D.DCM_FORCE_THREAD
+    F0, t0 = forces(D, box, pos, rc, prec=prec, force_kernel=walk, lx=lx)
+    F1, t1 = forces(D, box, pos, rc, prec=prec, lx=lx)
+    assert t1[2] == t0[2]
+    tol = MIXED_RMS if prec == "mixed" else FP64_RMS
+    assert np.sqrt(((F1 - F0)[:, :3] ** 2).mean()) <= tol * np.sqrt((F0[:, :3] ** 2).mean())
+    assert abs(t1[0] - t0[0]) <= 4 * tol * np.abs(F0[:, 3]).sum()
+
+
+def test_lists_and_adjoint_of_long_bundles(D):
+    box = (480.0, 33.0, 34.5)
+    pos = lattice(box, 93)
+    rng = np.random.default_rng(94)
+    res = []
+    for skin in (0.5, 0.0):
+        ctx = D.Context(D.make_params(box, n_max=len(pos), skin=skin, lx=0.5))
+        st = D.State(ctx, D.to_real4(torch.from_numpy(pos)), torch.zeros(len(pos), 4))
+        D.dcm_step_init(ctx, st)
+        assert D.dcm_status(ctx) == D.DCM_OK
+        ids = st.current()[3].cpu().numpy()
+        F = np.empty((len(pos), 3))
+        F[ids] = st.force.double().cpu().numpy()[:, :3]
+        res.append((F, st.thermo.cpu().numpy()))
+        ctx.close()
+    (F0, t0), (F1, t1) = res
+    assert t0[3] == t1[3]
+    assert np.sqrt(((F0 - F1) ** 2).mean()) <= 1e-5 * np.sqrt((F1 ** 2).mean())
+    types = rng.integers(0, 2, len(pos)).astype(np.float32)  # bounds as in test_adjoint_forms_against_fp64
+    A = np.concatenate([rng.normal(size=(len(pos), 3)), np.zeros((len(pos), 1))], 1).astype(np.float32)
+    rc = cutoffs(pos, box, "ramp", rng).astype(np.float32).astype(np.float64)
+    assert len(pos) > 49152
+    G0, d0 = by_input(D, box, pos, rc, types, A, lx=0.5, precision=D.DCM_PREC_FP64)
+    G1, d1 = by_input(D, box, pos, rc, types, A, lx=0.5)
+    assert np.sqrt(((G1 - G0)[:, :3] ** 2).mean()) <= 5e-6 * np.sqrt((G0[:, :3] ** 2).mean())
+    assert np.all(np.abs(d1 - d0) <= 5e-6 * np.abs(d0).max())
