@@ -439,8 +439,16 @@ TilePlan tile_plan(const dcm_params& p, const int64_t* nc, int64_t n) {
   t.cfg.nby = (int)((nc[1] + t.cfg.ry - 1) / t.cfg.ry);
   t.cfg.nbz = (int)((nc[2] + t.cfg.rz - 1) / t.cfg.rz);
   const double lx = p.lx > 0.0 ? p.lx : p.l, Lx = (double)nc[0] * lx;
-  const double cap = std::min(24.0 * p.rc_max, 0.5 * Lx - 2.0 * p.rc_max);
-  t.cfg.cap = (int)std::max(1.0, std::min(std::floor(cap / lx), 65535.0));
+  // Longest tile.  A launch of few tiles per warp (up to 16 on average) ends on its
+  // longest ones, in the vapor beside an interface along x: 260K particles, 164 x 41 x 41
+  // density boxes, 24 / 12 / 8 rc_max: 291 / 251 / 245 us.  A long launch wants them as
+  // full as they get: a step of 15.5M particles 5430 / 5487 / 5588 us.
+  auto longest = [&](double reach) {
+    const double cap = std::min(reach * p.rc_max, 0.5 * Lx - 2.0 * p.rc_max);
+    return (int)std::max(1.0, std::min(std::floor(cap / lx), 65535.0));
+  };
+  const int full = longest(24.0);
+  t.cfg.cap = p.n_max < (int64_t)32 * 16 * 152 * 16 ? longest(12.0) : full;
   int k;
   std::frexp(p.rc_max, &k);  // rc_max = f 2^k, f in [0.5, 1)
   t.cfg.scale = std::ldexp(1.0f, 3 - k);
@@ -456,8 +464,8 @@ TilePlan tile_plan(const dcm_params& p, const int64_t* nc, int64_t n) {
   const int64_t pieces = std::max<int64_t>(1, std::min(most, (152 * 8 + nb - 1) / nb));
   t.cfg.px = (int)((nc[0] + pieces - 1) / pieces);
   t.cfg.np = (int)((nc[0] + t.cfg.px - 1) / t.cfg.px);
-  auto spare = [&](int64_t cells) { return 2 + (int)((cells + t.cfg.cap - 1) / t.cfg.cap); };
-  t.cfg.cmax = spare(t.cfg.px);
+  auto spare = [&](int64_t cells, int cap) { return 2 + (int)((cells + cap - 1) / cap); };
+  t.cfg.cmax = spare(t.cfg.px, t.cfg.cap);
   t.slots = n / 32 + nb * t.cfg.np * t.cfg.cmax + 1;
   // A box of at least 4 rc_max (in a smaller one most tiles at an interface
   // reach past both ends of an axis), cells no wider than the cutoff sphere
@@ -465,7 +473,7 @@ TilePlan tile_plan(const dcm_params& p, const int64_t* nc, int64_t n) {
   // to the particles.
   const double Lmin = std::min(Lx, std::min((double)nc[1], (double)nc[2]) * p.l);
   t.usable = Lmin >= 4.0 * p.rc_max && p.l <= 2.0 * p.rc_max && lx <= 2.0 * p.rc_max &&
-             8 * nb * spare(nc[0]) <= n + 65536 && 32 * t.slots < (int64_t)1 << 31;
+             8 * nb * spare(nc[0], full) <= n + 65536 && 32 * t.slots < (int64_t)1 << 31;
   return t;
 }
 

@@ -493,3 +493,36 @@ def test_lists_and_adjoint_of_long_bundles(D):
     G1, d1 = by_input(D, box, pos, rc, types, A, lx=0.5)
     assert np.sqrt(((G1 - G0)[:, :3] ** 2).mean()) <= 5e-6 * np.sqrt((G0[:, :3] ** 2).mean())
     assert np.all(np.abs(d1 - d0) <= 5e-6 * np.abs(d0).max())
+
+
+@pytest.mark.parametrize("prec", ["mixed", "fp64"])
+@pytest.mark.parametrize("n_max", [0, 1_300_000])
+def test_long_tiles(D, n_max, prec):
+    """A thin gas in a long box: tiles end at their longest (12 rc_max, and 24 in
+    contexts of more than 1.2M particles), far from full."""
+    box = (450.0, 60.0, 60.0)
+    rng = np.random.default_rng(95)
+    n = 36000
+    pos = (rng.random((n, 3)) * np.array(box)).astype(np.float32)
+    pos = np.minimum(pos, np.nextafter(np.array(box, np.float32), np.float32(0)))
+    rc = rng.choice([3.0, 6.0], n)
+    res = []
+    real = torch.float32 if prec == "mixed" else torch.float64
+    for kernel in (D.DCM_FORCE_THREAD, D.DCM_FORCE_AUTO):
+        ctx = D.Context(D.make_params(box, n_max=max(n, n_max), lx=0.5, force_kernel=kernel,
+                                      precision=D.DCM_PREC_MIXED if prec == "mixed" else D.DCM_PREC_FP64))
+        p4 = D.to_real4(torch.from_numpy(pos), None, real)
+        i32 = dict(dtype=torch.int32, device="cuda")
+        cell, start, perm = torch.empty(n, **i32), torch.empty(ctx.ncell + 1, **i32), torch.empty(n, **i32)
+        ps = torch.empty_like(p4)
+        D.dcm_bin(ctx, n, p4, cell, start, perm, ps)
+        F, tot = torch.empty_like(ps), torch.zeros(3, dtype=torch.float64, device="cuda")
+        D.dcm_forces(ctx, n, ps, torch.from_numpy(rc).to(real).cuda()[perm.long()].contiguous(), start, F, tot)
+        assert D.dcm_status(ctx) == D.DCM_OK
+        res.append((F.double().cpu().numpy(), tot.cpu().numpy()))
+        ctx.close()
+    (F0, t0), (F1, t1) = res
+    assert t0[2] == t1[2]
+    mag = np.sqrt((F0[:, :3] ** 2).sum(1))  # overlapping particles: each against its own force
+    close = np.abs(F1 - F0)[:, :3].max(1) <= (2e-5 if prec == "mixed" else 1e-11) * np.maximum(mag, np.median(mag))
+    assert close.all()
