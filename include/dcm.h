@@ -75,11 +75,12 @@ enum dcm_status_code {
  * kernel serves FP32 runs (DCM_PREC_MIXED) of one or two types; otherwise
  * kernel 1 runs.  AUTO finds the candidates over tiles of 32 particles with a
  * tensor-core filter where that is faster: boxes of at least 4 rc_max, the
- * default accumulation, more than 32,768 particles in the mixed form (20,480
- * where the cells are no narrower than rc_min) and 4,000 in the FP64 form.  Smaller
- * systems of the mixed form take 16 lanes per particle (AUTO and PACKED; the same
- * sums bit for bit as one thread each; PACKED, and AUTO without tiles, up to 23,552
- * there).
+ * default accumulation, more than 32,768 particles in the mixed form and 4,000
+ * in the FP64 form.  Smaller systems of the mixed form take 16 lanes per
+ * particle (AUTO and PACKED; the same sums bit for bit as one thread each).  Where
+ * the cells are no narrower than rc_min these lines lie at 20,480 (23,552 without
+ * tiles), and with cells of rc_min to 1.5 rc_min a gas of fewer than 3 particles per
+ * sphere of rc_min runs no tiles in the mixed form.
  * Values 2, 4 and 5 are not used (invalid). */
 enum {
   DCM_FORCE_AUTO = 0,        /* tiles where they serve, else kernel 3 where it applies, else kernel 1 */

@@ -526,3 +526,19 @@ def test_long_tiles(D, n_max, prec):
     mag = np.sqrt((F0[:, :3] ** 2).sum(1))  # overlapping particles: each against its own force
     close = np.abs(F1 - F0)[:, :3].max(1) <= (2e-5 if prec == "mixed" else 1e-11) * np.maximum(mag, np.median(mag))
     assert close.all()
+
+
+@pytest.mark.parametrize("n,same", [(36000, True), (52000, False)])
+def test_thin_gas_in_wide_cells(D, n, same):
+    """Below 3 particles per sphere of rc_min (26.5 per 1000 sigma^3) AUTO is
+    the row walk, with its sums bit for bit; above it runs tiles."""
+    box = (120.0, 120.0, 114.0)
+    rng = np.random.default_rng(97)
+    g = np.stack(np.meshgrid(*[(np.arange(60) + 0.5) * (L / 60) for L in box], indexing="ij"), -1).reshape(-1, 3)
+    pos = (g + rng.uniform(-0.4, 0.4, g.shape))[rng.permutation(len(g))[:n]].astype(np.float32)
+    rc = np.full(n, 6.0)
+    F0, t0 = forces(D, box, pos, rc, l=3.0, h=1.5, force_kernel=D.DCM_FORCE_PACKED)
+    F1, t1 = forces(D, box, pos, rc, l=3.0, h=1.5)
+    assert t1[2] == t0[2]
+    assert np.array_equal(F1, F0) == same
+    assert np.sqrt(((F1 - F0)[:, :3] ** 2).mean()) <= MIXED_RMS * np.sqrt((F0[:, :3] ** 2).mean())
