@@ -104,25 +104,27 @@ __device__ __forceinline__ void walk_segments(const int32_t* __restrict__ start,
 // Which particle of a pair keeps it in a half list (Newton's third law form):
 // the one with the larger cutoff, the lower index on a tie, so that its walk
 // radius (its own cutoff plus the skin) covers the pair and every pair is
-// kept exactly once.  Full lists (n3 = 0) keep every candidate.
-template <typename R>
+// kept exactly once.  Full lists (N3 false) keep every candidate, and the builds of
+// the two kinds are compiled apart: a flag looked at per candidate cost the row walk 15%
+// (387K particles in a box 24 wide, one build and five force launches: 2131 -> 2007 us).
+template <typename R, bool N3>
 struct Owner {
   const R* __restrict__ rc;
   R rci, rc_max;
-  int self, n3;
+  int self;
   __device__ __forceinline__ bool keeps(int j) const {
-    if (!n3) return true;
+    if constexpr (!N3) return true;
     const R rcj = clamp_cutoff<R>(__ldg(rc + j), rc_max);
     return rci > rcj || (rci == rcj && self < j);
   }
 };
 
-template <typename R>
+template <typename R, bool N3>
 struct CountVisitor {
   const typename RT<R>::R4* __restrict__ pos;
   R rl2;
   int cnt;
-  Owner<R> own;
+  Owner<R, N3> own;
   __device__ __forceinline__ void plain(int j0, int j1, R xi, R yi, R zi) {
     for (int j = j0; j < j1; ++j) {
       auto pj = ldg4(pos + j);
@@ -182,12 +184,12 @@ struct ListColumn {
   }
 };
 
-template <typename R>
+template <typename R, bool N3>
 struct FillVisitor {
   const typename RT<R>::R4* __restrict__ pos;
   R rl2;
   ListColumn col;
-  Owner<R> own;
+  Owner<R, N3> own;
   __device__ __forceinline__ void plain(int j0, int j1, R xi, R yi, R zi) {
     int j = j0;
     if constexpr (sizeof(R) == 4) {  // two candidates per packed r^2 (the same roundings as one at a time)
@@ -229,17 +231,17 @@ __device__ __forceinline__ R list_radius(R rc, R rc_max, R skin) {
   return rc + skin;
 }
 
-template <typename R>
+template <typename R, bool N3>
 __global__ void __launch_bounds__(128) k_list_count(int64_t n, const typename RT<R>::R4* __restrict__ pos,
                                                     const R* __restrict__ rc, const int32_t* __restrict__ start,
-                                                    Grid<R> g, R rc_max, R skin, int n3,
+                                                    Grid<R> g, R rc_max, R skin,
                                                     int32_t* __restrict__ capw) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   int cnt = 0;
   if (i < n) {
     auto pi = ldg4(pos + i);
     R rl = list_radius<R>(rc[i], rc_max, skin);
-    CountVisitor<R> v{pos, rl * rl, 0, Owner<R>{rc, clamp_cutoff<R>(rc[i], rc_max), rc_max, (int)i, n3}};
+    CountVisitor<R, N3> v{pos, rl * rl, 0, Owner<R, N3>{rc, clamp_cutoff<R>(rc[i], rc_max), rc_max, (int)i}};
     walk_segments<R>(start, g, (int)i, pi, rl, v);
     cnt = v.cnt;
   }
@@ -249,16 +251,16 @@ __global__ void __launch_bounds__(128) k_list_count(int64_t n, const typename RT
 }
 
 // The list of particle i by the row walk.
-template <typename R>
+template <typename R, bool N3>
 __device__ __forceinline__ bool fill_one(int i, const typename RT<R>::R4* __restrict__ pos, const R* __restrict__ rc,
-                                         const int32_t* __restrict__ start, const Grid<R>& g, R rc_max, R skin, int n3,
+                                         const int32_t* __restrict__ start, const Grid<R>& g, R rc_max, R skin,
                                          const int32_t* __restrict__ capw, const int32_t* __restrict__ offw,
                                          uint32_t* __restrict__ list, int32_t* __restrict__ nnb,
                                          int32_t* __restrict__ nimg) {
   auto pi = ldg4(pos + i);
   R rl = list_radius<R>(rc[i], rc_max, skin);
-  FillVisitor<R> v{pos, rl * rl, ListColumn{lane_column(list, offw, i), capw[i >> 5], 0, 0, {0, 0, 0, 0}},
-                   Owner<R>{rc, clamp_cutoff<R>(rc[i], rc_max), rc_max, i, n3}};
+  FillVisitor<R, N3> v{pos, rl * rl, ListColumn{lane_column(list, offw, i), capw[i >> 5], 0, 0, {0, 0, 0, 0}},
+                   Owner<R, N3>{rc, clamp_cutoff<R>(rc[i], rc_max), rc_max, i}};
   walk_segments<R>(start, g, i, pi, rl, v);
   nnb[i] = v.col.kf;
   nimg[i] = v.col.kb;
@@ -268,17 +270,17 @@ __device__ __forceinline__ bool fill_one(int i, const typename RT<R>::R4* __rest
 // Fill lane columns of capacity capw[warp]: plain entries from the front,
 // image entries from the back.  More than capw entries raise *flag (the lists
 // are then incomplete and the caller counts exactly and fills again).
-template <typename R>
+template <typename R, bool N3>
 __global__ void __maxnreg__(80) k_list_fill(int64_t n, const typename RT<R>::R4* __restrict__ pos,
                                                    const R* __restrict__ rc, const int32_t* __restrict__ start,
-                                                   Grid<R> g, R rc_max, R skin, int n3,
+                                                   Grid<R> g, R rc_max, R skin,
                                                    const int32_t* __restrict__ capw,
                                                    const int32_t* __restrict__ offw, uint32_t* __restrict__ list,
                                                    int32_t* __restrict__ nnb, int32_t* __restrict__ nimg,
                                                    int32_t* __restrict__ flag) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  if (!fill_one<R>((int)i, pos, rc, start, g, rc_max, skin, n3, capw, offw, list, nnb, nimg)) atomicExch(flag, 1);
+  if (!fill_one<R, N3>((int)i, pos, rc, start, g, rc_max, skin, capw, offw, list, nnb, nimg)) atomicExch(flag, 1);
 }
 
 // What the tiles stage: position and index (-0 becomes +0, so that a sign bit
@@ -371,9 +373,10 @@ __global__ void __launch_bounds__(32 * kListTileWarps, 1) k_list_tiles(
 }
 
 // The tiles that the filter does not serve, by the row walk.
+template <bool N3>
 __global__ void __launch_bounds__(64) k_list_rest(const float4* __restrict__ pos, const float* __restrict__ rc,
                                                   const int32_t* __restrict__ start, Grid<float> g, TileTable t,
-                                                  float rc_max, float skin, int n3,
+                                                  float rc_max, float skin,
                                                   const int32_t* __restrict__ capw, const int32_t* __restrict__ offw,
                                                   uint32_t* __restrict__ list, int32_t* __restrict__ nnb,
                                                   int32_t* __restrict__ nimg, int32_t* __restrict__ flag) {
@@ -381,7 +384,7 @@ __global__ void __launch_bounds__(64) k_list_rest(const float4* __restrict__ pos
   for (int k = blockIdx.x * 2 + (threadIdx.x >> 5); k < n; k += gridDim.x * 2) {
     const int slot = __ldg(t.rest + k);
     const int i = __ldg(t.idx + 32 * (int64_t)slot + lane);
-    if (i >= 0 && !fill_one<float>(i, pos, rc, start, g, rc_max, skin, n3, capw, offw, list, nnb, nimg))
+    if (i >= 0 && !fill_one<float, N3>(i, pos, rc, start, g, rc_max, skin, capw, offw, list, nnb, nimg))
       atomicExch(flag, 1);
   }
 }
@@ -1009,14 +1012,15 @@ static int list_fill(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, con
       DCM_LAUNCH(ctx, k, (unsigned)std::min<int64_t>((tp.slots + kListTileWarps - 1) / kListTileWarps, sms),
                  32 * kListTileWarps, smem, st, rec, rc, ctx->cell_start, g, tp.cfg, t, tp.slots, rcm, skin, ctx->capw,
                  ctx->offw, ctx->list, ctx->nnb, ctx->nimg, ctx->lflag);
-      DCM_LAUNCH(ctx, k_list_rest, (unsigned)std::min<int64_t>((tp.slots + 1) / 2, 8 * sms), 64, 0, st, pos, rc,
-                 ctx->cell_start, g, t, rcm, skin, n3, ctx->capw, ctx->offw, ctx->list, ctx->nnb, ctx->nimg,
+      auto kr = n3 ? k_list_rest<true> : k_list_rest<false>;
+      DCM_LAUNCH(ctx, kr, (unsigned)std::min<int64_t>((tp.slots + 1) / 2, 8 * sms), 64, 0, st, pos, rc,
+                 ctx->cell_start, g, t, rcm, skin, ctx->capw, ctx->offw, ctx->list, ctx->nnb, ctx->nimg,
                  ctx->lflag);
       return DCM_OK;
     }
   }
   if (n > 0)
-    DCM_LAUNCH(ctx, k_list_fill<R>, nblk, 128, 0, st, n, pos, rc, ctx->cell_start, g, rcm, skin, n3, ctx->capw,
+    DCM_LAUNCH(ctx, (n3 ? k_list_fill<R, true> : k_list_fill<R, false>), nblk, 128, 0, st, n, pos, rc, ctx->cell_start, g, rcm, skin, ctx->capw,
                ctx->offw, ctx->list, ctx->nnb, ctx->nimg, ctx->lflag);
   DCM_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->xbuild, pos, sizeof(typename RT<R>::R4) * n, cudaMemcpyDeviceToDevice, st));
   return DCM_OK;
@@ -1043,7 +1047,7 @@ int list_build(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, const R* 
   if (ctx->host_status[3]) {
     // some list outgrew its bound: count exactly, then fill again
     if (n > 0)
-      DCM_LAUNCH(ctx, k_list_count<R>, (unsigned)nblk, 128, 0, st, n, pos, rc, ctx->cell_start, g, rcm, skin, n3,
+      DCM_LAUNCH(ctx, (n3 ? k_list_count<R, true> : k_list_count<R, false>), (unsigned)nblk, 128, 0, st, n, pos, rc, ctx->cell_start, g, rcm, skin,
                  ctx->capw);
     if ((r = exclusive_scan(ctx, ctx->capw, ctx->offw, nw, st))) return r;
     DCM_CUDA_TRY(ctx, cudaMemsetAsync(ctx->lflag, 0, sizeof(int32_t), st));

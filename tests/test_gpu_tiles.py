@@ -542,3 +542,11 @@ def test_thin_gas_in_wide_cells(D, n, same):
     assert t1[2] == t0[2]
     assert np.array_equal(F1, F0) == same
     assert np.sqrt(((F1 - F0)[:, :3] ** 2).mean()) <= MIXED_RMS * np.sqrt((F0[:, :3] ** 2).mean())
+
+
+@pytest.mark.parametrize("box", [(18.0, 21.0, 24.0), (24.0, 24.0, 120.0)])
+@pytest.mark.parametrize("typed,kw", [(False, dict()), (True, dict(newton3=1)), (False, dict(newton3=1, lx=0.5)),
+                                      (True, dict(lx=0.75))])
+def test_lists_by_the_row_walk(D, box, typed, kw):
+    """Boxes of less than 5 (rc_max + skin): full and half lists of the row walk."""
+    test_lists_over_tiles(D, box, None, 1.12, typed, kw)
