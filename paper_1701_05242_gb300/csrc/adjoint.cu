@@ -594,21 +594,21 @@ __global__ void __launch_bounds__(kAdjX2Block) k_adjoint_x2(int64_t n, const flo
 // particle, the candidates within its reverse reach, and the packed step above
 // runs on those alone (the row walk evaluates every candidate of the inner
 // window, forward and reverse, 2.1 per accepted pair, with 51% of the lanes
-// active).  Staged per candidate: position and type, upstream gradient, cutoff.
+// active).  Staged per candidate: position and type, upstream gradient, cutoff, the
+// first from the caller's positions, the others from an array of 16 bytes per particle
+// written for the launch over the binning's scratch.
 // ----------------------------------------------------------------------------
 struct __align__(32) AdjRec {
   float x, y, z, w, ax, ay, az, rc;
 };
 
-__global__ void __launch_bounds__(256) k_adj_records(int64_t n, const float4* __restrict__ pos,
-                                                     const float* __restrict__ rc, const float4* __restrict__ A,
-                                                     float rc_max, AdjRec* __restrict__ rec) {
+__global__ void __launch_bounds__(256) k_adj_records(int64_t n, const float* __restrict__ rc,
+                                                     const float4* __restrict__ A, float rc_max,
+                                                     float4* __restrict__ rec) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const float4 p = __ldg(pos + i), v = __ldg(A + i);
-  float4* q = reinterpret_cast<float4*>(rec + i);
-  q[0] = p;
-  q[1] = make_float4(v.x, v.y, v.z, clamp_cutoff<float>(__ldg(rc + i), rc_max));
+  const float4 v = __ldg(A + i);
+  rec[i] = make_float4(v.x, v.y, v.z, clamp_cutoff<float>(__ldg(rc + i), rc_max));
 }
 
 // Largest cutoff of the 27 blocks around each block.
@@ -632,9 +632,9 @@ __global__ void k_block_reach(const int32_t* __restrict__ bmax, BlockGrid bg, in
 constexpr int kAdjTileWarps = 12;
 
 __global__ void __launch_bounds__(32 * kAdjTileWarps, 1) k_adjoint_tiles(
-    const AdjRec* __restrict__ rec, const int32_t* __restrict__ start, const __grid_constant__ ForceArgs<float> a,
-    TileCfg cfg, const __grid_constant__ TileTable t, float half_dlde, BlockGrid bg, const int32_t* __restrict__ block_reach,
-    float4* __restrict__ G, double* __restrict__ part, int64_t nslot) {
+    const float4* __restrict__ pos, const float4* __restrict__ rec, const int32_t* __restrict__ start,
+    const __grid_constant__ ForceArgs<float> a, TileCfg cfg, const __grid_constant__ TileTable t, float half_dlde,
+    BlockGrid bg, const int32_t* __restrict__ block_reach, float4* __restrict__ G, double* __restrict__ part, int64_t nslot) {
   const unsigned full = 0xffffffffu;
   extern __shared__ __align__(32) unsigned char smem_raw[];
   TileSmem<AdjRec>& sm = reinterpret_cast<TileSmem<AdjRec>*>(smem_raw)[threadIdx.x >> 5];
@@ -655,8 +655,7 @@ __global__ void __launch_bounds__(32 * kAdjTileWarps, 1) k_adjoint_tiles(
     const int t1 = take();  // the next tile, asked for early
     const int i = __ldg(t.idx + 32 * (int64_t)slot + lane);
     const bool active = i >= 0;
-    const float4* self = reinterpret_cast<const float4*>(rec + max(i, 0));
-    const float4 pi = __ldg(self), ak = __ldg(self + 1);  // ak.w: the cutoff
+    const float4 pi = __ldg(pos + max(i, 0)), ak = __ldg(rec + max(i, 0));  // ak.w: the cutoff
     const float rck = ak.w, rck2 = rck * rck;
     const int b0 = block_coord(pi.x, bg.inv_be[0], bg.nb[0]), b1 = block_coord(pi.y, bg.inv_be[1], bg.nb[1]),
               b2 = block_coord(pi.z, bg.inv_be[2], bg.nb[2]);
@@ -667,7 +666,7 @@ __global__ void __launch_bounds__(32 * kAdjTileWarps, 1) k_adjoint_tiles(
     AdjAcc2 c;
     float xi[3] = {pi.x, pi.y, pi.z};
     const bool met = outside && tile_meets_outside<float>(cfg, t.outside, a.g, active, pi.y, pi.z, reach);
-    const bool done = !met && tile_candidates<float, AdjRec>(sm, rec, start, a.g, cfg, active, i, xi, rck, reach,
+    const bool done = !met && tile_candidates<float, AdjRec>(sm, HalvesSource{pos, rec}, start, a.g, cfg, active, i, xi, rck, reach,
                                                           [](const AdjRec& q) { return q.rc; }, []() {}, [&](int last) {
       ListWalk l;
       l.begin(shared_addr(&sm.list[0][lane]), last);
@@ -985,12 +984,12 @@ int lj_adjoint(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, const R* 
   static_assert(kAdjX2Block == adj_block<float>(), "the partials layout assumes equal blocks");
   if constexpr (sizeof(R) == 4) {
     if (tiled) {
-      AdjRec* rec = (AdjRec*)ctx->adj_rec;
+      float4* rec = (float4*)ctx->adj_rec;
       TileTable tt;
       int r0 = tile_cut<float>(ctx, tp, pos, rc, cell_start, a.g, tt, st);
       if (r0) return r0;
       if (part) DCM_CUDA_TRY(ctx, cudaMemsetAsync(part, 0, sizeof(double) * (size_t)(2 * nt * nt * nwarp), st));
-      DCM_LAUNCH(ctx, k_adj_records, (unsigned)((n + 255) / 256), 256, 0, st, n, pos, rc, A, a.rc_max, rec);
+      DCM_LAUNCH(ctx, k_adj_records, (unsigned)((n + 255) / 256), 256, 0, st, n, rc, A, a.rc_max, rec);
       DCM_LAUNCH(ctx, k_block_reach, (unsigned)((ctx->nblk + 127) / 128), 128, 0, st, (const int32_t*)ctx->blk_max, bg,
                  ctx->blk_max + ctx->nblk);
       const int smem = kAdjTileWarps * (int)sizeof(TileSmem<AdjRec>);
@@ -998,7 +997,7 @@ int lj_adjoint(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, const R* 
       int sms = 0;
       DCM_CUDA_TRY(ctx, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
       DCM_LAUNCH(ctx, k_adjoint_tiles, (unsigned)std::min<int64_t>((nwarp + kAdjTileWarps - 1) / kAdjTileWarps, sms),
-                 32 * kAdjTileWarps, smem, st, rec, cell_start, a, tp.cfg, tt, (float)(0.5 * dlde), bg,
+                 32 * kAdjTileWarps, smem, st, pos, (const float4*)rec, cell_start, a, tp.cfg, tt, (float)(0.5 * dlde), bg,
                  (const int32_t*)(ctx->blk_max + ctx->nblk), G, part, nwarp);
       DCM_LAUNCH(ctx, k_adjoint_rest, (unsigned)std::min<int64_t>(nwarp, 4 * sms), 32 * kAdjRestWarps, 0, st, pos, rc,
                  cell_start, a, tt, A, (float)(0.5 * dlde), G, part, nwarp, bg, (const int32_t*)ctx->blk_max);

@@ -273,6 +273,10 @@ struct ScratchPlan {
   }
   // the tiled adjoint: mixed form, systems that the warp-per-particle kernel is too slow for
   bool adj_tiles() const { return rsize == 4 && tile_cap > 0 && n_max > kAdjWarpMaxN; }
+  // the binning's slot, cell and perm, one after the other; the tiled adjoint, which
+  // bins nothing, keeps 16 bytes per particle there
+  int64_t sort_stride() const { return (n_max + 63) / 64 * 64; }
+  int64_t sort_bytes() const { return 4 * (adj_tiles() ? 4 : 3) * (sort_stride() > 0 ? sort_stride() : 64); }
   int64_t adj_doubles() const {
     const int64_t a = 32 * adj_slots(), b = adj_tiles() ? 8 * tile_cap : 0;
     return a > b ? a : b;
@@ -280,9 +284,9 @@ struct ScratchPlan {
   double skin;
   int32_t min_component, segmentation, ms_outer;
   int64_t total() const {
-    return 4 * 4 + 16 + 3 * 4 * n_max + 4 * (ncell + 1) + 4 * ncell + 8 * (scan_cap + 1) + 3 * 4 * nbox + 2 * nbox +
+    return 4 * 4 + 16 + sort_bytes() + 4 * (ncell + 1) + 4 * ncell + 8 * (scan_cap + 1) + 3 * 4 * nbox + 2 * nbox +
            2 * rsize * nbox + 4 * flags + 4 * (int64_t)kHistCap + 4 * 8 + 8 * 3 * red_slots() + 8 * 8 + 8 * 8 * 256 +
-           8 * adj_doubles() + (adj_tiles() ? 32 * n_max : 0) + 8 * 48 + (skin > 0 ? 8 * n_max + 8 * (n_max / 32 + 16) + 4 * rsize * n_max + 32 : 0) +
+           8 * adj_doubles() + 8 * 48 + (skin > 0 ? 8 * n_max + 8 * (n_max / 32 + 16) + 4 * rsize * n_max + 32 : 0) +
            (min_component > 0 ? 9 * nbox + 4 * 80 : 0) + 13 * nbox + 4 * (flags + 2) + 8 * nblk +
            4 * tile_scratch_ints(n_max) + (tile_cap > 0 ? 4 * tile_ints(tile_cap) : 0) +
            (segmentation ? 10 * rsize * nbox + 32 * ms_outer + 16 + 4 * (ms_outer + 2) : 0);
@@ -333,12 +337,12 @@ extern "C" const char* dcm_version(void) { return "dcm-gb300 0.1 (sm_103a)"; }
 // ---------------------------------------------------------------------------
 extern "C" void dcm_destroy(dcm_ctx* ctx) {
   if (!ctx) return;
-  void* dev[] = {ctx->status, ctx->coop_sync, ctx->slot,  ctx->cell,  ctx->perm,  ctx->cell_start, ctx->cell_count,
+  void* dev[] = {ctx->status, ctx->coop_sync, ctx->slot, ctx->cell_start, ctx->cell_count,
                  ctx->scan_state, ctx->box_count, ctx->g, ctx->g_tmp, ctx->s, ctx->iface,
                  ctx->D[1], ctx->flags, ctx->hist, ctx->thr, ctx->red, ctx->totals, ctx->D[0], ctx->red_tmp, ctx->adj_part, ctx->adj_pairs,
                  ctx->nnb, ctx->nimg, ctx->capw, ctx->offw, ctx->list, ctx->xbuild, ctx->dmax, ctx->lflag,
                  ctx->cc_lab, ctx->cc_cnt, ctx->cc_flags, ctx->cc_s0, ctx->dq[0], ctx->dq[1], ctx->dqlen,
-                 ctx->dstamp, ctx->dfixed, ctx->blk_max, ctx->tile_scratch, ctx->tiles, ctx->adj_rec, ctx->ms_u, ctx->ms_ub, ctx->ms_p, ctx->ms_w,
+                 ctx->dstamp, ctx->dfixed, ctx->blk_max, ctx->tile_scratch, ctx->tiles, ctx->ms_u, ctx->ms_ub, ctx->ms_p, ctx->ms_w,
                  ctx->ms_sums, ctx->ms_c, ctx->ms_flags};
   for (void* q : dev)
     if (q) cudaFree(q);
@@ -382,9 +386,12 @@ extern "C" int dcm_create(const dcm_params* p, dcm_ctx** out) {
   };
   alloc((void**)&ctx->status, 16);
   alloc((void**)&ctx->coop_sync, 16);
-  alloc((void**)&ctx->slot, 4 * nm);
-  alloc((void**)&ctx->cell, 4 * nm);
-  alloc((void**)&ctx->perm, 4 * nm);
+  alloc((void**)&ctx->slot, s.sort_bytes());
+  if (ok) {
+    ctx->cell = ctx->slot + s.sort_stride();
+    ctx->perm = ctx->cell + s.sort_stride();
+    if (s.adj_tiles()) ctx->adj_rec = ctx->slot;
+  }
   alloc((void**)&ctx->cell_start, 4 * (s.ncell + 1));
   alloc((void**)&ctx->cell_count, 4 * s.ncell);
   alloc((void**)&ctx->scan_state, 8 * (s.scan_cap + 1));
@@ -404,7 +411,6 @@ extern "C" int dcm_create(const dcm_params* p, dcm_ctx** out) {
   alloc((void**)&ctx->adj_part, 8 * s.adj_doubles());
   ctx->adj_cap = s.adj_slots();
   ctx->adj_doubles = s.adj_doubles();
-  if (s.adj_tiles()) alloc(&ctx->adj_rec, 32 * nm);
   if (p->skin > 0.0) {
     alloc((void**)&ctx->nnb, 4 * nm);
     alloc((void**)&ctx->nimg, 4 * nm);

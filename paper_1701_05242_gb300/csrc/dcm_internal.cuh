@@ -94,7 +94,7 @@ struct dcm_ctx {
   int32_t* status;          // [4]: first device-side error code, ...
   uint32_t* coop_sync;      // [4]: grid-barrier words of the cooperative distance sweeps
   int64_t wait_budget;      // nanoseconds a block waits at one of those barriers before DCM_ERR_TIMEOUT
-  int32_t* slot;            // n_max: rank of a particle inside its cell (atomics)
+  int32_t* slot;            // n_max: rank of a particle inside its cell (atomics); cell and perm follow in the same allocation
   int32_t* cell;            // n_max: cell of each particle (step)
   int32_t* perm;            // n_max
   int32_t* cell_start;      // ncell + 1
@@ -114,7 +114,8 @@ struct dcm_ctx {
   double* adj_part;         // [32][adj_cap] adjoint parameter-gradient partials
   int64_t adj_cap;          // partial slots per quantity
   int64_t adj_doubles;      // doubles in adj_part
-  void* adj_rec;            // n_max x 32 bytes: what the tiled adjoint stages per particle (or null: not served)
+  void* adj_rec;            // n_max x 16 bytes over slot, cell and perm: what the tiled adjoint stages per particle
+                            // beside its position (or null: not served)
   double* adj_pairs;        // [48]: per-pair eps sums, per-pair sigma sums
   double* totals;           // [4]
   int32_t* host_status;     // pinned host mirror

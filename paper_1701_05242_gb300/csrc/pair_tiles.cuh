@@ -106,8 +106,9 @@ __device__ __forceinline__ uint32_t shared_addr(const void* p) { return (uint32_
 
 // Copy element `at` (of BYTES bytes, counted from dst and src) to shared memory
 // if at < n: predicated, with the element's offset in the instruction.
-template <int BYTES, int AT>
-__device__ __forceinline__ void copy_if(uint32_t dst, const void* src, int n) {
+template <int AT, typename E>
+__device__ __forceinline__ void copy_if(uint32_t dst, const E* src, int n) {
+  constexpr int BYTES = sizeof(E);
   if constexpr (BYTES == 16)
     asm volatile("{\n\t.reg .pred p;\n\tsetp.gt.s32 p, %2, %3;\n\t@p cp.async.cg.shared.global [%0 + %4], [%1 + %4], 16;\n\t}"
                  ::"r"(dst), "l"(src), "r"(n), "n"(AT), "n"(BYTES * AT)
@@ -117,6 +118,18 @@ __device__ __forceinline__ void copy_if(uint32_t dst, const void* src, int n) {
                  "@p cp.async.cg.shared.global [%0 + %5], [%1 + %5], 16;\n\t}"
                  ::"r"(dst), "l"(src), "r"(n), "n"(AT), "n"(BYTES * AT), "n"(BYTES * AT + 16)
                  : "memory");
+}
+// The same for elements whose two halves come from two arrays.
+struct HalvesSource {
+  const float4 *first, *second;
+  __device__ __forceinline__ HalvesSource operator+(int k) const { return {first + k, second + k}; }
+};
+template <int AT>
+__device__ __forceinline__ void copy_if(uint32_t dst, const HalvesSource& src, int n) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.gt.s32 p, %3, %4;\n\t@p cp.async.cg.shared.global [%0 + %5], [%1 + %7], 16;\n\t"
+               "@p cp.async.cg.shared.global [%0 + %6], [%2 + %7], 16;\n\t}"
+               ::"r"(dst), "l"(src.first), "l"(src.second), "r"(n), "n"(AT), "n"(32 * AT), "n"(32 * AT + 16), "n"(16 * AT)
+               : "memory");
 }
 __device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
@@ -297,6 +310,7 @@ static __device__ __noinline__ bool tile_meets_outside(const TileCfg& cfg, const
 // (after possibly some chunks) if the tile cannot be evaluated this way; the
 // caller then discards what it summed.
 //
+//   pos    where the elements come from: const E*, or HalvesSource
 //   i      the lane's particle (ignored where !active), xi its position (out:
 //          in the tile's frame), ri its cutoff (clamped)
 //   ahead  called once, when the tile's own loads are done with
@@ -304,8 +318,8 @@ static __device__ __noinline__ bool tile_meets_outside(const TileCfg& cfg, const
 //          own_cutoff(candidate) gives the candidates a cutoff of their own, which
 //          then counts too (NoCutoff: it does not)
 struct NoCutoff {};
-template <typename R, typename E, typename Own, typename A, typename F>
-__device__ __forceinline__ bool tile_candidates(TileSmem<E>& sm, const E* __restrict__ pos,
+template <typename R, typename E, typename Src, typename Own, typename A, typename F>
+__device__ __forceinline__ bool tile_candidates(TileSmem<E>& sm, const Src pos,
                                                 const int32_t* __restrict__ start, const Grid<R>& g,
                                                 const TileCfg& cfg, bool active, int i, R (&xi)[3], float ri,
                                                 float reach, Own own_cutoff, A&& ahead, F&& consume) {
@@ -455,12 +469,12 @@ __device__ __forceinline__ bool tile_candidates(TileSmem<E>& sm, const E* __rest
         const int src = r + (lane >> 3);
         const int nn = __shfl_sync(full, len, src) - sub, jj = __shfl_sync(full, from, src) + sub;
         const uint32_t dst = pos_s + (uint32_t)((__shfl_sync(full, to, src) + sub) * (int)sizeof(E));
-        const E* p = pos + jj;
-        copy_if<sizeof(E), 0>(dst, p, nn);
-        copy_if<sizeof(E), 8>(dst, p, nn);
-        copy_if<sizeof(E), 16>(dst, p, nn);
+        const Src p = pos + jj;
+        copy_if<0>(dst, p, nn);
+        copy_if<8>(dst, p, nn);
+        copy_if<16>(dst, p, nn);
         if (most > 24)
-          for (int q = 24; q < most; q += 8) copy_if<sizeof(E), 0>(dst + (uint32_t)(q * sizeof(E)), p + q, nn - q);
+          for (int q = 24; q < most; q += 8) copy_if<0>(dst + (uint32_t)(q * sizeof(E)), p + q, nn - q);
       }
       if (images) {  // shift the image rows in place
         copy_async_wait();

@@ -105,6 +105,19 @@ def test_grid_dims_and_scratch(lib):
     assert b"sm_103a" in D.lib.dcm_version()
 
 
+def test_scratch_per_particle(lib):
+    """Mixed form: 12 bytes of binning scratch and 4 more under the adjoint's
+    records, 8 of adjoint partials, 4.4 of tile table, about 1 of force partials and
+    launch order; stepping alone never needs records of its own for the adjoint."""
+    sizes = []
+    for n in (8_000_000, 16_000_000):
+        D, p = _params(lib, box=(240.0, 240.0, 960.0), n_max=n, lx=0.5)
+        b = ctypes.c_int64()
+        assert D.lib.dcm_scratch_bytes(ctypes.byref(p), ctypes.byref(b)) == 0
+        sizes.append(b.value)
+    assert (sizes[1] - sizes[0]) / 8e6 <= 32
+
+
 def test_tensors_must_be_on_device(lib):
     import torch
     D, _ = _params(lib)

@@ -550,3 +550,41 @@ def test_thin_gas_in_wide_cells(D, n, same):
 def test_lists_by_the_row_walk(D, box, typed, kw):
     """Boxes of less than 5 (rc_max + skin): full and half lists of the row walk."""
     test_lists_over_tiles(D, box, None, 1.12, typed, kw)
+
+
+@pytest.mark.parametrize("skin", [0.0, 0.5])
+def test_adjoint_between_steps(D, skin):
+    """The tiled adjoint keeps its records in the binning's scratch: steps
+    around it give what they give without it, and it gives the same twice."""
+    box = (63.0, 61.5, 72.0)
+    pos = lattice(box, 98)
+    n = len(pos)
+    assert n > 49152
+    rng = np.random.default_rng(99)
+    vel = torch.from_numpy(rng.normal(size=(n, 4)).astype(np.float32))
+    vel[:, 3] = 0
+    A = torch.from_numpy(rng.normal(size=(n, 4)).astype(np.float32)).cuda()
+    i32 = dict(dtype=torch.int32, device="cuda")
+    res, grads = [], []
+    for adjoint in (False, True):
+        ctx = D.Context(D.make_params(box, n_max=n, skin=skin, recompute_every=3))
+        st = D.State(ctx, D.to_real4(torch.from_numpy(pos)), vel)
+        D.dcm_step_init(ctx, st)
+        p4 = D.to_real4(torch.from_numpy(pos))
+        cell, start, perm = torch.empty(n, **i32), torch.empty(ctx.ncell + 1, **i32), torch.empty(n, **i32)
+        ps = torch.empty_like(p4)
+        D.dcm_bin(ctx, n, p4, cell, start, perm, ps)
+        rc = torch.full((n,), 3.5, device="cuda")
+        for k in range(4):
+            if adjoint:
+                G, d = torch.empty_like(ps), torch.empty(2, dtype=torch.float64, device="cuda")
+                D.dcm_forces_backward(ctx, n, ps, rc, start, A, 0.7, G, d)
+                grads.append((G.cpu(), d.cpu()))
+            D.dcm_step(ctx, st, 0.002, 2)
+        assert D.dcm_status(ctx) == D.DCM_OK
+        res.append([t.cpu() for t in st.current()] + [st.force.cpu()])
+        ctx.close()
+    for a, b in zip(*res):
+        assert torch.equal(a, b)
+    for G, d in grads[1:]:
+        assert torch.equal(G, grads[0][0]) and torch.allclose(d, grads[0][1], rtol=1e-12, atol=0)
