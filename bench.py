@@ -597,9 +597,7 @@ def run_gb300(args):
     instr_pp = (FLOP_PER_PAIR * n_ew + FLOP_PER_PAIR_FORCES * (f_cnt - n_ew)) / max(f_cnt, 1)
     achieved = pairs * instr_pp / f_avg_s / 1e12 if f_avg_s > 0 else None
     acc_name = D.ACC_NAMES[D.dcm_accumulation(ctx)]
-    fkern = "k_forces_list" if args.skin > 0 else D.FORCE_KERNEL_NAMES[D.dcm_force_kernel(ctx)]
-    if fkern == "k_forces_x2" and args.force_kernel == D.DCM_FORCE_AUTO and acc_name == "plane_kahan":
-        fkern = "k_forces_tiles"  # the same pair arithmetic over tiles
+    fkern = "k_forces_list" if args.skin > 0 else D.force_kernel_name(ctx, n)
     cells = (args.cell_edge, args.cell_edge_x if args.cell_edge_x > 0 else args.cell_edge)
     roof = {"bound": "alu", "kernel": fkern, "achieved": achieved, "peak": peak_tinstr,
             "unit": "T FP32-instr/s", "frac": (achieved / peak_tinstr) if achieved else None,

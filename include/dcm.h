@@ -88,6 +88,9 @@ enum {
   DCM_FORCE_PACKED = 3       /* two candidates per FP32x2 instruction; one thread per particle i, in small systems 16 */
 };
 
+/* How a force launch finds its candidates (dcm_force_search). */
+enum { DCM_SEARCH_ROWS = 0, DCM_SEARCH_LANES = 1, DCM_SEARCH_TILES = 2 };
+
 /* Per-particle accumulation of the mixed precision form (dcm_params.
  * accumulation): how the FP32 pair terms of particle i (its force, energy and
  * virial) are summed.  Totals E and W are always reduced in FP64.  A "row
@@ -531,6 +534,12 @@ int dcm_launch_count(dcm_ctx* ctx, int64_t* count, int32_t reset);
  * the cell lists for this context's parameters (params.force_kernel with AUTO
  * and the kernels' limits resolved; the same over tiles), written to *kernel.  Host only. */
 int dcm_force_kernel(const dcm_ctx* ctx, int32_t* kernel);
+
+/* How dcm_forces and dcm_step find the candidates of n particles on the cell
+ * lists: cell rows by one thread per particle (DCM_SEARCH_ROWS), by 16 lanes per
+ * particle (DCM_SEARCH_LANES), or tiles of 32 particles (DCM_SEARCH_TILES), written
+ * to *search.  Host only. */
+int dcm_force_search(const dcm_ctx* ctx, int64_t n, int32_t* search);
 
 /* The DCM_ACC_* form in which this context's force launches sum each
  * particle's pair terms (params.accumulation with AUTO and the kernels'

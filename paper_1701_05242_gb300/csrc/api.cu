@@ -669,6 +669,12 @@ extern "C" int dcm_force_kernel(const dcm_ctx* ctx, int32_t* kernel) {
   return DCM_OK;
 }
 
+extern "C" int dcm_force_search(const dcm_ctx* ctx, int64_t n, int32_t* search) {
+  if (!ctx || !search || n < 0) return DCM_ERR_INVALID_ARG;
+  *search = force_search(ctx, n);
+  return DCM_OK;
+}
+
 extern "C" int dcm_accumulation(const dcm_ctx* ctx, int32_t* form) {
   if (!ctx || !form) return DCM_ERR_INVALID_ARG;
   *form = resolve_accumulation(ctx);

@@ -319,7 +319,8 @@ inline TilePlan list_tile_plan(dcm_params p, const int64_t* nc, int64_t n) {
 }
 constexpr int64_t kListTilesMinN = 4000;  // below: the row walk, as the forces (kTilesMinN)
 constexpr int64_t tile_ints(int64_t slots) { return 8 + 35 * slots; }
-bool tiles_serve(const dcm_ctx* ctx, int64_t n);  // whether lj_forces runs over tiles
+bool tiles_serve(const dcm_ctx* ctx, int64_t n);  // whether AUTO may run n particles over tiles
+int force_search(const dcm_ctx* ctx, int64_t n);   // how lj_forces finds the candidates (DCM_SEARCH_*)
 template <typename R>
 struct ForceArgs;
 // Forces (and with part, 3 quantities of tile_plan(...).slots partials) over tiles.

@@ -148,6 +148,18 @@ int resolve_accumulation(const dcm_ctx* ctx) {
   return m;
 }
 
+// How a force launch of n particles finds its candidates: 16 lanes per
+// particle and tiles serve the default accumulation of the packed pair loop (the
+// tiles' sums carried by the same Kahan compensation), tiles also the FP64 form.
+int force_search(const dcm_ctx* ctx, int64_t n) {
+  const bool kahan =
+      resolve_force_kernel(ctx) == DCM_FORCE_PACKED && resolve_accumulation(ctx) == DCM_ACC_PLANE_KAHAN;
+  const bool fp64 = ctx->p.precision == DCM_PREC_FP64;
+  const bool tiles = ctx->p.force_kernel == DCM_FORCE_AUTO && (fp64 || kahan) && tiles_serve(ctx, n);
+  if (kahan && n <= planes_max_n(ctx->p, tiles)) return DCM_SEARCH_LANES;
+  return tiles ? DCM_SEARCH_TILES : DCM_SEARCH_ROWS;
+}
+
 namespace {
 
 // Cost key of the packed kernel's tiles (tile_order.cuh): the largest cutoff
@@ -224,12 +236,9 @@ int lj_forces(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, const R* r
   a.rc_max = (R)ctx->p.rc_max;
   const bool typed = lj_general(t);
   const int kind = resolve_force_kernel(ctx);
-  // the default accumulation of the packed pair loop; AUTO runs over tiles where
-  // they serve (their sums carried by the same Kahan compensation), or FP64
-  const bool kahan = kind == DCM_FORCE_PACKED && resolve_accumulation(ctx) == DCM_ACC_PLANE_KAHAN;
-  const bool tiles = ctx->p.force_kernel == DCM_FORCE_AUTO && (sizeof(R) == 8 || kahan) && tiles_serve(ctx, n);
+  const int search = force_search(ctx, n);
   if constexpr (sizeof(R) == 4) {
-    if (kahan && n <= planes_max_n(ctx->p, tiles)) {
+    if (search == DCM_SEARCH_LANES) {
       const bool ew = energies || totals;
       double* part = totals ? ctx->red : nullptr;
       const int64_t nblk = plane_slots(n);
@@ -244,7 +253,7 @@ int lj_forces(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, const R* r
       return DCM_OK;
     }
   }
-  if (tiles) {
+  if (search == DCM_SEARCH_TILES) {
     double* part = totals ? ctx->red : nullptr;
     stage_begin(ctx, DCM_STAGE_FORCES, st);
     int r = tile_forces<R>(ctx, typed, energies || totals, n, pos, rc, cell_start, a, force, part, st);

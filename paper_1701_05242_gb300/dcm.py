@@ -32,6 +32,7 @@ DCM_PREC_MIXED = 1
 DCM_FORCE_AUTO = 0
 DCM_FORCE_THREAD = 1
 DCM_FORCE_PACKED = 3
+DCM_SEARCH_ROWS, DCM_SEARCH_LANES, DCM_SEARCH_TILES = 0, 1, 2
 DCM_ACC_AUTO = 0
 DCM_ACC_FP32 = 1
 DCM_ACC_ROW_FP64 = 2
@@ -123,6 +124,7 @@ _SIGS = {
     "dcm_stage_times": (_i32, [_vp, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(_i64)]),
     "dcm_launch_count": (_i32, [_vp, ctypes.POINTER(_i64), _i32]),
     "dcm_force_kernel": (_i32, [_vp, ctypes.POINTER(ctypes.c_int32)]),
+    "dcm_force_search": (_i32, [_vp, _i64, ctypes.POINTER(ctypes.c_int32)]),
     "dcm_accumulation": (_i32, [_vp, ctypes.POINTER(ctypes.c_int32)]),
 }
 
@@ -355,6 +357,12 @@ def dcm_force_kernel(ctx: Context) -> int:
     return k.value
 
 
+def dcm_force_search(ctx: Context, n: int) -> int:
+    k = ctypes.c_int32()
+    ctx.check(lib.dcm_force_search(ctx.handle, int(n), ctypes.byref(k)))
+    return k.value
+
+
 def dcm_accumulation(ctx: Context) -> int:
     k = ctypes.c_int32()
     ctx.check(lib.dcm_accumulation(ctx.handle, ctypes.byref(k)))
@@ -362,6 +370,14 @@ def dcm_accumulation(ctx: Context) -> int:
 
 
 FORCE_KERNEL_NAMES = {DCM_FORCE_THREAD: "k_forces", DCM_FORCE_PACKED: "k_forces_x2"}
+
+
+def force_kernel_name(ctx: Context, n: int) -> str:
+    """The kernel that dcm_forces and dcm_step launch on n particles' cell lists."""
+    search = dcm_force_search(ctx, n)
+    if search == DCM_SEARCH_ROWS:
+        return FORCE_KERNEL_NAMES[dcm_force_kernel(ctx)]
+    return "k_forces_tiles" if search == DCM_SEARCH_TILES else "k_forces_planes"
 
 
 # ---------------------------------------------------------------- batched form

@@ -588,3 +588,25 @@ def test_adjoint_between_steps(D, skin):
         assert torch.equal(a, b)
     for G, d in grads[1:]:
         assert torch.equal(G, grads[0][0]) and torch.allclose(d, grads[0][1], rtol=1e-12, atol=0)
+
+
+@pytest.mark.parametrize("n,box,kw,name", [
+    (2000, (12.0, 12.0, 48.0), dict(), "k_forces_planes"),
+    (32768, (61.5, 61.5, 61.5), dict(), "k_forces_planes"),
+    (32769, (61.5, 61.5, 61.5), dict(), "k_forces_tiles"),
+    (32769, (22.5, 61.5, 61.5), dict(), "k_forces_x2"),              # narrower than 4 rc_max
+    (32769, (61.5, 61.5, 61.5), dict(force_kernel=3), "k_forces_x2"),
+    (32769, (61.5, 61.5, 61.5), dict(accumulation=1), "k_forces_x2"),
+    (2000, (12.0, 12.0, 48.0), dict(force_kernel=1), "k_forces"),
+    (32769, (61.5, 61.5, 61.5), dict(ntypes=3, eps=(1, 1, 1), sigma=(1, 1, 1)), "k_forces"),
+    (20480, (60.0, 60.0, 60.0), dict(l=3.0, h=1.5), "k_forces_planes"),
+    (20481, (60.0, 60.0, 60.0), dict(l=3.0, h=1.5), "k_forces_tiles"),
+    (23553, (60.0, 60.0, 60.0), dict(l=3.0, h=1.5, force_kernel=3), "k_forces_x2"),
+    (3999, (24.0, 24.0, 48.0), dict(precision=0), "k_forces"),
+    (4000, (24.0, 24.0, 48.0), dict(precision=0), "k_forces_tiles"),
+])
+def test_force_search(D, n, box, kw, name):
+    """Which kernel a force launch of n particles runs."""
+    ctx = D.Context(D.make_params(box, n_max=40000, **kw))
+    assert D.force_kernel_name(ctx, n) == name
+    ctx.close()
