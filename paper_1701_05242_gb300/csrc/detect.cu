@@ -296,7 +296,7 @@ int detect_interface(dcm_ctx* ctx, const int32_t* box_count, uint8_t* s, uint8_t
   const int64_t cols = (int64_t)((nx + 31) / 32) * ((ny + 7) / 8);
   const int zc = (int)std::max<int64_t>(8, std::min<int64_t>(64, (int64_t)nz * cols / (152 * 8)));
   const dim3 grid((nx + 31) / 32, (ny + 7) / 8, (nz + zc - 1) / zc);
-  if (w <= 4 && grid.y <= 65535 && grid.z <= 65535) {
+  if (w <= 4) {
     auto k = w == 0 ? k_box_sum3<0> : w == 1 ? k_box_sum3<1> : w == 2 ? k_box_sum3<2> : w == 3 ? k_box_sum3<3> : k_box_sum3<4>;
     DCM_LAUNCH(ctx, k, grid, 256, 0, st, box_count, g, nx, ny, nz, zc, thr);
   } else {

@@ -90,27 +90,20 @@ __device__ __forceinline__ void dist_push(bool push, int b, int x, int y, int z,
   }
 }
 
-// Loads of the iterates: COH through L2 (__ldcg), for the cooperative sweep
-// kernel, whose blocks read what other blocks wrote earlier in the same
-// launch (behind a grid barrier); ordinary loads otherwise.
-template <typename R, bool COH>
-__device__ __forceinline__ R dld(const R* p) {
-  if constexpr (COH) return __ldcg(p);
-  else return *p;
-}
-
-// Update of one box from the previous iterate; true if it changed.
-template <typename R, bool COH = false>
+// Update of one box from the previous iterate; true if it changed.  The
+// iterates are read through L2 (__ldcg): other blocks wrote them earlier in the same
+// launch, behind a grid barrier.
+template <typename R>
 __device__ __forceinline__ bool dist_update(const R* Din, R* Dout, int64_t b, int x, int y, int z, int nx, int ny,
                                             int nz, R h, R r_grid) {
-  R cur = dld<R, COH>(Din + b);
+  R cur = __ldcg(Din + b);
   int xm = x == 0 ? nx - 1 : x - 1, xp = x == nx - 1 ? 0 : x + 1;
   int ym = y == 0 ? ny - 1 : y - 1, yp = y == ny - 1 ? 0 : y + 1;
   int zm = z == 0 ? nz - 1 : z - 1, zp = z == nz - 1 ? 0 : z + 1;
   int64_t row = (int64_t)nx * (y + (int64_t)ny * z);
-  R a0 = fmin(dld<R, COH>(Din + row + xm), dld<R, COH>(Din + row + xp));
-  R a1 = fmin(dld<R, COH>(Din + x + nx * (ym + (int64_t)ny * z)), dld<R, COH>(Din + x + nx * (yp + (int64_t)ny * z)));
-  R a2 = fmin(dld<R, COH>(Din + x + nx * (y + (int64_t)ny * zm)), dld<R, COH>(Din + x + nx * (y + (int64_t)ny * zp)));
+  R a0 = fmin(__ldcg(Din + row + xm), __ldcg(Din + row + xp));
+  R a1 = fmin(__ldcg(Din + x + nx * (ym + (int64_t)ny * z)), __ldcg(Din + x + nx * (yp + (int64_t)ny * z)));
+  R a2 = fmin(__ldcg(Din + x + nx * (y + (int64_t)ny * zm)), __ldcg(Din + x + nx * (y + (int64_t)ny * zp)));
   R d = godunov3<R>(a0, a1, a2, h);
   bool ch = d < cur && d <= r_grid;
   Dout[b] = ch ? d : cur;
@@ -258,7 +251,7 @@ __global__ void __launch_bounds__(kCoopBlock) k_dist_coop(R* D0, R* D1, int nx, 
         x = b - yz * nx;
         z = yz / ny;
         y = yz - z * ny;
-        changed = dist_update<R, true>(Din, Dout, b, x, y, z, nx, ny, nz, h, r_grid);
+        changed = dist_update<R>(Din, Dout, b, x, y, z, nx, ny, nz, h, r_grid);
       }
       any |= changed;
       dist_push(changed, b, x, y, z, nx, ny, nz, fixed0, stamp, qout, qlen, it);
@@ -308,8 +301,6 @@ int distance_sweeps(dcm_ctx* ctx, const uint8_t* s, const uint8_t* iface, R* D, 
   DCM_CUDA_TRY(ctx, cudaMemsetAsync(ctx->dstamp, 0xff, sizeof(int32_t) * (size_t)nbox, st));
   const int64_t cols = (int64_t)((nx + 31) / 32) * ((ny + 7) / 8);
   const int zc = (int)std::max<int64_t>(1, std::min<int64_t>(64, (int64_t)nz * cols / (152 * 8)));
-  if ((ny + 7) / 8 > 65535 || (nz + zc - 1) / zc > 65535)
-    return set_error(ctx, DCM_ERR_CAPACITY, "distance sweeps: density grid too long");
   bool four = false;
   if constexpr (sizeof(R) == 4) {
     four = nx % 4 == 0 && (((uintptr_t)s | (uintptr_t)iface) & 3) == 0 && ((uintptr_t)D & 15) == 0;
