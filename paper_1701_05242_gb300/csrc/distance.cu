@@ -233,7 +233,11 @@ __global__ void __launch_bounds__(kCoopBlock) k_dist_coop(R* D0, R* D1, int nx, 
                                                    uint32_t* sync, int64_t budget_ns, int32_t* status) {
   const unsigned full = 0xffffffffu;
   const uint32_t expected = gridDim.x;
-  const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, gs = (int64_t)gridDim.x * blockDim.x;
+  // neighbouring warps of the queue on different SMs: a sweep's queue fills a part
+  // of the launch only, and the FP64 form needs every SM's units (64^3 boxes, 17
+  // sweeps of two flat interfaces: 262 us with whole blocks in turn)
+  const int64_t gt = ((int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31),
+                gs = (int64_t)gridDim.x * blockDim.x;
   for (int it = 1; it < budget; ++it) {
     if (((volatile int32_t*)flags)[it - 1] == 0) break;  // the previous sweep changed nothing
     const R* Din = (it & 1) ? D1 : D0;
