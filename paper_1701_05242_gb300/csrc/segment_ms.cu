@@ -105,16 +105,36 @@ __global__ void k_ms_start(const int32_t* __restrict__ g, const uint8_t* __restr
 // half the launches, which is what counts for grids that stay in L2: 1.05M
 // boxes, 800 iterations, 11.7 -> 5.95 ms (7.4 us per iteration, of which the
 // launch and the drain of one wave of blocks are most).
+//
+// The FP64 form is bound by the FP64 units: its blocks take 64 columns in a row,
+// whatever the shape (blocks of 32 x 8 left 36% to 71% of their lanes idle in planes of
+// 41 x 41, 33 x 9 and 16 x 16 boxes), and above kMsFused boxes the duals are not formed
+// twice: two kernels, 17 FP64 operations per box instead of 26.  800 iterations, FP64,
+// 32 x 8 / 64 in a row / two kernels: 41 x 41 x 164 boxes 22.3 / 13.2 / 14.1 ms, 1.05M
+// 37.1 / 37.1 / 30.6, 4.1M 131 / 131 / 101.
+constexpr int64_t kMsFused = 600000;
 template <typename R>
-__global__ void __launch_bounds__(256) k_ms_step(const R* __restrict__ ub, const R* __restrict__ p,
+constexpr int ms_block() { return sizeof(R) == 8 ? 64 : 256; }
+
+template <typename R>
+__global__ void __launch_bounds__(ms_block<R>()) k_ms_step(const R* __restrict__ ub, const R* __restrict__ p,
                                                  const R* __restrict__ w, R* __restrict__ u, R* __restrict__ ub1,
                                                  R* __restrict__ p1, int nx, int ny, int nz, int zc, R sigma, R tau,
                                                  R nu, const int32_t* flags, int o) {
   if (!ms_active(flags, o)) return;
-  const int x = blockIdx.x * 32 + (threadIdx.x & 31), y = blockIdx.y * 8 + (threadIdx.x >> 5);
+  const int nxy = nx * ny;  // fewer than 2^31 boxes
+  int x, y;
+  if constexpr (sizeof(R) == 8) {
+    const int c = blockIdx.x * ms_block<R>() + threadIdx.x;
+    y = c / nx;
+    x = c - nx * y;
+  } else {
+    x = blockIdx.x * 32 + (threadIdx.x & 31);
+    y = blockIdx.y * 8 + (threadIdx.x >> 5);
+  }
   if (x >= nx || y >= ny) return;
   const int z0 = blockIdx.z * zc, z1 = min(z0 + zc, nz);
-  const int nxy = nx * ny, col = x + nx * y;  // fewer than 2^31 boxes
+  const int col = x + nx * y;
   const int64_t nbox = (int64_t)nxy * nz;
   const R *px = p, *py = p + nbox, *pz = p + 2 * nbox;
   R *qx = p1, *qy = p1 + nbox, *qz = p1 + 2 * nbox;
@@ -153,6 +173,46 @@ __global__ void __launch_bounds__(256) k_ms_step(const R* __restrict__ ub, const
   }
 }
 
+// The two steps of an iteration apart, in place (p: px, py, pz).
+template <typename R>
+__global__ void __launch_bounds__(256) k_ms_dual(const R* __restrict__ ub, R* __restrict__ p, int nx, int ny, int nz,
+                                                 R sigma, R nu, const int32_t* flags, int o) {
+  if (!ms_active(flags, o)) return;
+  const int64_t nxy = (int64_t)nx * ny, nbox = nxy * nz;
+  for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < nbox; b += (int64_t)gridDim.x * blockDim.x) {
+    const int x = (int)(b % nx), y = (int)((b / nx) % ny), z = (int)(b / nxy);
+    const int64_t ahead[3] = {x == nx - 1 ? b - x : b + 1, y == ny - 1 ? b - (int64_t)y * nx : b + nx,
+                              z == nz - 1 ? b - z * nxy : b + nxy};
+    const R here = ub[b];
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+      const R q = r_add(p[e * nbox + b], r_mul(sigma, r_sub(ub[ahead[e]], here)));
+      p[e * nbox + b] = q < -nu ? -nu : (q > nu ? nu : q);
+    }
+  }
+}
+
+template <typename R>
+__global__ void __launch_bounds__(256) k_ms_primal(const R* __restrict__ p, const R* __restrict__ w, R* __restrict__ u,
+                                                   R* __restrict__ ub, int nx, int ny, int nz, R tau,
+                                                   const int32_t* flags, int o) {
+  if (!ms_active(flags, o)) return;
+  const int64_t nxy = (int64_t)nx * ny, nbox = nxy * nz;
+  for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < nbox; b += (int64_t)gridDim.x * blockDim.x) {
+    const int x = (int)(b % nx), y = (int)((b / nx) % ny), z = (int)(b / nxy);
+    const int64_t behind[3] = {x == 0 ? b + nx - 1 : b - 1, y == 0 ? b + (int64_t)(ny - 1) * nx : b - nx,
+                               z == 0 ? b + (nz - 1) * nxy : b - nxy};
+    R dtp = (R)0;
+#pragma unroll
+    for (int e = 0; e < 3; ++e) dtp = r_add(dtp, r_sub(p[e * nbox + behind[e]], p[e * nbox + b]));
+    const R u0 = u[b];
+    R v = r_sub(u0, r_mul(tau, r_add(dtp, w[b])));
+    v = v < (R)0 ? (R)0 : (v > (R)1 ? (R)1 : v);
+    ub[b] = r_sub(r_mul((R)2, v), u0);
+    u[b] = v;
+  }
+}
+
 // s = (u >= 1/2); flags[o + 1] = 1 if any box changed.
 template <typename R>
 __global__ void k_ms_threshold(const R* __restrict__ u, uint8_t* __restrict__ s, int64_t nbox, int32_t* flags,
@@ -177,19 +237,28 @@ int ms_run(dcm_ctx* ctx, const int32_t* count, uint8_t* s, cudaStream_t st) {
   R* ub[2] = {(R*)ctx->ms_ub, (R*)ctx->ms_ub + nbox};
   R* p[2] = {(R*)ctx->ms_p, (R*)ctx->ms_p + 3 * nbox};
   R* w = (R*)ctx->ms_w;
-  // columns of 32 x 8 boxes, cut along z so that small grids fill the chip
-  const int64_t cols = (int64_t)((nx + 31) / 32) * ((ny + 7) / 8);
-  int zc = (int)std::max<int64_t>(4, std::min<int64_t>(32, (int64_t)nz * cols / (152 * 6)));
-  const dim3 blocks((nx + 31) / 32, (ny + 7) / 8, (nz + zc - 1) / zc);
+  // columns of boxes, cut along z so that small grids fill the chip
+  constexpr bool kRow = sizeof(R) == 8;
+  constexpr int kBlock = ms_block<R>();
+  const int cx = kRow ? (int)(((int64_t)nx * ny + kBlock - 1) / kBlock) : (nx + 31) / 32, cy = kRow ? 1 : (ny + 7) / 8;
+  const int zc = (int)std::max<int64_t>(4, std::min<int64_t>(32, (int64_t)nz * cx * cy / (152 * 6 * (256 / kBlock))));
+  const dim3 blocks(cx, cy, (nz + zc - 1) / zc);
   DCM_CUDA_TRY(ctx, cudaMemsetAsync(ctx->ms_flags, 0, sizeof(int32_t) * (size_t)(outer + 2), st));
   DCM_CUDA_TRY(ctx, cudaMemsetAsync(ctx->ms_sums, 0, sizeof(unsigned long long) * 4 * (size_t)outer, st));
   for (int o = 0; o < outer; ++o) {
     DCM_LAUNCH(ctx, k_ms_sums, grid, 256, 0, st, count, s, nbox, ctx->ms_sums, ctx->ms_flags, o);
     DCM_LAUNCH(ctx, k_ms_start<R>, grid, 256, 0, st, count, s, nbox, ctx->ms_sums, ctx->ms_flags, ctx->ms_c, o, w, u,
                ub[0], p[0]);
-    for (int it = 0; it < inner; ++it)
-      DCM_LAUNCH(ctx, k_ms_step<R>, blocks, 256, 0, st, ub[it & 1], p[it & 1], w, u, ub[(it + 1) & 1], p[(it + 1) & 1],
-                 nx, ny, nz, zc, (R)kMsSigma, (R)kMsTau, (R)ctx->p.ms_nu, ctx->ms_flags, o);
+    for (int it = 0; it < inner; ++it) {
+      if (kRow && nbox >= kMsFused) {
+        DCM_LAUNCH(ctx, k_ms_dual<R>, grid, 256, 0, st, ub[0], p[0], nx, ny, nz, (R)kMsSigma, (R)ctx->p.ms_nu,
+                   ctx->ms_flags, o);
+        DCM_LAUNCH(ctx, k_ms_primal<R>, grid, 256, 0, st, p[0], w, u, ub[0], nx, ny, nz, (R)kMsTau, ctx->ms_flags, o);
+      } else {
+        DCM_LAUNCH(ctx, k_ms_step<R>, blocks, kBlock, 0, st, ub[it & 1], p[it & 1], w, u, ub[(it + 1) & 1],
+                   p[(it + 1) & 1], nx, ny, nz, zc, (R)kMsSigma, (R)kMsTau, (R)ctx->p.ms_nu, ctx->ms_flags, o);
+      }
+    }
     DCM_LAUNCH(ctx, k_ms_threshold<R>, grid, 256, 0, st, u, s, nbox, ctx->ms_flags, o);
   }
   return check_launch(ctx, "ms_segment");

@@ -132,3 +132,14 @@ def test_segmentation_validation(D):
     p = D.make_params((1, 1, 1), segmentation=1)
     with pytest.raises(D.DcmError):
         D.Batch(p, [(12.0, 12.0, 48.0)], [10])
+
+
+@pytest.mark.parametrize("nh", [(84, 85, 84), (85, 85, 84), (4, 400, 400), (33, 9, 40)])
+def test_fp64_bit_exact_on_both_sides_of_600000_boxes(D, nh):
+    """Below 600,000 boxes one kernel per iteration, blocks of 64 columns in a
+    row; above two kernels."""
+    count = noisy_counts(nh, 11, waves=1.0)
+    s, iface, T = run(D, count, nh, "fp64", 1.5, 11, 2)
+    so, io, To, _ = oracle(count, nh, 1.5, 11, 2)
+    assert T == To
+    assert np.array_equal(s, so) and np.array_equal(iface, io)
