@@ -8,10 +8,14 @@
 
 namespace dcm {
 
+// Towards zero, saturating (NaN: some integer).
+__device__ __forceinline__ int to_int(float v) { return __float2int_rz(v); }
+__device__ __forceinline__ int to_int(double v) { return __double2int_rz(v); }
+
 template <typename R>
 __device__ __forceinline__ void centre_coord(R x, R h, R inv_h, int& k, R& t) {
   R q = floor(x * inv_h - (R)0.5);
-  k = (int)fmin(fmax(q, (R)-1e9), (R)1e9);  // room for the steps below (NaN: -1e9)
+  k = min(max(to_int(q), -1000000000), 1000000000);  // room for the steps below
   if (((R)k + (R)0.5) * h > x)
     --k;
   else if (((R)k + (R)1.5) * h <= x)
