@@ -650,7 +650,7 @@ __global__ void __launch_bounds__(32 * kAdjTileWarps, 1) k_adjoint_tiles(
     const int q = __shfl_sync(full, q0, 0);
     return q < ntile ? __ldg(q < nfirst ? t.list + q : t.list + (nslot - 1 - (q - nfirst))) : -1;
   };
-  int slot = slot_of(take());
+  int slot = slot_of(first_tile());
   while (slot >= 0) {
     const int t1 = take();  // the next tile, asked for early
     const int i = __ldg(t.idx + 32 * (int64_t)slot + lane);
@@ -986,7 +986,10 @@ int lj_adjoint(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, const R* 
     if (tiled) {
       float4* rec = (float4*)ctx->adj_rec;
       TileTable tt;
-      int r0 = tile_cut<float>(ctx, tp, pos, rc, cell_start, a.g, tt, st);
+      int sms = 0;
+      DCM_CUDA_TRY(ctx, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
+      const int grid = (int)std::min<int64_t>(nwarp, sms);
+      int r0 = tile_cut<float>(ctx, tp, pos, rc, cell_start, a.g, tt, grid * kAdjTileWarps, st);
       if (r0) return r0;
       if (part) DCM_CUDA_TRY(ctx, cudaMemsetAsync(part, 0, sizeof(double) * (size_t)(2 * nt * nt * nwarp), st));
       DCM_LAUNCH(ctx, k_adj_records, (unsigned)((n + 255) / 256), 256, 0, st, n, rc, A, a.rc_max, rec);
@@ -994,11 +997,8 @@ int lj_adjoint(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, const R* 
                  ctx->blk_max + ctx->nblk);
       const int smem = kAdjTileWarps * (int)sizeof(TileSmem<AdjRec>);
       DCM_CUDA_TRY(ctx, cudaFuncSetAttribute(k_adjoint_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-      int sms = 0;
-      DCM_CUDA_TRY(ctx, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
-      DCM_LAUNCH(ctx, k_adjoint_tiles, (unsigned)std::min<int64_t>((nwarp + kAdjTileWarps - 1) / kAdjTileWarps, sms),
-                 32 * kAdjTileWarps, smem, st, pos, (const float4*)rec, cell_start, a, tp.cfg, tt, (float)(0.5 * dlde), bg,
-                 (const int32_t*)(ctx->blk_max + ctx->nblk), G, part, nwarp);
+      DCM_LAUNCH(ctx, k_adjoint_tiles, grid, 32 * kAdjTileWarps, smem, st, pos, (const float4*)rec, cell_start, a, tp.cfg,
+                 tt, (float)(0.5 * dlde), bg, (const int32_t*)(ctx->blk_max + ctx->nblk), G, part, nwarp);
       DCM_LAUNCH(ctx, k_adjoint_rest, (unsigned)std::min<int64_t>(nwarp, 4 * sms), 32 * kAdjRestWarps, 0, st, pos, rc,
                  cell_start, a, tt, A, (float)(0.5 * dlde), G, part, nwarp, bg, (const int32_t*)ctx->blk_max);
     }

@@ -37,7 +37,8 @@ namespace dcm {
 // of few tiles per warp does not end on them (300K particles, a cylinder of
 // liquid: 259 -> 246 us against full tiles alone first).  Coordinates
 // outside the box are looked for in the boundary cells, the only ones that may
-// hold them; the piece's flag says whether there are any.  NR: cell rows of a bundle, at most; the starts of the next 32
+// hold them; the piece's flag says whether there are any.  queue: tiles that the warps
+// of the next launch take by their number (first_tile), before they ask.  NR: cell rows of a bundle, at most; the starts of the next 32
 // steps are loaded while these are dealt.
 template <typename R, int NR>
 __global__ void __launch_bounds__(128) k_tile_cut(const int32_t* __restrict__ start,
@@ -45,12 +46,13 @@ __global__ void __launch_bounds__(128) k_tile_cut(const int32_t* __restrict__ st
                                                   const R* __restrict__ rc, R wide, Grid<R> g, TileCfg cfg,
                                                   int32_t* __restrict__ idx, int32_t* __restrict__ list,
                                                   int32_t* __restrict__ counters, int32_t* __restrict__ flag,
-                                                  int64_t nslot) {
+                                                  int64_t nslot, int queue) {
   const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const int piece = blockIdx.x * 4 + (threadIdx.x >> 5), b = piece / cfg.np;
   if (b >= cfg.nby * cfg.nbz) return;
+  if (piece == 0 && lane == 0) counters[kTileQueue] = queue;
   const int by = b % cfg.nby, bz = b / cfg.nby;
   const int xs = (piece - b * cfg.np) * cfg.px, xe = min(xs + cfg.px, nx);
   const int y0 = by * cfg.ry, z0 = bz * cfg.rz, nr_y = min(cfg.ry, ny - y0), nr_z = min(cfg.rz, nz - z0);
@@ -305,7 +307,7 @@ __global__ void __launch_bounds__(32 * tile_warps<R>(), 1) k_forces_tiles(
     const int t = __shfl_sync(full, t0, 0);
     return t < ntile ? __ldg(t < nfirst ? list + t : list + (nslot - 1 - (t - nfirst))) : -1;
   };
-  int slot = slot_of(take()), slot1 = slot_of(take());
+  int slot = slot_of(first_tile()), slot1 = slot_of(take());
   int i = slot >= 0 ? __ldg(idx + 32 * (int64_t)slot + lane) : -1;
   R4 pi = ldg4(pos + max(i, 0));
   R ri = rc[max(i, 0)];
@@ -385,7 +387,7 @@ __global__ void __launch_bounds__(kRestBlock, sizeof(R) == 4 ? 2 : 1) k_forces_r
   const int n = __ldg(t.counters + kTileRest);
   if (n >= rest_many<R>()) {
     constexpr int kWarps = kRestBlock / 32;
-    for (int k = blockIdx.x * kWarps + (threadIdx.x >> 5); k < n; k += gridDim.x * kWarps) {
+    for (int k = first_tile(); k < n; k += gridDim.x * kWarps) {
       const int slot = __ldg(t.rest + k);
       const int i = __ldg(t.idx + 32 * (int64_t)slot + (threadIdx.x & 31));
       double e = 0, w = 0;
@@ -498,7 +500,7 @@ bool tiles_serve(const dcm_ctx* ctx, int64_t n) {
 
 template <typename R>
 int tile_cut(dcm_ctx* ctx, const TilePlan& tp, const typename RT<R>::R4* pos, const R* rc, const int32_t* cell_start,
-             const Grid<R>& g, TileTable& t, cudaStream_t st) {
+             const Grid<R>& g, TileTable& t, int warps, cudaStream_t st) {
   t.counters = ctx->tiles;
   t.list = t.counters + kTileCounters;
   t.rest = t.list + tp.slots;
@@ -508,11 +510,11 @@ int tile_cut(dcm_ctx* ctx, const TilePlan& tp, const typename RT<R>::R4* pos, co
   DCM_CUDA_TRY(ctx, cudaMemsetAsync(t.counters, 0, kTileCounters * sizeof(int32_t), st));
   auto kc = tp.cfg.ry * tp.cfg.rz <= 4 ? k_tile_cut<R, 4> : k_tile_cut<R, 16>;
   DCM_LAUNCH(ctx, kc, (unsigned)((nb + 3) / 4), 128, 0, st, cell_start, pos, rc, (R)(1.2 * ctx->p.rc_min), g, tp.cfg,
-             t.idx, t.list, t.counters, t.outside, tp.slots);
+             t.idx, t.list, t.counters, t.outside, tp.slots, warps);
   return DCM_OK;
 }
 template int tile_cut<float>(dcm_ctx*, const TilePlan&, const float4*, const float*, const int32_t*,
-                             const Grid<float>&, TileTable&, cudaStream_t);
+                             const Grid<float>&, TileTable&, int, cudaStream_t);
 
 template <typename R>
 int tile_forces(dcm_ctx* ctx, bool typed, bool ew, int64_t n, const typename RT<R>::R4* pos, const R* rc,
@@ -520,18 +522,18 @@ int tile_forces(dcm_ctx* ctx, bool typed, bool ew, int64_t n, const typename RT<
                 cudaStream_t st) {
   const TilePlan tp = tile_plan(ctx->p, ctx->nc, n);
   if (part) DCM_CUDA_TRY(ctx, cudaMemsetAsync(part, 0, 3 * sizeof(double) * (size_t)tp.slots, st));
+  int sms = 0;
+  DCM_CUDA_TRY(ctx, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
+  constexpr int warps = tile_warps<R>(), smem = warps * (int)sizeof(TileSmem<typename RT<R>::R4>);
+  const int grid = (int)std::min<int64_t>(tp.slots, sms);
   TileTable t;
-  int r = tile_cut<R>(ctx, tp, pos, rc, cell_start, a.g, t, st);
+  int r = tile_cut<R>(ctx, tp, pos, rc, cell_start, a.g, t, grid * warps, st);
   if (r) return r;
   auto k = typed ? (ew ? k_forces_tiles<R, true, true> : k_forces_tiles<R, true, false>)
                  : (ew ? k_forces_tiles<R, false, true> : k_forces_tiles<R, false, false>);
   auto kr = typed ? (ew ? k_forces_rest<R, true, true> : k_forces_rest<R, true, false>)
                   : (ew ? k_forces_rest<R, false, true> : k_forces_rest<R, false, false>);
-  constexpr int warps = tile_warps<R>(), smem = warps * (int)sizeof(TileSmem<typename RT<R>::R4>);
   DCM_CUDA_TRY(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  int sms = 0;
-  DCM_CUDA_TRY(ctx, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
-  const unsigned grid = (unsigned)std::min<int64_t>((tp.slots + warps - 1) / warps, sms);
   DCM_LAUNCH(ctx, k, grid, 32 * warps, smem, st, pos, rc, cell_start, a, tp.cfg, t, force, part, tp.slots);
   DCM_LAUNCH(ctx, kr, (unsigned)std::min<int64_t>(tp.slots, 2 * sms), kRestBlock, 0, st, pos, rc, cell_start, a, t,
              force, part, tp.slots);

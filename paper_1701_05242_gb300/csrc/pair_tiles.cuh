@@ -78,7 +78,7 @@ struct TileTable {
 };
 template <typename R>
 int tile_cut(dcm_ctx* ctx, const TilePlan& tp, const typename RT<R>::R4* pos, const R* rc, const int32_t* cell_start,
-             const Grid<R>& g, TileTable& t, cudaStream_t st);
+             const Grid<R>& g, TileTable& t, int warps, cudaStream_t st);
 
 // First bit (from the most significant) of a nonzero word.
 __device__ __forceinline__ int first_bit(uint32_t w) {
@@ -282,6 +282,12 @@ __device__ __forceinline__ int warp_incl_sum(int v) {
   }
   return v;
 }
+
+// A warp's first tile; it asks the queue, which starts behind them, for the others.  Neighbours in the list
+// go to different SMs: a launch of few tiles took them on the SMs whose warps asked
+// first, two per warp (FP64 forces of 6,451 particles 1150 - 1550 us from run to run,
+// 760 so; mixed, 47,455 particles with cells of 3: 311 -> 171 us).
+__device__ __forceinline__ int first_tile() { return (threadIdx.x >> 5) * gridDim.x + blockIdx.x; }
 
 // Whether a tile may meet a coordinate outside the box: whether its own bundle
 // or one of those within its largest reach holds any (y, z, reach: of the lanes'

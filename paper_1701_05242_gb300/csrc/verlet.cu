@@ -314,11 +314,7 @@ __global__ void __launch_bounds__(32 * kListTileWarps, 1) k_list_tiles(
   const int lane = threadIdx.x & 31;
   const int nfirst = __ldg(t.counters + kTileFirst), ntile = nfirst + __ldg(t.counters + kTileLater);
   const bool outside = __ldg(t.counters + kTileOutside) != 0;
-  for (;;) {
-    int k = 0;
-    if (lane == 0) k = atomicAdd(t.counters + kTileQueue, 1);
-    k = __shfl_sync(full, k, 0);
-    if (k >= ntile) break;
+  for (int k = first_tile(); k < ntile;) {
     const int slot = __ldg(k < nfirst ? t.list + k : t.list + (nslot - 1 - (k - nfirst)));
     const int i = __ldg(t.idx + 32 * (int64_t)slot + lane);
     const bool active = i >= 0;
@@ -369,6 +365,8 @@ __global__ void __launch_bounds__(32 * kListTileWarps, 1) k_list_tiles(
       nimg[i] = col.kb;
       if (!col.finish()) atomicExch(flag, 1);
     }
+    if (lane == 0) k = atomicAdd(t.counters + kTileQueue, 1);
+    k = __shfl_sync(full, k, 0);
   }
 }
 
@@ -1000,17 +998,17 @@ static int list_fill(dcm_ctx* ctx, int64_t n, const typename RT<R>::R4* pos, con
     if (ctx->tiles && tp.usable && n >= kListTilesMinN) {
       float4* rec = (float4*)ctx->xbuild;
       TileTable t;
-      int r = tile_cut<float>(ctx, tp, pos, rc, ctx->cell_start, g, t, st);
+      int sms = 0;
+      DCM_CUDA_TRY(ctx, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
+      const int grid = (int)std::min<int64_t>(tp.slots, sms);
+      int r = tile_cut<float>(ctx, tp, pos, rc, ctx->cell_start, g, t, grid * kListTileWarps, st);
       if (r) return r;
       auto k = n3 ? k_list_tiles<true> : k_list_tiles<false>;
       constexpr int smem = kListTileWarps * (int)sizeof(TileSmem<float4>);
       static_assert(smem <= 227 * 1024, "one block per SM");
       DCM_CUDA_TRY(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-      int sms = 0;
-      DCM_CUDA_TRY(ctx, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
       DCM_LAUNCH(ctx, k_list_records, (unsigned)((n + 255) / 256), 256, 0, st, n, pos, rec);
-      DCM_LAUNCH(ctx, k, (unsigned)std::min<int64_t>((tp.slots + kListTileWarps - 1) / kListTileWarps, sms),
-                 32 * kListTileWarps, smem, st, rec, rc, ctx->cell_start, g, tp.cfg, t, tp.slots, rcm, skin, ctx->capw,
+      DCM_LAUNCH(ctx, k, grid, 32 * kListTileWarps, smem, st, rec, rc, ctx->cell_start, g, tp.cfg, t, tp.slots, rcm, skin, ctx->capw,
                  ctx->offw, ctx->list, ctx->nnb, ctx->nimg, ctx->lflag);
       auto kr = n3 ? k_list_rest<true> : k_list_rest<false>;
       DCM_LAUNCH(ctx, kr, (unsigned)std::min<int64_t>((tp.slots + 1) / 2, 8 * sms), 64, 0, st, pos, rc,
