@@ -11,8 +11,8 @@
 // tensor pipe 11% busy, HBM nearly idle.  Sixteen warps of 512 staged
 // candidates fill the SM's shared memory; 13 of 640 and 20 of 384 (at 96
 // registers) were slower.  Kernel times against the row walk, energies included:
-// 15.5M particles 6140 -> 4525 us, 1.0M 525 -> 426, 260K of two types 255 -> 180,
-// 260K in FP64 6000 -> 1725.
+// 15.5M particles 6140 -> 4498 us, 1.0M 525 -> 380 (cells of 0.5 x 1.5 x 1.5; cubic
+// ones 410), 260K in FP64 6000 -> 1725.
 #include <algorithm>
 #include <climits>
 #include <cmath>
