@@ -492,14 +492,14 @@ struct Walker {
   }
 };
 
-// The rows of the z-plane uz of particle `self`'s walk (walk_rows); false if
-// the plane is out of reach.
+// The rows y0 .. y1 of the z-plane uz of particle `self`'s walk (walk_rows);
+// false if the plane is out of reach.
 template <typename R, bool TYPED, bool X2, Accum M, bool NC = true, Walk MODE = Walk::kAll, bool EW = true>
 __device__ __forceinline__ bool walk_plane(const typename RT<R>::R4* __restrict__ pos,
                                            const int32_t* __restrict__ start, const Grid<R>& g,
                                            const ForceArgs<R>& a, int self, const typename RT<R>::R4& pi,
-                                           const Walker<R>& wk, int uz, int ti, const R* ushift, Acc<R>& c, Acc2& c2,
-                                           Sums<M>& S) {
+                                           const Walker<R>& wk, int uz, int y0, int y1, int ti, const R* ushift,
+                                           Acc<R>& c, Acc2& c2, Sums<M>& S) {
   constexpr bool kImg = MODE == Walk::kImagesOnly;
   const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
   const R l = g.edge, il = g.inv_edge, ilx = g.inv_edge_x;
@@ -511,7 +511,7 @@ __device__ __forceinline__ bool walk_plane(const typename RT<R>::R4* __restrict_
   int wz = uz < 0 ? uz + nz : (uz >= nz ? uz - nz : uz);
   R zi = uz >= nz ? pi.z - g.L[2] : pi.z;  // image +L: shift i
   R zsh = uz < 0 ? -g.L[2] : (R)0;          // image -L: shift j
-  for (int uy = cy - H; uy <= cy + H; ++uy) {
+  for (int uy = y0; uy <= y1; ++uy) {
     R gy = uy > cy ? (R)uy * l - pi.y : (uy < cy ? pi.y - (R)(uy + 1) * l : (R)0);
     R gyz2 = gz2 + gy * gy;
     if (gyz2 >= rc2s) continue;
@@ -571,7 +571,9 @@ __device__ __forceinline__ void walk_rows(const typename RT<R>::R4* __restrict__
                                           int ti, const R* ushift, Acc<R>& c, Acc2& c2, Sums<M>& S) {
   const Walker<R> wk(g, pi, rci);
   for (int uz = wk.cz - wk.H; uz <= wk.cz + wk.H; ++uz) {
-    if (!walk_plane<R, TYPED, X2, M, NC, MODE, EW>(pos, start, g, a, self, pi, wk, uz, ti, ushift, c, c2, S)) continue;
+    if (!walk_plane<R, TYPED, X2, M, NC, MODE, EW>(pos, start, g, a, self, pi, wk, uz, wk.cy - wk.H, wk.cy + wk.H, ti,
+                                                   ushift, c, c2, S))
+      continue;
     if constexpr (plane_form(M)) flush_partials<M, R, X2, EW>(c, c2, S);
   }
 }
@@ -702,12 +704,13 @@ __device__ __forceinline__ typename RT<R>::R4 force_one(const typename RT<R>::R4
 }
 
 // Force, energy and virial of particle i (in: whether there is one) with 16
-// lanes, by a whole warp for its two half-warps' particles: each lane walks one
-// z-plane of the stencil (or every 16th, where the cells are fine).  FP32: the
+// lanes, by a whole warp for its two half-warps' particles.  FP32: each lane walks
+// one z-plane of the stencil (or every 16th, where the cells are fine), and the
 // planes' partial sums are then added in the order of the planes with the
 // compensation of the plane-Kahan form, so the results are bit for bit those of
-// force_one in that form; FP64: the lanes' sums are added in a fixed tree.  All 16
-// lanes return the results.
+// force_one in that form.  FP64: the lanes take the stencil's rows in turn (five or
+// nine planes would leave half of the lanes idle, and the FP64 units are what counts),
+// and their sums are added in a fixed tree.  All 16 lanes return the results.
 template <typename R, bool TYPED, bool EW>
 __device__ __forceinline__ typename RT<R>::R4 force_planes(const typename RT<R>::R4* __restrict__ pos,
                                                            const int32_t* __restrict__ start, const ForceArgs<R>& a,
@@ -734,7 +737,8 @@ __device__ __forceinline__ typename RT<R>::R4 force_planes(const typename RT<R>:
       const int q = q0 + sub;
       c2.fx = c2.fy = c2.fz = c2.en = c2.vir = make_float2(0.f, 0.f);
       const bool reached = q < np && walk_plane<R, TYPED, true, M, true, Walk::kAll, EW>(
-                                         pos, start, a.g, a, i, pi, wk, wk.cz - wk.H + q, ti, k8, c, c2, S);
+                                         pos, start, a.g, a, i, pi, wk, wk.cz - wk.H + q, wk.cy - wk.H, wk.cy + wk.H, ti, k8, c, c2,
+                                         S);
       __syncwarp();
       const float v[5] = {c2.fx.x + c2.fx.y, c2.fy.x + c2.fy.y, c2.fz.x + c2.fz.y, c2.en.x + c2.en.y,
                           c2.vir.x + c2.vir.y};
@@ -749,9 +753,11 @@ __device__ __forceinline__ typename RT<R>::R4 force_planes(const typename RT<R>:
     }
     for (int o = kPlaneLanes / 2; o > 0; o >>= 1) c2.np += __shfl_xor_sync(full, c2.np, o);
   } else {
-    for (int q = sub; q < np; q += kPlaneLanes)
-      walk_plane<R, TYPED, false, M, true, Walk::kAll, true>(pos, start, a.g, a, i, pi, wk, wk.cz - wk.H + q, ti, k8, c,
-                                                            c2, S);
+    for (int q = sub; q < np * np; q += kPlaneLanes) {  // row q of the stencil
+      const int uy = wk.cy - wk.H + q % np;
+      walk_plane<R, TYPED, false, M, true, Walk::kAll, true>(pos, start, a.g, a, i, pi, wk, wk.cz - wk.H + q / np, uy, uy,
+                                                            ti, k8, c, c2, S);
+    }
     __syncwarp();
 #pragma unroll
     for (int o = kPlaneLanes / 2; o > 0; o >>= 1) {

@@ -367,11 +367,11 @@ __global__ void __launch_bounds__(32 * tile_warps<R>(), 1) k_forces_tiles(
 
 // The tiles that the filter does not serve, by the row walk.  Few of them: a
 // block per tile, 16 lanes per particle (force_planes), because such a launch lasts
-// as long as its longest walk (FP64, a quarter of 7,738 particles: 1180 us with a
-// thread per particle, about 500 so).  Many of them (coordinates outside the box all
-// over it): a warp per tile, a thread per particle, which keeps more lanes busy (all
-// 8,900 tiles of 260K particles: 680 us with 16 lanes, 260 with one; FP64, 2,000
-// tiles: 4700 and 2000).
+// as long as its longest walk (FP64 forces of 7,738 particles in a box of 4.25 rc_max,
+// a quarter left over: 2480 us with a thread per particle, 1430 so).  Many of them
+// (coordinates outside the box all over it): a warp per tile, a thread per particle,
+// which keeps more lanes busy (all 8,900 tiles of 260K particles: 680 us with 16 lanes,
+// 260 with one; the call with 2,000 tiles in FP64: 3430 and 2770).
 constexpr int kRestBlock = 32 * kPlaneLanes;
 template <typename R>
 constexpr int rest_many() { return sizeof(R) == 4 ? 1500 : 600; }
